@@ -7,6 +7,7 @@
 #include <stdio.h>
 
 #include <string>
+#include <vector>
 
 #include "../../include/cagra_gb.h"
 
@@ -72,6 +73,22 @@ int exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaSt
 int radix_sort_pairs(const uint32_t* keys_in, const int32_t* vals_in,
                      uint32_t* keys_out, int32_t* vals_out, int64_t n, int bits,
                      cudaStream_t s);
+
+// Stream-ordered scratch, given back when it goes out of scope.
+struct Scratch {
+  std::vector<void*> ptrs;
+  cudaStream_t s;
+  explicit Scratch(cudaStream_t st) : s(st) {}
+  template <typename T>
+  cudaError_t get(T** p, size_t n) {
+    cudaError_t e = cudaMallocAsync((void**)p, sizeof(T) * (n > 0 ? n : 1), s);
+    if (e == cudaSuccess) ptrs.push_back((void*)*p);
+    return e;
+  }
+  ~Scratch() {
+    for (void* p : ptrs) cudaFreeAsync(p, s);
+  }
+};
 
 // ---------------------------------------------------------------------------
 // Device helpers

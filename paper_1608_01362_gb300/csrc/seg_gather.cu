@@ -1,7 +1,7 @@
 // Flagged-edge segment gather: plan construction and the kernel.
 #include <algorithm>
 
-#include "seg_gather.cuh"
+#include "staged_stream.cuh"
 
 namespace cg {
 namespace {
@@ -59,12 +59,11 @@ __global__ void export_col_kernel(const uint32_t* __restrict__ colf,
 __global__ void open_row_kernel(const int32_t* __restrict__ rp,
                                 const int64_t* __restrict__ row_base,
                                 const int64_t* __restrict__ edge_base,
-                                const int64_t* __restrict__ chunk_base, int k, int m, int chunk_a,
-                                int chunk_b, int64_t nchunks, int32_t* __restrict__ open_row) {
+                                const int64_t* __restrict__ chunk_base, int k, int64_t size,
+                                int64_t nchunks, int32_t* __restrict__ open_row) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nchunks;
        c += (int64_t)gridDim.x * blockDim.x) {
     const int s = last_le(chunk_base, k + 1, c);
-    const int64_t size = s < m ? chunk_a : chunk_b;
     const int64_t e0 = edge_base[s] + (c - chunk_base[s]) * size;
     const int64_t e = min(e0 + size, edge_base[s + 1]) - 1;  // the chunk's last edge
     int64_t lo = row_base[s], hi = row_base[s + 1];  // last row with rp[row] <= e
@@ -110,17 +109,17 @@ __global__ void seg_fixup_kernel(const int4* __restrict__ pieces, int64_t npiece
   }
 }
 
-// Subgraph row of each chunk's first edge (segments [0, m) use chunks of
-// chunk_a edges, the others chunks of chunk_b).
+// Subgraph row of each chunk's first edge (chunks of `size` edges; the staged
+// segments have none).
 __global__ void first_row_kernel(const int32_t* __restrict__ rp,
                                  const int64_t* __restrict__ row_base,
                                  const int64_t* __restrict__ edge_base,
-                                 const int64_t* __restrict__ chunk_base, int k, int m, int chunk_a,
-                                 int chunk_b, int64_t nchunks, int32_t* __restrict__ first_row) {
+                                 const int64_t* __restrict__ chunk_base, int k, int64_t size,
+                                 int64_t nchunks, int32_t* __restrict__ first_row) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nchunks;
        c += (int64_t)gridDim.x * blockDim.x) {
     const int s = last_le(chunk_base, k + 1, c);
-    const int64_t e = edge_base[s] + (c - chunk_base[s]) * (s < m ? chunk_a : chunk_b);
+    const int64_t e = edge_base[s] + (c - chunk_base[s]) * size;
     int64_t lo = row_base[s], hi = row_base[s + 1];  // last row with rp[row] <= e
     while (lo < hi) {
       const int64_t mid = (lo + hi) >> 1;
@@ -254,195 +253,24 @@ seg_gather_kernel(const uint32_t* __restrict__ colf, const typename Op::T* __res
   }
 }
 
-// Copy n values into shared memory with many independent loads in flight per
-// thread (16-byte loads when the source is 16-byte aligned), so staging a
-// table costs a few memory round trips rather than one per element.
-// nt: threads taking part (tid in [0, nt)).
+// Copy n values into shared memory by threads [0, nt): 16-byte asynchronous
+// copies where the source is 16-byte aligned (all of a thread's copies are in
+// flight at once and pass no register), 4-byte ones otherwise.  The caller's
+// next barrier publishes the table.
 template <typename T>
 __device__ __forceinline__ void stage_table(const T* __restrict__ src, int n, T* dst, int tid,
                                             int nt) {
   static_assert(sizeof(T) == 4, "4-byte values");
-  if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-    const int n4 = n >> 2;
-    const uint4* s4 = reinterpret_cast<const uint4*>(src);
-    uint4* d4 = reinterpret_cast<uint4*>(dst);
-    for (int b = 0; b < n4; b += nt * 4) {
-      uint4 r[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = b + u * nt + tid;
-        if (i < n4) r[u] = __ldg(s4 + i);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = b + u * nt + tid;
-        if (i < n4) d4[i] = r[u];
-      }
-    }
-    for (int i = (n4 << 2) + tid; i < n; i += nt) dst[i] = src[i];
-  } else {
-    for (int b = 0; b < n; b += nt * 8) {
-      T r[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int i = b + u * nt + tid;
-        if (i < n) r[u] = __ldg(src + i);
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int i = b + u * nt + tid;
-        if (i < n) dst[i] = r[u];
-      }
-    }
-  }
-}
-
-// Staged chunk stream, per 512-edge chunk (1168 bytes):
-//   [0, 1024)     512 uint16 segment-local source indices, lane l's 16 edges
-//                 at bytes [32l, 32l + 32)
-//   [1024, 1152)  32 uint32, lane l's: bits 0-15 its row-end mask (bit u:
-//                 edge u ends a row), bits 16-31 the row ends in lanes before l
-//   [1152, 1156)  int32 subgraph row of the chunk's first edge
-constexpr int kStagedIPL = 16;
-constexpr int kStagedChunk = 32 * kStagedIPL;  // 512 edges
-constexpr int kStagedChunkBytes = 2 * kStagedChunk + 64 + 64 + 16;  // 1168
-
-// One warp per staged chunk: pack its 512 edges, the lanes' row-end masks and
-// their exclusive prefix, and the chunk's first subgraph row.
-__global__ void staged_fill_kernel(const uint32_t* __restrict__ colf,
-                                   const int64_t* __restrict__ seg_chunk,
-                                   const int64_t* __restrict__ seg_cstart,
-                                   const int32_t* __restrict__ seg_E,
-                                   const int32_t* __restrict__ first_row, int m,
-                                   int64_t nchunks_a, uint8_t* __restrict__ cs) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nchunks_a;
-       c += nw) {
-    const int s = last_le(seg_chunk, m + 1, c);
-    const int64_t e_begin = (c - seg_chunk[s]) * kStagedChunk + lane * kStagedIPL;
-    uint32_t packed[kStagedIPL / 2];
-    uint32_t fl = 0;
-#pragma unroll
-    for (int u = 0; u < kStagedIPL; ++u) {
-      const int64_t e = e_begin + u;
-      uint32_t idx = 0;
-      if (e < seg_E[s]) {
-        const uint32_t wv = colf[seg_cstart[s] + e];
-        idx = wv & 0xFFFFu;  // segment-local index (< 65536 for staged segments)
-        fl |= (wv >> 31) << u;
-      }
-      if (u & 1) packed[u >> 1] |= idx << 16; else packed[u >> 1] = idx;
-    }
-    const int F = __popc(fl);
-    int incl = F;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    uint8_t* base = cs + c * kStagedChunkBytes;
-    uint4* dst = reinterpret_cast<uint4*>(base + lane * 32);
-    dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-    dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
-    reinterpret_cast<uint32_t*>(base + 2 * kStagedChunk)[lane] =
-        (fl & 0xFFFFu) | ((uint32_t)(incl - F) << 16);
-    if (lane == 0) {
-      int32_t* tail = reinterpret_cast<int32_t*>(base + 2 * kStagedChunk + 128);
-      tail[0] = first_row[c];
-      tail[1] = tail[2] = tail[3] = 0;
-    }
-  }
-}
-
-// One staged chunk whose stream words are loaded: pk (16 indices), fl (row
-// ends), pre (row ends before this lane), frow (first subgraph row).
-template <class Op>
-__device__ __forceinline__ void staged_chunk(const uint32_t (&pk)[8], uint32_t fl, int pre,
-                                             int n, int32_t c, int32_t frow,
-                                             const typename Op::T* tab, uint32_t tmax,
-                                             typename Op::T* __restrict__ out,
-                                             typename Op::T* __restrict__ carry) {
-  using T = typename Op::T;
-  constexpr int IPL = kStagedIPL;
-  constexpr int CHUNK = kStagedChunk;
-  const int lane = threadIdx.x & 31;
-  T v[IPL];
-  const uint32_t tmax2 = tmax | (tmax << 16);  // both 16-bit halves clamped at once
-  if (n == CHUNK) {
-#pragma unroll
-    for (int u = 0; u < IPL; u += 2) {
-      const uint32_t q = __vminu2(pk[u >> 1], tmax2);
-      v[u] = tab[q & 0xFFFFu];
-      v[u + 1] = tab[q >> 16];
-    }
-  } else {  // a segment's last chunk: lanes past its end hold nothing
-    const int nl = n - lane * IPL;
-#pragma unroll
-    for (int u = 0; u < IPL; u += 2) {
-      const uint32_t q = __vminu2(pk[u >> 1], tmax2);
-      v[u] = u < nl ? tab[q & 0xFFFFu] : Op::identity();
-      v[u + 1] = u + 1 < nl ? tab[q >> 16] : Op::identity();
-    }
-    fl &= nl >= IPL ? 0xFFFFu : (nl <= 0 ? 0u : ((1u << nl) - 1u));
-  }
-  const int F = __popc(fl);
-  const int32_t row0 = frow + pre;
-  // sequential fold; rows that start and end in this lane are final
-  T acc = Op::identity(), first_val = Op::identity();
-  int nf = 0;
-#pragma unroll
-  for (int u = 0; u < IPL; ++u) {
-    acc = Op::op(acc, v[u]);
-    if (fl & (1u << u)) {
-      if (nf == 0)
-        first_val = acc;
-      else
-        out[row0 + nf] = acc;
-      ++nf;
-      acc = Op::identity();
-    }
-  }
-  // the part of each lane's first row held by earlier lanes: one exchange
-  // when every lane ends a row, a segmented scan otherwise
-  T S = acc;
-  if (!__all_sync(0xffffffffu, F > 0)) {
-    int h = F > 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const T y = __shfl_up_sync(0xffffffffu, S, o);
-      const int g = __shfl_up_sync(0xffffffffu, h, o);
-      if (lane >= o) {
-        if (!h) S = Op::op(y, S);
-        h |= g;
-      }
-    }
-  }
-  const T P = __shfl_up_sync(0xffffffffu, S, 1);
-  if (F > 0) out[row0] = lane > 0 ? Op::op(P, first_val) : first_val;
-  // the row open at the chunk's end (completed by the carry pieces)
-  const uint32_t lf = __shfl_sync(0xffffffffu, fl, (n - 1) / IPL);
-  if (lane == 31 && !((lf >> ((n - 1) % IPL)) & 1u)) carry[c] = S;
-}
-
-// Bulk prefetch of [p, p + bytes) into L2 (TMA; p and bytes 16-byte aligned).
-__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void staged_load(const uint8_t* __restrict__ cs, int32_t c,
-                                            uint32_t (&pk)[8], uint32_t& fl, int& pre,
-                                            int32_t& frow) {
-  const int lane = threadIdx.x & 31;
-  const uint8_t* base = cs + (int64_t)c * kStagedChunkBytes;
-  const uint4 qa = __ldcs(reinterpret_cast<const uint4*>(base + lane * 32));
-  const uint4 qb = __ldcs(reinterpret_cast<const uint4*>(base + lane * 32 + 16));
-  const uint32_t w = __ldcs(reinterpret_cast<const unsigned*>(base + 2 * kStagedChunk) + lane);
-  fl = w & 0xFFFFu;
-  pre = (int)(w >> 16);
-  frow = __ldcs(reinterpret_cast<const int32_t*>(base + 2 * kStagedChunk + 128));
-  pk[0] = qa.x; pk[1] = qa.y; pk[2] = qa.z; pk[3] = qa.w;
-  pk[4] = qb.x; pk[5] = qb.y; pk[6] = qb.z; pk[7] = qb.w;
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  const int n4 = (reinterpret_cast<uintptr_t>(src) & 15) == 0 ? n >> 2 : 0;
+  for (int i = tid; i < n4; i += nt)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 16 * i),
+                 "l"(src + 4 * i)
+                 : "memory");
+  for (int i = (n4 << 2) + tid; i < n; i += nt)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4 * i), "l"(src + i)
+                 : "memory");
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // Barrier among threads [0, nt) of the block: the whole block, or named
@@ -454,74 +282,86 @@ __device__ __forceinline__ void group_sync(int nt) {
     asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
 }
 
+// What the staged schedule's blocks share: block b owns tasks
+// [blk_task[b], blk_task[b+1]) (equal stretches of the stream); next[b] of
+// them have been taken.
+struct StagedShare {
+  const int32_t* blk_task;  // [grid+1]
+  unsigned* next;           // [grid]
+  const int32_t* seg_lo;
+  const int32_t* seg_tab;
+  int m;                    // the staged segments are [0, m)
+};
+struct StagedSlots {  // a block's shared words
+  int32_t lo, hi;
+  unsigned fullest;
+};
+
+constexpr int kStealMin = 64;  // a range with fewer tasks left is not worth a table copy
+
 // The staged schedule, run by threads [0, nt) of a block: segments [0, m)
-// are read from a shared-memory copy of their source values.  Work pieces
-// of consecutive block-groups (nt/32 chunks each; at most `piece`, shrinking
-// towards the end) are handed out in increasing order by an atomic counter
-// of block-groups: a block's groups only move forward (so it stages each
-// segment's table at most once) and a slow block simply takes fewer pieces.
-// A warp's chunk is 512 edges of the compressed stream (lane l holds 16);
-// while it works on one chunk the TMA unit prefetches its next one into L2.
+// are read from a shared-memory copy of their source values.  A block works
+// through its own range of tasks, which meets one or two segments, half of
+// what is left at a time; when it runs dry it takes half of what is left of
+// the fullest range.  (The earlier schedule handed out small pieces of all
+// the tasks in order, so every block met nearly every segment: 31 table
+// copies per block on RMAT-25, each as long as 1.8 us of L2 reads at 64
+// bytes per cycle and SM, and two barriers per piece.)
 template <class Op>
 __device__ __forceinline__ void staged_pieces(
-    const uint8_t* __restrict__ cs, const typename Op::T* __restrict__ x,
-    const int32_t* __restrict__ seg_E, const int64_t* __restrict__ seg_chunk,
-    const int32_t* __restrict__ seg_ctile, const int32_t* __restrict__ seg_lo,
-    const int32_t* __restrict__ seg_tab, int32_t ct_end, int32_t piece,
-    unsigned* __restrict__ next_piece, typename Op::T* __restrict__ out,
-    typename Op::T* __restrict__ carry, typename Op::T* tab, int nt, int32_t* s_piece,
-    int32_t* s_size) {
+    const StagedTasks& q, const StagedShare& sh, const typename Op::T* __restrict__ x,
+    typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry, typename Op::T* tab,
+    int nt, StagedSlots* slots) {
   using T = typename Op::T;
-  constexpr int CHUNK = kStagedChunk;
-  const int warps = nt >> 5;
-  const int tid = threadIdx.x, w = tid >> 5;
-  int s = 0;
-  int32_t Es = 0, cbase = 0, ctbase = 0, ctnext = -1;
-  uint32_t tmax = 0;
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  int s = -1;              // the segment in the table
+  int v = (int)blockIdx.x;  // the range being worked on
+  if (tid == 0) tab[q.pad] = Op::identity();  // the first table's barrier publishes it
 
   for (;;) {
-    group_sync(nt);  // everyone is done with the previous piece's s_piece
+    group_sync(nt);  // everyone is done with the previous piece's slots
     if (tid == 0) {
-      // guided self-scheduling: a piece is the remaining block-groups over
-      // twice the grid, at most `piece` and at least one, so the last
-      // pieces are small and the blocks finish together
-      const int32_t cur = (int32_t)*(volatile unsigned*)next_piece;
-      int32_t sz = (ct_end - cur) / (2 * (int32_t)gridDim.x);
-      sz = sz < 1 ? 1 : (sz > piece ? piece : sz);
-      *s_piece = (int32_t)atomicAdd(next_piece, (unsigned)sz);
-      *s_size = sz;
+      const int32_t b0 = sh.blk_task[v], n = sh.blk_task[v + 1] - b0;
+      const int32_t taken = (int32_t)*(volatile unsigned*)(sh.next + v);
+      const int32_t sz = max((n - taken) / 2, kStealMin);
+      const int32_t lo = taken < n ? (int32_t)atomicAdd(sh.next + v, (unsigned)sz) : n;
+      slots->lo = b0 + min(lo, n);
+      slots->hi = b0 + min(lo + sz, n);
+      slots->fullest = 0u;
     }
     group_sync(nt);
-    const int32_t my_lo = *s_piece;
-    if (my_lo >= ct_end) break;
-    const int32_t my_hi = my_lo + *s_size < ct_end ? my_lo + *s_size : ct_end;
-    for (int32_t ct = my_lo; ct < my_hi;) {
-      if (ct >= ctnext) {  // a new segment (uniform across the group)
-        while (ct >= seg_ctile[s + 1]) ++s;
-        Es = seg_E[s];
-        cbase = (int32_t)seg_chunk[s];
-        ctbase = seg_ctile[s];
-        ctnext = seg_ctile[s + 1];
-        const int32_t lo = seg_lo[s], tn = seg_tab[s];
-        tmax = tn > 0 ? (uint32_t)(tn - 1) : 0u;
+    int32_t t = slots->lo;
+    const int32_t hi = slots->hi;
+    if (t >= hi) {  // this range is done: find the fullest one
+      for (int b = tid; b < (int)gridDim.x; b += nt) {
+        const int32_t left = sh.blk_task[b + 1] - sh.blk_task[b] -
+                             (int32_t)*(volatile unsigned*)(sh.next + b);
+        if (left >= kStealMin)
+          atomicMax(&slots->fullest, ((unsigned)min(left, 0x1FFFFF) << 11) | (unsigned)b);
+      }
+      group_sync(nt);
+      if (slots->fullest == 0u) break;
+      v = (int)(slots->fullest & 0x7FFu);
+      continue;
+    }
+    while (t < hi) {
+      int sn = 0;  // the segment of task t: segments whose tasks all precede it
+      for (int i = 0; i < sh.m; i += 32) {
+        const bool before = i + lane < sh.m && __ldg(q.seg_task + i + lane + 1) <= t;
+        const unsigned bal = __ballot_sync(0xffffffffu, before);
+        sn += __popc(bal);
+        if (bal != 0xffffffffu) break;
+      }
+      const int32_t te = __ldg(q.seg_task + sn + 1);
+      if (sn != s) {
+        s = sn;
         group_sync(nt);  // every warp is done reading the previous table
-        stage_table<T>(x + lo, tn, tab, tid, nt);
+        stage_table<T>(x + sh.seg_lo[s], sh.seg_tab[s], tab, tid, nt);
         group_sync(nt);
       }
-      const int32_t j = (ct - ctbase) * warps + w;
-      if (j * CHUNK < Es) {  // warp-uniform
-        const int32_t c = cbase + j;
-        // ask the TMA unit to pull this warp's next chunk into L2 meanwhile
-        if ((threadIdx.x & 31) == 0 && ct + 1 < my_hi && (j + warps) * CHUNK < Es)
-          prefetch_l2(cs + (int64_t)(c + warps) * kStagedChunkBytes, kStagedChunkBytes);
-        uint32_t pk[8], fl;
-        int pre;
-        int32_t frow;
-        staged_load(cs, c, pk, fl, pre, frow);
-        staged_chunk<Op>(pk, fl, pre, Es - j * CHUNK < CHUNK ? Es - j * CHUNK : CHUNK, c, frow,
-                         tab, tmax, out, carry);
-      }
-      ++ct;
+      const int32_t e = min(hi, te);
+      staged_run<Op>(q, t, e, w, nt >> 5, tab, out, carry);
+      t = e;
     }
   }
 }
@@ -529,18 +369,12 @@ __device__ __forceinline__ void staged_pieces(
 // The staged launch: every thread of the block runs the staged schedule.
 template <class Op, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
-staged_gather_kernel(const uint8_t* __restrict__ cs, const typename Op::T* __restrict__ x,
-                     const int32_t* __restrict__ seg_E, const int64_t* __restrict__ seg_chunk,
-                     const int32_t* __restrict__ seg_ctile, const int32_t* __restrict__ seg_lo,
-                     const int32_t* __restrict__ seg_tab, int32_t ct_end, int32_t piece,
-                     unsigned* __restrict__ next_piece, typename Op::T* __restrict__ out,
-                     typename Op::T* __restrict__ carry) {
+staged_gather_kernel(StagedTasks q, StagedShare sh, const typename Op::T* __restrict__ x,
+                     typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int32_t s_piece, s_size;
-  staged_pieces<Op>(cs, x, seg_E, seg_chunk, seg_ctile, seg_lo, seg_tab, ct_end, piece,
-                    next_piece, out, carry, reinterpret_cast<T*>(smem_raw), THREADS, &s_piece,
-                    &s_size);
+  __shared__ StagedSlots slots;
+  staged_pieces<Op>(q, sh, x, out, carry, reinterpret_cast<T*>(smem_raw), THREADS, &slots);
 }
 
 // The segment-affine staged launch (the nested form of two-level segmenting:
@@ -548,44 +382,31 @@ staged_gather_kernel(const uint8_t* __restrict__ cs, const typename Op::T* __res
 // with random L2 reads, cut into shared-memory-sized segments).  Each block
 // takes whole segments of [m, m2) from a counter, in order (heaviest first
 // after clustering), stages the segment's table once and streams all its
-// chunks with every warp; low-degree segments thus pay one table copy each
+// tasks with every warp; low-degree segments thus pay one table copy each
 // instead of one per block.
 template <class Op>
 __global__ void __launch_bounds__(1024, 1)
-affine_gather_kernel(const uint8_t* __restrict__ cs, const typename Op::T* __restrict__ x,
-                     const int32_t* __restrict__ seg_E, const int64_t* __restrict__ seg_chunk,
+affine_gather_kernel(StagedTasks q, const typename Op::T* __restrict__ x,
                      const int32_t* __restrict__ seg_lo, const int32_t* __restrict__ seg_tab,
                      int m, int m2, unsigned* __restrict__ next_seg,
                      typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   using T = typename Op::T;
-  constexpr int CHUNK = kStagedChunk;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
   __shared__ int32_t s_seg;
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, w = tid >> 5;
+  if (tid == 0) tab[q.pad] = Op::identity();
   for (;;) {
     __syncthreads();  // every warp is done with the previous table and s_seg
     if (tid == 0) s_seg = m + (int32_t)atomicAdd(next_seg, 1u);
     __syncthreads();
     const int s = s_seg;
     if (s >= m2) break;
-    const int32_t Es = seg_E[s], cbase = (int32_t)seg_chunk[s], tn = seg_tab[s];
-    const int32_t nch = (Es + CHUNK - 1) / CHUNK;
-    if (nch == 0) continue;
-    stage_table<T>(x + seg_lo[s], tn, tab, tid, 1024);
+    const int32_t tb = q.seg_task[s], te = q.seg_task[s + 1];
+    if (tb == te) continue;
+    stage_table<T>(x + seg_lo[s], seg_tab[s], tab, tid, 1024);
     __syncthreads();
-    const uint32_t tmax = tn > 0 ? (uint32_t)(tn - 1) : 0u;
-    for (int32_t j = w; j < nch; j += 32) {
-      const int32_t c = cbase + j;
-      if (lane == 0 && j + 32 < nch)
-        prefetch_l2(cs + (int64_t)(c + 32) * kStagedChunkBytes, kStagedChunkBytes);
-      uint32_t pk[8], fl;
-      int pre;
-      int32_t frow;
-      staged_load(cs, c, pk, fl, pre, frow);
-      staged_chunk<Op>(pk, fl, pre, Es - j * CHUNK < CHUNK ? Es - j * CHUNK : CHUNK, c, frow, tab,
-                       tmax, out, carry);
-    }
+    staged_run<Op>(q, tb, te, w, 32, tab, out, carry);
   }
 }
 
@@ -641,24 +462,36 @@ __device__ __forceinline__ void cached_queue(
 // shared memory, so the two kinds of lookup proceed side by side.
 template <class Op>
 __global__ void __launch_bounds__(1024, 1)
-overlap_gather_kernel(const uint8_t* __restrict__ cs, const uint32_t* __restrict__ colf,
+overlap_gather_kernel(StagedTasks q, StagedShare sh, const uint32_t* __restrict__ colf,
                       const typename Op::T* __restrict__ x, int32_t nx,
                       const int32_t* __restrict__ first_row,
                       const int64_t* __restrict__ seg_cstart, const int32_t* __restrict__ seg_E,
-                      const int64_t* __restrict__ seg_chunk,
-                      const int32_t* __restrict__ seg_ctile, const int32_t* __restrict__ seg_lo,
-                      const int32_t* __restrict__ seg_tab, int m, int k, int32_t ct_end,
-                      int32_t piece, int staged_threads, unsigned* __restrict__ counters,
+                      const int64_t* __restrict__ seg_chunk, const int32_t* __restrict__ seg_lo,
+                      int m, int k, int staged_threads, unsigned* __restrict__ next_chunk,
                       typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int32_t s_piece, s_size;
+  __shared__ StagedSlots slots;
   if ((int)threadIdx.x < staged_threads)
-    staged_pieces<Op>(cs, x, seg_E, seg_chunk, seg_ctile, seg_lo, seg_tab, ct_end, piece,
-                      counters, out, carry, reinterpret_cast<T*>(smem_raw), staged_threads,
-                      &s_piece, &s_size);
-  cached_queue<Op>(colf, x, nx, first_row, seg_cstart, seg_E, seg_chunk, seg_lo, m, k,
-                   counters + 1, out, carry);
+    staged_pieces<Op>(q, sh, x, out, carry, reinterpret_cast<T*>(smem_raw), staged_threads, &slots);
+  cached_queue<Op>(colf, x, nx, first_row, seg_cstart, seg_E, seg_chunk, seg_lo, m, k, next_chunk,
+                   out, carry);
+}
+
+// Block b's first task: equal stretches of the stream.
+__global__ void staged_share_kernel(const uint4* __restrict__ desc, int32_t ntasks, int grid,
+                                    int32_t* __restrict__ blk_task) {
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b <= grid; b += gridDim.x * blockDim.x) {
+    const uint4 e = desc[ntasks - 1];
+    const int64_t total = (int64_t)e.x + (e.y >> 16);
+    const int64_t want = total * b / grid;
+    int32_t lo = 0, hi = ntasks;
+    while (lo < hi) {
+      const int32_t mid = (lo + hi) >> 1;
+      if ((int64_t)desc[mid].x < want) lo = mid + 1; else hi = mid;
+    }
+    blk_task[b] = b == grid ? ntasks : lo;
+  }
 }
 
 }  // namespace
@@ -753,7 +586,8 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   CG_TRY(device_info(&di));
   const int cap = seg_table_capacity(ctas_per_sm);
   int tab = tab_vertices < 0 ? cap : std::min(tab_vertices, cap);
-  tab = std::min(tab, 65536) & ~3;  // staged sources are 16-bit segment-local indices
+  // staged sources are 16-bit segment-local indices, one of them the identity's
+  tab = std::min(tab, 65532) & ~3;
   const int k = p->k;
   // staged prefix: leading segments that fit the table and carry enough
   // edges (>= 4 per source) for staging them in shared memory to pay
@@ -796,38 +630,36 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
     return CG_ERR_INVALID_ARG;
   }
   p->overlap = (m > 0 && cached_edges) ? p->overlap_request : 0;
-  const int chunk_a = kStagedChunk, chunk_b = kCachedChunk;
-  const int warps_a = p->overlap > 0 ? 32 - p->overlap : threads / 32, warps_b = 1024 / 32;
+  const int warps_b = 1024 / 32;
+  const int tab_cap = (int)((tabmax + 3) & ~3LL);
+  // chunks of the segments read through L1/L2
   std::vector<int64_t> chunk(k + 1, 0);
   std::vector<int32_t> ctile(k + 1, 0), tn(k > 0 ? k : 1, 0);
   for (int q = 0; q < k; ++q) {
-    const int64_t Eq = p->edge_base[q + 1] - p->edge_base[q];
-    const int64_t nch = ceil_div(Eq, q < m2 ? chunk_a : chunk_b);
-    chunk[q + 1] = chunk[q] + nch;
-    // block-groups of the sweeping launches (none for the segment-affine segments)
-    ctile[q + 1] = ctile[q] + (q < m ? (int32_t)ceil_div(nch, warps_a)
-                                     : q < m2 ? 0 : (int32_t)ceil_div(nch, warps_b));
+    chunk[q + 1] =
+        chunk[q] + (q < m2 ? 0 : ceil_div(p->edge_base[q + 1] - p->edge_base[q], kCachedChunk));
     tn[q] = q < m2 ? (int32_t)(p->src_bounds[q + 1] - p->src_bounds[q]) : 0;
   }
-  const int64_t nchunks = chunk[k];
-  if (nchunks > p->chunk_cap) {
+  const int64_t ncached = chunk[k];
+  // the staged segments' tasks; their extra carries follow the chunks' carries
+  std::vector<int32_t> extra_row;
+  CG_TRY(staged_build(p, m2, tab_cap, ncached, &extra_row, s));
+  const int64_t ncarry = ncached + (int64_t)extra_row.size();
+  for (int q = 0; q < k; ++q)  // block-groups of the L1/L2 launch
+    ctile[q + 1] = ctile[q] + (int32_t)ceil_div(chunk[q + 1] - chunk[q], warps_b);
+  if (ncached > p->chunk_cap) {
     cudaFree(p->first_row);
-    cudaFree(p->carry);
     p->first_row = nullptr;
-    p->carry = nullptr;
     p->chunk_cap = 0;
-    const size_t nc = (size_t)(nchunks > 0 ? nchunks : 1);
-    CG_CUDA(cudaMalloc((void**)&p->first_row, sizeof(int32_t) * nc));
-    CG_CUDA(cudaMalloc(&p->carry, sizeof(int32_t) * nc));
-    p->chunk_cap = nchunks;
+    CG_CUDA(cudaMalloc((void**)&p->first_row, sizeof(int32_t) * (size_t)ncached));
+    p->chunk_cap = ncached;
   }
-  const int64_t cs_bytes = chunk[m2] * kStagedChunkBytes;
-  if (cs_bytes > p->cs_cap) {
-    cudaFree(p->cs);
-    p->cs = nullptr;
-    p->cs_cap = 0;
-    CG_CUDA(cudaMalloc((void**)&p->cs, (size_t)cs_bytes));
-    p->cs_cap = cs_bytes;
+  if (ncarry > p->carry_cap) {
+    cudaFree(p->carry);
+    p->carry = nullptr;
+    p->carry_cap = 0;
+    CG_CUDA(cudaMalloc(&p->carry, sizeof(int32_t) * (size_t)ncarry));
+    p->carry_cap = ncarry;
   }
   CG_CUDA(cudaMemcpyAsync(p->seg_chunk, chunk.data(), sizeof(int64_t) * (k + 1),
                           cudaMemcpyHostToDevice, s));
@@ -836,15 +668,9 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   if (k > 0)
     CG_CUDA(cudaMemcpyAsync(p->seg_tab, tn.data(), sizeof(int32_t) * k, cudaMemcpyHostToDevice,
                             s));
-  if (nchunks > 0) {
-    first_row_kernel<<<grid_for(nchunks, 256), 256, 0, s>>>(
-        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, m2, chunk_a, chunk_b, nchunks,
-        p->first_row);
-    CG_LAUNCH_CHECK();
-  }
-  if (chunk[m2] > 0) {
-    staged_fill_kernel<<<grid_for(chunk[m2] * 32, 256), 256, 0, s>>>(
-        p->colf, p->seg_chunk, p->seg_cstart, p->seg_E, p->first_row, m2, chunk[m2], p->cs);
+  if (ncached > 0) {
+    first_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
+        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, kCachedChunk, ncached, p->first_row);
     CG_LAUNCH_CHECK();
   }
   // static runs of carries, cut into pieces for the parallel completion
@@ -857,24 +683,28 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   p->fx_sum = nullptr;
   p->fx_done = nullptr;
   p->fx_npieces = p->fx_nruns = 0;
-  if (nchunks > 0) {
-    int32_t* orow = nullptr;
-    CG_CUDA(cudaMallocAsync((void**)&orow, sizeof(int32_t) * (size_t)nchunks, s));
-    open_row_kernel<<<grid_for(nchunks, 256), 256, 0, s>>>(
-        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, m2, chunk_a, chunk_b, nchunks, orow);
-    cudaError_t ce = cudaGetLastError();
-    std::vector<int32_t> hc((size_t)nchunks);
-    if (ce == cudaSuccess)
-      ce = cudaMemcpyAsync(hc.data(), orow, sizeof(int32_t) * (size_t)nchunks,
-                           cudaMemcpyDeviceToHost, s);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-    cudaFreeAsync(orow, s);
-    if (ce != cudaSuccess) return cuda_fail(ce, "segmented gather: carry runs", __FILE__, __LINE__);
+  if (ncarry > 0) {
+    std::vector<int32_t> hc((size_t)ncarry, -1);  // the row each carry belongs to
+    std::copy(extra_row.begin(), extra_row.end(), hc.begin() + ncached);
+    if (ncached > 0) {
+      int32_t* orow = nullptr;
+      CG_CUDA(cudaMallocAsync((void**)&orow, sizeof(int32_t) * (size_t)ncached, s));
+      open_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
+          p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, kCachedChunk, ncached, orow);
+      cudaError_t ce = cudaGetLastError();
+      if (ce == cudaSuccess)
+        ce = cudaMemcpyAsync(hc.data(), orow, sizeof(int32_t) * (size_t)ncached,
+                             cudaMemcpyDeviceToHost, s);
+      if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+      cudaFreeAsync(orow, s);
+      if (ce != cudaSuccess)
+        return cuda_fail(ce, "segmented gather: carry runs", __FILE__, __LINE__);
+    }
     std::vector<int4> hp, hr;
-    for (int64_t c = 0; c < nchunks;) {
+    for (int64_t c = 0; c < ncarry;) {
       if (hc[c] < 0) { ++c; continue; }
       int64_t e = c + 1;
-      while (e < nchunks && hc[e] == hc[c]) ++e;
+      while (e < ncarry && hc[e] == hc[c]) ++e;
       const int32_t run = (int32_t)hr.size(), p0 = (int32_t)hp.size();
       for (int64_t x = c; x < e; x += 32)
         hp.push_back(make_int4((int32_t)x, (int32_t)std::min<int64_t>(32, e - x), run, 0));
@@ -898,29 +728,42 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   CG_CUDA(cudaStreamSynchronize(s));  // host vectors go out of scope
   p->threads = threads;
   p->ctas_per_sm = ctas_per_sm;
-  p->tab_cap = (int)((tabmax + 3) & ~3LL);
+  p->tab_cap = tab_cap;
   p->table_request = tab;
   p->m = m;
   p->m2 = m2;
   p->grid_affine = di.sm_count;
-  p->nchunks = nchunks;
-  p->ct_split = ctile[m];
+  p->nchunks = p->h_seg_task[k] + ncached;
   p->n_ctiles = ctile[k];
-  p->grid = (int)std::max<int64_t>(
-      1, std::min<int64_t>(p->ct_split, (int64_t)di.sm_count * ctas_per_sm));
-  if (p->overlap > 0) p->grid = di.sm_count;  // every SM serves the L1/L2 queue too
-  // about eight pieces per block: balance without many table reloads
-  p->piece = (int32_t)std::max<int64_t>(1, ceil_div(p->ct_split, 8LL * p->grid));
-  if (!p->counter) CG_CUDA(cudaMalloc((void**)&p->counter, 3 * sizeof(unsigned)));
+  // the staged launch: one block per resident slot, or per task where there are fewer
+  // (every SM serves the L1/L2 queue too in an overlapped launch)
+  const int32_t head = p->h_seg_task[m];
+  p->grid = (int)std::max<int64_t>(1, std::min<int64_t>(head, (int64_t)di.sm_count * ctas_per_sm));
+  if (p->overlap > 0) p->grid = di.sm_count;
+  p->head_tasks = head;
+  if (!p->counter) {
+    const size_t most = (size_t)di.sm_count * 2;  // blocks of any staged shape
+    CG_CUDA(cudaMalloc((void**)&p->counter, sizeof(unsigned) * (2 + most)));
+    CG_CUDA(cudaMalloc((void**)&p->blk_task, sizeof(int32_t) * (most + 1)));
+  }
+  if (head > 0) {
+    staged_share_kernel<<<grid_for(p->grid + 1, 128), 128, 0, s>>>(p->desc, head, p->grid,
+                                                                   p->blk_task);
+    CG_LAUNCH_CHECK();
+    CG_CUDA(cudaStreamSynchronize(s));
+  }
   p->grid_l2 = (int)std::max<int64_t>(
-      1, std::min<int64_t>(p->n_ctiles - p->ct_split, (int64_t)di.sm_count * 2));
+      1, std::min<int64_t>(p->n_ctiles, (int64_t)di.sm_count * 2));
   return CG_OK;
 }
 
 void seg_plan_free(SegPlan* p) {
   cudaFree(p->counter);
+  cudaFree(p->blk_task);
   cudaFree(p->colf);
   cudaFree(p->cs);
+  cudaFree(p->desc);
+  cudaFree(p->seg_task);
   cudaFree(p->meta);
   cudaFree(p->seg_cstart);
   cudaFree(p->seg_E);
@@ -938,7 +781,8 @@ void seg_plan_free(SegPlan* p) {
 }
 
 int64_t seg_plan_bytes(const SegPlan& p) {
-  return 4 * p.colf_len + p.cs_cap + 8 * p.chunk_cap + 72 * (int64_t)p.k + 20 * p.fx_npieces +
+  return 4 * p.colf_len + p.cs_cap + 16 * p.desc_cap + 4 * (p.chunk_cap + p.carry_cap) +
+         76 * (int64_t)p.k + 20 * p.fx_npieces +
          20 * p.fx_nruns;
 }
 
@@ -953,18 +797,28 @@ int seg_plan_export_col(const SegPlan& p, const int32_t* rp, int32_t* col, cudaS
   return CG_OK;
 }
 
+static StagedTasks staged_tasks(const SegPlan& p) {
+  return StagedTasks{p.cs, p.desc, p.seg_task, p.tab_cap};
+}
+
+static StagedShare staged_share(const SegPlan& p) {
+  return StagedShare{p.blk_task, p.counter + 2, p.seg_lo, p.seg_tab, p.m};
+}
+
+// the table and, behind it, the identity's entry
+static size_t staged_smem(const SegPlan& p) { return 4 * (size_t)p.tab_cap + 16; }
+
 template <class Op, int THREADS>
 static int launch_staged(const SegPlan& p, const typename Op::T* x, typename Op::T* out,
                          cudaStream_t s) {
   using T = typename Op::T;
-  const size_t smem = (size_t)p.tab_cap * sizeof(T);
+  const size_t smem = staged_smem(p);
   auto fn = staged_gather_kernel<Op, THREADS>;
-  CG_CUDA(cudaMemsetAsync(p.counter, 0, sizeof(unsigned), s));
+  CG_CUDA(cudaMemsetAsync(p.counter, 0, sizeof(unsigned) * (2 + p.grid), s));
   if (smem > 48 * 1024)
     CG_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
-  fn<<<p.grid, THREADS, smem, s>>>(p.cs, x, p.seg_E, p.seg_chunk, p.seg_ctile, p.seg_lo,
-                                   p.seg_tab, p.ct_split, p.piece, p.counter, out,
+  fn<<<p.grid, THREADS, smem, s>>>(staged_tasks(p), staged_share(p), x, out,
                                    reinterpret_cast<T*>(p.carry));
   CG_LAUNCH_CHECK();
   return CG_OK;
@@ -974,15 +828,15 @@ template <class Op>
 static int launch_overlap(const SegPlan& p, const typename Op::T* x, int32_t nx,
                           typename Op::T* out, cudaStream_t s) {
   using T = typename Op::T;
-  const size_t smem = (size_t)p.tab_cap * sizeof(T);
+  const size_t smem = staged_smem(p);
   auto fn = overlap_gather_kernel<Op>;
-  CG_CUDA(cudaMemsetAsync(p.counter, 0, 2 * sizeof(unsigned), s));
+  CG_CUDA(cudaMemsetAsync(p.counter, 0, sizeof(unsigned) * (2 + p.grid), s));
   if (smem > 48 * 1024)
     CG_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
-  fn<<<p.grid, 1024, smem, s>>>(p.cs, p.colf, x, nx, p.first_row, p.seg_cstart, p.seg_E,
-                                p.seg_chunk, p.seg_ctile, p.seg_lo, p.seg_tab, p.m, p.k,
-                                p.ct_split, p.piece, 1024 - 32 * p.overlap, p.counter, out,
+  fn<<<p.grid, 1024, smem, s>>>(staged_tasks(p), staged_share(p), p.colf, x, nx, p.first_row,
+                                p.seg_cstart, p.seg_E, p.seg_chunk, p.seg_lo, p.m, p.k,
+                                1024 - 32 * p.overlap, p.counter, out,
                                 reinterpret_cast<T*>(p.carry));
   CG_LAUNCH_CHECK();
   return CG_OK;
@@ -998,7 +852,7 @@ int run_seg_gather(const SegPlan& p, const typename Op::T* x, int32_t nx, typena
     phases &= ~(kPhaseStaged | kPhaseCached);
   }
   // staged segments [0, m): read from a shared-memory copy
-  if ((phases & kPhaseStaged) && p.m > 0 && p.ct_split > 0) {
+  if ((phases & kPhaseStaged) && p.head_tasks > 0) {
     if (p.threads == 1024)
       CG_TRY((launch_staged<Op, 1024>(p, x, out, s)));
     else
@@ -1006,21 +860,21 @@ int run_seg_gather(const SegPlan& p, const typename Op::T* x, int32_t nx, typena
   }
   // the table-sized cold segments, one block per segment
   if ((phases & kPhaseCached) && p.m2 > p.m) {
-    const size_t smem = (size_t)p.tab_cap * sizeof(T);
+    const size_t smem = staged_smem(p);
     auto fn = affine_gather_kernel<Op>;
-    CG_CUDA(cudaMemsetAsync(p.counter + 2, 0, sizeof(unsigned), s));
+    CG_CUDA(cudaMemsetAsync(p.counter + 1, 0, sizeof(unsigned), s));
     if (smem > 48 * 1024)
       CG_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)smem));
-    fn<<<p.grid_affine, 1024, smem, s>>>(p.cs, x, p.seg_E, p.seg_chunk, p.seg_lo, p.seg_tab, p.m,
-                                         p.m2, p.counter + 2, out, reinterpret_cast<T*>(p.carry));
+    fn<<<p.grid_affine, 1024, smem, s>>>(staged_tasks(p), x, p.seg_lo, p.seg_tab, p.m, p.m2,
+                                         p.counter + 1, out, reinterpret_cast<T*>(p.carry));
     CG_LAUNCH_CHECK();
   }
   // the rest through L1/L2: no shared memory, so the whole on-chip store is L1
-  if ((phases & kPhaseCached) && p.n_ctiles > p.ct_split) {
+  if ((phases & kPhaseCached) && p.n_ctiles > 0) {
     seg_gather_kernel<Op, 1024><<<p.grid_l2, 1024, 0, s>>>(
         p.colf, x, nx, p.first_row, p.seg_cstart, p.seg_E, p.seg_chunk, p.seg_ctile, p.seg_lo,
-        p.k, p.ct_split, (int32_t)p.n_ctiles, out, reinterpret_cast<T*>(p.carry));
+        p.k, 0, (int32_t)p.n_ctiles, out, reinterpret_cast<T*>(p.carry));
     CG_LAUNCH_CHECK();
   }
   if ((phases & kPhaseFixup) && p.fx_npieces > 0) {

@@ -6,14 +6,15 @@
 // one edge, so row i is the (i+1)-th flagged edge: the gather needs no row
 // pointers at all.
 //
-// Work unit: a warp owns a chunk of 32*IPL consecutive edges of one segment
-// (IPL = 8, or 16 in the staged launch at one block per SM); lane l holds
-// edges [IPL*l, IPL*l + IPL) of it (16-byte streaming loads).  Lanes
+// Work unit of the segments read through L1/L2: a warp owns a chunk of 256
+// consecutive edges of one segment; lane l holds edges [8l, 8l + 8) of it
+// (16-byte streaming loads).  Lanes
 // fold their 8 values sequentially, emit every row that starts and ends
 // inside them, and a warp-wide segmented scan over the lanes' open-row parts
 // completes each lane's first row.  The row still open at the chunk's end
 // goes to carry[chunk], folded in afterwards in chunk order.  No shared
-// staging of edges and no block barriers between chunks.
+// staging of edges and no block barriers between chunks.  The staged segments
+// have a layout of their own (staged_stream.cuh).
 //
 // Two launches per pass.  The leading segments that fit an SM's shared
 // memory (after clustering, the hot head: the paper's cache-sized segment,
@@ -33,26 +34,34 @@
 namespace cg {
 
 constexpr uint32_t kRowEndFlag = 0x80000000u;
-constexpr int kMaxChunkEdges = 512;  // 32 lanes x 16 edges (staged launch, 1 block/SM)
+constexpr int kMaxChunkEdges = 512;  // padding behind the edges: a chunk may read past the end
 
 struct SegPlan {
   int k = 0;
   int64_t E = 0, rows = 0, nchunks = 0;
   uint32_t* colf = nullptr;        // [colf_len] flagged, padded segment-local sources
-  uint8_t* cs = nullptr;           // staged chunk stream (16-bit local indices + masks)
+  uint8_t* cs = nullptr;           // staged segments' edge stream (staged_stream.cuh)
   int64_t cs_cap = 0;
+  uint4* desc = nullptr;           // one descriptor per staged task
+  int64_t desc_cap = 0;
+  int32_t* seg_task = nullptr;     // [k+1] first staged task of each segment
+  std::vector<int32_t> h_seg_task;
+  int32_t head_tasks = 0;          // tasks of the segments [0, m)
+  int32_t* blk_task = nullptr;     // [grid+1] first task of each staged block's range
   int64_t colf_len = 0;
   int64_t* seg_cstart = nullptr;   // [k]   first colf entry of each segment
   int32_t* seg_E = nullptr;        // [k]   edges of each segment
   int64_t* seg_chunk = nullptr;    // [k+1] first global chunk of each segment
-  int32_t* seg_ctile = nullptr;    // [k+1] first block-group of each segment
+  int32_t* seg_ctile = nullptr;    // [k+1] first L1/L2 block-group of each segment
   int32_t* seg_lo = nullptr;       // [k]   first source of each segment
   int32_t* seg_tab = nullptr;      // [k]   table entries used for each segment
-  int32_t* first_row = nullptr;    // [nchunks] subgraph row of each chunk's first edge
-  void* carry = nullptr;           // [nchunks] 4-byte values
+  int32_t* first_row = nullptr;    // subgraph row of each L1/L2 chunk's first edge
+  void* carry = nullptr;           // [carry_cap] 4-byte values: the L1/L2 chunks', then the
+                                   // full pieces' of long staged rows
+  int64_t carry_cap = 0;
   int64_t* meta = nullptr;         // [4(k+1)] row_base, edge_base, cstart, bounds (device)
   const int32_t* rp32 = nullptr;   // subgraph row starts (owned by the handle)
-  int64_t chunk_cap = 0;           // capacity of first_row / carry
+  int64_t chunk_cap = 0;           // capacity of first_row
   std::vector<int64_t> h_cstart, src_bounds, edge_base, row_base;
   int threads = 1024;       // staged-segment launch shape
   int ctas_per_sm = 1;
@@ -63,12 +72,10 @@ struct SegPlan {
   double affine_head = 0.0;  // > 0: head threshold (edges per source) of the segment-affine
                             // plan; the table-sized segments after the head go one per block
   int grid_affine = 0;      // blocks of the segment-affine launch
-  int32_t ct_split = 0;     // first block-group of the unstaged segments
-  int64_t n_ctiles = 0;
+  int64_t n_ctiles = 0;     // block-groups of the L1/L2 launch
   int grid = 0;             // staged launch blocks
-  int32_t piece = 1;        // block-groups per work piece of the staged launch
-  unsigned* counter = nullptr;  // [3] next staged work piece, next L1/L2 chunk (overlap),
-                                //     next segment-affine segment
+  unsigned* counter = nullptr;  // next L1/L2 chunk (overlap), next segment-affine segment,
+                                // tasks taken of each staged block's range
   int overlap_request = 0;  // warps per block given to the L1/L2 segments (0: two launches)
   int overlap = 0;          // the same, in effect (0 when one kind of segment is absent)
   int grid_l2 = 0;          // unstaged launch blocks (1024 threads, 2 per SM)
@@ -96,6 +103,13 @@ int seg_plan_build(const int32_t* col, const int64_t* rp, const int32_t* rp32, i
 // (-1: the capacity; 0: none).  Synchronizes the stream.
 int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertices,
                        cudaStream_t s);
+
+// Lay out the staged segments [0, m2): their tasks, descriptors and stream (pad:
+// the table entry that holds the identity).  extra_row: the rows of the full
+// pieces of rows longer than kStagedMost, whose carry slots start at
+// carry_base.  Synchronizes.
+int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base,
+                 std::vector<int32_t>* extra_row, cudaStream_t s);
 
 void seg_plan_free(SegPlan* p);
 int64_t seg_plan_bytes(const SegPlan& p);

@@ -275,21 +275,6 @@ __global__ void blk_transpose_kernel(const int32_t* __restrict__ blk_sm, int k, 
   }
 }
 
-struct Scratch {
-  std::vector<void*> ptrs;
-  cudaStream_t s;
-  explicit Scratch(cudaStream_t st) : s(st) {}
-  template <typename T>
-  cudaError_t get(T** p, size_t n) {
-    cudaError_t e = cudaMallocAsync((void**)p, sizeof(T) * (n > 0 ? n : 1), s);
-    if (e == cudaSuccess) ptrs.push_back((void*)*p);
-    return e;
-  }
-  ~Scratch() {
-    for (void* p : ptrs) cudaFreeAsync(p, s);
-  }
-};
-
 int build_impl(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E, int32_t k,
                const std::vector<int64_t>& bounds, int32_t B, cg_segmented* g, cudaStream_t s) {
   Scratch tmp(s);
