@@ -62,33 +62,58 @@ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 // Grid size for grid-stride kernels: a multiple of the SM count.
 int grid_for(int64_t n, int threads, int per_sm = 8);
 
+// Stream-ordered scratch, given back when it goes out of scope.  Taken in
+// slabs: an allocation from the stream-ordered pool costs 10-60 us of host
+// time after every synchronisation (the pool gives its memory back then), and
+// a build wants dozens of arrays.  `first` sizes the first slab.
+struct Scratch {
+  std::vector<void*> slabs;
+  cudaStream_t s;
+  size_t first;
+  char* cur = nullptr;
+  size_t left = 0;
+  explicit Scratch(cudaStream_t st, size_t first_slab = 0) : s(st), first(first_slab) {}
+  Scratch(const Scratch&) = delete;
+  Scratch& operator=(const Scratch&) = delete;
+  static size_t round(size_t b) { return (b + 255) & ~(size_t)255; }
+  template <typename T>
+  cudaError_t get(T** p, size_t n) {
+    const size_t b = round(sizeof(T) * (n > 0 ? n : 1));
+    if (b > left) {
+      const size_t slab = b > first ? b : first;
+      void* q = nullptr;
+      cudaError_t e = cudaMallocAsync(&q, slab, s);
+      if (e != cudaSuccess) return e;
+      slabs.push_back(q);
+      cur = static_cast<char*>(q);
+      left = slab;
+      first = (size_t)1 << 20;  // a slab that was sized too small goes on in small ones
+    }
+    *p = reinterpret_cast<T*>(cur);
+    cur += b;
+    left -= b;
+    return cudaSuccess;
+  }
+  ~Scratch() {
+    for (void* p : slabs) cudaFreeAsync(p, s);
+  }
+};
+
 // ---------------------------------------------------------------------------
-// Scans and sorts (scan.cu).  All stream-ordered; scratch from the stream-
-// ordered allocator.
+// Scans and sorts (scan.cu).  All stream-ordered; scratch from ws, or of their
+// own.  scan_scratch / sort_scratch: the bytes they take for n items.
 // ---------------------------------------------------------------------------
 // out[i] = sum_{j<i} in[j] for i in [0, n]; out has n+1 entries.
-int exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s);
-int exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s);
+int exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s,
+                       Scratch* ws = nullptr);
+int exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s,
+                              Scratch* ws = nullptr);
+size_t scan_scratch(int64_t n);
+size_t sort_scratch(int64_t n);
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits of key.
 int radix_sort_pairs(const uint32_t* keys_in, const int32_t* vals_in,
                      uint32_t* keys_out, int32_t* vals_out, int64_t n, int bits,
-                     cudaStream_t s);
-
-// Stream-ordered scratch, given back when it goes out of scope.
-struct Scratch {
-  std::vector<void*> ptrs;
-  cudaStream_t s;
-  explicit Scratch(cudaStream_t st) : s(st) {}
-  template <typename T>
-  cudaError_t get(T** p, size_t n) {
-    cudaError_t e = cudaMallocAsync((void**)p, sizeof(T) * (n > 0 ? n : 1), s);
-    if (e == cudaSuccess) ptrs.push_back((void*)*p);
-    return e;
-  }
-  ~Scratch() {
-    for (void* p : ptrs) cudaFreeAsync(p, s);
-  }
-};
+                     cudaStream_t s, Scratch* ws = nullptr);
 
 // ---------------------------------------------------------------------------
 // Device helpers

@@ -21,10 +21,11 @@ struct cg_segmented {
   int32_t nb = 0;
   int64_t rows = 0;
   std::vector<int64_t> bounds, row_base, edge_base;  // host copies, k+1 each
-  int32_t* row_ptr = nullptr;  // [rows+1] (export only; the gather reads flagged edges)
-  int32_t* idx_map = nullptr;  // [rows]
+  int32_t* idx_map = nullptr;  // [rows]; row_ptr and blk lie in the same allocation
+  int32_t* row_ptr = nullptr;  // [rows+1] (builds and export; the gathers do not read it)
   int32_t* blk = nullptr;      // [(nb+1)*k] block-major
   cg::SegPlan plan;            // flagged padded edges + chunk index + launch shape
+  char* state = nullptr;         // one allocation that holds the arrays below
   void* interm = nullptr;        // [rows] 4-byte values (intermBuf)
   double* partials = nullptr;    // [2*nb] per-block FP64 partial sums
   unsigned* counter = nullptr;   // last-block detection

@@ -70,7 +70,7 @@ __global__ void tile_scan_kernel(const TI* __restrict__ in, int64_t n,
 }
 
 template <typename TI>
-int exclusive_scan_impl(const TI* in, int64_t* out, int64_t n, cudaStream_t s) {
+int exclusive_scan_impl(const TI* in, int64_t* out, int64_t n, cudaStream_t s, Scratch* ws) {
   if (n <= 0) {
     CG_CUDA(cudaMemsetAsync(out, 0, sizeof(int64_t), s));
     return CG_OK;
@@ -81,20 +81,16 @@ int exclusive_scan_impl(const TI* in, int64_t* out, int64_t n, cudaStream_t s) {
     CG_LAUNCH_CHECK();
     return CG_OK;
   }
+  Scratch own(s, scan_scratch(n));
+  if (!ws) ws = &own;
   int64_t* buf = nullptr;  // tile sums [tiles], tile offsets [tiles+1]
-  CG_CUDA(cudaMallocAsync((void**)&buf, sizeof(int64_t) * (2 * tiles + 1), s));
+  CG_CUDA(ws->get(&buf, 2 * tiles + 1));
   tile_reduce_kernel<TI><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, buf);
-  int st = CG_OK;
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) st = cuda_fail(e, "tile_reduce", __FILE__, __LINE__);
-  if (st == CG_OK) st = exclusive_scan_impl<int64_t>(buf, buf + tiles, tiles, s);
-  if (st == CG_OK) {
-    tile_scan_kernel<TI><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, buf + tiles, out);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) st = cuda_fail(e, "tile_scan", __FILE__, __LINE__);
-  }
-  cudaFreeAsync(buf, s);
-  return st;
+  CG_LAUNCH_CHECK();
+  CG_TRY(exclusive_scan_impl<int64_t>(buf, buf + tiles, tiles, s, ws));
+  tile_scan_kernel<TI><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, buf + tiles, out);
+  CG_LAUNCH_CHECK();
+  return CG_OK;
 }
 
 // ---------------------------------------------------------------- radix sort
@@ -174,54 +170,60 @@ __global__ void radix_scatter_kernel(const uint32_t* __restrict__ kin,
 
 }  // namespace
 
-int exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s) {
-  return exclusive_scan_impl<int64_t>(in, out, n, s);
+size_t scan_scratch(int64_t n) {
+  size_t b = 0;
+  for (int64_t t = ceil_div(n, kScanTile); t > 1; t = ceil_div(t, kScanTile))
+    b += Scratch::round(sizeof(int64_t) * (size_t)(2 * t + 1));
+  return b;
 }
-int exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s) {
-  return exclusive_scan_impl<int32_t>(in, out, n, s);
+int exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t s, Scratch* ws) {
+  return exclusive_scan_impl<int64_t>(in, out, n, s, ws);
+}
+int exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s,
+                              Scratch* ws) {
+  return exclusive_scan_impl<int32_t>(in, out, n, s, ws);
+}
+
+// the ping-pong pair, the digit counts and their scan (one scan's scratch per pass)
+size_t sort_scratch(int64_t n) {
+  const int64_t ntiles = ceil_div(n, kSortTile);
+  return 2 * Scratch::round(4 * (size_t)n) + Scratch::round(4 * 256 * (size_t)ntiles) +
+         Scratch::round(8 * (256 * (size_t)ntiles + 1)) + 4 * scan_scratch(256 * ntiles);
 }
 
 int radix_sort_pairs(const uint32_t* keys_in, const int32_t* vals_in, uint32_t* keys_out,
-                     int32_t* vals_out, int64_t n, int bits, cudaStream_t s) {
+                     int32_t* vals_out, int64_t n, int bits, cudaStream_t s, Scratch* ws) {
   if (n <= 0) return CG_OK;
   const int passes = bits <= 0 ? 1 : (bits + 7) / 8;
   const int64_t ntiles = ceil_div(n, kSortTile);
+  Scratch own(s, sort_scratch(n));
+  if (!ws) ws = &own;
   uint32_t* kb = nullptr;
   int32_t* vb = nullptr;
   int32_t* counts = nullptr;
   int64_t* offs = nullptr;
-  int st = CG_OK;
-  cudaError_t e;
-  e = cudaMallocAsync((void**)&kb, sizeof(uint32_t) * n, s);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&vb, sizeof(int32_t) * n, s);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&counts, sizeof(int32_t) * 256 * ntiles, s);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&offs, sizeof(int64_t) * (256 * ntiles + 1), s);
-  if (e != cudaSuccess) st = cuda_fail(e, "radix scratch", __FILE__, __LINE__);
+  CG_CUDA(ws->get(&kb, n));
+  CG_CUDA(ws->get(&vb, n));
+  CG_CUDA(ws->get(&counts, 256 * ntiles));
+  CG_CUDA(ws->get(&offs, 256 * ntiles + 1));
   // ping-pong so that the last pass lands in (keys_out, vals_out)
   const uint32_t* ksrc = keys_in;
   const int32_t* vsrc = vals_in;
-  for (int p = 0; p < passes && st == CG_OK; ++p) {
+  for (int p = 0; p < passes; ++p) {
     // passes alternate between the scratch pair and the output pair, ending in the output
     const bool to_out = ((passes - 1 - p) % 2) == 0;
     uint32_t* kdst = to_out ? keys_out : kb;
     int32_t* vdst = to_out ? vals_out : vb;
     radix_hist_kernel<<<(unsigned)ntiles, kSortThreads, 0, s>>>(ksrc, n, 8 * p, counts, ntiles);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) { st = cuda_fail(e, "radix_hist", __FILE__, __LINE__); break; }
-    st = exclusive_scan_i32_to_i64(counts, offs, 256 * ntiles, s);
-    if (st != CG_OK) break;
+    CG_LAUNCH_CHECK();
+    CG_TRY(exclusive_scan_i32_to_i64(counts, offs, 256 * ntiles, s, ws));
     radix_scatter_kernel<<<(unsigned)ntiles, kSortThreads, 0, s>>>(ksrc, vsrc, n, 8 * p, offs,
                                                                     ntiles, kdst, vdst);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) { st = cuda_fail(e, "radix_scatter", __FILE__, __LINE__); break; }
+    CG_LAUNCH_CHECK();
     ksrc = kdst;
     vsrc = vdst;
   }
-  if (kb) cudaFreeAsync(kb, s);
-  if (vb) cudaFreeAsync(vb, s);
-  if (counts) cudaFreeAsync(counts, s);
-  if (offs) cudaFreeAsync(offs, s);
-  return st;
+  return CG_OK;
 }
 
 }  // namespace cg

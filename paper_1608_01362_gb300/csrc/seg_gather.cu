@@ -16,26 +16,6 @@ __device__ __forceinline__ int last_le(const int64_t* a, int n, int64_t v) {
   return lo - 1;
 }
 
-// One warp per subgraph row: copy its sources, as indices local to their
-// segment, into the padded layout and flag the last one.
-__global__ void colf_fill_kernel(const int32_t* __restrict__ col, const int64_t* __restrict__ rp,
-                                 int64_t rows, const int64_t* __restrict__ row_base,
-                                 const int64_t* __restrict__ edge_base,
-                                 const int64_t* __restrict__ cstart,
-                                 const int64_t* __restrict__ bounds, int k,
-                                 uint32_t* __restrict__ colf) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < rows; i += nw) {
-    const int s = last_le(row_base, k + 1, i);
-    const int64_t lo = rp[i], hi = rp[i + 1];
-    const int64_t shift = cstart[s] - edge_base[s];
-    const int32_t src0 = (int32_t)bounds[s];
-    for (int64_t e = lo + lane; e < hi; e += 32)
-      colf[e + shift] = (uint32_t)(col[e] - src0) | (e == hi - 1 ? kRowEndFlag : 0u);
-  }
-}
-
 __global__ void export_col_kernel(const uint32_t* __restrict__ colf,
                                   const int32_t* __restrict__ rp, int64_t rows,
                                   const int64_t* __restrict__ row_base,
@@ -75,37 +55,59 @@ __global__ void open_row_kernel(const int32_t* __restrict__ rp,
   }
 }
 
-// Completion of the rows that span chunks, one thread per piece (<= 32
-// consecutive chunks of one run of carries on the same row).  A one-piece
-// run folds its carries into the row directly; otherwise every piece stores
-// its fold and the last piece of the run to finish (an atomic count, no
-// waiting) folds the pieces in order into the row.  Deterministic, and a hub
-// row spanning many chunks is spread over many threads.
+// Completion of the rows that span chunks: carry c belongs to row carry_row[c]
+// (-1: none), and the carries of one row are consecutive (a run).  A warp
+// takes 32 carries and finishes the runs that begin among them: those that
+// also end there by one segmented scan, the last one by reading on, 128
+// carries at a time, until its row ends.  The order is fixed: deterministic.
+// (The run lists this replaces were made by the host from a copy of the rows,
+// 0.7 ms of a new 65 M-edge graph.)
 template <class Op>
-__global__ void seg_fixup_kernel(const int4* __restrict__ pieces, int64_t npieces,
-                                 const int4* __restrict__ runs,
-                                 const typename Op::T* __restrict__ carry,
-                                 typename Op::T* __restrict__ psum, unsigned* __restrict__ done,
-                                 typename Op::T* __restrict__ out) {
+__global__ void __launch_bounds__(256)
+seg_fixup_kernel(const int32_t* __restrict__ carry_row, const typename Op::T* __restrict__ carry,
+                 int64_t n, typename Op::T* __restrict__ out) {
   using T = typename Op::T;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < npieces;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int4 pc = pieces[p];  // (first chunk, chunks, run)
-    const int4 rn = runs[pc.z]; // (row, first piece, pieces)
-    T v = carry[pc.x];
-    for (int j = 1; j < pc.y; ++j) v = Op::op(v, carry[pc.x + j]);
-    if (rn.z == 1) {
-      out[rn.x] = Op::op(v, out[rn.x]);
-      continue;
+  constexpr unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t c0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) << 5; c0 < n;
+       c0 += step) {
+    const int64_t c = c0 + lane;
+    const int32_t r = c < n ? __ldg(carry_row + c) : -1;
+    int32_t prev = __shfl_up_sync(kFull, r, 1), next = __shfl_down_sync(kFull, r, 1);
+    if (lane == 0) prev = c0 > 0 ? __ldg(carry_row + c0 - 1) : -1;
+    if (lane == 31) next = c0 + 32 < n ? __ldg(carry_row + c0 + 32) : -1;
+    T S = r >= 0 ? carry[c] : Op::identity();
+    int h = r < 0 || r != prev;  // a run begins (or none lies) here
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const T y = __shfl_up_sync(kFull, S, o);
+      const int g = __shfl_up_sync(kFull, h, o);
+      if (lane >= o) {
+        if (!h) S = Op::op(y, S);
+        h |= g;
+      }
     }
-    psum[p] = v;
-    __threadfence();
-    if (atomicAdd(done + pc.z, 1u) != (unsigned)rn.z - 1) continue;
-    __threadfence();
-    T t = __ldcg(psum + rn.y);
-    for (int j = 1; j < rn.z; ++j) t = Op::op(t, __ldcg(psum + rn.y + j));
-    out[rn.x] = Op::op(t, out[rn.x]);
-    done[pc.z] = 0u;  // ready for the next pass
+    if (r >= 0 && h && next != r) out[r] = Op::op(S, out[r]);
+    if (!__shfl_sync(kFull, (int)(r >= 0 && h && next == r), 31)) continue;
+    const int32_t row = __shfl_sync(kFull, r, 31);
+    T t = __shfl_sync(kFull, S, 31);
+    bool more = true;
+    for (int64_t b = c0 + 32; more; b += 128) {
+      T v = Op::identity();
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t i = b + 32 * u + lane;
+        const unsigned m = __ballot_sync(kFull, i < n && __ldg(carry_row + (i < n ? i : 0)) == row);
+        const int len = !more ? 0 : m == kFull ? 32 : __ffs(~m) - 1;
+        if (lane < len) v = Op::op(v, carry[i]);
+        more = more && len == 32;
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) v = Op::op(v, __shfl_xor_sync(kFull, v, o));
+      t = Op::op(t, v);
+    }
+    if (lane == 0) out[row] = Op::op(t, out[row]);
   }
 }
 
@@ -511,15 +513,10 @@ int seg_table_capacity(int ctas) {
   return (int)((per / 4) & ~31LL);
 }
 
-int seg_plan_build(const int32_t* col, const int64_t* rp, const int32_t* rp32, int64_t rows,
-                   int64_t E, int k, const std::vector<int64_t>& row_base,
-                   const std::vector<int64_t>& edge_base, const std::vector<int64_t>& src_bounds,
-                   SegPlan* p, cudaStream_t s) {
+int seg_plan_alloc(int64_t E, int k, const std::vector<int64_t>& edge_base,
+                   const std::vector<int64_t>& src_bounds, SegPlan* p, cudaStream_t s) {
   p->k = k;
   p->E = E;
-  p->rows = rows;
-  p->rp32 = rp32;
-  p->row_base = row_base;
   p->edge_base = edge_base;
   p->src_bounds = src_bounds;
   p->h_cstart.assign(k + 1, 0);
@@ -533,41 +530,46 @@ int seg_plan_build(const int32_t* col, const int64_t* rp, const int32_t* rp32, i
     return CG_ERR_UNSUPPORTED;
   }
   CG_CUDA(cudaMalloc((void**)&p->colf, sizeof(uint32_t) * p->colf_len));
-  CG_CUDA(cudaMemsetAsync(p->colf, 0, sizeof(uint32_t) * p->colf_len, s));
-  const size_t kk = (size_t)(k > 0 ? k : 1);
-  CG_CUDA(cudaMalloc((void**)&p->seg_cstart, sizeof(int64_t) * kk));
-  CG_CUDA(cudaMalloc((void**)&p->seg_E, sizeof(int32_t) * kk));
-  CG_CUDA(cudaMalloc((void**)&p->seg_chunk, sizeof(int64_t) * (kk + 1)));
-  CG_CUDA(cudaMalloc((void**)&p->seg_ctile, sizeof(int32_t) * (kk + 1)));
-  CG_CUDA(cudaMalloc((void**)&p->seg_lo, sizeof(int32_t) * kk));
-  CG_CUDA(cudaMalloc((void**)&p->seg_tab, sizeof(int32_t) * kk));
-  CG_CUDA(cudaMalloc((void**)&p->meta, sizeof(int64_t) * 4 * (kk + 1)));
+  // The segments' arrays, one allocation and one upload: meta (row_base, which
+  // the caller's build writes, edge_base, cstart, bounds), then seg_E and
+  // seg_lo; behind them what seg_plan_configure uploads in its turn (seg_chunk,
+  // seg_ctile, seg_tab), and the staged launch's counters and shares.
+  DeviceInfo di{};
+  CG_TRY(device_info(&di));
+  const size_t n = (size_t)k + 1, most = (size_t)di.sm_count * 2;  // blocks of any staged shape
+  const size_t words = 2 * 4 * n + 2 * n + 2 * n + 3 * n + (2 + most) + (most + 1);
+  CG_CUDA(cudaMalloc((void**)&p->meta, 4 * words));
+  int32_t* w = reinterpret_cast<int32_t*>(p->meta) + 2 * 4 * n;
+  p->seg_cstart = p->meta + 2 * n;
+  p->seg_E = w;
+  p->seg_lo = w + n;
+  w += 2 * n;  // 8-byte aligned: an even number of words before it
+  p->seg_chunk = reinterpret_cast<int64_t*>(w);
+  p->seg_ctile = w + 2 * n;
+  p->seg_tab = w + 3 * n;
+  p->seg_task = w + 4 * n;
+  p->counter = reinterpret_cast<unsigned*>(w + 5 * n);
+  p->blk_task = w + 5 * n + 2 + most;
+  std::vector<int64_t> up(4 * n, 0);  // edge_base, cstart, bounds, then seg_E and seg_lo
+  int32_t* eo = reinterpret_cast<int32_t*>(up.data() + 3 * n);
+  for (size_t q = 0; q < n; ++q) {
+    up[q] = edge_base[q];
+    up[n + q] = p->h_cstart[q];
+    up[2 * n + q] = src_bounds[q];
+    eo[q] = q + 1 < n ? (int32_t)(edge_base[q + 1] - edge_base[q]) : 0;
+    eo[n + q] = (int32_t)src_bounds[q];
+  }
+  // (a copy from pageable memory returns once the source has been read)
+  CG_CUDA(cudaMemcpyAsync(p->meta + n, up.data(), sizeof(int64_t) * up.size(),
+                          cudaMemcpyHostToDevice, s));
+  return CG_OK;
+}
 
-  std::vector<int32_t> segE(kk, 0), lo(kk, 0);
-  for (int q = 0; q < k; ++q) {
-    segE[q] = (int32_t)(edge_base[q + 1] - edge_base[q]);
-    lo[q] = (int32_t)src_bounds[q];
-  }
-  CG_CUDA(cudaMemcpyAsync(p->seg_cstart, p->h_cstart.data(), sizeof(int64_t) * k,
-                          cudaMemcpyHostToDevice, s));
-  CG_CUDA(cudaMemcpyAsync(p->seg_E, segE.data(), sizeof(int32_t) * k, cudaMemcpyHostToDevice, s));
-  CG_CUDA(cudaMemcpyAsync(p->seg_lo, lo.data(), sizeof(int32_t) * k, cudaMemcpyHostToDevice, s));
-  // meta: row_base, edge_base, cstart, bounds (k+1 each), for chunk indexing and export
-  CG_CUDA(cudaMemcpyAsync(p->meta, row_base.data(), sizeof(int64_t) * (k + 1),
-                          cudaMemcpyHostToDevice, s));
-  CG_CUDA(cudaMemcpyAsync(p->meta + (k + 1), edge_base.data(), sizeof(int64_t) * (k + 1),
-                          cudaMemcpyHostToDevice, s));
-  CG_CUDA(cudaMemcpyAsync(p->meta + 2 * (k + 1), p->h_cstart.data(), sizeof(int64_t) * (k + 1),
-                          cudaMemcpyHostToDevice, s));
-  CG_CUDA(cudaMemcpyAsync(p->meta + 3 * (k + 1), src_bounds.data(), sizeof(int64_t) * (k + 1),
-                          cudaMemcpyHostToDevice, s));
-  if (rows > 0) {
-    colf_fill_kernel<<<grid_for(rows * 32, 256, 16), 256, 0, s>>>(
-        col, rp, rows, p->meta, p->meta + (k + 1), p->meta + 2 * (k + 1), p->meta + 3 * (k + 1),
-        k, p->colf);
-    CG_LAUNCH_CHECK();
-  }
-  CG_CUDA(cudaStreamSynchronize(s));  // host vectors above go out of scope
+int seg_plan_finish(SegPlan* p, const int32_t* rp32, int64_t rows,
+                    const std::vector<int64_t>& row_base, cudaStream_t s) {
+  p->rows = rows;
+  p->rp32 = rp32;
+  p->row_base = row_base;
   return seg_plan_configure(p, 1024, 1, -1, s);
 }
 
@@ -641,91 +643,28 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
     tn[q] = q < m2 ? (int32_t)(p->src_bounds[q + 1] - p->src_bounds[q]) : 0;
   }
   const int64_t ncached = chunk[k];
-  // the staged segments' tasks; their extra carries follow the chunks' carries
-  std::vector<int32_t> extra_row;
-  CG_TRY(staged_build(p, m2, tab_cap, ncached, &extra_row, s));
-  const int64_t ncarry = ncached + (int64_t)extra_row.size();
+  // the staged segments' tasks; the carries of their full pieces follow the chunks'
+  CG_TRY(staged_build(p, m2, tab_cap, ncached, s));
   for (int q = 0; q < k; ++q)  // block-groups of the L1/L2 launch
     ctile[q + 1] = ctile[q] + (int32_t)ceil_div(chunk[q + 1] - chunk[q], warps_b);
-  if (ncached > p->chunk_cap) {
-    cudaFree(p->first_row);
-    p->first_row = nullptr;
-    p->chunk_cap = 0;
-    CG_CUDA(cudaMalloc((void**)&p->first_row, sizeof(int32_t) * (size_t)ncached));
-    p->chunk_cap = ncached;
+  {  // seg_chunk, seg_ctile, seg_tab lie one behind the other
+    const size_t n = (size_t)k + 1;
+    std::vector<int32_t> up(4 * n, 0);
+    std::copy(chunk.begin(), chunk.end(), reinterpret_cast<int64_t*>(up.data()));
+    std::copy(ctile.begin(), ctile.end(), up.begin() + 2 * n);
+    std::copy(tn.begin(), tn.begin() + k, up.begin() + 3 * n);
+    CG_CUDA(cudaMemcpyAsync(p->seg_chunk, up.data(), sizeof(int32_t) * up.size(),
+                            cudaMemcpyHostToDevice, s));
   }
-  if (ncarry > p->carry_cap) {
-    cudaFree(p->carry);
-    p->carry = nullptr;
-    p->carry_cap = 0;
-    CG_CUDA(cudaMalloc(&p->carry, sizeof(int32_t) * (size_t)ncarry));
-    p->carry_cap = ncarry;
-  }
-  CG_CUDA(cudaMemcpyAsync(p->seg_chunk, chunk.data(), sizeof(int64_t) * (k + 1),
-                          cudaMemcpyHostToDevice, s));
-  CG_CUDA(cudaMemcpyAsync(p->seg_ctile, ctile.data(), sizeof(int32_t) * (k + 1),
-                          cudaMemcpyHostToDevice, s));
-  if (k > 0)
-    CG_CUDA(cudaMemcpyAsync(p->seg_tab, tn.data(), sizeof(int32_t) * k, cudaMemcpyHostToDevice,
-                            s));
   if (ncached > 0) {
     first_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
         p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, kCachedChunk, ncached, p->first_row);
     CG_LAUNCH_CHECK();
+    open_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
+        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, kCachedChunk, ncached,
+        p->carry_row);
+    CG_LAUNCH_CHECK();
   }
-  // static runs of carries, cut into pieces for the parallel completion
-  cudaFree(p->fx_pieces);
-  cudaFree(p->fx_runs);
-  cudaFree(p->fx_sum);
-  cudaFree(p->fx_done);
-  p->fx_pieces = nullptr;
-  p->fx_runs = nullptr;
-  p->fx_sum = nullptr;
-  p->fx_done = nullptr;
-  p->fx_npieces = p->fx_nruns = 0;
-  if (ncarry > 0) {
-    std::vector<int32_t> hc((size_t)ncarry, -1);  // the row each carry belongs to
-    std::copy(extra_row.begin(), extra_row.end(), hc.begin() + ncached);
-    if (ncached > 0) {
-      int32_t* orow = nullptr;
-      CG_CUDA(cudaMallocAsync((void**)&orow, sizeof(int32_t) * (size_t)ncached, s));
-      open_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
-          p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, kCachedChunk, ncached, orow);
-      cudaError_t ce = cudaGetLastError();
-      if (ce == cudaSuccess)
-        ce = cudaMemcpyAsync(hc.data(), orow, sizeof(int32_t) * (size_t)ncached,
-                             cudaMemcpyDeviceToHost, s);
-      if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-      cudaFreeAsync(orow, s);
-      if (ce != cudaSuccess)
-        return cuda_fail(ce, "segmented gather: carry runs", __FILE__, __LINE__);
-    }
-    std::vector<int4> hp, hr;
-    for (int64_t c = 0; c < ncarry;) {
-      if (hc[c] < 0) { ++c; continue; }
-      int64_t e = c + 1;
-      while (e < ncarry && hc[e] == hc[c]) ++e;
-      const int32_t run = (int32_t)hr.size(), p0 = (int32_t)hp.size();
-      for (int64_t x = c; x < e; x += 32)
-        hp.push_back(make_int4((int32_t)x, (int32_t)std::min<int64_t>(32, e - x), run, 0));
-      hr.push_back(make_int4(hc[c], p0, (int32_t)hp.size() - p0, 0));
-      c = e;
-    }
-    p->fx_npieces = (int64_t)hp.size();
-    p->fx_nruns = (int64_t)hr.size();
-    if (!hp.empty()) {
-      CG_CUDA(cudaMalloc((void**)&p->fx_pieces, sizeof(int4) * hp.size()));
-      CG_CUDA(cudaMalloc((void**)&p->fx_runs, sizeof(int4) * hr.size()));
-      CG_CUDA(cudaMalloc(&p->fx_sum, 4 * hp.size()));
-      CG_CUDA(cudaMalloc((void**)&p->fx_done, sizeof(unsigned) * hr.size()));
-      CG_CUDA(cudaMemcpyAsync(p->fx_pieces, hp.data(), sizeof(int4) * hp.size(),
-                              cudaMemcpyHostToDevice, s));
-      CG_CUDA(cudaMemcpyAsync(p->fx_runs, hr.data(), sizeof(int4) * hr.size(),
-                              cudaMemcpyHostToDevice, s));
-      CG_CUDA(cudaMemsetAsync(p->fx_done, 0, sizeof(unsigned) * hr.size(), s));
-    }
-  }
-  CG_CUDA(cudaStreamSynchronize(s));  // host vectors go out of scope
   p->threads = threads;
   p->ctas_per_sm = ctas_per_sm;
   p->tab_cap = tab_cap;
@@ -741,49 +680,42 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   p->grid = (int)std::max<int64_t>(1, std::min<int64_t>(head, (int64_t)di.sm_count * ctas_per_sm));
   if (p->overlap > 0) p->grid = di.sm_count;
   p->head_tasks = head;
-  if (!p->counter) {
-    const size_t most = (size_t)di.sm_count * 2;  // blocks of any staged shape
-    CG_CUDA(cudaMalloc((void**)&p->counter, sizeof(unsigned) * (2 + most)));
-    CG_CUDA(cudaMalloc((void**)&p->blk_task, sizeof(int32_t) * (most + 1)));
-  }
   if (head > 0) {
     staged_share_kernel<<<grid_for(p->grid + 1, 128), 128, 0, s>>>(p->desc, head, p->grid,
                                                                    p->blk_task);
     CG_LAUNCH_CHECK();
-    CG_CUDA(cudaStreamSynchronize(s));
   }
   p->grid_l2 = (int)std::max<int64_t>(
       1, std::min<int64_t>(p->n_ctiles, (int64_t)di.sm_count * 2));
+  CG_CUDA(cudaStreamSynchronize(s));
+  return CG_OK;
+}
+
+int seg_plan_carries(SegPlan* p, int64_t n) {
+  p->ncarry = n;
+  if (n <= p->carry_cap) return CG_OK;
+  cudaFree(p->first_row);
+  p->first_row = nullptr;
+  p->carry_cap = 0;
+  CG_CUDA(cudaMalloc((void**)&p->first_row, 3 * sizeof(int32_t) * (size_t)n));
+  p->carry_row = p->first_row + n;
+  p->carry = p->first_row + 2 * n;
+  p->carry_cap = n;
   return CG_OK;
 }
 
 void seg_plan_free(SegPlan* p) {
-  cudaFree(p->counter);
-  cudaFree(p->blk_task);
   cudaFree(p->colf);
   cudaFree(p->cs);
   cudaFree(p->desc);
-  cudaFree(p->seg_task);
   cudaFree(p->meta);
-  cudaFree(p->seg_cstart);
-  cudaFree(p->seg_E);
-  cudaFree(p->seg_chunk);
-  cudaFree(p->seg_ctile);
-  cudaFree(p->seg_lo);
-  cudaFree(p->seg_tab);
   cudaFree(p->first_row);
-  cudaFree(p->carry);
-  cudaFree(p->fx_pieces);
-  cudaFree(p->fx_runs);
-  cudaFree(p->fx_sum);
-  cudaFree(p->fx_done);
   *p = SegPlan();
 }
 
 int64_t seg_plan_bytes(const SegPlan& p) {
-  return 4 * p.colf_len + p.cs_cap + 16 * p.desc_cap + 4 * (p.chunk_cap + p.carry_cap) +
-         76 * (int64_t)p.k + 20 * p.fx_npieces +
-         20 * p.fx_nruns;
+  return 4 * p.colf_len + p.cs_cap + 16 * p.desc_cap + 12 * p.carry_cap +
+         76 * (int64_t)p.k;
 }
 
 int seg_plan_export_col(const SegPlan& p, const int32_t* rp, int32_t* col, cudaStream_t s) {
@@ -877,10 +809,9 @@ int run_seg_gather(const SegPlan& p, const typename Op::T* x, int32_t nx, typena
         p.k, 0, (int32_t)p.n_ctiles, out, reinterpret_cast<T*>(p.carry));
     CG_LAUNCH_CHECK();
   }
-  if ((phases & kPhaseFixup) && p.fx_npieces > 0) {
-    seg_fixup_kernel<Op><<<grid_for(p.fx_npieces, 256, 4), 256, 0, s>>>(
-        p.fx_pieces, p.fx_npieces, p.fx_runs, reinterpret_cast<const T*>(p.carry),
-        reinterpret_cast<T*>(p.fx_sum), p.fx_done, out);
+  if ((phases & kPhaseFixup) && p.ncarry > 0) {
+    seg_fixup_kernel<Op><<<grid_for(p.ncarry, 256, 8), 256, 0, s>>>(
+        p.carry_row, reinterpret_cast<const T*>(p.carry), p.ncarry, out);
     CG_LAUNCH_CHECK();
   }
   return CG_OK;

@@ -49,19 +49,20 @@ struct SegPlan {
   int32_t head_tasks = 0;          // tasks of the segments [0, m)
   int32_t* blk_task = nullptr;     // [grid+1] first task of each staged block's range
   int64_t colf_len = 0;
+  int64_t* meta = nullptr;         // one allocation: row_base, edge_base, cstart, bounds (k+1
+                                   // each), then the segments' arrays below
   int64_t* seg_cstart = nullptr;   // [k]   first colf entry of each segment
   int32_t* seg_E = nullptr;        // [k]   edges of each segment
   int64_t* seg_chunk = nullptr;    // [k+1] first global chunk of each segment
   int32_t* seg_ctile = nullptr;    // [k+1] first L1/L2 block-group of each segment
   int32_t* seg_lo = nullptr;       // [k]   first source of each segment
   int32_t* seg_tab = nullptr;      // [k]   table entries used for each segment
+  // carries: one per L1/L2 chunk, then one per full piece of a long staged row; one allocation
   int32_t* first_row = nullptr;    // subgraph row of each L1/L2 chunk's first edge
-  void* carry = nullptr;           // [carry_cap] 4-byte values: the L1/L2 chunks', then the
-                                   // full pieces' of long staged rows
-  int64_t carry_cap = 0;
-  int64_t* meta = nullptr;         // [4(k+1)] row_base, edge_base, cstart, bounds (device)
+  int32_t* carry_row = nullptr;    // [ncarry] the row a carry belongs to (-1: none)
+  void* carry = nullptr;           // [ncarry] 4-byte values
+  int64_t ncarry = 0, carry_cap = 0;
   const int32_t* rp32 = nullptr;   // subgraph row starts (owned by the handle)
-  int64_t chunk_cap = 0;           // capacity of first_row
   std::vector<int64_t> h_cstart, src_bounds, edge_base, row_base;
   int threads = 1024;       // staged-segment launch shape
   int ctas_per_sm = 1;
@@ -79,25 +80,19 @@ struct SegPlan {
   int overlap_request = 0;  // warps per block given to the L1/L2 segments (0: two launches)
   int overlap = 0;          // the same, in effect (0 when one kind of segment is absent)
   int grid_l2 = 0;          // unstaged launch blocks (1024 threads, 2 per SM)
-  // rows spanning chunks: runs of carries (a static structure) cut into
-  // pieces of <= 32 chunks, completed in parallel (see run_seg_gather)
-  int4* fx_pieces = nullptr;   // [fx_npieces] (first chunk, chunks, run, -)
-  int4* fx_runs = nullptr;     // [fx_nruns] (row, first piece, pieces, -)
-  void* fx_sum = nullptr;      // [fx_npieces] 4-byte piece sums
-  unsigned* fx_done = nullptr; // [fx_nruns] finished pieces per run
-  int64_t fx_npieces = 0, fx_nruns = 0;
 };
 
 // Largest shared table (entries, multiple of 32) for `ctas` blocks per SM.
 int seg_table_capacity(int ctas);
 
-// Build colf, the chunk index and the carry buffers from the unpadded
-// segmented CSR (col[E] int32 global sources, rp[rows+1] int64 row starts;
-// rp32: the same row starts in int32, kept by the handle).  Synchronizes.
-int seg_plan_build(const int32_t* col, const int64_t* rp, const int32_t* rp32, int64_t rows,
-                   int64_t E, int k, const std::vector<int64_t>& row_base,
-                   const std::vector<int64_t>& edge_base, const std::vector<int64_t>& src_bounds,
-                   SegPlan* p, cudaStream_t s);
+// Allocate a plan for E edges in k segments (colf and the segments' arrays;
+// the caller fills colf and meta's row_base), then, with the rows known (rp32:
+// their first edges, kept by the handle), choose the default launch shape.
+// Both synchronize.
+int seg_plan_alloc(int64_t E, int k, const std::vector<int64_t>& edge_base,
+                   const std::vector<int64_t>& src_bounds, SegPlan* p, cudaStream_t s);
+int seg_plan_finish(SegPlan* p, const int32_t* rp32, int64_t rows,
+                    const std::vector<int64_t>& row_base, cudaStream_t s);
 
 // Launch shape: threads per block (512 or 1024), blocks per SM, table size
 // (-1: the capacity; 0: none).  Synchronizes the stream.
@@ -105,11 +100,12 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
                        cudaStream_t s);
 
 // Lay out the staged segments [0, m2): their tasks, descriptors and stream (pad:
-// the table entry that holds the identity).  extra_row: the rows of the full
-// pieces of rows longer than kStagedMost, whose carry slots start at
-// carry_base.  Synchronizes.
-int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base,
-                 std::vector<int32_t>* extra_row, cudaStream_t s);
+// the table entry that holds the identity).  The carries of the full pieces of
+// rows longer than kStagedMost follow the first carry_base ones; their rows are
+// written to carry_row.  Synchronizes.
+int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s);
+// Room for n carries (their contents are lost when it grows).
+int seg_plan_carries(SegPlan* p, int64_t n);
 
 void seg_plan_free(SegPlan* p);
 int64_t seg_plan_bytes(const SegPlan& p);

@@ -172,22 +172,24 @@ staged_fill_kernel(const uint32_t* __restrict__ colf, const int32_t* __restrict_
 
 }  // namespace
 
-int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base,
-                 std::vector<int32_t>* extra_row, cudaStream_t s) {
+int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s) {
   const int k = p->k;
   const int64_t rows = p->row_base[m2];
-  extra_row->clear();
   p->h_seg_task.assign(k + 1, 0);
-  if (!p->seg_task) CG_CUDA(cudaMalloc((void**)&p->seg_task, sizeof(int32_t) * (size_t)(k + 1)));
   if (rows == 0) {
     CG_CUDA(cudaMemsetAsync(p->seg_task, 0, sizeof(int32_t) * (size_t)(k + 1), s));
-    return CG_OK;
+    return seg_plan_carries(p, carry_base);
   }
   std::vector<int64_t> wbase(m2 + 1, 0);
   for (int q = 0; q < m2; ++q)
     wbase[q + 1] = wbase[q] + ceil_div(p->row_base[q + 1] - p->row_base[q], kStagedWindow);
   const int64_t nb = wbase[m2] << kClassBits;
-  Scratch tmp(s);
+  const int64_t edges = p->edge_base[m2];
+  const int64_t most = rows + edges / kStagedMost;  // rows and at most their full pieces
+  Scratch tmp(s, 6 * Scratch::round(4 * (size_t)most) + sort_scratch(most) +
+                     3 * Scratch::round(8 * (size_t)(nb + 1)) + 2 * Scratch::round(4 * (size_t)nb) +
+                     2 * scan_scratch(nb) + Scratch::round(8 * (size_t)(rows + 1)) +
+                     scan_scratch(rows) + Scratch::round(8 * (size_t)(m2 + 1)) + 4096);
   int64_t *d_wbase = nullptr, *pos = nullptr, *start = nullptr, *task_base = nullptr,
           *unit_base = nullptr;
   uint32_t *key = nullptr, *skey = nullptr;
@@ -200,9 +202,6 @@ int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base,
   CG_CUDA(cudaMemcpyAsync(d_wbase, wbase.data(), sizeof(int64_t) * (m2 + 1),
                           cudaMemcpyHostToDevice, s));
   CG_CUDA(cudaMemsetAsync(total, 0, sizeof(unsigned long long), s));
-  // an upper bound of the full pieces sizes the sort's arrays
-  const int64_t edges = p->edge_base[m2];
-  const int64_t most = rows + edges / kStagedMost;
   CG_CUDA(tmp.get(&key, most));
   CG_CUDA(tmp.get(&skey, most));
   CG_CUDA(tmp.get(&val, most));
@@ -213,22 +212,20 @@ int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base,
   unsigned long long nx = 0;
   CG_CUDA(cudaMemcpyAsync(&nx, total, sizeof(nx), cudaMemcpyDeviceToHost, s));
   CG_CUDA(cudaStreamSynchronize(s));
-  CG_CUDA(tmp.get(&xrow, nx));
+  CG_TRY(seg_plan_carries(p, carry_base + (int64_t)nx));
+  xrow = p->carry_row + carry_base;
   CG_CUDA(tmp.get(&xpiece, nx));
   if (nx > 0) {
     CG_CUDA(tmp.get(&pos, rows + 1));
-    CG_TRY(exclusive_scan_i32_to_i64(nfull, pos, rows, s));
+    CG_TRY(exclusive_scan_i32_to_i64(nfull, pos, rows, s, &tmp));
     staged_extra_kernel<<<grid_for(rows, 256), 256, 0, s>>>(nfull, pos, rows, key, val, xrow,
                                                             xpiece);
     CG_LAUNCH_CHECK();
-    extra_row->resize(nx);
-    CG_CUDA(cudaMemcpyAsync(extra_row->data(), xrow, sizeof(int32_t) * nx,
-                            cudaMemcpyDeviceToHost, s));
   }
   const int64_t n = rows + (int64_t)nx;
   int bits = kClassBits;
   while (bits < 32 && ((int64_t)1 << bits) < nb) ++bits;
-  CG_TRY(radix_sort_pairs(key, val, skey, item, n, bits, s));
+  CG_TRY(radix_sort_pairs(key, val, skey, item, n, bits, s, &tmp));
   CG_CUDA(tmp.get(&start, nb + 1));
   CG_CUDA(tmp.get(&tasks, nb));
   CG_CUDA(tmp.get(&units, nb));
@@ -236,8 +233,8 @@ int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base,
   CG_CUDA(tmp.get(&unit_base, nb + 1));
   staged_bucket_kernel<<<grid_for(nb + 1, 256), 256, 0, s>>>(skey, n, nb, start, tasks, units);
   CG_LAUNCH_CHECK();
-  CG_TRY(exclusive_scan_i32_to_i64(tasks, task_base, nb, s));
-  CG_TRY(exclusive_scan_i32_to_i64(units, unit_base, nb, s));
+  CG_TRY(exclusive_scan_i32_to_i64(tasks, task_base, nb, s, &tmp));
+  CG_TRY(exclusive_scan_i32_to_i64(units, unit_base, nb, s, &tmp));
   staged_seg_task_kernel<<<grid_for(k + 1, 128), 128, 0, s>>>(task_base, d_wbase, m2, k,
                                                               p->seg_task);
   CG_LAUNCH_CHECK();
@@ -267,7 +264,6 @@ int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base,
       rows, xrow, xpiece, start, task_base, unit_base, (int)nb, ntasks, pad, carry_base, p->desc,
       p->cs);
   CG_LAUNCH_CHECK();
-  CG_CUDA(cudaStreamSynchronize(s));  // wbase and the copies into extra_row
   return CG_OK;
 }
 
