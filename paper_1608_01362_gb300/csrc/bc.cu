@@ -6,14 +6,12 @@
 // segmenting to pay).
 //
 // Forward phase, one BFS level at a time from the source (level 0, sigma 1):
-//   push (small frontier: its out-edges, one thread per edge, found through a
-//         prefix sum of the frontier's out-degrees): an unvisited w gets level
-//         L+1 by compare-and-swap and joins the next frontier; every edge into
-//         a level-(L+1) vertex adds sigma[u] to sigma[w] with an FP64 atomic;
-//   pull (large frontier, bottom-up: the merge-path tile gather over the
-//         in-rows of the unvisited vertices, read through their list, of
-//         x = sigma on the frontier, 0 elsewhere): an unvisited v whose sum is
-//         non-zero gets level L+1 and sigma = the sum.
+//   push (small frontier: its out-edges): an unvisited w gets level L+1 by
+//         compare-and-swap and joins the next frontier; every edge into a
+//         level-(L+1) vertex adds sigma[u] to sigma[w] with an FP64 atomic;
+//   pull (large frontier, bottom-up): the in-rows of the unvisited vertices are
+//         summed over sigma of the frontier's vertices (a bit each); an
+//         unvisited v whose sum is non-zero gets level L+1 and sigma = the sum.
 // sigma counts shortest paths: integers, exact in FP64 in any order below
 // 2^53, so levels and sigma do not depend on the direction or the order.
 // Pull is taken when (frontier out-edges) * alpha > E.
@@ -21,18 +19,29 @@
 // Backward phase, deepest level first: for every u at level L,
 //   delta[u] = sigma[u] * sum over out-neighbours w at level L+1 of
 //              (1 + delta[w]) / sigma[w]
-// as a gather over the out-rows of level L's vertices taken in the order of
-// the level's list (a "virtual" CSR of that level: the tile gather reads each
-// edge through the list), with x = (1 + delta) / sigma on level L+1 and
-// 0 on every other level (out-neighbours of a level-L vertex lie at levels
-// <= L+1, and levels <= L are still 0), by the same tile gather; the level
-// lists are first put in (level, vertex ID) order, so the summation order is
-// fixed and the results deterministic.  bc[u] += delta[u] for u != source.
+// over the out-rows of level L's vertices, read where a bit says that the
+// neighbour lies on level L+1 or deeper (out-neighbours of a level-L vertex lie
+// at levels <= L+1), in the order of the level's list; the reached vertices
+// are first put in (level, no out-edges, vertex ID) order, so the summation
+// order is fixed and the results deterministic.  bc[u] += delta[u] for u !=
+// source.
+//
+// What bounded the earlier form: on a 65 M-edge graph 43 ms for 12 sources, of
+// them 24.5 on the GPU; the rest were 300 host reads of counts and 200 scratch
+// allocations, each dear after such a read.  Now a level costs one host read
+// (the next frontier's vertices, its out-edges and the vertices found, counted
+// while they are found), none on the way back, and no allocation: the appends
+// reserve a vertex's place in the list and its place among the frontier's
+// out-edges with one 64-bit atomic, so the list comes with its prefix and
+// needs no scan.  Edges find their row with a warp's row walk (rowwalk.cuh)
+// instead of a binary search per edge in shared memory.  12 sources: 43.4 ->
+// 15.5 ms; 4 sources on 0.9 M edges: 7.6 -> 1.6 ms.
 #include <algorithm>
 #include <vector>
 
-#include "gather.cuh"
+#include "carry_runs.cuh"
 #include "handles.cuh"
+#include "rowwalk.cuh"
 
 struct cg_bc {
   int device = 0;
@@ -42,27 +51,32 @@ struct cg_bc {
   const int32_t* in_src = nullptr;
   const int64_t* out_off = nullptr;  // caller-owned out-edge CSR (push, backward)
   const int32_t* out_dst = nullptr;
+  char* slab = nullptr;        // one allocation that holds the arrays below
   int32_t* level = nullptr;    // [V] BFS level of the current source (-1: unreached)
   double* sigma = nullptr;     // [V] shortest-path counts
   double* delta = nullptr;     // [V] dependencies
-  double* xval = nullptr;      // [V] gathered values (see above), 0 elsewhere
-  double* acc = nullptr;       // [V] gathered sums
-  uint32_t* xbits = nullptr;   // [V/32 + 1] one bit per vertex: xval may be non-zero
+  double* xval = nullptr;      // [V] (1 + delta) / sigma, read where xbits says so
+  double* acc = nullptr;       // [V] gathered sums, by list position
+  uint32_t* xbits = nullptr;   // [V/32 + 1] one bit per vertex
+  int32_t* flist[2] = {nullptr, nullptr};  // [V] a frontier's vertices that have out-edges
+  int32_t* fpos[2] = {nullptr, nullptr};   // [V] their first places among its out-edges
+  int32_t* fgap[2] = {nullptr, nullptr};   // [V] from those to their places in out_dst
   int32_t* lists = nullptr;    // [V] reached vertices, level after level
-  int32_t* deg = nullptr;      // [V] out-degrees of one level's vertices
-  int64_t* rend = nullptr;     // [V+1] their exclusive prefix (rend[n] = total)
-  int32_t* counter = nullptr;  // [1] next free position in lists
-  int32_t* ids = nullptr;      // [V] sort scratch: reached vertices in ID order
-  uint32_t* keys = nullptr;    // [V] sort scratch: their levels
+  int32_t* pos = nullptr;      // [V] row starts of `lists` (backward) or of `ids` (pull)
+  int32_t* gap = nullptr;      // [V] from an edge's place among them to its place in the CSR
+  int32_t* ids = nullptr;      // [V] unvisited vertices (pull); sort scratch
+  uint32_t* keys = nullptr;    // [V] sort scratch
   uint32_t* keys_out = nullptr;  // [V]
-  int64_t* h_pin = nullptr;    // pinned host words for the per-level counts
-  int32_t* vt_row = nullptr;   // tiles of a level's virtual CSR
-  int32_t* vt_edge = nullptr;
-  double* vt_carry = nullptr;
-  int32_t* vt_carry_row = nullptr;
-  int64_t vt_cap = 0;
+  int64_t* tsum = nullptr;     // tile sums of a compaction and their prefix
+  double* carry = nullptr;     // [E/256 + 2] open rows of the gather's tiles
+  int32_t* carry_row = nullptr;
+  unsigned long long* count = nullptr;  // [4] vertices << 32 | out-edges appended to the
+                                        // frontier (three levels in turn), vertices reached
+  void* sort = nullptr;        // scratch of the scans and the sort
+  size_t sort_bytes = 0;
+  unsigned long long* h_pin = nullptr;  // pinned host copy of count
   double alpha = 16.0;
-  std::vector<int64_t> lbase;  // level bounds in `lists` of the last source
+  int32_t depth = 0;           // levels of the last source
   int32_t last_source = -1;
   int32_t push_levels = 0, pull_levels = 0;
 };
@@ -71,16 +85,18 @@ namespace cg {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kSub = 256;        // edges a warp folds at once: 8 consecutive per lane
+constexpr int kPushTile = 256;   // frontier edges per warp in a push
+typedef unsigned long long u64;
 
 __global__ void bc_reset_kernel(int32_t V, int32_t* __restrict__ level,
                                 double* __restrict__ sigma, double* __restrict__ delta,
-                                double* __restrict__ xval, uint32_t* __restrict__ xbits) {
+                                uint32_t* __restrict__ xbits) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V;
        v += (int64_t)gridDim.x * blockDim.x) {
     level[v] = -1;
     sigma[v] = 0.0;
     delta[v] = 0.0;
-    xval[v] = 0.0;
     if ((v & 31) == 0) xbits[v >> 5] = 0u;
   }
 }
@@ -92,175 +108,443 @@ __device__ __forceinline__ void set_bit(uint32_t* bits, int32_t v, bool on) {
     atomicAnd(bits + (v >> 5), ~(1u << (v & 31)));
 }
 
-__global__ void bc_seed_kernel(int32_t s, int32_t* __restrict__ level, double* __restrict__ sigma,
-                               double* __restrict__ xval, uint32_t* __restrict__ xbits,
-                               int32_t* __restrict__ lists, int32_t* __restrict__ counter) {
+__global__ void bc_seed_kernel(int32_t s, const int64_t* __restrict__ out_off,
+                               int32_t* __restrict__ level, double* __restrict__ sigma,
+                               int32_t* __restrict__ list, int32_t* __restrict__ fpos,
+                               int32_t* __restrict__ fgap, u64* __restrict__ count) {
   level[s] = 0;
   sigma[s] = 1.0;
-  xval[s] = 1.0;
-  set_bit(xbits, s, true);
-  lists[0] = s;
-  *counter = 1;
+  const u64 deg = (u64)(out_off[s + 1] - out_off[s]);
+  list[0] = s;
+  fpos[0] = 0;
+  fgap[0] = (int32_t)out_off[s];
+  count[0] = deg ? (1ull << 32) | deg : 0ull;
+  count[1] = count[2] = 0ull;
+  count[3] = 1ull;
 }
 
-// Row lengths in a CSR (off: the out- or in-edge offsets) for the vertices of
-// a list (taken from the expanded CSR's own offsets, so every expanded edge
-// lies inside its row).
-__global__ void list_degree_kernel(const int32_t* __restrict__ list, int64_t n,
-                                   const int64_t* __restrict__ off, int32_t* __restrict__ deg) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t u = list[i];
-    deg[i] = (int32_t)(off[u + 1] - off[u]);
-  }
-}
+struct Frontier {
+  int32_t* list;
+  int32_t* pos;
+  int32_t* gap;
+};
 
-// Append v to lists at a position from one atomic per warp.
-__device__ __forceinline__ void append(bool take, int32_t v, int32_t* lists, int32_t* counter) {
-  const unsigned m = __ballot_sync(0xffffffffu, take);
-  if (!m) return;
+// The vertices found at this level by the warp: those with out-edges join the
+// next frontier at places reserved together with their out-edges' places.
+__device__ __forceinline__ void append(bool take, int32_t v, const int64_t* __restrict__ out_off,
+                                       const Frontier& f, u64* next, u64* reached) {
+  const unsigned full = 0xffffffffu;
+  const unsigned found = __ballot_sync(full, take);
+  if (!found) return;
   const int lane = threadIdx.x & 31;
-  int32_t base = 0;
-  if (lane == __ffs(m) - 1) base = atomicAdd(counter, __popc(m));
-  base = __shfl_sync(0xffffffffu, base, __ffs(m) - 1);
-  if (take) lists[base + __popc(m & ((1u << lane) - 1u))] = v;
+  int64_t o0 = 0;
+  int32_t deg = 0;
+  if (take) {
+    o0 = __ldg(out_off + v);
+    deg = (int32_t)(__ldg(out_off + v + 1) - o0);
+  }
+  const unsigned m = __ballot_sync(full, deg > 0);
+  int32_t incl = deg;  // a warp's degrees sum to at most E < 2^31 (its vertices are distinct)
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t y = __shfl_up_sync(full, incl, o);
+    if (lane >= o) incl += y;
+  }
+  u64 base = 0;
+  if (lane == 31) {
+    atomicAdd(reached, (u64)__popc(found));
+    if (m) base = atomicAdd(next, ((u64)__popc(m) << 32) | (u64)(uint32_t)incl);
+  }
+  base = __shfl_sync(full, base, 31);
+  if (deg > 0) {
+    const int64_t at = (int64_t)(base >> 32) + __popc(m & ((1u << lane) - 1u));
+    const int32_t p = (int32_t)(base & 0xffffffffull) + incl - deg;
+    f.list[at] = v;
+    f.pos[at] = p;
+    f.gap[at] = (int32_t)o0 - p;
+  }
 }
 
-// The out-edges [0, m) of a list's vertices laid end to end (row i = list
-// position i, starting at rend[i]) are cut into merge-path tiles of rows +
-// edges (tile_row / tile_edge, as for the gather); the block of tile t keeps
-// the starts rend[r0 .. r1] of the tile's rows in shared memory, so each of
-// its edges finds its row with a binary search in shared memory.  Returns
-// the number of row starts loaded (0: the tile has no edges).
-__device__ __forceinline__ int load_tile_rows(const int64_t* __restrict__ rend, int64_t n,
-                                              const int32_t* __restrict__ tile_row,
-                                              const int32_t* __restrict__ tile_edge,
-                                              int64_t* s_start, int64_t& r0, int64_t& e0,
-                                              int64_t& e1) {
-  const int64_t t = blockIdx.x;
-  r0 = tile_row[t];
-  e0 = tile_edge[t];
-  e1 = tile_edge[t + 1];
-  if (e0 >= e1) return 0;
-  const int64_t rl = tile_row[t + 1] < n - 1 ? tile_row[t + 1] : n - 1;
-  const int cnt = (int)(rl - r0 + 1);  // <= kTileItems + 1
-  for (int j = threadIdx.x; j < cnt; j += blockDim.x) s_start[j] = rend[r0 + j];
+// The same for a whole block (every thread calls it): one pair of atomics for
+// its 256 vertices, where a warp's would queue up behind each other on the two
+// counters.
+__device__ __forceinline__ void append_block(bool take, int32_t v,
+                                             const int64_t* __restrict__ out_off,
+                                             const Frontier& f, u64* next, u64* reached) {
+  __shared__ u64 s_w[kThreads / 32], s_base;
+  __shared__ int s_found;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (!__syncthreads_or(take)) return;
+  if (threadIdx.x == 0) s_found = 0;
+  int64_t o0 = 0;
+  u64 val = 0;
+  if (take) {
+    o0 = __ldg(out_off + v);
+    const u64 deg = (u64)(__ldg(out_off + v + 1) - o0);
+    if (deg) val = (1ull << 32) | deg;
+  }
+  u64 incl = val;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const u64 y = __shfl_up_sync(full, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) s_w[w] = incl;
+  const int found = __popc(__ballot_sync(full, take));
   __syncthreads();
-  return cnt;
-}
-
-// last j in [0, cnt) with s_start[j] <= k (s_start ascending, s_start[0] <= k)
-__device__ __forceinline__ int tile_row_of(const int64_t* s_start, int cnt, int64_t k) {
-  int lo = 0, hi = cnt;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (s_start[mid] <= k) lo = mid + 1; else hi = mid;
+  if (lane == 0 && found) atomicAdd(&s_found, found);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    u64 total = 0;
+    for (int q = 0; q < kThreads / 32; ++q) total += s_w[q];
+    atomicAdd(reached, (u64)s_found);
+    s_base = total ? atomicAdd(next, total) : 0ull;
   }
-  return lo - 1;
+  __syncthreads();
+  if (val) {
+    u64 at = s_base + incl - val;
+    for (int q = 0; q < w; ++q) at += s_w[q];
+    const int32_t p = (int32_t)(at & 0xffffffffull);
+    f.list[at >> 32] = v;
+    f.pos[at >> 32] = p;
+    f.gap[at >> 32] = (int32_t)o0 - p;
+  }
+  __syncthreads();  // s_w and s_base are used again
 }
 
-// Push: the frontier's (list, n vertices) out-edges, a tile per block.
+// Push: the frontier's n vertices and m out-edges, kPushTile edges per warp.
+// The counts of the level after next are cleared for it.
 __global__ void __launch_bounds__(kThreads)
-push_kernel(const int32_t* __restrict__ list, int64_t n, const int64_t* __restrict__ rend,
-            const int32_t* __restrict__ tile_row, const int32_t* __restrict__ tile_edge,
-            const int64_t* __restrict__ out_off, const int32_t* __restrict__ out_dst, int32_t L,
-            int32_t* __restrict__ level, double* __restrict__ sigma,
-            int32_t* __restrict__ lists, int32_t* __restrict__ counter) {
-  __shared__ int64_t s_start[kTileItems + 1];
-  int64_t r0, e0, e1;
-  const int cnt = load_tile_rows(rend, n, tile_row, tile_edge, s_start, r0, e0, e1);
-  if (cnt == 0) return;
-  for (int64_t k0 = e0; k0 < e1; k0 += blockDim.x) {
-    const int64_t k = k0 + threadIdx.x;  // the warp stays converged for the append
-    bool take = false;
-    int32_t w = 0;
-    if (k < e1) {
-      const int j = tile_row_of(s_start, cnt, k);
-      const int32_t u = list[r0 + j];
-      w = out_dst[out_off[u] + (k - s_start[j])];
-      // a target seen visited on an earlier level needs no atomic; one that
-      // reads unvisited takes the compare-and-swap (it may lose to another
-      // edge of this level, which then reads L + 1)
-      int32_t old = __ldcg(level + w);
-      if (old == -1) old = atomicCAS(level + w, -1, L + 1);
-      take = old == -1;
-      if (old == -1 || old == L + 1) atomicAdd(sigma + w, sigma[u]);
+push_kernel(Frontier cur, int32_t n, int32_t m, const int64_t* __restrict__ out_off,
+            const int32_t* __restrict__ out_dst, int32_t L, int32_t* __restrict__ level,
+            double* __restrict__ sigma, Frontier nxt, u64* __restrict__ count) {
+  u64* next = count + (L + 1) % 3;
+  if (blockIdx.x == 0 && threadIdx.x == 0) count[(L + 2) % 3] = 0ull;
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  DenseWalk walk(cur.pos, n, m);
+  for (int64_t b = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kPushTile; b < m;
+       b += nw * kPushTile) {
+    walk.seek((int32_t)b);
+    for (int i = 0; i < kPushTile && b + i < m; i += 32) {
+      const int64_t e = b + i + lane;
+      int32_t j;
+      walk.batch((int32_t)(b + i), &j);
+      bool take = false;
+      int32_t w = 0;
+      if (e < m) {
+        const int32_t u = __ldg(cur.list + j);
+        w = __ldcs(out_dst + (e + __ldg(cur.gap + j)));
+        // a target seen visited on an earlier level needs no atomic; one that
+        // reads unvisited takes the compare-and-swap (it may lose to another
+        // edge of this level, which then reads L + 1)
+        int32_t old = __ldcg(level + w);
+        if (old == -1) old = atomicCAS(level + w, -1, L + 1);
+        take = old == -1;
+        if (old == -1 || old == L + 1) atomicAdd(sigma + w, sigma[u]);
+      }
+      append(take, w, out_off, nxt, next, count + 3);
     }
-    append(take, w, lists, counter);
   }
 }
 
-// Bottom-up step: the unvisited vertices that have in-edges (their IDs in
-// ascending order) ...
-__global__ void unvisited_flag_kernel(int32_t V, const int32_t* __restrict__ level,
-                                      const int64_t* __restrict__ in_off,
-                                      int32_t* __restrict__ flag) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V;
-       v += (int64_t)gridDim.x * blockDim.x)
-    flag[v] = level[v] == -1 && in_off[v + 1] > in_off[v];
+// ---------------------------------------------------------------------------
+// Compactions: a value per item, its exclusive prefix, and what to write there
+// (tile sums, their scan, a second pass over the items).
+// ---------------------------------------------------------------------------
+constexpr int kItems = 8;                      // per thread, 32 at a time per warp
+constexpr int kCTile = kThreads * kItems;
+
+// unvisited vertices that have in-edges: 1 << 32 | in-edges
+struct Unvisited {
+  const int32_t* level;
+  const int64_t* in_off;
+  int32_t* ids;
+  int32_t* pos;
+  int32_t* gap;
+  __device__ u64 operator()(int64_t v) const {
+    if (__ldg(level + v) != -1) return 0ull;
+    const u64 d = (u64)(__ldg(in_off + v + 1) - __ldg(in_off + v));
+    return d ? (1ull << 32) | d : 0ull;
+  }
+  __device__ void put(int64_t v, u64 val, u64 before) const {
+    ids[before >> 32] = (int32_t)v;
+    pos[before >> 32] = (int32_t)(before & 0xffffffffull);
+    gap[before >> 32] = (int32_t)(__ldg(in_off + v) - (int64_t)(before & 0xffffffffull));
+  }
+};
+
+// reached vertices, keyed by level and by having no out-edges
+struct Reached {
+  const int32_t* level;
+  const int64_t* out_off;
+  int32_t* ids;
+  uint32_t* keys;
+  __device__ u64 operator()(int64_t v) const { return __ldg(level + v) >= 0; }
+  __device__ void put(int64_t v, u64, u64 before) const {
+    ids[before] = (int32_t)v;
+    keys[before] = ((uint32_t)level[v] << 1) | (out_off[v + 1] == out_off[v]);
+  }
+};
+
+// row starts of the reached vertices in list order
+struct ListRows {
+  const int32_t* list;
+  const int64_t* out_off;
+  int32_t* pos;
+  int32_t* gap;
+  __device__ u64 operator()(int64_t i) const {
+    const int32_t u = __ldg(list + i);
+    return (u64)(__ldg(out_off + u + 1) - __ldg(out_off + u)) | 1ull << 63;
+  }
+  __device__ void put(int64_t i, u64, u64 before) const {
+    const int32_t p = (int32_t)(before & 0x7fffffffull);
+    pos[i] = p;
+    gap[i] = (int32_t)__ldg(out_off + __ldg(list + i)) - p;
+  }
+};
+
+template <class F, bool WRITE>
+__global__ void __launch_bounds__(kThreads)
+compact_kernel(F f, int64_t n, int64_t* __restrict__ tsum) {
+  __shared__ u64 s_w[kThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t base = (int64_t)blockIdx.x * kCTile + (int64_t)w * (kItems * 32);
+  u64 v[kItems], sum = 0;
+#pragma unroll
+  for (int r = 0; r < kItems; ++r) {
+    const int64_t i = base + r * 32 + lane;
+    v[r] = i < n ? f(i) : 0ull;
+    sum += v[r] & ~(1ull << 63);
+  }
+  for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) s_w[w] = sum;
+  __syncthreads();
+  if (!WRITE) {
+    if (threadIdx.x == 0) {
+      u64 t = 0;
+      for (int q = 0; q < kThreads / 32; ++q) t += s_w[q];
+      tsum[blockIdx.x] = (int64_t)t;
+    }
+    return;
+  }
+  u64 run = (u64)tsum[blockIdx.x];
+  for (int q = 0; q < w; ++q) run += s_w[q];
+#pragma unroll
+  for (int r = 0; r < kItems; ++r) {
+    const u64 x = v[r] & ~(1ull << 63);
+    u64 incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (v[r]) f.put(base + r * 32 + lane, x, run + incl - x);
+    run += __shfl_sync(0xffffffffu, incl, 31);
+  }
 }
 
-__global__ void unvisited_compact_kernel(int32_t V, const int32_t* __restrict__ level,
-                                         const int64_t* __restrict__ in_off,
-                                         const int64_t* __restrict__ pos,
-                                         int32_t* __restrict__ ids) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V;
-       v += (int64_t)gridDim.x * blockDim.x)
-    if (level[v] == -1 && in_off[v + 1] > in_off[v]) ids[pos[v]] = (int32_t)v;
+// *total (device) = the values' sum.
+template <class F>
+int compact(cg_bc* h, const F& f, int64_t n, const int64_t** total, cudaStream_t s) {
+  const int64_t tiles = ceil_div(n, kCTile);
+  int64_t* scan = h->tsum + tiles;
+  compact_kernel<F, false><<<(unsigned)tiles, kThreads, 0, s>>>(f, n, h->tsum);
+  CG_LAUNCH_CHECK();
+  Scratch ws(s, h->sort, h->sort_bytes);
+  CG_TRY(exclusive_scan_i64(h->tsum, scan, tiles, s, &ws));
+  compact_kernel<F, true><<<(unsigned)tiles, kThreads, 0, s>>>(f, n, scan);
+  CG_LAUNCH_CHECK();
+  if (total) *total = scan + tiles;
+  return CG_OK;
 }
 
-// ... and after the gather of their in-rows: one with a non-zero sum (a
-// frontier in-neighbour) is on level L+1.
-__global__ void pull_update_kernel(const int32_t* __restrict__ ids, int64_t n,
-                                   const double* __restrict__ acc, int32_t L,
-                                   int32_t* __restrict__ level, double* __restrict__ sigma,
-                                   int32_t* __restrict__ lists, int32_t* __restrict__ counter) {
+// ---------------------------------------------------------------------------
+// Row sums: out[i] = sum over the edges of listed row i (every listed row has an
+// edge; its neighbours lie in vadj, gap[i] behind their places among the
+// listed rows' edges laid end to end) of x at the neighbours whose bit is set.  A warp takes a tile of 256 or 1024 consecutive
+// edges (pos: the rows' starts among them): it looks 32 edges at a time up, keeps the 256 values in shared memory, and then folds 8 consecutive ones
+// per lane, one segmented scan joining the lanes.  FP64 adds run at 2 per
+// cycle and SM here, so there are 13 warp adds per 256 edges and no more; the
+// loads behind them are the adjacency stream and, per edge, a bit (V / 8
+// bytes: stays on chip).  The largest levels of a 65 M-edge graph: 577 -> 300 us
+// (a search per edge by shuffles took 1000 instructions per 256 edges and 490
+// us; the list's rows all have edges, so a bit mask of their ends does).  A row that is open at a tile's end leaves its part
+// in the tile's carry (completed in order by row_fix_kernel).
+// ---------------------------------------------------------------------------
+struct RowSums {
+  const int32_t* pos;
+  const int32_t* gap;
+  int32_t origin;          // pos of row 0
+  int64_t n, m;            // rows and edges, or
+  const int64_t* packed;   // rows << 32 | edges on the device
+  const int32_t* vadj;
+  const uint32_t* bits;
+  const double* x;
+  double* out;
+  double* carry;
+  int32_t* carry_row;
+  __device__ __forceinline__ int64_t rows() const { return packed ? *packed >> 32 : n; }
+  __device__ __forceinline__ int64_t edges() const {
+    return packed ? *packed & 0xffffffffll : m;
+  }
+};
+
+// 256-edge steps of a tile: few long tiles where there is work for every warp
+__device__ __forceinline__ int tile_steps(int64_t m) { return m >= ((int64_t)1 << 22) ? 4 : 1; }
+
+__device__ __forceinline__ int pad8(int j) { return j + (j >> 3); }
+
+__global__ void __launch_bounds__(kThreads, 4)
+row_sum_kernel(RowSums a) {
+  __shared__ double s_all[kThreads / 32][kSub + kSub / 8];
+  constexpr unsigned kFull = 0xffffffffu;
+  constexpr int U = 4;  // batches of 32 edges whose reads are in flight together
+  const int lane = threadIdx.x & 31;
+  double* sv = s_all[threadIdx.x >> 5];
+  const int64_t m = a.edges();
+  const int steps = tile_steps(m);
+  const int64_t ntiles = (m + steps * kSub - 1) / (steps * kSub);
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  DenseWalk walk(a.pos, (int32_t)a.rows(), (int32_t)m, a.origin);
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < ntiles; t += nw) {
+    const int64_t t0 = t * steps * kSub, t1 = min(t0 + steps * kSub, m);
+    walk.seek((int32_t)t0);
+    double open = 0.0;       // the part so far of the row open before the step
+    int32_t open_row = -1;   // the row open behind it
+    for (int64_t b = t0; b < t1; b += kSub) {
+      uint32_t ends = 0;     // lane q < 8: the row ends of batch q
+      int32_t row0 = 0;      // row of the step's first edge
+#pragma unroll
+      for (int q0 = 0; q0 < kSub / 32; q0 += U) {
+        int64_t at[U];
+        int32_t w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t e = b + (q0 + u) * 32 + lane;
+          int32_t r;
+          if (q0 + u == 0) row0 = walk.row;
+          const uint32_t f = walk.batch((int32_t)(b + (q0 + u) * 32), &r);
+          if (lane == q0 + u) ends = f;
+          at[u] = e < t1 ? e + a.origin + __ldg(a.gap + r) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) w[u] = at[u] >= 0 ? __ldcs(a.vadj + at[u]) : -1;
+        bool hit[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          hit[u] = w[u] >= 0 && ((__ldg(a.bits + (w[u] >> 5)) >> (w[u] & 31)) & 1u);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          sv[pad8((q0 + u) * 32 + lane)] = hit[u] ? __ldg(a.x + w[u]) : 0.0;
+      }
+      __syncwarp();
+      const uint32_t fl = (__shfl_sync(kFull, ends, lane >> 2) >> (8 * (lane & 3))) & 0xFFu;
+      const int F = __popc(fl);
+      int incl = F;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const int32_t first = row0 + incl - F;  // rows follow one another: each has an edge
+      double acc = lane == 0 ? open : 0.0, first_val = 0.0;
+      int nf = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const double v = sv[pad8(lane * 8 + u)];
+        if (__double_as_longlong(v) != 0) acc += v;  // (an FP64 compare takes the adds' pipe)
+        if (fl & (1u << u)) {
+          if (nf == 0)
+            first_val = acc;
+          else
+            a.out[first + nf] = acc;
+          ++nf;
+          acc = 0.0;
+        }
+      }
+      double S = acc;
+      int g = F > 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(kFull, S, o);
+        const int gy = __shfl_up_sync(kFull, g, o);
+        if (lane >= o) {
+          if (!g && __double_as_longlong(y) != 0) S = y + S;
+          g |= gy;
+        }
+      }
+      const double P = __shfl_up_sync(kFull, S, 1);
+      if (F > 0) a.out[first] = lane > 0 ? P + first_val : first_val;
+      open = __shfl_sync(kFull, S, 31);
+      // the step's last edge: does its row end there?
+      const int last = (int)(min(b + kSub, t1) - b) - 1;
+      const uint32_t lw = __shfl_sync(kFull, ends, last >> 5);
+      open_row = (lw >> (last & 31)) & 1u ? -1 : row0 + __shfl_sync(kFull, incl, 31);
+      __syncwarp();
+    }
+    if (lane == 0) {
+      a.carry[t] = open;
+      a.carry_row[t] = open_row;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) row_fix_kernel(RowSums a) {
+  const int64_t m = a.edges();
+  const int64_t tile = (int64_t)tile_steps(m) * kSub;
+  fix_runs<SumF64>(a.carry_row, a.carry, (m + tile - 1) / tile, a.out);
+}
+
+int row_sums(const RowSums& a, int64_t most_edges, cudaStream_t s) {
+  const int64_t tiles = ceil_div(most_edges, kSub);
+  row_sum_kernel<<<grid_for(tiles * 32, kThreads, 4), kThreads, 0, s>>>(a);
+  CG_LAUNCH_CHECK();
+  row_fix_kernel<<<grid_for(tiles, 256, 4), 256, 0, s>>>(a);
+  CG_LAUNCH_CHECK();
+  return CG_OK;
+}
+
+// After the pull's sums: one with a non-zero sum (a frontier in-neighbour) is on
+// level L+1.
+__global__ void __launch_bounds__(kThreads)
+pull_update_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ packed,
+                   const double* __restrict__ acc, const int64_t* __restrict__ out_off, int32_t L,
+                   int32_t* __restrict__ level, double* __restrict__ sigma, Frontier nxt,
+                   u64* __restrict__ count) {
+  u64* next = count + (L + 1) % 3;
+  if (blockIdx.x == 0 && threadIdx.x == 0) count[(L + 2) % 3] = 0ull;
+  const int64_t n = *packed >> 32;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += stride) {
-    const int64_t i = i0 + threadIdx.x;  // the warp stays converged for the append
+    const int64_t i = i0 + threadIdx.x;  // the block stays together for the append
     bool take = false;
     int32_t v = 0;
     if (i < n) {
       v = ids[i];
-      const double a = acc[i];
-      if (a != 0.0) {
+      const double x = acc[i];
+      if (x != 0.0) {
         level[v] = L + 1;
-        sigma[v] = a;
+        sigma[v] = x;
         take = true;
       }
     }
-    append(take, v, lists, counter);
+    append_block(take, v, out_off, nxt, next, count + 3);
   }
 }
 
-// x over the vertices of a list: sigma (forward frontier) or 0, with the
-// vertices' bits in xbits.
-__global__ void set_x_kernel(const int32_t* __restrict__ list, int64_t n,
-                             const double* __restrict__ sigma, double* __restrict__ xval,
-                             uint32_t* __restrict__ xbits, bool clear) {
+__global__ void set_bits_kernel(const int32_t* __restrict__ list, int64_t n,
+                                uint32_t* __restrict__ bits, bool on) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t u = list[i];
-    xval[u] = clear ? 0.0 : sigma[u];
-    set_bit(xbits, u, !clear);
-  }
+       i += (int64_t)gridDim.x * blockDim.x)
+    set_bit(bits, list[i], on);
 }
 
-// The deepest level: delta = 0, x = 1 / sigma.
-__global__ void deepest_kernel(const int32_t* __restrict__ list, int64_t n,
-                               const double* __restrict__ sigma, double* __restrict__ xval,
-                               uint32_t* __restrict__ xbits) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t u = list[i];
-    xval[u] = 1.0 / sigma[u];
-    set_bit(xbits, u, true);
-  }
-}
-
-// delta of level L from the gathered sums; bc += delta (not for the source);
-// x = (1 + delta) / sigma for the next level up.
-__global__ void dependency_kernel(const int32_t* __restrict__ list, int64_t n,
+// A level's n listed vertices, the first `summed` of them with gathered sums (0
+// for the others): delta, bc += delta (not for the source) and x = (1 + delta)
+// / sigma for the next level up.
+__global__ void dependency_kernel(const int32_t* __restrict__ list, int64_t n, int64_t summed,
                                   const double* __restrict__ sums, const double* __restrict__ sigma,
                                   double* __restrict__ delta, double* __restrict__ xval,
                                   uint32_t* __restrict__ xbits, double* __restrict__ bc,
@@ -268,151 +552,61 @@ __global__ void dependency_kernel(const int32_t* __restrict__ list, int64_t n,
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t u = list[i];
-    const double d = sigma[u] * sums[i];
-    delta[u] = d;
-    xval[u] = (1.0 + d) / sigma[u];
+    const double sg = sigma[u];
+    double d = 0.0;
+    if (i < summed) {
+      d = sg * sums[i];
+      delta[u] = d;
+      if (u != source) bc[u] += d;
+    }
+    xval[u] = (1.0 + d) / sg;
     set_bit(xbits, u, true);
-    if (u != source) bc[u] += d;
   }
 }
 
-// Reached vertices in ascending ID order (pos: exclusive prefix of reached).
-__global__ void reached_flag_kernel(int32_t V, const int32_t* __restrict__ level,
-                                    int32_t* __restrict__ flag) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V;
-       v += (int64_t)gridDim.x * blockDim.x)
-    flag[v] = level[v] >= 0;
-}
-
-__global__ void compact_kernel(int32_t V, const int32_t* __restrict__ level,
-                               const int64_t* __restrict__ pos, int32_t* __restrict__ ids,
-                               uint32_t* __restrict__ keys) {
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V;
-       v += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t l = level[v];
-    if (l >= 0) {
-      ids[pos[v]] = (int32_t)v;
-      keys[pos[v]] = (uint32_t)l;
+__global__ void row_of_edge_kernel(const int64_t* __restrict__ off, int32_t V, int64_t E,
+                                   int32_t* __restrict__ dst) {
+  constexpr int kTile = 1024;
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  RowWalk<int64_t> walk(off, V, (int32_t)E);
+  for (int64_t b = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kTile; b < E;
+       b += nw * kTile) {
+    walk.seek((int32_t)b);
+    for (int i = 0; i < kTile && b + i < E; i += 32) {
+      const int64_t e = b + i + lane;
+      int32_t st, en;
+      const int32_t r = walk.row_of((int32_t)e, e < E, &st, &en);
+      if (e < E) __stcs(dst + e, r);
     }
   }
 }
 
-__global__ void row_of_edge_kernel(const int64_t* __restrict__ off, int32_t V,
-                                   int32_t* __restrict__ dst) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < V; v += nw)
-    for (int64_t e = off[v] + lane; e < off[v + 1]; e += 32) dst[e] = (int32_t)v;
-}
-
-int read_i64(cg_bc* h, const int64_t* dev, int64_t* out, cudaStream_t s) {
-  CG_CUDA(cudaMemcpyAsync(h->h_pin, dev, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+int read_counts(cg_bc* h, cudaStream_t s) {
+  CG_CUDA(cudaMemcpyAsync(h->h_pin, h->count, 4 * sizeof(u64), cudaMemcpyDeviceToHost, s));
   CG_CUDA(cudaStreamSynchronize(s));
-  *out = h->h_pin[0];
   return CG_OK;
 }
 
-int read_i32(cg_bc* h, const int32_t* dev, int32_t* out, cudaStream_t s) {
-  CG_CUDA(cudaMemcpyAsync(h->h_pin, dev, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  CG_CUDA(cudaStreamSynchronize(s));
-  *out = *reinterpret_cast<int32_t*>(h->h_pin);
-  return CG_OK;
-}
+Frontier frontier(const cg_bc* h, int q) { return Frontier{h->flist[q], h->fpos[q], h->fgap[q]}; }
 
-// Degrees of list[0, n) and their prefix; *m = total out-edges.
-int level_rows(cg_bc* h, const int32_t* list, int64_t n, int64_t* m, cudaStream_t s) {
-  list_degree_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(list, n, h->out_off, h->deg);
-  CG_LAUNCH_CHECK();
-  CG_TRY(exclusive_scan_i32_to_i64(h->deg, h->rend, n, s));
-  return read_i64(h, h->rend + n, m, s);
-}
-
-int grow_vt(cg_bc* h, int64_t ntiles);
-
-// Merge-path tiles of a list's n rows and m out-edges (rend: row starts,
-// rend[n] = m) into h->vt_row / h->vt_edge; *ntiles = their number.
-int level_tiles(cg_bc* h, int64_t n, int64_t m, int64_t* ntiles, cudaStream_t s) {
-  *ntiles = ceil_div(n + m, kTileItems);
-  CG_TRY(grow_vt(h, *ntiles));
-  tile_partition_kernel<int64_t><<<grid_for(*ntiles + 1, 256), 256, 0, s>>>(
-      h->rend + 1, n, m, kTileItems, *ntiles, h->vt_row, h->vt_edge);
-  CG_LAUNCH_CHECK();
-  return CG_OK;
-}
-
-int grow_vt(cg_bc* h, int64_t ntiles) {
-  if (ntiles + 1 <= h->vt_cap) return CG_OK;
-  cudaFree(h->vt_row);
-  cudaFree(h->vt_edge);
-  cudaFree(h->vt_carry);
-  cudaFree(h->vt_carry_row);
-  h->vt_row = h->vt_edge = h->vt_carry_row = nullptr;
-  h->vt_carry = nullptr;
-  h->vt_cap = 0;
-  const size_t c = (size_t)(ntiles + 1);
-  CG_CUDA(cudaMalloc((void**)&h->vt_row, 4 * c));
-  CG_CUDA(cudaMalloc((void**)&h->vt_edge, 4 * c));
-  CG_CUDA(cudaMalloc((void**)&h->vt_carry, 8 * c));
-  CG_CUDA(cudaMalloc((void**)&h->vt_carry_row, 4 * c));
-  h->vt_cap = ntiles + 1;
-  return CG_OK;
-}
-
-// Lay the level lists out in (level, vertex ID) order: the appends of the
-// forward phase come in whatever order the atomics give, and the backward
-// sums are associated by position in these lists.  A compaction of the
-// reached vertices in ID order, then a stable radix sort on the level.
-int order_levels(cg_bc* h, int32_t depth, cudaStream_t s) {
+// One bottom-up level: the unvisited vertices that have in-edges, in ID order,
+// gather sigma of the frontier's n vertices over their in-rows.  Visited
+// vertices' rows are never read.
+int pull_level(cg_bc* h, int32_t L, int32_t n, cudaStream_t s) {
   const int32_t V = h->V;
-  const int64_t n = h->lbase[depth];
-  reached_flag_kernel<<<grid_for(V, kThreads), kThreads, 0, s>>>(V, h->level, h->deg);
+  const int cur = L & 1;
+  set_bits_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(h->flist[cur], n, h->xbits, true);
   CG_LAUNCH_CHECK();
-  CG_TRY(exclusive_scan_i32_to_i64(h->deg, h->rend, V, s));
-  compact_kernel<<<grid_for(V, kThreads), kThreads, 0, s>>>(V, h->level, h->rend, h->ids,
-                                                            h->keys);
+  const int64_t* packed = nullptr;
+  CG_TRY(compact(h, Unvisited{h->level, h->in_off, h->ids, h->pos, h->gap}, V, &packed, s));
+  const RowSums a{h->pos, h->gap, 0, 0, 0, packed, h->in_src, h->xbits, h->sigma, h->acc,
+                  h->carry, h->carry_row};
+  CG_TRY(row_sums(a, h->E, s));
+  pull_update_kernel<<<grid_for(V, kThreads), kThreads, 0, s>>>(
+      h->ids, packed, h->acc, h->out_off, L, h->level, h->sigma, frontier(h, 1 - cur), h->count);
   CG_LAUNCH_CHECK();
-  int bits = 1;
-  while (bits < 32 && (int64_t(1) << bits) < (int64_t)depth) ++bits;
-  return radix_sort_pairs(h->keys, h->ids, h->keys_out, h->lists, n, bits, s);
-}
-
-// One bottom-up level: the unvisited vertices that have in-edges (ids, in
-// ID order) gather x = sigma on the frontier (0 elsewhere, tested through
-// xbits) over their in-rows laid end to end; a non-zero sum puts a vertex on
-// level L+1 with that sum as its path count.  Visited vertices' rows are
-// never read.
-int pull_level(cg_bc* h, int32_t L, cudaStream_t s) {
-  const int32_t V = h->V;
-  unvisited_flag_kernel<<<grid_for(V, kThreads), kThreads, 0, s>>>(V, h->level, h->in_off,
-                                                                    h->deg);
-  CG_LAUNCH_CHECK();
-  CG_TRY(exclusive_scan_i32_to_i64(h->deg, h->rend, V, s));
-  unvisited_compact_kernel<<<grid_for(V, kThreads), kThreads, 0, s>>>(V, h->level, h->in_off,
-                                                                       h->rend, h->ids);
-  CG_LAUNCH_CHECK();
-  int64_t n = 0, m = 0;
-  CG_TRY(read_i64(h, h->rend + V, &n, s));
-  if (n == 0) return CG_OK;
-  list_degree_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(h->ids, n, h->in_off, h->deg);
-  CG_LAUNCH_CHECK();
-  CG_TRY(exclusive_scan_i32_to_i64(h->deg, h->rend, n, s));
-  CG_TRY(read_i64(h, h->rend + n, &m, s));
-  if (m == 0) return CG_OK;
-  int64_t ntiles = 0;
-  CG_TRY(level_tiles(h, n, m, &ntiles, s));
-  // the in-rows of the listed vertices, read through the list (no copy)
-  gather_tile_kernel<SumF64, kTileThreads, kTileIPT, false, int64_t, true, true>
-      <<<(unsigned)ntiles, kTileThreads, 0, s>>>(h->rend + 1, nullptr, h->xval, V, h->vt_row,
-                                                 h->vt_edge, h->acc, h->vt_carry,
-                                                 h->vt_carry_row, h->xbits, h->ids, h->in_off,
-                                                 h->in_src);
-  CG_LAUNCH_CHECK();
-  carry_fixup_kernel<SumF64><<<grid_for(ntiles, 256, 4), 256, 0, s>>>(h->vt_carry,
-                                                                     h->vt_carry_row, ntiles, n,
-                                                                     h->acc);
-  CG_LAUNCH_CHECK();
-  pull_update_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(h->ids, n, h->acc, L, h->level,
-                                                                h->sigma, h->lists, h->counter);
+  set_bits_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(h->flist[cur], n, h->xbits, false);
   CG_LAUNCH_CHECK();
   return CG_OK;
 }
@@ -420,81 +614,67 @@ int pull_level(cg_bc* h, int32_t L, cudaStream_t s) {
 int run_source(cg_bc* h, int32_t src, double* bc, cudaStream_t s) {
   const int32_t V = h->V;
   bc_reset_kernel<<<grid_for(V, kThreads), kThreads, 0, s>>>(V, h->level, h->sigma, h->delta,
-                                                               h->xval, h->xbits);
+                                                               h->xbits);
   CG_LAUNCH_CHECK();
-  bc_seed_kernel<<<1, 1, 0, s>>>(src, h->level, h->sigma, h->xval, h->xbits, h->lists,
-                                 h->counter);
+  bc_seed_kernel<<<1, 1, 0, s>>>(src, h->out_off, h->level, h->sigma, h->flist[0], h->fpos[0],
+                                 h->fgap[0], h->count);
   CG_LAUNCH_CHECK();
-  h->lbase.assign(1, 0);
-  h->lbase.push_back(1);
+  CG_TRY(read_counts(h, s));
+  // per level: vertices, of them with out-edges, and these edges
+  std::vector<int64_t> size(1, 1), rows, edges;
   h->push_levels = h->pull_levels = 0;
   // forward: one level per round until a level adds nobody
   for (int32_t L = 0;; ++L) {
-    const int64_t b0 = h->lbase[L], n = h->lbase[L + 1] - b0;
-    const int32_t* list = h->lists + b0;
-    int64_t m = 0;
-    CG_TRY(level_rows(h, list, n, &m, s));
-    if (m > 0) {
-      if ((double)m * h->alpha > (double)h->E) {  // pull (bottom-up)
-        CG_TRY(pull_level(h, L, s));
-        ++h->pull_levels;
-      } else {  // push from the frontier's out-edges
-        int64_t ntiles = 0;
-        CG_TRY(level_tiles(h, n, m, &ntiles, s));
-        push_kernel<<<(unsigned)ntiles, kThreads, 0, s>>>(list, n, h->rend, h->vt_row,
-                                                          h->vt_edge, h->out_off, h->out_dst, L,
-                                                          h->level, h->sigma, h->lists,
-                                                          h->counter);
-        CG_LAUNCH_CHECK();
-        ++h->push_levels;
-      }
+    const u64 packed = h->h_pin[L % 3], reached = h->h_pin[3];
+    const int32_t n = (int32_t)(packed >> 32), m = (int32_t)(packed & 0xffffffffull);
+    rows.push_back(n);
+    edges.push_back(m);
+    if (m == 0) break;  // L is the deepest level
+    if ((double)m * h->alpha > (double)h->E) {  // pull (bottom-up)
+      CG_TRY(pull_level(h, L, n, s));
+      ++h->pull_levels;
+    } else {  // push from the frontier's out-edges
+      const int cur = L & 1;
+      push_kernel<<<grid_for(ceil_div(m, kPushTile) * 32, kThreads), kThreads, 0, s>>>(
+          frontier(h, cur), n, m, h->out_off, h->out_dst, L, h->level, h->sigma,
+          frontier(h, 1 - cur), h->count);
+      CG_LAUNCH_CHECK();
+      ++h->push_levels;
     }
-    int32_t cnt = 0;
-    CG_TRY(read_i32(h, h->counter, &cnt, s));
-    if (cnt == h->lbase[L + 1]) break;  // nothing new: L is the deepest level
-    h->lbase.push_back(cnt);
-    // the frontier moves on: x = sigma on level L+1 only
-    set_x_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(list, n, h->sigma, h->xval, h->xbits,
-                                                            true);
-    CG_LAUNCH_CHECK();
-    const int64_t n1 = cnt - h->lbase[L + 1];
-    set_x_kernel<<<grid_for(n1, kThreads), kThreads, 0, s>>>(h->lists + h->lbase[L + 1], n1,
-                                                             h->sigma, h->xval, h->xbits, false);
-    CG_LAUNCH_CHECK();
+    CG_TRY(read_counts(h, s));
+    if (h->h_pin[3] == reached) break;  // nothing new
+    size.push_back((int64_t)(h->h_pin[3] - reached));
   }
-  const int32_t depth = (int32_t)h->lbase.size() - 1;  // levels 0 .. depth-1
-  CG_TRY(order_levels(h, depth, s));
+  const int32_t depth = (int32_t)size.size();  // levels 0 .. depth-1
+  h->depth = depth;
+  int64_t reached = 0;
+  for (int64_t q : size) reached += q;
+  // the reached vertices in (level, no out-edges, ID) order, and their row starts
+  CG_TRY(compact(h, Reached{h->level, h->out_off, h->ids, h->keys}, V, nullptr, s));
+  int bits = 1;
+  while (bits < 32 && (int64_t(1) << bits) < 2 * (int64_t)depth) ++bits;
   {
-    const int64_t b = h->lbase[depth - 1], n = h->lbase[depth] - b;
-    deepest_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(h->lists + b, n, h->sigma,
-                                                              h->xval, h->xbits);
-    CG_LAUNCH_CHECK();
+    Scratch ws(s, h->sort, h->sort_bytes);
+    CG_TRY(radix_sort_pairs(h->keys, h->ids, h->keys_out, h->lists, reached, bits, s, &ws));
   }
-  // backward: levels depth-2 .. 0
-  for (int32_t L = depth - 2; L >= 0; --L) {
-    const int64_t b0 = h->lbase[L], n = h->lbase[L + 1] - b0;
+  CG_TRY(compact(h, ListRows{h->lists, h->out_off, h->pos, h->gap}, reached, nullptr, s));
+  // backward: the deepest level, whose sums are all 0, then levels depth-2 .. 0
+  int64_t b0 = reached, e0 = 0;
+  for (int32_t L = 0; L < depth; ++L) e0 += edges[L];
+  for (int32_t L = depth - 1; L >= 0; --L) {
+    const int64_t n = size[L];
+    b0 -= n;
+    e0 -= edges[L];
     const int32_t* list = h->lists + b0;
-    int64_t m = 0;
-    CG_TRY(level_rows(h, list, n, &m, s));
-    if (m > 0) {
-      int64_t ntiles = 0;
-      CG_TRY(level_tiles(h, n, m, &ntiles, s));
-      // the out-rows of level L's vertices, read through the level list
-      gather_tile_kernel<SumF64, kTileThreads, kTileIPT, false, int64_t, true, true>
-          <<<(unsigned)ntiles, kTileThreads, 0, s>>>(h->rend + 1, nullptr, h->xval, V,
-                                                     h->vt_row, h->vt_edge, h->acc, h->vt_carry,
-                                                     h->vt_carry_row, h->xbits, list, h->out_off,
-                                                     h->out_dst);
-      CG_LAUNCH_CHECK();
-      carry_fixup_kernel<SumF64><<<grid_for(ntiles, 256, 4), 256, 0, s>>>(
-          h->vt_carry, h->vt_carry_row, ntiles, n, h->acc);
-      CG_LAUNCH_CHECK();
-    } else {
-      CG_CUDA(cudaMemsetAsync(h->acc, 0, sizeof(double) * (size_t)n, s));
+    int64_t summed = 0;
+    if (L < depth - 1) {
+      summed = rows[L];
+      const RowSums a{h->pos + b0, h->gap + b0, (int32_t)e0, rows[L], edges[L], nullptr,
+                      h->out_dst, h->xbits, h->xval, h->acc, h->carry, h->carry_row};
+      CG_TRY(row_sums(a, edges[L], s));
     }
-    dependency_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(list, n, h->acc, h->sigma,
-                                                                h->delta, h->xval, h->xbits, bc,
-                                                                src);
+    dependency_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(
+        list, n, summed, h->acc, h->sigma, h->delta, h->xval, h->xbits, bc, src);
     CG_LAUNCH_CHECK();
   }
   h->last_source = src;
@@ -525,7 +705,8 @@ int cg_transpose_csr(const int64_t* in_offsets, const int32_t* in_src, int32_t V
     e = cudaMallocAsync((void**)&rows, sizeof(int32_t) * (size_t)E, stream);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&kout, sizeof(uint32_t) * (size_t)E, stream);
     if (e == cudaSuccess) {
-      row_of_edge_kernel<<<grid_for((int64_t)V * 32, 256), 256, 0, stream>>>(in_offsets, V, rows);
+      row_of_edge_kernel<<<grid_for(ceil_div(E, 1024) * 32, 256), 256, 0, stream>>>(in_offsets, V,
+                                                                                    E, rows);
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) st = cuda_fail(e, "cg_transpose_csr", __FILE__, __LINE__);
@@ -560,22 +741,46 @@ int bc_create(const int64_t* in_offsets, const int32_t* in_src, const int64_t* o
   h->in_src = in_src;
   h->out_off = out_offsets;
   h->out_dst = out_dst;
-  const size_t v4 = sizeof(int32_t) * (size_t)V, v8 = sizeof(double) * (size_t)V;
-  cudaError_t e = cudaMalloc((void**)&h->level, v4);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->sigma, v8);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->delta, v8);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->xval, v8);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->acc, v8);
-  if (e == cudaSuccess)
-    e = cudaMalloc((void**)&h->xbits, sizeof(uint32_t) * ((size_t)V / 32 + 1));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->lists, v4);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->deg, v4);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->rend, sizeof(int64_t) * ((size_t)V + 1));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->counter, sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->ids, v4);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->keys, v4);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->keys_out, v4);
-  if (e == cudaSuccess) e = cudaHostAlloc((void**)&h->h_pin, 2 * sizeof(int64_t), 0);
+  const size_t v4 = Scratch::round(4 * (size_t)V), v8 = Scratch::round(8 * (size_t)V);
+  const int64_t tiles = ceil_div(V, kCTile);
+  const size_t nc = (size_t)(E / kSub + 2);
+  h->sort_bytes = sort_scratch(V) + scan_scratch(tiles) + 4096;
+  const size_t ts = Scratch::round(8 * (size_t)(2 * tiles + 2));
+  const size_t xb = Scratch::round(4 * ((size_t)V / 32 + 1));
+  const size_t c8 = Scratch::round(8 * nc), c4 = Scratch::round(4 * nc);
+  cudaError_t e = cudaMalloc((void**)&h->slab, 13 * v4 + 4 * v8 + xb + ts + c8 + c4 + 256 +
+                                                   h->sort_bytes);
+  if (e == cudaSuccess) {
+    char* p = h->slab;
+    auto take = [&](size_t bytes) {
+      char* q = p;
+      p += bytes;
+      return q;
+    };
+    h->sigma = reinterpret_cast<double*>(take(v8));
+    h->delta = reinterpret_cast<double*>(take(v8));
+    h->xval = reinterpret_cast<double*>(take(v8));
+    h->acc = reinterpret_cast<double*>(take(v8));
+    h->level = reinterpret_cast<int32_t*>(take(v4));
+    for (int q = 0; q < 2; ++q) {
+      h->flist[q] = reinterpret_cast<int32_t*>(take(v4));
+      h->fpos[q] = reinterpret_cast<int32_t*>(take(v4));
+      h->fgap[q] = reinterpret_cast<int32_t*>(take(v4));
+    }
+    h->lists = reinterpret_cast<int32_t*>(take(v4));
+    h->pos = reinterpret_cast<int32_t*>(take(v4));
+    h->gap = reinterpret_cast<int32_t*>(take(v4));
+    h->ids = reinterpret_cast<int32_t*>(take(v4));
+    h->keys = reinterpret_cast<uint32_t*>(take(v4));
+    h->keys_out = reinterpret_cast<uint32_t*>(take(v4));
+    h->xbits = reinterpret_cast<uint32_t*>(take(xb));
+    h->tsum = reinterpret_cast<int64_t*>(take(ts));
+    h->carry = reinterpret_cast<double*>(take(c8));
+    h->carry_row = reinterpret_cast<int32_t*>(take(c4));
+    h->count = reinterpret_cast<unsigned long long*>(take(256));
+    h->sort = take(h->sort_bytes);
+    e = cudaHostAlloc((void**)&h->h_pin, 4 * sizeof(unsigned long long), 0);
+  }
   int st = e == cudaSuccess ? CG_OK : cuda_fail(e, "bc_create", __FILE__, __LINE__);
   if (st == CG_OK) {
     e = cudaStreamSynchronize(stream);
@@ -595,23 +800,7 @@ int bc_destroy(cg_bc* h) {
   cudaGetDevice(&cur);
   if (cur != h->device) cudaSetDevice(h->device);
   cudaDeviceSynchronize();
-  cudaFree(h->level);
-  cudaFree(h->sigma);
-  cudaFree(h->delta);
-  cudaFree(h->xval);
-  cudaFree(h->acc);
-  cudaFree(h->xbits);
-  cudaFree(h->lists);
-  cudaFree(h->deg);
-  cudaFree(h->rend);
-  cudaFree(h->counter);
-  cudaFree(h->ids);
-  cudaFree(h->keys);
-  cudaFree(h->keys_out);
-  cudaFree(h->vt_row);
-  cudaFree(h->vt_edge);
-  cudaFree(h->vt_carry);
-  cudaFree(h->vt_carry_row);
+  cudaFree(h->slab);
   if (h->h_pin) cudaFreeHost(h->h_pin);
   if (cur != h->device) cudaSetDevice(cur);
   delete h;
@@ -644,7 +833,7 @@ int bc_source_state(const cg_bc* h, int32_t* level, double* sigma, double* delta
   if (level) CG_CUDA(cudaMemcpyAsync(level, h->level, v4, cudaMemcpyDeviceToDevice, stream));
   if (sigma) CG_CUDA(cudaMemcpyAsync(sigma, h->sigma, v8, cudaMemcpyDeviceToDevice, stream));
   if (delta) CG_CUDA(cudaMemcpyAsync(delta, h->delta, v8, cudaMemcpyDeviceToDevice, stream));
-  if (depth) *depth = (int32_t)h->lbase.size() - 1;
+  if (depth) *depth = h->depth;
   if (push_levels) *push_levels = h->push_levels;
   if (pull_levels) *pull_levels = h->pull_levels;
   return CG_OK;

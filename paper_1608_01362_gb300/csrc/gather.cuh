@@ -95,26 +95,13 @@ __global__ void tile_partition_kernel(const RowEndT* __restrict__ row_end, int64
 
 // The gather tile kernel.  row_end[i] = first edge after row i (global edge
 // index); col: global source IDs; PROBE sends every gathered read to x[0].
-// MASKED: xmask holds one bit per source; x is read only where the bit is
-// set (the identity elsewhere), so a sparse x (a frontier) costs a bit test
-// from a small, cache-resident array instead of a value read per edge.
-// VIRT: the rows are rows of another CSR (voff, vadj) taken in the order of
-// a vertex list vlist (row i = vertex vlist[i]; row_end: their lengths'
-// inclusive prefix); each edge's source is read through the list
-// (vadj[voff[vlist[i]] + position in the row]) instead of from col, so a
-// subset of a graph's rows is gathered without being copied out first.
-template <class Op, int THREADS, int IPT, bool PROBE, typename RowEndT, bool MASKED = false,
-          bool VIRT = false>
+template <class Op, int THREADS, int IPT, bool PROBE, typename RowEndT>
 __global__ void __launch_bounds__(THREADS)
 gather_tile_kernel(const RowEndT* __restrict__ row_end, const int32_t* __restrict__ col,
                    const typename Op::T* __restrict__ x, int32_t nx,
                    const int32_t* __restrict__ tile_row, const int32_t* __restrict__ tile_edge,
                    typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry,
-                   int32_t* __restrict__ carry_row,
-                   const uint32_t* __restrict__ xmask = nullptr,
-                   const int32_t* __restrict__ vlist = nullptr,
-                   const int64_t* __restrict__ voff = nullptr,
-                   const int32_t* __restrict__ vadj = nullptr) {
+                   int32_t* __restrict__ carry_row) {
   using T = typename Op::T;
   constexpr int TILE = THREADS * IPT;
   constexpr int WARPS = THREADS / 32;
@@ -124,11 +111,9 @@ gather_tile_kernel(const RowEndT* __restrict__ row_end, const int32_t* __restric
   // Row results.  A row emitted during the walk lies wholly inside the
   // emitting thread's items (a row that began in an earlier thread's items is
   // the thread's first row, written only after the block scan), so no other
-  // thread reads its end any more and a 4-byte result can take its place.  An
-  // 8-byte result written there would cover two row ends, one of them
-  // possibly another thread's current row: wider values get their own array.
-  __shared__ T s_res_wide[sizeof(T) > 4 ? PADT : 1];
-  T* s_res = sizeof(T) > 4 ? s_res_wide : reinterpret_cast<T*>(s_rend);
+  // thread reads its end any more and a 4-byte result can take its place.
+  static_assert(sizeof(T) == 4, "a row result takes its row end's place");
+  T* s_res = reinterpret_cast<T*>(s_rend);
   __shared__ T s_wval[WARPS];
   __shared__ int32_t s_wrow[WARPS];
   __shared__ T s_prev_val[THREADS];
@@ -145,43 +130,19 @@ gather_tile_kernel(const RowEndT* __restrict__ row_end, const int32_t* __restric
   const int nr = min(max(r1 - r0, 0), TILE);
   const int ne = min(max(e1 - e0, 0), TILE - nr);
 
-  if constexpr (VIRT) {  // row ends first: each edge finds its row among them
-    for (int i = tid; i < nr; i += THREADS)
-      s_rend[pad32(i)] = (int32_t)((int64_t)row_end[r0 + i] - e0);
-    __syncthreads();
-  }
-  // 1. edges: stream col (or read the sources through the list), gather x
+  // 1. edges: stream col, gather x
   {
     int32_t c[IPT];
-    if constexpr (VIRT) {
-      const int64_t start0 = r0 > 0 ? (int64_t)row_end[r0 - 1] : 0;  // row r0's first edge
 #pragma unroll
-      for (int u = 0; u < IPT; ++u) {
-        const int j = u * THREADS + tid;
-        c[u] = -1;
-        if (j < ne) {
-          int lo = 0, hi = nr;  // rows of the tile ending at or before edge j
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (s_rend[pad32(mid)] <= j) lo = mid + 1; else hi = mid;
-          }
-          const int64_t start = lo == 0 ? start0 : (int64_t)e0 + s_rend[pad32(lo - 1)];
-          c[u] = __ldg(vadj + __ldg(voff + __ldg(vlist + r0 + lo)) + ((int64_t)e0 + j - start));
-        }
-      }
-    } else {
-#pragma unroll
-      for (int u = 0; u < IPT; ++u) {
-        const int j = u * THREADS + tid;
-        c[u] = j < ne ? __ldcs(col + e0 + j) : -1;
-      }
+    for (int u = 0; u < IPT; ++u) {
+      const int j = u * THREADS + tid;
+      c[u] = j < ne ? __ldcs(col + e0 + j) : -1;
     }
     T v[IPT];
 #pragma unroll
     for (int u = 0; u < IPT; ++u) {
       const int32_t cu = c[u];
-      bool ok = cu >= 0 && cu < nx;
-      if constexpr (MASKED) ok = ok && ((__ldg(xmask + (cu >> 5)) >> (cu & 31)) & 1u);
+      const bool ok = cu >= 0 && cu < nx;
       v[u] = ok ? ld_gather(x + (PROBE ? 0 : cu)) : Op::identity();
     }
 #pragma unroll
@@ -191,9 +152,8 @@ gather_tile_kernel(const RowEndT* __restrict__ row_end, const int32_t* __restric
     }
   }
   // 2. row ends relative to e0 (in [0, ne] for the tile's rows)
-  if constexpr (!VIRT)
-    for (int i = tid; i < nr; i += THREADS)
-      s_rend[pad32(i)] = (int32_t)((int64_t)row_end[r0 + i] - e0);
+  for (int i = tid; i < nr; i += THREADS)
+    s_rend[pad32(i)] = (int32_t)((int64_t)row_end[r0 + i] - e0);
   __syncthreads();
 
   // 3. sequential walk over this thread's merged items
@@ -302,10 +262,9 @@ constexpr int kTileIPT = 8;
 constexpr int kTileItems = kTileThreads * kTileIPT;
 
 // Allocate and fill a plan (cudaMalloc: the plan lives with its handle).
-// carry_bytes: size of the gathered values (4, or 8 for SumF64).
 template <typename RowEndT>
 int plan_tiles(const RowEndT* row_end, int64_t nrows, int64_t nedges, TilePlan* p,
-                cudaStream_t s, int carry_bytes = 4) {
+                cudaStream_t s) {
   p->nrows = nrows;
   p->nedges = nedges;
   p->tile = kTileItems;
@@ -313,7 +272,7 @@ int plan_tiles(const RowEndT* row_end, int64_t nrows, int64_t nedges, TilePlan* 
   const size_t nb = sizeof(int32_t) * (size_t)(p->ntiles + 1);
   CG_CUDA(cudaMalloc((void**)&p->tile_row, nb));
   CG_CUDA(cudaMalloc((void**)&p->tile_edge, nb));
-  CG_CUDA(cudaMalloc(&p->carry, (size_t)carry_bytes * (size_t)(p->ntiles + 1)));
+  CG_CUDA(cudaMalloc(&p->carry, 4 * (size_t)(p->ntiles + 1)));
   CG_CUDA(cudaMalloc((void**)&p->carry_row, nb));
   tile_partition_kernel<RowEndT><<<grid_for(p->ntiles + 1, 256), 256, 0, s>>>(
       row_end, nrows, nedges, kTileItems, p->ntiles, p->tile_row, p->tile_edge);
@@ -331,23 +290,15 @@ inline void free_tile_plan(TilePlan* p) {
 
 inline int64_t tile_plan_bytes(const TilePlan& p) { return 16 * (p.ntiles + 1); }
 
-// Launch gather + fix-up.  row_end points at the first row's end.  xmask
-// (optional): one bit per source, x read only where it is set.
+// Launch gather + fix-up.  row_end points at the first row's end.
 template <class Op, bool PROBE, typename RowEndT>
 int run_tile_gather(const TilePlan& p, const RowEndT* row_end, const int32_t* col,
-                    const typename Op::T* x, int32_t nx, typename Op::T* out, cudaStream_t s,
-                    const uint32_t* xmask = nullptr) {
+                    const typename Op::T* x, int32_t nx, typename Op::T* out, cudaStream_t s) {
   if (p.ntiles == 0) return CG_OK;
-  if (xmask)
-    gather_tile_kernel<Op, kTileThreads, kTileIPT, PROBE, RowEndT, true>
-        <<<(unsigned)p.ntiles, kTileThreads, 0, s>>>(
-            row_end, col, x, nx, p.tile_row, p.tile_edge, out,
-            reinterpret_cast<typename Op::T*>(p.carry), p.carry_row, xmask);
-  else
-    gather_tile_kernel<Op, kTileThreads, kTileIPT, PROBE, RowEndT>
-        <<<(unsigned)p.ntiles, kTileThreads, 0, s>>>(
-            row_end, col, x, nx, p.tile_row, p.tile_edge, out,
-            reinterpret_cast<typename Op::T*>(p.carry), p.carry_row);
+  gather_tile_kernel<Op, kTileThreads, kTileIPT, PROBE, RowEndT>
+      <<<(unsigned)p.ntiles, kTileThreads, 0, s>>>(
+          row_end, col, x, nx, p.tile_row, p.tile_edge, out,
+          reinterpret_cast<typename Op::T*>(p.carry), p.carry_row);
   CG_LAUNCH_CHECK();
   carry_fixup_kernel<Op><<<grid_for(p.ntiles, 256, 4), 256, 0, s>>>(
       reinterpret_cast<const typename Op::T*>(p.carry), p.carry_row, p.ntiles, p.nrows, out);

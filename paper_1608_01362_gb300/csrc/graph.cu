@@ -76,7 +76,7 @@ relabel_copy_kernel(const int64_t* __restrict__ offsets, const int32_t* __restri
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t n = min(E, out_offsets[V]);  // an old_of_new that is no permutation
-  RowWalk<int64_t> walk{out_offsets, V, 0, 0, 0, 0};
+  RowWalk<int64_t> walk(out_offsets, V, (int32_t)out_offsets[V]);
   for (int64_t b = ((((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5)) * kRelabelTile; b < n;
        b += nw * kRelabelTile) {
     walk.seek((int32_t)b);
@@ -86,8 +86,8 @@ relabel_copy_kernel(const int64_t* __restrict__ offsets, const int32_t* __restri
 #pragma unroll
       for (int j = 0; j < U; ++j) {
         const int64_t e = b + i + 32 * j + lane;
-        int32_t st = 0;
-        const int32_t r = walk.row_of((int32_t)e, e < n, &st);
+        int32_t st, en;
+        const int32_t r = walk.row_of((int32_t)e, e < n, &st, &en);
         at[j] = -1;
         if (e < n) {
           const int64_t o = __ldg(old_of_new + r);  // in [0, V): its row is not empty

@@ -118,13 +118,13 @@ split_kernel(const int64_t* __restrict__ offsets, const int32_t* __restrict__ sr
   if (!SCATTER) return;
   __syncthreads();
   if (base >= E) return;
-  RowWalk<int64_t> walk{offsets, V, 0, 0, 0, 0};
+  RowWalk<int64_t> walk(offsets, V, (int32_t)E);
   walk.seek((int32_t)base);
 #pragma unroll
   for (int r = 0; r < kSplitRounds; ++r) {
     const int64_t e = base + r * 32 + lane;
-    int32_t st;
-    const int32_t row = walk.row_of((int32_t)e, e < E, &st);
+    int32_t st, en;
+    const int32_t row = walk.row_of((int32_t)e, e < E, &st, &en);
     if (e < E) {
       const int s = sr[r] >> 16;
       const int32_t pos = pl[s] + mine[s] + (sr[r] & 0xFFFF);
