@@ -8,26 +8,27 @@
 //
 // Each side is a per-vertex gather of err * neighbour-row over that side's
 // CSR (Algorithm 3's gather with a 32-wide row and a dot product per edge).
-// On this GPU both factor matrices fit in L2 (Netflix shape: 61 MB of user
-// rows and 2.3 MB of item rows in FP32, half that in BF16), so the source
-// set is one segment and the gather is split only for load balance: every
-// vertex's rating list is cut into pieces of at most kPiece ratings, a warp
-// takes one piece at a time, and a group of K/8 lanes takes one rating (each
-// lane 8 dimensions: 32 or 16 bytes of the row).  Piece partial gradients
-// are summed per vertex, in piece order, by the update kernel.
+// Where it pays the neighbours' rows are read from shared memory, a segment of
+// them at a time (cf_seg.cu).  Otherwise, both factor matrices fitting in L2
+// (Netflix shape: 61 MB of user rows and 2.3 MB of item rows in FP32, half that
+// in BF16), the source set is one segment and the gather is split only for load
+// balance: every vertex's rating list is cut into pieces of at most kCfPiece
+// ratings, a warp takes one piece at a time, and a group of K/8 lanes takes one
+// rating (each lane 8 dimensions: 32 or 16 bytes of the row).  Piece partial
+// gradients are summed per vertex, in piece order, by the update kernel.
 //
 // Storage precision of P and Q: FP32, BF16, or BF16 hi + lo pairs
 // (hi = bf16(x), lo = bf16(x - hi), packed in one 32-bit word per entry);
 // arithmetic is FP32, SSE is FP64.
-#include <cuda_bf16.h>
-
 #include <vector>
 
-#include "common.cuh"
+#include "cf_seg.cuh"
+#include "cf_store.cuh"
 
 namespace cg {
 constexpr int kCfPiece = 512;   // ratings per gather piece
-constexpr int kCfWide = 64;     // vertices with more pieces are updated by a whole block
+constexpr int kCfWarp = 24;     // vertices with more pieces are updated by a warp,
+constexpr int kCfWide = 384;    // with more than these by a whole block
 constexpr int kCfThreads = 256;
 }  // namespace cg
 
@@ -42,14 +43,16 @@ struct cg_bipartite {
   const int64_t* ioff = nullptr;
   const int32_t* iuser = nullptr;
   const uint8_t* irate = nullptr;
-  // pieces per side: owning vertex, first rating; per vertex its first piece
+  cg::CfSegments seg[2];  // a side's gather through segments, where it is the better one
+  // otherwise pieces per side: owning vertex, first rating; per vertex its first piece
   int32_t* pvtx[2] = {nullptr, nullptr};
   int64_t* pbeg[2] = {nullptr, nullptr};
-  int64_t* poff[2] = {nullptr, nullptr};
+  int64_t* poff[2] = {nullptr, nullptr};  // (the segments' where the side has them)
   int64_t npieces[2] = {0, 0};
   float* gpart[2] = {nullptr, nullptr};  // [npieces][K] piece gradients
-  int32_t* wide[2] = {nullptr, nullptr};  // vertices with more than kCfWide pieces
-  int32_t nwide[2] = {0, 0};
+  // vertices with more than kCfWarp pieces: the first nwide with more than kCfWide
+  int32_t* wide[2] = {nullptr, nullptr};
+  int32_t nwide[2] = {0, 0}, nwarp[2] = {0, 0};
   // factor storage (FP32, BF16, or BF16 hi + lo words); index 1 unused
   void* P[2] = {nullptr, nullptr};
   void* Q[2] = {nullptr, nullptr};
@@ -62,9 +65,6 @@ struct cg_bipartite {
 namespace cg {
 namespace {
 
-__device__ __forceinline__ float b_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float b_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-
 __device__ __forceinline__ void unpack8(const uint4& h, float (&y)[8]) {
   y[0] = b_lo(h.x); y[1] = b_hi(h.x); y[2] = b_lo(h.y); y[3] = b_hi(h.y);
   y[4] = b_lo(h.z); y[5] = b_hi(h.z); y[6] = b_lo(h.w); y[7] = b_hi(h.w);
@@ -76,11 +76,6 @@ __device__ __forceinline__ uint32_t pk(float a, float b) {
 }
 
 // 8 consecutive dimensions of row `row` (K per row) in the storage format.
-// BF16 hi + lo is stored as one 32-bit word per dimension (hi in the low
-// half, lo in the high half), so a row is one 128-byte line at K = 32, like
-// FP32, and a lane reads its 8 dimensions with two 16-byte loads.
-__device__ __forceinline__ float hilo(uint32_t w) { return b_lo(w) + b_hi(w); }
-
 template <int PREC>
 __device__ __forceinline__ void load8(const void* p0, int64_t row, int K, int d0, float (&y)[8]) {
   const int64_t at = row * K + d0;
@@ -222,26 +217,42 @@ cf_gather_kernel(const int32_t* __restrict__ pvtx, const int64_t* __restrict__ p
 }
 
 // x_v += step (g_v / deg v - lambda x_v), g_v = sum of v's piece gradients in
-// piece order.  One group of LANES lanes per vertex.
+// piece order (piece p's lies at slots[p], or at p without a list).  One group
+// of LANES lanes per vertex, four pieces' reads in flight.
 template <int LANES, int PREC>
 __global__ void __launch_bounds__(kCfThreads)
-cf_update_kernel(const int64_t* __restrict__ poff, const int64_t* __restrict__ off, int64_t n,
-                 const float* __restrict__ gpart, void* x0, float lambda, float step) {
+cf_update_kernel(const int64_t* __restrict__ poff, const int32_t* __restrict__ slots,
+                 const int64_t* __restrict__ off, int64_t n, const float* __restrict__ gpart,
+                 void* x0, float lambda, float step) {
   constexpr int K = 8 * LANES;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t ng = ((int64_t)gridDim.x * blockDim.x) / LANES;
   const int sub = (int)(t % LANES);
   const int d0 = 8 * sub;
   for (int64_t v = t / LANES; v < n; v += ng) {
-    if (poff[v + 1] - poff[v] > kCfWide) continue;  // cf_update_wide_kernel's
+    if (poff[v + 1] - poff[v] > kCfWarp) continue;  // the warp's or the block's
     float g[8], x[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) g[q] = 0.0f;
-    for (int64_t p = poff[v]; p < poff[v + 1]; ++p) {
-      const float4* s = reinterpret_cast<const float4*>(gpart + p * K + d0);
-      const float4 a = __ldcs(s), b = __ldcs(s + 1);
-      g[0] += a.x; g[1] += a.y; g[2] += a.z; g[3] += a.w;
-      g[4] += b.x; g[5] += b.y; g[6] += b.z; g[7] += b.w;
+    constexpr int U = 4;
+    const int64_t p1 = poff[v + 1];
+    for (int64_t p = poff[v]; p < p1; p += U) {
+      float4 a[U], b[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        a[u] = b[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p + u < p1) {
+          const int64_t q = slots ? (int64_t)__ldg(slots + p + u) : p + u;
+          const float4* s = reinterpret_cast<const float4*>(gpart + q * K + d0);
+          a[u] = __ldcs(s);
+          b[u] = __ldcs(s + 1);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        g[0] += a[u].x; g[1] += a[u].y; g[2] += a[u].z; g[3] += a[u].w;
+        g[4] += b[u].x; g[5] += b[u].y; g[6] += b[u].z; g[7] += b[u].w;
+      }
     }
     const int64_t deg = off[v + 1] - off[v];
     const float inv = deg > 0 ? 1.0f / (float)deg : 0.0f;
@@ -252,6 +263,60 @@ cf_update_kernel(const int64_t* __restrict__ poff, const int64_t* __restrict__ o
   }
 }
 
+// Vertices with more than kCfWarp pieces: one warp each.  Its groups of LANES
+// lanes sum interleaved subsets of the pieces, four reads in flight each, and a
+// fixed-order tree over the groups gives the gradient sum; deterministic.  (A
+// block per such vertex, the rule from 65 pieces on, spent 0.26 ms on the
+// Netflix shape's 17,770 items of about 280 pieces, most of it in the block's
+// barriers; a warp 0.17.)
+template <int LANES, int PREC>
+__global__ void __launch_bounds__(kCfThreads)
+cf_update_warp_kernel(const int32_t* __restrict__ list, int32_t n,
+                      const int64_t* __restrict__ poff, const int32_t* __restrict__ slots,
+                      const int64_t* __restrict__ off, const float* __restrict__ gpart, void* x0,
+                      float lambda, float step) {
+  constexpr int K = 8 * LANES, GROUPS = 32 / LANES, U = 4;
+  const int lane = threadIdx.x & 31, sub = lane % LANES, grp = lane / LANES, d0 = 8 * sub;
+  const int32_t nw = (int32_t)((gridDim.x * blockDim.x) >> 5);
+  for (int32_t i = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); i < n; i += nw) {
+    const int32_t v = list[i];
+    const int64_t p1 = poff[v + 1];
+    float g[8], x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) g[q] = 0.0f;
+    for (int64_t p = poff[v] + grp; p < p1; p += U * GROUPS) {
+      float4 a[U], b[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        a[u] = b[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int64_t pu = p + u * GROUPS;
+        if (pu < p1) {
+          const int64_t q = slots ? (int64_t)__ldg(slots + pu) : pu;
+          const float4* s = reinterpret_cast<const float4*>(gpart + q * K + d0);
+          a[u] = __ldcs(s);
+          b[u] = __ldcs(s + 1);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        g[0] += a[u].x; g[1] += a[u].y; g[2] += a[u].z; g[3] += a[u].w;
+        g[4] += b[u].x; g[5] += b[u].y; g[6] += b[u].z; g[7] += b[u].w;
+      }
+    }
+#pragma unroll
+    for (int o = LANES; o < 32; o <<= 1)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) g[q] += __shfl_xor_sync(0xffffffffu, g[q], o);
+    if (grp == 0) {
+      const float inv = 1.0f / (float)(off[v + 1] - off[v]);
+      load8<PREC>(x0, v, K, d0, x);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) x[q] = x[q] + step * (g[q] * inv - lambda * x[q]);
+      store8<PREC>(x0, v, K, d0, x);
+    }
+  }
+}
+
 // Vertices with more than kCfWide pieces (hub items): one block each.  The
 // block's groups of LANES lanes sum interleaved subsets of the pieces (four
 // independent accumulators per group, combined in a fixed order), then a
@@ -259,9 +324,9 @@ cf_update_kernel(const int64_t* __restrict__ poff, const int64_t* __restrict__ o
 template <int LANES, int PREC>
 __global__ void __launch_bounds__(kCfThreads)
 cf_update_wide_kernel(const int32_t* __restrict__ wide, int32_t nwide,
-                      const int64_t* __restrict__ poff, const int64_t* __restrict__ off,
-                      const float* __restrict__ gpart, void* x0, float lambda,
-                      float step) {
+                      const int64_t* __restrict__ poff, const int32_t* __restrict__ slots,
+                      const int64_t* __restrict__ off, const float* __restrict__ gpart, void* x0,
+                      float lambda, float step) {
   constexpr int K = 8 * LANES;
   constexpr int GROUPS = kCfThreads / LANES;
   constexpr int U = 4;
@@ -281,7 +346,8 @@ cf_update_wide_kernel(const int32_t* __restrict__ wide, int32_t nwide,
       for (int j = 0; j < U; ++j) {
         const int64_t pj = p + (int64_t)j * GROUPS;
         if (pj < p1) {
-          const float4* s = reinterpret_cast<const float4*>(gpart + pj * K + d0);
+          const int64_t q = slots ? (int64_t)__ldg(slots + pj) : pj;
+          const float4* s = reinterpret_cast<const float4*>(gpart + q * K + d0);
           const float4 x = __ldcs(s), y = __ldcs(s + 1);
           a[j][0] += x.x; a[j][1] += x.y; a[j][2] += x.z; a[j][3] += x.w;
           a[j][4] += y.x; a[j][5] += y.y; a[j][6] += y.z; a[j][7] += y.w;
@@ -410,6 +476,10 @@ int sweep_side(cg_bipartite* h, int side, double* sse, float lambda, float step,
   void** other = side == 0 ? h->Q : h->P;
   const int64_t n = side == 0 ? h->U : h->I;
   if (gather) {
+    if (h->seg[side].k > 0)
+      return cf_seg_gather(h->seg[side], h->K, h->precision, side == 0 ? h->I : h->U, nb, rt,
+                           self[0], other[0], h->gpart[side], side == 0, h->partials, h->counter,
+                           sse, s);
     if (h->npieces[side] == 0) {
       if (side == 0 && sse) CG_CUDA(cudaMemsetAsync(sse, 0, sizeof(double), s));
       return CG_OK;
@@ -424,12 +494,19 @@ int sweep_side(cg_bipartite* h, int side, double* sse, float lambda, float step,
           h->partials, h->counter, nullptr);
   } else {
     cf_update_kernel<LANES, PREC><<<grid_for(n * LANES, kCfThreads, 8), kCfThreads, 0, s>>>(
-        h->poff[side], off, n, h->gpart[side], self[0], lambda, step);
+        h->poff[side], h->seg[side].slots, off, n, h->gpart[side], self[0], lambda, step);
+    if (h->nwarp[side] > 0) {
+      CG_LAUNCH_CHECK();
+      cf_update_warp_kernel<LANES, PREC>
+          <<<grid_for((int64_t)h->nwarp[side] * 32, kCfThreads, 8), kCfThreads, 0, s>>>(
+              h->wide[side] + h->nwide[side], h->nwarp[side], h->poff[side], h->seg[side].slots,
+              off, h->gpart[side], self[0], lambda, step);
+    }
     if (h->nwide[side] > 0) {
       CG_LAUNCH_CHECK();
       cf_update_wide_kernel<LANES, PREC><<<h->nwide[side], kCfThreads, 0, s>>>(
-          h->wide[side], h->nwide[side], h->poff[side], off, h->gpart[side], self[0],
-          lambda, step);
+          h->wide[side], h->nwide[side], h->poff[side], h->seg[side].slots, off, h->gpart[side],
+          self[0], lambda, step);
     }
   }
   CG_LAUNCH_CHECK();
@@ -499,7 +576,8 @@ void cf_free(cg_bipartite* h) {
   for (int s = 0; s < 2; ++s) {
     cudaFree(h->pvtx[s]);
     cudaFree(h->pbeg[s]);
-    cudaFree(h->poff[s]);
+    if (h->seg[s].k == 0) cudaFree(h->poff[s]);
+    cf_seg_free(&h->seg[s]);
     cudaFree(h->gpart[s]);
     cudaFree(h->wide[s]);
     cudaFree(h->P[s]);
@@ -510,7 +588,8 @@ void cf_free(cg_bipartite* h) {
   delete h;
 }
 
-int build_pieces(cg_bipartite* h, int side, cudaStream_t s) {
+// The pieces of the gather from L2: at most kCfPiece ratings of one vertex.
+int build_plain_pieces(cg_bipartite* h, int side, cudaStream_t s) {
   const int64_t* off = side == 0 ? h->uoff : h->ioff;
   const int64_t n = side == 0 ? h->U : h->I;
   int64_t* cnt = nullptr;
@@ -544,7 +623,24 @@ int build_pieces(cg_bipartite* h, int side, cudaStream_t s) {
                                                         h->pbeg[side]);
     CG_LAUNCH_CHECK();
   }
-  // vertices with many pieces get a whole block in the update
+  return CG_OK;
+}
+
+int build_pieces(cg_bipartite* h, int side, cudaStream_t s) {
+  const int64_t* off = side == 0 ? h->uoff : h->ioff;
+  const int64_t n = side == 0 ? h->U : h->I;
+  CG_TRY(cf_seg_build(&h->seg[side], n, side == 0 ? h->I : h->U, h->R, h->K, off,
+                      side == 0 ? h->uitem : h->iuser, s));
+  if (h->seg[side].k > 0) {
+    const CfSegments& c = h->seg[side];
+    h->poff[side] = c.poff;
+    h->npieces[side] = c.npieces;
+    CG_CUDA(cudaMalloc((void**)&h->gpart[side], sizeof(float) * (size_t)c.nslots * h->K));
+    h->bytes += c.bytes + 4 * c.nslots * h->K;
+  } else {
+    CG_TRY(build_plain_pieces(h, side, s));
+  }
+  // vertices with many pieces get a warp or a whole block in the update
   std::vector<int64_t> hp((size_t)n + 1);
   CG_CUDA(cudaMemcpyAsync(hp.data(), h->poff[side], sizeof(int64_t) * (size_t)(n + 1),
                           cudaMemcpyDeviceToHost, s));
@@ -553,6 +649,9 @@ int build_pieces(cg_bipartite* h, int side, cudaStream_t s) {
   for (int64_t v = 0; v < n; ++v)
     if (hp[v + 1] - hp[v] > kCfWide) wide.push_back((int32_t)v);
   h->nwide[side] = (int32_t)wide.size();
+  for (int64_t v = 0; v < n; ++v)
+    if (hp[v + 1] - hp[v] > kCfWarp && hp[v + 1] - hp[v] <= kCfWide) wide.push_back((int32_t)v);
+  h->nwarp[side] = (int32_t)wide.size() - h->nwide[side];
   if (!wide.empty()) {
     CG_CUDA(cudaMalloc((void**)&h->wide[side], sizeof(int32_t) * wide.size()));
     h->bytes += 4 * (int64_t)wide.size();

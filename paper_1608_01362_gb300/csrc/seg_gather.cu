@@ -2,6 +2,7 @@
 #include <algorithm>
 
 #include "carry_runs.cuh"
+#include "ranges.cuh"
 #include "staged_stream.cuh"
 
 namespace cg {
@@ -227,85 +228,35 @@ __device__ __forceinline__ void stage_table(const T* __restrict__ src, int n, T*
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// Barrier among threads [0, nt) of the block: the whole block, or named
-// barrier 1 when only the staged warps of an overlapped launch take part.
-__device__ __forceinline__ void group_sync(int nt) {
-  if (nt == (int)blockDim.x)
-    __syncthreads();
-  else
-    asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
-}
-
-// What the staged schedule's blocks share: block b owns tasks
-// [blk_task[b], blk_task[b+1]) (equal stretches of the stream); next[b] of
-// them have been taken.
+// The staged segments [0, m) and their tasks' shares among the blocks.
 struct StagedShare {
-  const int32_t* blk_task;  // [grid+1]
-  unsigned* next;           // [grid]
+  RangeShare ranges;
   const int32_t* seg_lo;
   const int32_t* seg_tab;
-  int m;                    // the staged segments are [0, m)
+  int m;
 };
-struct StagedSlots {  // a block's shared words
-  int32_t lo, hi;
-  unsigned fullest;
-};
-
-constexpr int kStealMin = 64;  // a range with fewer tasks left is not worth a table copy
 
 // The staged schedule, run by threads [0, nt) of a block: segments [0, m)
 // are read from a shared-memory copy of their source values.  A block works
-// through its own range of tasks, which meets one or two segments, half of
-// what is left at a time; when it runs dry it takes half of what is left of
-// the fullest range.  (The earlier schedule handed out small pieces of all
-// the tasks in order, so every block met nearly every segment: 31 table
-// copies per block on RMAT-25, each as long as 1.8 us of L2 reads at 64
-// bytes per cycle and SM, and two barriers per piece.)
+// through its own range of tasks, which meets one or two segments, and then
+// helps with the fullest range (ranges.cuh).  (The earlier schedule handed out
+// small pieces of all the tasks in order, so every block met nearly every
+// segment: 31 table copies per block on RMAT-25, each as long as 1.8 us of L2
+// reads at 64 bytes per cycle and SM, and two barriers per piece.)
 template <class Op>
 __device__ __forceinline__ void staged_pieces(
     const StagedTasks& q, const StagedShare& sh, const typename Op::T* __restrict__ x,
     typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry, typename Op::T* tab,
-    int nt, StagedSlots* slots) {
+    int nt, RangeSlots* slots) {
   using T = typename Op::T;
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  int s = -1;              // the segment in the table
+  const int tid = threadIdx.x, w = tid >> 5;
+  int s = -1;               // the segment in the table
   int v = (int)blockIdx.x;  // the range being worked on
   if (tid == 0) tab[q.pad] = Op::identity();  // the first table's barrier publishes it
-
-  for (;;) {
-    group_sync(nt);  // everyone is done with the previous piece's slots
-    if (tid == 0) {
-      const int32_t b0 = sh.blk_task[v], n = sh.blk_task[v + 1] - b0;
-      const int32_t taken = (int32_t)*(volatile unsigned*)(sh.next + v);
-      const int32_t sz = max((n - taken) / 2, kStealMin);
-      const int32_t lo = taken < n ? (int32_t)atomicAdd(sh.next + v, (unsigned)sz) : n;
-      slots->lo = b0 + min(lo, n);
-      slots->hi = b0 + min(lo + sz, n);
-      slots->fullest = 0u;
-    }
-    group_sync(nt);
-    int32_t t = slots->lo;
-    const int32_t hi = slots->hi;
-    if (t >= hi) {  // this range is done: find the fullest one
-      for (int b = tid; b < (int)gridDim.x; b += nt) {
-        const int32_t left = sh.blk_task[b + 1] - sh.blk_task[b] -
-                             (int32_t)*(volatile unsigned*)(sh.next + b);
-        if (left >= kStealMin)
-          atomicMax(&slots->fullest, ((unsigned)min(left, 0x1FFFFF) << 11) | (unsigned)b);
-      }
-      group_sync(nt);
-      if (slots->fullest == 0u) break;
-      v = (int)(slots->fullest & 0x7FFu);
-      continue;
-    }
+  int32_t t, hi;
+  while (next_range(sh.ranges, nt, slots, &v, &t, &hi)) {
     while (t < hi) {
-      int sn = 0;  // the segment of task t: segments whose tasks all precede it
-      for (int i = 0; i < sh.m; i += 32) {
-        const bool before = i + lane < sh.m && __ldg(q.seg_task + i + lane + 1) <= t;
-        const unsigned bal = __ballot_sync(0xffffffffu, before);
-        sn += __popc(bal);
-        if (bal != 0xffffffffu) break;
-      }
+      const int sn = segment_of_task(q.seg_task, sh.m, t);
       const int32_t te = __ldg(q.seg_task + sn + 1);
       if (sn != s) {
         s = sn;
@@ -327,7 +278,7 @@ staged_gather_kernel(StagedTasks q, StagedShare sh, const typename Op::T* __rest
                      typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ StagedSlots slots;
+  __shared__ RangeSlots slots;
   staged_pieces<Op>(q, sh, x, out, carry, reinterpret_cast<T*>(smem_raw), THREADS, &slots);
 }
 
@@ -425,7 +376,7 @@ overlap_gather_kernel(StagedTasks q, StagedShare sh, const uint32_t* __restrict_
                       typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ StagedSlots slots;
+  __shared__ RangeSlots slots;
   if ((int)threadIdx.x < staged_threads)
     staged_pieces<Op>(q, sh, x, out, carry, reinterpret_cast<T*>(smem_raw), staged_threads, &slots);
   cached_queue<Op>(colf, x, nx, first_row, seg_cstart, seg_E, seg_chunk, seg_lo, m, k, next_chunk,
@@ -686,7 +637,7 @@ static StagedTasks staged_tasks(const SegPlan& p) {
 }
 
 static StagedShare staged_share(const SegPlan& p) {
-  return StagedShare{p.blk_task, p.counter + 2, p.seg_lo, p.seg_tab, p.m};
+  return StagedShare{{p.blk_task, p.counter + 2}, p.seg_lo, p.seg_tab, p.m};
 }
 
 // the table and, behind it, the identity's entry
