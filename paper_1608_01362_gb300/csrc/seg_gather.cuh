@@ -103,7 +103,10 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
 // the table entry that holds the identity).  The carries of the full pieces of
 // rows longer than kStagedMost follow the first carry_base ones; their rows are
 // written to carry_row.  Synchronizes.
-int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s);
+// place (optional): where each row's sum goes, below 65535, in the place of its
+// position in its window (the tasks' base row is then 0).
+int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s,
+                 const int32_t* place = nullptr);
 // Room for n carries (their contents are lost when it grows).
 int seg_plan_carries(SegPlan* p, int64_t n);
 

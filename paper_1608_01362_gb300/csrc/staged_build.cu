@@ -103,7 +103,8 @@ staged_fill_kernel(const uint32_t* __restrict__ colf, const int32_t* __restrict_
                    const int32_t* __restrict__ xrow, const int32_t* __restrict__ xpiece,
                    const int64_t* __restrict__ start, const int64_t* __restrict__ task_base,
                    const int64_t* __restrict__ unit_base, int nb, int64_t ntasks, int pad,
-                   int64_t carry_base, uint4* __restrict__ desc, uint8_t* __restrict__ cs) {
+                   int64_t carry_base, const int32_t* __restrict__ place,
+                   uint4* __restrict__ desc, uint8_t* __restrict__ cs) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < ntasks; t += nw) {
@@ -119,7 +120,8 @@ staged_fill_kernel(const uint32_t* __restrict__ colf, const int32_t* __restrict_
     const int words = class_words(c), slots = class_slots(c), lg = class_lg(c);
     uint8_t* base = cs + off * 32;
     if (lane == 0) {
-      const int64_t z = c == kClassFull ? carry_base + (item[first] - rows) : row0;
+      const int64_t z =
+          c == kClassFull ? carry_base + (item[first] - rows) : place ? 0 : row0;
       desc[t] = make_uint4((uint32_t)off, class_word(c), (uint32_t)z, 0u);
     }
     // edges [e0, e0 + len) of the row slot j of the task (len 0: unused)
@@ -134,7 +136,7 @@ staged_fill_kernel(const uint32_t* __restrict__ colf, const int32_t* __restrict_
       const int piece = it < rows ? full : xpiece[it - rows];
       *e0 = (int64_t)rp[r] + (int64_t)piece * kStagedMost;
       *len = it < rows ? whole - full * kStagedMost : kStagedMost;
-      return (int32_t)(r - row0);
+      return place ? place[r] : (int32_t)(r - row0);
     };
     auto put = [&](int slot, uint32_t v) {
       reinterpret_cast<uint16_t*>(base)[2 * word_at(words, slot >> 1, lane) + (slot & 1)] =
@@ -172,7 +174,8 @@ staged_fill_kernel(const uint32_t* __restrict__ colf, const int32_t* __restrict_
 
 }  // namespace
 
-int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s) {
+int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s,
+                 const int32_t* place) {
   const int k = p->k;
   const int64_t rows = p->row_base[m2];
   p->h_seg_task.assign(k + 1, 0);
@@ -184,6 +187,10 @@ int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s
   for (int q = 0; q < m2; ++q)
     wbase[q + 1] = wbase[q] + ceil_div(p->row_base[q + 1] - p->row_base[q], kStagedWindow);
   const int64_t nb = wbase[m2] << kClassBits;
+  if (nb >= 0x7FFFFFFFLL) {
+    set_error("staged segments: too many of them (%d)", m2);
+    return CG_ERR_UNSUPPORTED;
+  }
   const int64_t edges = p->edge_base[m2];
   const int64_t most = rows + edges / kStagedMost;  // rows and at most their full pieces
   Scratch tmp(s, 6 * Scratch::round(4 * (size_t)most) + sort_scratch(most) +
@@ -261,8 +268,8 @@ int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s
   }
   staged_fill_kernel<<<grid_for(ntasks * 32, 256), 256, 0, s>>>(
       p->colf, p->rp32, p->meta, p->meta + (k + 1), p->meta + 2 * (k + 1), d_wbase, m2, item,
-      rows, xrow, xpiece, start, task_base, unit_base, (int)nb, ntasks, pad, carry_base, p->desc,
-      p->cs);
+      rows, xrow, xpiece, start, task_base, unit_base, (int)nb, ntasks, pad, carry_base, place,
+      p->desc, p->cs);
   CG_LAUNCH_CHECK();
   return CG_OK;
 }
