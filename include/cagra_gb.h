@@ -19,7 +19,8 @@
  *    on the host before anything is enqueued; on error nothing is enqueued
  *    and cg_last_error_message() (thread-local) explains.  Calls that must
  *    read a device result on the host (noted below) synchronize the stream.
- *  - No entry point spins on device flags; no kernel waits on another.
+ *  - No entry point spins on device flags; a kernel waits on another only for its
+ *    end, in stream order.
  *  - Handles are bound to the device that was current when they were built;
  *    use them with that device current.
  */

@@ -9,7 +9,7 @@
 // in segment order.  Subgraph row i (global row index over all segments)
 // holds edges [row_ptr[i], row_ptr[i+1]) (stored flagged and padded in
 // plan.colf) and its destination is idx_map[i].  blk[b*k + s] is the first
-// (global) row of segment s whose destination is >= b*B (block-major: a
+// (global) row of segment s whose destination is >= b*mB (block-major: a
 // merge block's starts of all segments are contiguous); rows of segment s
 // inside merge block b are [blk[b*k + s], blk[(b+1)*k + s]).
 struct cg_segmented {
@@ -19,11 +19,13 @@ struct cg_segmented {
   int32_t k = 0;
   int32_t B = 0;
   int32_t nb = 0;
+  int32_t mB = 0;              // destinations per warp of the merge (at most B, see merge_block)
+  int32_t mnb = 0;             // merge blocks of mB destinations
   int64_t rows = 0;
   std::vector<int64_t> bounds, row_base, edge_base;  // host copies, k+1 each
   int32_t* idx_map = nullptr;  // [rows]; row_ptr and blk lie in the same allocation
   int32_t* row_ptr = nullptr;  // [rows+1] (builds and export; the gathers do not read it)
-  int32_t* blk = nullptr;      // [(nb+1)*k] block-major
+  int32_t* blk = nullptr;      // [(mnb+1)*k] block-major
   cg::SegPlan plan;            // flagged padded edges + chunk index + launch shape
   char* state = nullptr;         // one allocation that holds the arrays below
   void* interm = nullptr;        // [rows] 4-byte values (intermBuf)
@@ -54,6 +56,14 @@ struct cg_plain {
 };
 
 namespace cg {
+// Destinations per warp of the merge: the caller's B, halved (down to 32) while
+// the GPU would have fewer than 48 such warps per SM.  One warp's merge is a
+// chain of dependent reads, so a small graph's time is that chain: with B = 512
+// a 20,011-vertex graph merged on 5 of 152 SMs (11.0 us, 4.9 with 32), a
+// 1 M-vertex graph on 13 warps per SM (18.8 us, 11.7 with 128); from about 4 M
+// vertices on B stays.
+int32_t merge_block(int32_t V, int32_t B, int sm_count);
+
 // Validate an in-edge CSR on the device (offsets monotone from 0 to E, every
 // source in [0, V)).  Synchronizes the stream.
 int validate_csr(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,

@@ -17,6 +17,7 @@ lp_merge_update_kernel(const int32_t* __restrict__ blk, const int32_t* __restric
                        const int32_t* __restrict__ labels_in, int32_t* __restrict__ labels_out,
                        unsigned long long* __restrict__ changed) {
   extern __shared__ int32_t lp_acc_all[];
+  chain_begin();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t mb = (int64_t)blockIdx.x * kMergeWarps + w;
   if (mb >= nb) return;
@@ -60,14 +61,14 @@ int lp_iterate(const cg_segmented* g, const int32_t* labels_in, int32_t* labels_
   if (!cnt) cnt = reinterpret_cast<unsigned long long*>(g->dslot + 3);
   CG_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), stream));
   CG_TRY(run_seg_gather<MinI32>(g->plan, labels_in, g->V, (int32_t*)g->interm, stream));
-  const size_t smem = (size_t)kMergeWarps * g->B * 4;
+  const size_t smem = (size_t)kMergeWarps * g->mB * 4;
   if (smem > 32 * 1024)
     CG_CUDA(cudaFuncSetAttribute((const void*)lp_merge_update_kernel,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  lp_merge_update_kernel<<<(unsigned)ceil_div(g->nb, kMergeWarps), kMergeWarps * 32, smem,
-                           stream>>>(g->blk, g->idx_map, (const int32_t*)g->interm, g->k, g->nb,
-                                     g->B, g->V, labels_in, labels_out, cnt);
-  CG_LAUNCH_CHECK();
+  CG_TRY(launch_chained(lp_merge_update_kernel, (unsigned)ceil_div(g->mnb, kMergeWarps),
+                        kMergeWarps * 32, smem, stream, g->blk, g->idx_map,
+                        (const int32_t*)g->interm, g->k, g->mnb, g->mB, g->V, labels_in,
+                        labels_out, cnt));
   if (host_changed) {
     unsigned long long h = 0;
     CG_CUDA(cudaMemcpyAsync(&h, cnt, sizeof(h), cudaMemcpyDeviceToHost, stream));

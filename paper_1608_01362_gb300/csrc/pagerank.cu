@@ -2,11 +2,9 @@
 // pull baseline (Algorithm 1), plus the stand-alone gather / merge entry
 // points.
 //
-// One iteration of pr_iterate = two kernels (+ a tiny carry fix-up):
-//   gather_tile_kernel   Algorithm 3 over every subgraph, segments in order
-//                        (tiles are dispatched in segment order, so the
-//                        random reads of contrib stay inside one segment's
-//                        slice at a time), writing intermBuf sequentially;
+// One iteration of pr_iterate = the gather's launches (Algorithm 3: the staged
+// segments, those read through L1/L2, the fix-up of rows that span chunks; see
+// seg_gather.cuh) and
 //   merge_update_kernel  Algorithm 4 per block of B destinations: the block's
 //                        rows of every subgraph are added, segment by
 //                        segment, into a shared-memory accumulator; then the
@@ -25,6 +23,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32, 6)
 merge_update_kernel(const int32_t* __restrict__ blk, const int32_t* __restrict__ idx_map,
                     const float* __restrict__ interm, int k, int nb, int B, PrArgs a) {
   extern __shared__ float acc_all[];
+  chain_begin();
   const double D = *a.D_in;
   const int w = threadIdx.x >> 5;
   const int64_t mb = (int64_t)blockIdx.x * kMergeWarps + w;
@@ -47,6 +46,7 @@ merge_only_kernel(const int32_t* __restrict__ blk, const int32_t* __restrict__ i
                   typename Op::T* __restrict__ out) {
   using T = typename Op::T;
   extern __shared__ unsigned char raw[];
+  chain_begin();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t mb = (int64_t)blockIdx.x * kMergeWarps + w;
   if (mb >= nb) return;
@@ -57,10 +57,16 @@ merge_only_kernel(const int32_t* __restrict__ blk, const int32_t* __restrict__ i
   for (int i = lane; i < n; i += 32) out[v0 + i] = acc[i];
 }
 
-__global__ void pr_init_kernel(const float* __restrict__ inv, int32_t V, float* __restrict__ rank,
-                               float* __restrict__ contrib, unsigned long long* __restrict__ ndang) {
+// D (zero before the launch) first counts: finished blocks in its high half,
+// dangling vertices in its low one; the last block turns it into their mass.
+__global__ void __launch_bounds__(256)
+pr_init_kernel(const float* __restrict__ inv, int32_t V, float* __restrict__ rank,
+               float* __restrict__ contrib, unsigned long long* __restrict__ D) {
+  __shared__ unsigned s_c;
+  if (threadIdx.x == 0) s_c = 0u;
+  __syncthreads();
   const float r = 1.0f / (float)V;
-  unsigned long long c = 0;
+  unsigned c = 0;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V;
        v += (int64_t)gridDim.x * blockDim.x) {
     const float iv = inv[v];
@@ -69,7 +75,14 @@ __global__ void pr_init_kernel(const float* __restrict__ inv, int32_t V, float* 
     c += iv == 0.0f;
   }
   c = warp_sum(c);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(ndang, c);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_c, c);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned long long mine = (1ull << 32) | s_c;
+    const unsigned long long now = atomicAdd(D, mine) + mine;
+    if ((unsigned)(now >> 32) == gridDim.x)
+      *reinterpret_cast<double*>(D) = (double)(now & 0xffffffffull) * (double)r;
+  }
 }
 
 // Personalised start: all mass on the seed; D = the seed's mass if it is
@@ -84,11 +97,6 @@ __global__ void ppr_init_kernel(const float* __restrict__ inv, int32_t V, int32_
     contrib[v] = r * inv[v];
     if (v == seed) *D = inv[v] == 0.0f ? 1.0 : 0.0;
   }
-}
-
-__global__ void pr_init_finish_kernel(const unsigned long long* __restrict__ ndang, int32_t V,
-                                      double* __restrict__ D) {
-  *D = (double)(*ndang) * (double)(1.0f / (float)V);
 }
 
 // contrib = rank * inv and per-block FP64 partials of the dangling mass.
@@ -181,19 +189,10 @@ extern "C" {
 int pr_init(const float* inv, int32_t V, float* rank, float* contrib, double* D,
             cudaStream_t stream) {
   CG_ARG(V >= 1 && inv && rank && contrib && D, "pr_init: bad arguments");
-  unsigned long long* nd = nullptr;
-  CG_CUDA(cudaMallocAsync((void**)&nd, sizeof(unsigned long long), stream));
-  cudaError_t e = cudaMemsetAsync(nd, 0, sizeof(unsigned long long), stream);
-  if (e == cudaSuccess) {
-    pr_init_kernel<<<grid_for(V, 256), 256, 0, stream>>>(inv, V, rank, contrib, nd);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) {
-    pr_init_finish_kernel<<<1, 1, 0, stream>>>(nd, V, D);
-    e = cudaGetLastError();
-  }
-  cudaFreeAsync(nd, stream);
-  if (e != cudaSuccess) return cuda_fail(e, "pr_init", __FILE__, __LINE__);
+  CG_CUDA(cudaMemsetAsync(D, 0, sizeof(double), stream));
+  pr_init_kernel<<<grid_for(V, 256), 256, 0, stream>>>(inv, V, rank, contrib,
+                                                       reinterpret_cast<unsigned long long*>(D));
+  CG_LAUNCH_CHECK();
   return CG_OK;
 }
 
@@ -245,23 +244,22 @@ int cg_seg_gather(const cg_segmented* g, int32_t op, const void* x, void* interm
 
 int merge(const cg_segmented* g, int32_t op, const void* interm, void* out, cudaStream_t stream) {
   CG_ARG(g && out && (interm || g->rows == 0), "merge: null argument");
-  const unsigned grid = (unsigned)ceil_div(g->nb, kMergeWarps);
-  const size_t smem = (size_t)kMergeWarps * g->B * 4;
+  const unsigned grid = (unsigned)ceil_div(g->mnb, kMergeWarps);
+  const size_t smem = (size_t)kMergeWarps * g->mB * 4;
   if (op == CG_OP_SUM_F32) {
     auto fn = merge_only_kernel<SumF32>;
     CG_TRY(set_merge_smem((const void*)fn, smem));
-    fn<<<grid, kMergeWarps * 32, smem, stream>>>(g->blk, g->idx_map, (const float*)interm, g->k,
-                                                 g->nb, g->B, g->V, (float*)out);
+    CG_TRY(launch_chained(fn, grid, kMergeWarps * 32, smem, stream, g->blk, g->idx_map,
+                          (const float*)interm, g->k, g->mnb, g->mB, g->V, (float*)out));
   } else if (op == CG_OP_MIN_I32) {
     auto fn = merge_only_kernel<MinI32>;
     CG_TRY(set_merge_smem((const void*)fn, smem));
-    fn<<<grid, kMergeWarps * 32, smem, stream>>>(g->blk, g->idx_map, (const int32_t*)interm,
-                                                 g->k, g->nb, g->B, g->V, (int32_t*)out);
+    CG_TRY(launch_chained(fn, grid, kMergeWarps * 32, smem, stream, g->blk, g->idx_map,
+                          (const int32_t*)interm, g->k, g->mnb, g->mB, g->V, (int32_t*)out));
   } else {
     set_error("merge: unknown op %d", op);
     return CG_ERR_INVALID_ARG;
   }
-  CG_LAUNCH_CHECK();
   return CG_OK;
 }
 
@@ -286,7 +284,7 @@ static int merge_update_seeded(const cg_segmented* g, const float* inv, const fl
   CG_ARG(damping >= 0.0 && damping <= 1.0, "pr_merge_update: damping must be in [0, 1]");
   CG_ARG(rank_out != rank_in && (const float*)contrib_out != rank_in && rank_out != contrib_out,
          "pr_merge_update: outputs must not alias the inputs or each other");
-  const size_t smem = (size_t)kMergeWarps * g->B * 4;
+  const size_t smem = (size_t)kMergeWarps * g->mB * 4;
   CG_TRY(set_merge_smem((const void*)merge_update_kernel, smem));
   PrArgs a;
   a.inv = inv;
@@ -303,11 +301,9 @@ static int merge_update_seeded(const cg_segmented* g, const float* inv, const fl
   a.counter = g->counter;
   a.V = g->V;
   a.seed = seed;
-  merge_update_kernel<<<(unsigned)ceil_div(g->nb, kMergeWarps), kMergeWarps * 32, smem,
-                        stream>>>(g->blk, g->idx_map, (const float*)g->interm, g->k, g->nb,
-                                  g->B, a);
-  CG_LAUNCH_CHECK();
-  return CG_OK;
+  return launch_chained(merge_update_kernel, (unsigned)ceil_div(g->mnb, kMergeWarps),
+                        kMergeWarps * 32, smem, stream, g->blk, g->idx_map,
+                        (const float*)g->interm, g->k, g->mnb, g->mB, a);
 }
 
 static int iterate_seeded(const cg_segmented* g, const float* inv, const float* rank_in,

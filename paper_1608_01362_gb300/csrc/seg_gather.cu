@@ -61,6 +61,7 @@ template <class Op>
 __global__ void __launch_bounds__(256)
 seg_fixup_kernel(const int32_t* __restrict__ carry_row, const typename Op::T* __restrict__ carry,
                  int64_t n, typename Op::T* __restrict__ out) {
+  chain_begin();
   fix_runs<Op>(carry_row, carry, n, out);
 }
 
@@ -176,6 +177,7 @@ seg_gather_kernel(const uint32_t* __restrict__ colf, const typename Op::T* __res
                   const int32_t* __restrict__ seg_lo, int k, int32_t ct_begin, int32_t ct_end,
                   typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   constexpr int WARPS = THREADS / 32;
+  chain_begin();
   const int w = threadIdx.x >> 5;
   const int32_t my_lo = ct_begin + (int32_t)blockIdx.x;
   const int32_t step = (int32_t)gridDim.x;
@@ -231,6 +233,7 @@ __device__ __forceinline__ void stage_table(const T* __restrict__ src, int n, T*
 // The staged segments [0, m) and their tasks' shares among the blocks.
 struct StagedShare {
   RangeShare ranges;
+  unsigned* done;           // blocks finished
   const int32_t* seg_lo;
   const int32_t* seg_tab;
   int m;
@@ -271,6 +274,22 @@ __device__ __forceinline__ void staged_pieces(
   }
 }
 
+// The last block to finish clears the n counters that the launch used, ready
+// for the next one (which then needs no memset before it).  Every thread of the
+// block calls it, when the block is done with the counters.
+__device__ __forceinline__ void counters_done(unsigned* counters, int n, unsigned* done) {
+  __shared__ bool s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) counters[i] = 0u;
+  if (threadIdx.x == 0) *done = 0u;
+}
+
 // The staged launch: every thread of the block runs the staged schedule.
 template <class Op, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
@@ -279,7 +298,9 @@ staged_gather_kernel(StagedTasks q, StagedShare sh, const typename Op::T* __rest
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ RangeSlots slots;
+  chain_begin();
   staged_pieces<Op>(q, sh, x, out, carry, reinterpret_cast<T*>(smem_raw), THREADS, &slots);
+  counters_done(sh.ranges.next, (int)gridDim.x, sh.done);
 }
 
 // The segment-affine staged launch (the nested form of two-level segmenting:
@@ -293,9 +314,10 @@ template <class Op>
 __global__ void __launch_bounds__(1024, 1)
 affine_gather_kernel(StagedTasks q, const typename Op::T* __restrict__ x,
                      const int32_t* __restrict__ seg_lo, const int32_t* __restrict__ seg_tab,
-                     int m, int m2, unsigned* __restrict__ next_seg,
+                     int m, int m2, unsigned* __restrict__ next_seg, unsigned* __restrict__ done,
                      typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   using T = typename Op::T;
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
   __shared__ int32_t s_seg;
@@ -313,6 +335,7 @@ affine_gather_kernel(StagedTasks q, const typename Op::T* __restrict__ x,
     __syncthreads();
     staged_run<Op>(q, tb, te, w, 32, tab, out, carry);
   }
+  counters_done(next_seg, 1, done);
 }
 
 // L1/L2 chunks of segments [m, k) taken from a queue (a global counter of
@@ -377,10 +400,12 @@ overlap_gather_kernel(StagedTasks q, StagedShare sh, const uint32_t* __restrict_
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ RangeSlots slots;
+  chain_begin();
   if ((int)threadIdx.x < staged_threads)
     staged_pieces<Op>(q, sh, x, out, carry, reinterpret_cast<T*>(smem_raw), staged_threads, &slots);
   cached_queue<Op>(colf, x, nx, first_row, seg_cstart, seg_E, seg_chunk, seg_lo, m, k, next_chunk,
                    out, carry);
+  counters_done(next_chunk, 4 + (int)gridDim.x, sh.done);  // the ranges' lie behind it
 }
 
 // Block b's first task: equal stretches of the stream.
@@ -440,7 +465,7 @@ int seg_plan_alloc(int64_t E, int k, const std::vector<int64_t>& edge_base,
   DeviceInfo di{};
   CG_TRY(device_info(&di));
   const size_t n = (size_t)k + 1, most = (size_t)di.sm_count * 2;  // blocks of any staged shape
-  const size_t words = 2 * 4 * n + 2 * n + 2 * n + 3 * n + (2 + most) + (most + 1);
+  const size_t words = 2 * 4 * n + 2 * n + 2 * n + 3 * n + (4 + most) + (most + 1);
   CG_CUDA(cudaMalloc((void**)&p->meta, 4 * words));
   int32_t* w = reinterpret_cast<int32_t*>(p->meta) + 2 * 4 * n;
   p->seg_cstart = p->meta + 2 * n;
@@ -452,7 +477,8 @@ int seg_plan_alloc(int64_t E, int k, const std::vector<int64_t>& edge_base,
   p->seg_tab = w + 3 * n;
   p->seg_task = w + 4 * n;
   p->counter = reinterpret_cast<unsigned*>(w + 5 * n);
-  p->blk_task = w + 5 * n + 2 + most;
+  p->blk_task = w + 5 * n + 4 + most;
+  CG_CUDA(cudaMemsetAsync(p->counter, 0, 4 * (4 + most), s));
   std::vector<int64_t> up(4 * n, 0);  // edge_base, cstart, bounds, then seg_E and seg_lo
   int32_t* eo = reinterpret_cast<int32_t*>(up.data() + 3 * n);
   for (size_t q = 0; q < n; ++q) {
@@ -476,8 +502,23 @@ int seg_plan_finish(SegPlan* p, const int32_t* rp32, int64_t rows,
   return seg_plan_configure(p, 1024, 1, -1, s);
 }
 
+// The staged kernels may take the largest table (a launch asks for its own).
+template <class Op>
+static int allow_tables() {
+  const void* fns[] = {(const void*)staged_gather_kernel<Op, 1024>,
+                       (const void*)staged_gather_kernel<Op, 512>,
+                       (const void*)affine_gather_kernel<Op>,
+                       (const void*)overlap_gather_kernel<Op>};
+  const int most = 4 * seg_table_capacity(1) + 16;
+  for (const void* f : fns)
+    CG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+  return CG_OK;
+}
+
 int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertices,
                        cudaStream_t s) {
+  CG_TRY(allow_tables<SumF32>());
+  CG_TRY(allow_tables<MinI32>());
   if (threads != 512 && threads != 1024) {
     set_error("gather threads must be 512 or 1024 (got %d)", threads);
     return CG_ERR_INVALID_ARG;
@@ -637,7 +678,7 @@ static StagedTasks staged_tasks(const SegPlan& p) {
 }
 
 static StagedShare staged_share(const SegPlan& p) {
-  return StagedShare{{p.blk_task, p.counter + 2}, p.seg_lo, p.seg_tab, p.m};
+  return StagedShare{{p.blk_task, p.counter + 4}, p.counter + 2, p.seg_lo, p.seg_tab, p.m};
 }
 
 // the table and, behind it, the identity's entry
@@ -649,14 +690,8 @@ static int launch_staged(const SegPlan& p, const typename Op::T* x, typename Op:
   using T = typename Op::T;
   const size_t smem = staged_smem(p);
   auto fn = staged_gather_kernel<Op, THREADS>;
-  CG_CUDA(cudaMemsetAsync(p.counter, 0, sizeof(unsigned) * (2 + p.grid), s));
-  if (smem > 48 * 1024)
-    CG_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
-  fn<<<p.grid, THREADS, smem, s>>>(staged_tasks(p), staged_share(p), x, out,
-                                   reinterpret_cast<T*>(p.carry));
-  CG_LAUNCH_CHECK();
-  return CG_OK;
+  return launch_chained(fn, p.grid, THREADS, smem, s, staged_tasks(p), staged_share(p), x, out,
+                        reinterpret_cast<T*>(p.carry));
 }
 
 template <class Op>
@@ -665,16 +700,9 @@ static int launch_overlap(const SegPlan& p, const typename Op::T* x, int32_t nx,
   using T = typename Op::T;
   const size_t smem = staged_smem(p);
   auto fn = overlap_gather_kernel<Op>;
-  CG_CUDA(cudaMemsetAsync(p.counter, 0, sizeof(unsigned) * (2 + p.grid), s));
-  if (smem > 48 * 1024)
-    CG_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
-  fn<<<p.grid, 1024, smem, s>>>(staged_tasks(p), staged_share(p), p.colf, x, nx, p.first_row,
-                                p.seg_cstart, p.seg_E, p.seg_chunk, p.seg_lo, p.m, p.k,
-                                1024 - 32 * p.overlap, p.counter, out,
-                                reinterpret_cast<T*>(p.carry));
-  CG_LAUNCH_CHECK();
-  return CG_OK;
+  return launch_chained(fn, p.grid, 1024, smem, s, staged_tasks(p), staged_share(p), p.colf, x, nx,
+                        p.first_row, p.seg_cstart, p.seg_E, p.seg_chunk, p.seg_lo, p.m, p.k,
+                        1024 - 32 * p.overlap, p.counter, out, reinterpret_cast<T*>(p.carry));
 }
 
 template <class Op>
@@ -696,26 +724,19 @@ int run_seg_gather(const SegPlan& p, const typename Op::T* x, int32_t nx, typena
   // the table-sized cold segments, one block per segment
   if ((phases & kPhaseCached) && p.m2 > p.m) {
     const size_t smem = staged_smem(p);
-    auto fn = affine_gather_kernel<Op>;
-    CG_CUDA(cudaMemsetAsync(p.counter + 1, 0, sizeof(unsigned), s));
-    if (smem > 48 * 1024)
-      CG_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)smem));
-    fn<<<p.grid_affine, 1024, smem, s>>>(staged_tasks(p), x, p.seg_lo, p.seg_tab, p.m, p.m2,
-                                         p.counter + 1, out, reinterpret_cast<T*>(p.carry));
-    CG_LAUNCH_CHECK();
+    CG_TRY(launch_chained(affine_gather_kernel<Op>, p.grid_affine, 1024, smem, s, staged_tasks(p),
+                          x, p.seg_lo, p.seg_tab, p.m, p.m2, p.counter + 1, p.counter + 3, out,
+                          reinterpret_cast<T*>(p.carry)));
   }
   // the rest through L1/L2: no shared memory, so the whole on-chip store is L1
   if ((phases & kPhaseCached) && p.n_ctiles > 0) {
-    seg_gather_kernel<Op, 1024><<<p.grid_l2, 1024, 0, s>>>(
-        p.colf, x, nx, p.first_row, p.seg_cstart, p.seg_E, p.seg_chunk, p.seg_ctile, p.seg_lo,
-        p.k, 0, (int32_t)p.n_ctiles, out, reinterpret_cast<T*>(p.carry));
-    CG_LAUNCH_CHECK();
+    CG_TRY(launch_chained(seg_gather_kernel<Op, 1024>, p.grid_l2, 1024, 0, s, p.colf, x, nx,
+                          p.first_row, p.seg_cstart, p.seg_E, p.seg_chunk, p.seg_ctile, p.seg_lo,
+                          p.k, 0, (int32_t)p.n_ctiles, out, reinterpret_cast<T*>(p.carry)));
   }
   if ((phases & kPhaseFixup) && p.ncarry > 0) {
-    seg_fixup_kernel<Op><<<grid_for(p.ncarry, 256, 8), 256, 0, s>>>(
-        p.carry_row, reinterpret_cast<const T*>(p.carry), p.ncarry, out);
-    CG_LAUNCH_CHECK();
+    CG_TRY(launch_chained(seg_fixup_kernel<Op>, grid_for(p.ncarry, 256, 8), 256, 0, s, p.carry_row,
+                          reinterpret_cast<const T*>(p.carry), p.ncarry, out));
   }
   return CG_OK;
 }

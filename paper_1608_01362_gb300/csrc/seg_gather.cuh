@@ -75,8 +75,9 @@ struct SegPlan {
   int grid_affine = 0;      // blocks of the segment-affine launch
   int64_t n_ctiles = 0;     // block-groups of the L1/L2 launch
   int grid = 0;             // staged launch blocks
-  unsigned* counter = nullptr;  // next L1/L2 chunk (overlap), next segment-affine segment,
-                                // tasks taken of each staged block's range
+  unsigned* counter = nullptr;  // next L1/L2 chunk (overlap), next segment-affine segment, blocks
+                                // finished of either, tasks taken of each staged block's range;
+                                // zero between launches (the last block of each clears them)
   int overlap_request = 0;  // warps per block given to the L1/L2 segments (0: two launches)
   int overlap = 0;          // the same, in effect (0 when one kind of segment is absent)
   int grid_l2 = 0;          // unstaged launch blocks (1024 threads, 2 per SM)

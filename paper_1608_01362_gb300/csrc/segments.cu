@@ -313,15 +313,22 @@ __global__ void to_i64_kernel(const int32_t* __restrict__ in, int64_t n,
     out[i] = in[i];
 }
 
-// Block-major merge index (blk[b*k + s]) -> segment-major local rows
-// (out[s*(nb+1) + b] = blk[b*k + s] - row_base[s]), the oracle's layout.
-__global__ void blk_local_kernel(const int32_t* __restrict__ blk, const int64_t* __restrict__ rb,
-                                 int k, int nb, int32_t* __restrict__ out) {
+// Merge-block indices of the caller's block size, segment-major and local to
+// the segment (out[s*(nb+1) + b]: rows of segment s with destination < b*B),
+// the oracle's layout.
+__global__ void blk_local_kernel(const int32_t* __restrict__ idx_map,
+                                 const int64_t* __restrict__ rb, int k, int B, int nb,
+                                 int32_t* __restrict__ out) {
   const int64_t n = (int64_t)k * (nb + 1);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t sg = i / (nb + 1), b = i % (nb + 1);
-    out[i] = (int32_t)(blk[b * k + sg] - rb[sg]);
+    const int64_t sg = i / (nb + 1), v = (i % (nb + 1)) * B;
+    int64_t lo = rb[sg], hi = rb[sg + 1];
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (idx_map[mid] < v) lo = mid + 1; else hi = mid;
+    }
+    out[i] = (int32_t)(lo - rb[sg]);
   }
 }
 
@@ -329,6 +336,10 @@ int build_impl(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,
                const std::vector<int64_t>& bounds, int32_t B, cg_segmented* g, cudaStream_t s) {
   const int64_t ntiles = ceil_div(E, kSplitTile);
   g->nb = (int32_t)ceil_div(V, B);
+  DeviceInfo di{};
+  CG_TRY(device_info(&di));
+  g->mB = merge_block(V, B, di.sm_count);
+  g->mnb = (int32_t)ceil_div(V, g->mB);
   const size_t e4 = Scratch::round(4 * (size_t)E), kt = (size_t)k * ntiles;
   Scratch tmp(s, e4 + Scratch::round(4 * kt) + Scratch::round(8 * (kt + 1)) +
                      scan_scratch((int64_t)kt) + scan_scratch(ntiles) +
@@ -387,7 +398,7 @@ int build_impl(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,
   }
   g->rows = rows;
   // idx_map, row_ptr and blk: one allocation
-  const size_t n1 = (size_t)(rows > 0 ? rows : 1), nbk = (size_t)k * (g->nb + 1);
+  const size_t n1 = (size_t)(rows > 0 ? rows : 1), nbk = (size_t)k * (g->mnb + 1);
   const size_t r4 = Scratch::round(4 * (n1 + 1));
   CG_CUDA(cudaMalloc((void**)&g->idx_map, 2 * r4 + 4 * nbk));
   g->row_ptr = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(g->idx_map) + r4);
@@ -405,13 +416,13 @@ int build_impl(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,
   CG_CUDA(cudaMemcpyAsync(g->row_base.data(), d_rb, sizeof(int64_t) * (k + 1),
                           cudaMemcpyDeviceToHost, s));
   // D
-  blk_kernel<<<grid_for((int64_t)nbk, 256), 256, 0, s>>>(d_rb, k, g->idx_map, B, g->nb, g->blk);
+  blk_kernel<<<grid_for((int64_t)nbk, 256), 256, 0, s>>>(d_rb, k, g->idx_map, g->mB, g->mnb, g->blk);
   CG_LAUNCH_CHECK();
   CG_CUDA(cudaStreamSynchronize(s));  // row_base
   // E
   CG_TRY(seg_plan_finish(p, g->row_ptr, rows, g->row_base, s));
   // the iteration state, one allocation: dslot, counter, partials, rank_tmp, contrib_tmp, interm
-  const size_t v4 = Scratch::round(4 * (size_t)V), pb = Scratch::round(16 * (size_t)g->nb);
+  const size_t v4 = Scratch::round(4 * (size_t)V), pb = Scratch::round(16 * (size_t)g->mnb);
   CG_CUDA(cudaMalloc((void**)&g->state, 256 + pb + 2 * v4 + 4 * n1));
   CG_CUDA(cudaMemsetAsync(g->state, 0, 256, s));
   g->dslot = reinterpret_cast<double*>(g->state);
@@ -421,8 +432,8 @@ int build_impl(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,
   g->contrib_tmp = reinterpret_cast<float*>(g->state + 256 + pb + v4);
   g->interm = g->state + 256 + pb + 2 * v4;
   CG_CUDA(cudaStreamSynchronize(s));
-  g->bytes = 4 * (rows + 1) + 4 * rows + 4 * (int64_t)k * (g->nb + 1) +
-             seg_plan_bytes(g->plan) + 4 * rows + 16 * (int64_t)g->nb + 4 + 32 + 8 * (int64_t)V;
+  g->bytes = 4 * (rows + 1) + 4 * rows + 4 * (int64_t)k * (g->mnb + 1) +
+             seg_plan_bytes(g->plan) + 4 * rows + 16 * (int64_t)g->mnb + 4 + 32 + 8 * (int64_t)V;
   return CG_OK;
 }
 
@@ -433,6 +444,12 @@ void free_segmented(cg_segmented* g) {
 }
 
 }  // namespace
+
+int32_t merge_block(int32_t V, int32_t B, int sm_count) {
+  int32_t b = B;
+  while (b > 32 && ceil_div(V, b) < (int64_t)sm_count * 48) b = std::max(32, (b + 1) / 2);
+  return b;
+}
 
 int validate_csr(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,
                  cudaStream_t s) {
@@ -662,7 +679,7 @@ int cg_segmented_export(const cg_segmented* g, int64_t* h_bounds, int64_t* h_row
                                     cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
       blk_local_kernel<<<grid_for((int64_t)g->k * (g->nb + 1), 256), 256, 0, s>>>(
-          g->blk, d_rb, g->k, g->nb, d_block_start);
+          g->idx_map, d_rb, g->k, g->B, g->nb, d_block_start);
       e = cudaGetLastError();
     }
     cudaFreeAsync(d_rb, s);
