@@ -50,8 +50,10 @@ struct cg_bipartite {
   int64_t* poff[2] = {nullptr, nullptr};  // (the segments' where the side has them)
   int64_t npieces[2] = {0, 0};
   float* gpart[2] = {nullptr, nullptr};  // [npieces][K] piece gradients
-  // vertices with more than kCfWarp pieces: the first nwide with more than kCfWide
+  // vertices with more than kCfWide pieces, and from the list's end those with
+  // more than kCfWarp
   int32_t* wide[2] = {nullptr, nullptr};
+  int32_t* warp[2] = {nullptr, nullptr};
   int32_t nwide[2] = {0, 0}, nwarp[2] = {0, 0};
   // factor storage (FP32, BF16, or BF16 hi + lo words); index 1 unused
   void* P[2] = {nullptr, nullptr};
@@ -499,7 +501,7 @@ int sweep_side(cg_bipartite* h, int side, double* sse, float lambda, float step,
       CG_LAUNCH_CHECK();
       cf_update_warp_kernel<LANES, PREC>
           <<<grid_for((int64_t)h->nwarp[side] * 32, kCfThreads, 8), kCfThreads, 0, s>>>(
-              h->wide[side] + h->nwide[side], h->nwarp[side], h->poff[side], h->seg[side].slots,
+              h->warp[side], h->nwarp[side], h->poff[side], h->seg[side].slots,
               off, h->gpart[side], self[0], lambda, step);
     }
     if (h->nwide[side] > 0) {
@@ -580,12 +582,24 @@ void cf_free(cg_bipartite* h) {
     cf_seg_free(&h->seg[s]);
     cudaFree(h->gpart[s]);
     cudaFree(h->wide[s]);
-    cudaFree(h->P[s]);
-    cudaFree(h->Q[s]);
   }
-  cudaFree(h->partials);
-  cudaFree(h->counter);
+  cudaFree(h->P[0]);  // with Q, the partials and the counter
   delete h;
+}
+
+// Lists the vertices with more than kCfWide pieces from the list's front and
+// those with more than kCfWarp from its end (cap is at least the number of
+// either together).  Each vertex's update is its own: the order is of no account.
+__global__ void many_pieces_kernel(const int64_t* __restrict__ poff, int64_t n, int32_t cap,
+                                   int32_t* __restrict__ list, int32_t* __restrict__ count) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t np = poff[v + 1] - poff[v];
+    if (np > kCfWide)
+      list[atomicAdd(count, 1)] = (int32_t)v;
+    else if (np > kCfWarp)
+      list[cap - 1 - atomicAdd(count + 1, 1)] = (int32_t)v;
+  }
 }
 
 // The pieces of the gather from L2: at most kCfPiece ratings of one vertex.
@@ -641,24 +655,22 @@ int build_pieces(cg_bipartite* h, int side, cudaStream_t s) {
     CG_TRY(build_plain_pieces(h, side, s));
   }
   // vertices with many pieces get a warp or a whole block in the update
-  std::vector<int64_t> hp((size_t)n + 1);
-  CG_CUDA(cudaMemcpyAsync(hp.data(), h->poff[side], sizeof(int64_t) * (size_t)(n + 1),
-                          cudaMemcpyDeviceToHost, s));
-  CG_CUDA(cudaStreamSynchronize(s));
-  std::vector<int32_t> wide;
-  for (int64_t v = 0; v < n; ++v)
-    if (hp[v + 1] - hp[v] > kCfWide) wide.push_back((int32_t)v);
-  h->nwide[side] = (int32_t)wide.size();
-  for (int64_t v = 0; v < n; ++v)
-    if (hp[v + 1] - hp[v] > kCfWarp && hp[v + 1] - hp[v] <= kCfWide) wide.push_back((int32_t)v);
-  h->nwarp[side] = (int32_t)wide.size() - h->nwide[side];
-  if (!wide.empty()) {
-    CG_CUDA(cudaMalloc((void**)&h->wide[side], sizeof(int32_t) * wide.size()));
-    h->bytes += 4 * (int64_t)wide.size();
-    CG_CUDA(cudaMemcpyAsync(h->wide[side], wide.data(), sizeof(int32_t) * wide.size(),
-                            cudaMemcpyHostToDevice, s));
-    CG_CUDA(cudaStreamSynchronize(s));
+  const int32_t cap = (int32_t)(h->npieces[side] / kCfWarp + 1);
+  CG_CUDA(cudaMalloc((void**)&h->wide[side], sizeof(int32_t) * ((size_t)cap + 2)));
+  h->bytes += 4 * ((int64_t)cap + 2);
+  int32_t* count = h->wide[side] + cap;
+  CG_CUDA(cudaMemsetAsync(count, 0, 2 * sizeof(int32_t), s));
+  if (n > 0) {
+    many_pieces_kernel<<<grid_for(n, 256), 256, 0, s>>>(h->poff[side], n, cap, h->wide[side],
+                                                        count);
+    CG_LAUNCH_CHECK();
   }
+  int32_t got[2] = {0, 0};
+  CG_CUDA(cudaMemcpyAsync(got, count, sizeof(got), cudaMemcpyDeviceToHost, s));
+  CG_CUDA(cudaStreamSynchronize(s));
+  h->nwide[side] = got[0];
+  h->nwarp[side] = got[1];
+  h->warp[side] = h->wide[side] + cap - got[1];
   return CG_OK;
 }
 
@@ -768,19 +780,22 @@ int cf_create(int64_t U, int64_t I, int32_t K, int32_t precision, const int64_t*
   if (st == CG_OK) st = build_pieces(h, 1, stream);
   cudaError_t e = cudaSuccess;
   const size_t el = precision == 1 ? 2 : 4;  // BF16 hi + lo: one 32-bit word per entry
-  const int planes = 1;
-  for (int pl = 0; pl < planes && st == CG_OK && e == cudaSuccess; ++pl) {
-    e = cudaMalloc(&h->P[pl], el * (size_t)U * K);
-    if (e == cudaSuccess) e = cudaMalloc(&h->Q[pl], el * (size_t)I * K);
-    h->bytes += (int64_t)(el * (size_t)(U + I) * K);
-  }
-  if (st == CG_OK && e == cudaSuccess) {
-    DeviceInfo di{};
-    st = device_info(&di);
+  DeviceInfo di{};
+  if (st == CG_OK) st = device_info(&di);
+  if (st == CG_OK) {
     h->gather_grid = di.sm_count * 8;  // 2048 threads per SM at 256 per block
-    if (st == CG_OK) e = cudaMalloc((void**)&h->partials, sizeof(double) * h->gather_grid);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->counter, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->counter, 0, sizeof(unsigned), stream);
+    const size_t pb = Scratch::round(el * (size_t)U * K), qb = Scratch::round(el * (size_t)I * K),
+                 sb = Scratch::round(sizeof(double) * h->gather_grid);
+    char* slab = nullptr;
+    e = cudaMalloc((void**)&slab, pb + qb + sb + sizeof(unsigned));
+    if (e == cudaSuccess) {
+      h->P[0] = slab;
+      h->Q[0] = slab + pb;
+      h->partials = reinterpret_cast<double*>(slab + pb + qb);
+      h->counter = reinterpret_cast<unsigned*>(slab + pb + qb + sb);
+      h->bytes += (int64_t)(el * (size_t)(U + I) * K);
+      e = cudaMemsetAsync(h->counter, 0, sizeof(unsigned), stream);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   }
   if (st == CG_OK && e != cudaSuccess) st = cuda_fail(e, "cf_create", __FILE__, __LINE__);

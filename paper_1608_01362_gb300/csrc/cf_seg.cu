@@ -540,9 +540,12 @@ int cf_seg_build(CfSegments* c, int64_t n, int64_t nn, int64_t R, int K, const i
   // (ratings that are not grouped by segment would break into single ones)
   if (bad || !segments_pay(K, R, nruns, di.l2_bytes)) return CG_OK;
   const int64_t most = nruns + R / kCfSegPiece;  // pieces at most
+  const size_t tasks = (size_t)(most / G + k);     // tasks at most
   Scratch t2(s, 4 * Scratch::round(4 * (size_t)nruns) + Scratch::round(8 * (size_t)(nruns + 1)) +
                     scan_scratch(nruns) + 5 * Scratch::round(4 * (size_t)most) +
-                    sort_scratch(most) + Scratch::round(8 * (size_t)(k + 1)) + 4096);
+                    sort_scratch(most) + Scratch::round(8 * (size_t)(k + 1)) +
+                    Scratch::round(4 * tasks) + Scratch::round(8 * tasks + 8) +
+                    scan_scratch((int64_t)tasks) + 8192);
   int32_t *begin = nullptr, *vtx = nullptr, *seg = nullptr, *np = nullptr, *item = nullptr,
           *sitem = nullptr, *run = nullptr;
   int64_t *run_first = nullptr, *seg_item = nullptr;
@@ -605,15 +608,13 @@ int cf_seg_build(CfSegments* c, int64_t n, int64_t nn, int64_t R, int K, const i
   CG_LAUNCH_CHECK();
   cf_poff_kernel<<<grid_for(n + 1, 256), 256, 0, s>>>(off, n, begin, nruns, run_first, c->poff);
   CG_LAUNCH_CHECK();
-  Scratch t3(s, Scratch::round(4 * (size_t)c->ntasks) + Scratch::round(8 * (size_t)c->ntasks + 8) +
-                    scan_scratch(c->ntasks) + 1024);
   int32_t* cost = nullptr;
   int64_t* before = nullptr;
-  CG_CUDA(t3.get(&cost, c->ntasks));
-  CG_CUDA(t3.get(&before, (size_t)c->ntasks + 1));
+  CG_CUDA(t2.get(&cost, c->ntasks));
+  CG_CUDA(t2.get(&before, (size_t)c->ntasks + 1));
   cf_cost_kernel<<<grid_for(c->ntasks, 256), 256, 0, s>>>(c->recs, G, c->ntasks, cost);
   CG_LAUNCH_CHECK();
-  CG_TRY(exclusive_scan_i32_to_i64(cost, before, c->ntasks, s, &t3));
+  CG_TRY(exclusive_scan_i32_to_i64(cost, before, c->ntasks, s, &t2));
   cf_share_kernel<<<grid_for(c->grid + 1, 128), 128, 0, s>>>(before, c->ntasks, c->grid,
                                                               c->blk_task);
   CG_LAUNCH_CHECK();
