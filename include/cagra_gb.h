@@ -490,10 +490,9 @@ typedef struct cg_ppr cg_ppr;
  * teleports to seed_j and returns its dangling mass there:
  *   R'[v][j] = d sum_{u->v} C[u][j] + [v == seed_j] ((1-d) + d D_j)
  *   C'[v][j] = R'[v][j] * inv[v],  D'_j = sum over inv[v] = 0 of R'[v][j]
- * The state C is held by the handle as BF16: planes = 2 stores hi = bf16(c)
- * and lo = bf16(c - hi) (about 16 significant bits), planes = 1 stores hi
- * only (8 bits, half the gather traffic); sums are FP32, D_j and residuals
- * FP64.  The segmented graph must outlive the handle and stay unchanged.
+ * The state C is held by the handle in 32 bits per value with planes = 2
+ * (FP32), as BF16 with planes = 1 (8 significant bits, half the gather
+ * traffic); sums are FP32, D_j and residuals FP64.  The segmented graph must outlive the handle and stay unchanged.
  * Memory: about rows*256 + V*(256 + 128*planes) + E/128*260 bytes.
  * Synchronizes.
  */

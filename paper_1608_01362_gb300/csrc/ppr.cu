@@ -7,11 +7,12 @@
 // (the teleport and the dangling mass of column j return to its seed).
 //
 // Storage.  The iteration state is C (the contributions R/outdeg) of the
-// non-dangling vertices, as BF16 planes: hi = bf16(c) and, with two planes,
-// lo = bf16(c - hi), 128 bytes per vertex per plane.  Gathers read the
-// planes and accumulate hi + lo in FP32.  R itself is written in FP32 only
-// when asked for (the last iteration, and the one before it for the L1
-// residual); D_j and the residual are FP64 with a fixed reduction order.
+// non-dangling vertices: with two planes FP32, 256 bytes per vertex (the bytes
+// of a BF16 hi + lo pair, at full precision: an edge is then four packed adds
+// and no unpacking), with one plane BF16, 128 bytes.  Gathers accumulate in
+// FP32.  R itself is written in FP32 only when asked for (the last iteration,
+// and the one before it for the L1 residual); D_j and the residual are FP64
+// with a fixed reduction order.
 //
 // Kernels per iteration:
 //   ppr_gather_kernel  an octet (8 lanes, 8 columns each) walks a 128-edge
@@ -22,7 +23,7 @@
 //                      to a carry slot;
 //   ppr_fixup_kernel   completes the rows that span chunks: each run of
 //                      carries (consecutive chunks open on the same row, a
-//                      static structure) is cut into pieces of <= 32 chunks
+//                      static structure) is cut into pieces of <= 16 chunks
 //                      summed in parallel; the last piece of a run adds the
 //                      pieces' sums, in order, into the row;
 //   ppr_merge_kernel   an octet takes 16 consecutive destinations, sums
@@ -39,18 +40,41 @@ namespace {
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-__device__ __forceinline__ void add_row(float (&acc)[8], const uint4& h) {
-  acc[0] += bf_lo(h.x); acc[1] += bf_hi(h.x);
-  acc[2] += bf_lo(h.y); acc[3] += bf_hi(h.y);
-  acc[4] += bf_lo(h.z); acc[5] += bf_hi(h.z);
-  acc[6] += bf_lo(h.w); acc[7] += bf_hi(h.w);
+// 8 FP32 values as 4 packed pairs: one 32-byte load, four packed adds
+// (rounded as the scalar ones).
+struct Row8 {
+  uint64_t p[4];
+};
+
+__device__ __forceinline__ uint64_t pair(float a, float b) {
+  return (uint64_t)__float_as_uint(b) << 32 | __float_as_uint(a);
 }
 
-__device__ __forceinline__ void add_row2(float (&acc)[8], const uint4& h, const uint4& l) {
-  acc[0] += bf_lo(h.x) + bf_lo(l.x); acc[1] += bf_hi(h.x) + bf_hi(l.x);
-  acc[2] += bf_lo(h.y) + bf_lo(l.y); acc[3] += bf_hi(h.y) + bf_hi(l.y);
-  acc[4] += bf_lo(h.z) + bf_lo(l.z); acc[5] += bf_hi(h.z) + bf_hi(l.z);
-  acc[6] += bf_lo(h.w) + bf_lo(l.w); acc[7] += bf_hi(h.w) + bf_hi(l.w);
+__device__ __forceinline__ void add_row(Row8& acc, const Row8& x) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc.p[q]) : "l"(x.p[q]));
+}
+
+// Columns 8 lane8 .. 8 lane8 + 7 of a contribution row.  FP32 rows are not kept
+// in L1: hardly one in eight is read again in time (274 us against 261 for a
+// gather of 15.7 M edges), and the edge words want the room.
+template <int PLANES>
+__device__ __forceinline__ Row8 load_contrib(const void* c, uint32_t row, int lane8) {
+  Row8 x;
+  if (PLANES == 2) {
+    const float* p = static_cast<const float*>(c) + ((int64_t)row * kCols + lane8 * 8);
+    asm volatile("ld.global.L1::no_allocate.v4.b64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(x.p[0]), "=l"(x.p[1]), "=l"(x.p[2]), "=l"(x.p[3])
+                 : "l"(p));
+  } else {
+    const uint4 h = __ldg(static_cast<const uint4*>(c) + ((int64_t)row * 8 + lane8));
+    x.p[0] = pair(bf_lo(h.x), bf_hi(h.x));
+    x.p[1] = pair(bf_lo(h.y), bf_hi(h.y));
+    x.p[2] = pair(bf_lo(h.z), bf_hi(h.z));
+    x.p[3] = pair(bf_lo(h.w), bf_hi(h.w));
+  }
+  return x;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
@@ -58,116 +82,138 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<const uint32_t*>(&p);
 }
 
-// hi = bf16(c); lo = bf16(c - hi) (c - hi is exact in FP32).
-__device__ __forceinline__ void split_row(const float (&c)[8], uint4* hi, uint4* lo) {
-  uint32_t h[4], l[4];
+// An octet's row moves in 32-byte pieces, one instruction and whole sectors a
+// lane; streaming (evict-first): intermBuf and carries must not push the
+// segment's C rows out of L2.
+__device__ __forceinline__ void store_row(float* dst, const Row8& a) {
+  asm volatile("st.global.cs.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(dst), "l"(a.p[0]), "l"(a.p[1]),
+               "l"(a.p[2]), "l"(a.p[3])
+               : "memory");
+}
+
+__device__ __forceinline__ Row8 load_row(const float* src) {
+  Row8 x;
+  asm volatile("ld.global.cs.v4.b64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(x.p[0]), "=l"(x.p[1]), "=l"(x.p[2]), "=l"(x.p[3])
+               : "l"(src)
+               : "memory");
+  return x;
+}
+
+__device__ __forceinline__ void unpack(const Row8& a, float (&x)[8]) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    h[q] = pack_bf16(c[2 * q], c[2 * q + 1]);
-    l[q] = pack_bf16(c[2 * q] - bf_lo(h[q]), c[2 * q + 1] - bf_hi(h[q]));
-  }
-  *hi = make_uint4(h[0], h[1], h[2], h[3]);
-  if (lo) *lo = make_uint4(l[0], l[1], l[2], l[3]);
+  for (int q = 0; q < 8; ++q) x[q] = __uint_as_float((uint32_t)(a.p[q >> 1] >> (32 * (q & 1))));
 }
 
-// streaming (evict-first) store: intermBuf and carries must not push the
-// segment's C rows out of L2
-__device__ __forceinline__ void store_row(float* dst, const float (&a)[8]) {
-  float4* p = reinterpret_cast<float4*>(dst);
-  __stcs(p, make_float4(a[0], a[1], a[2], a[3]));
-  __stcs(p + 1, make_float4(a[4], a[5], a[6], a[7]));
+__device__ __forceinline__ Row8 pack(const float (&x)[8]) {
+  return {{pair(x[0], x[1]), pair(x[2], x[3]), pair(x[4], x[5]), pair(x[6], x[7])}};
 }
 
-__device__ __forceinline__ void load_row(const float* src, float (&a)[8]) {
-  const float4* p = reinterpret_cast<const float4*>(src);
-  const float4 x = __ldcs(p), y = __ldcs(p + 1);
-  a[0] = x.x; a[1] = x.y; a[2] = x.z; a[3] = x.w;
-  a[4] = y.x; a[5] = y.y; a[6] = y.z; a[7] = y.w;
-}
-
-__device__ __forceinline__ uint32_t pick(const uint4& v, int c) {
-  return c == 0 ? v.x : c == 1 ? v.y : c == 2 ? v.z : v.w;
+template <int PLANES>
+__device__ __forceinline__ void store_contrib(void* c, int64_t v, int lane8, const float (&x)[8]) {
+  if (PLANES == 2)
+    store_row(static_cast<float*>(c) + v * kCols + lane8 * 8, pack(x));
+  else
+    __stcs(static_cast<uint4*>(c) + v * 8 + lane8,
+           make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]),
+                      pack_bf16(x[6], x[7])));
 }
 
 // ---------------------------------------------------------------------------
 // Gather (Algorithm 3, 64-wide).  Octet o takes chunks o, o + #octets, ...:
 // all octets sweep the chunks in segment order together, so the C rows read
 // at any moment belong to one or two segments' source slices.
+//
+// What bounds it is the row reads' way from L2: 256 bytes an edge at 64 bytes
+// per cycle and SM, 215 us for 15.7 M edges at 1.92 GHz (two planes); the
+// kernel takes 246.  Reading rows as two BF16 planes it took 335: 67
+// instructions for four octets' edge, 32 of them unpacking.  Rows in flight
+// per octet beyond the one or two that fit in 40 registers, or more than 6
+// blocks per SM, cost (two rows at 5 blocks 316 us, 7 blocks 296): they evict
+// one another from L2 and the edge words from L1.
 // ---------------------------------------------------------------------------
 template <int PLANES>
-__global__ void __launch_bounds__(kThreads, 6)
+__global__ void __launch_bounds__(kThreads, kGatherBlocks)
 ppr_gather_kernel(const uint32_t* __restrict__ colf, const PprSeg* __restrict__ segs,
-                  const int2* __restrict__ chunks, int64_t nchunks,
-                  const uint4* __restrict__ c_hi, const uint4* __restrict__ c_lo,
+                  const int2* __restrict__ chunks, int64_t nchunks, const void* __restrict__ contrib,
                   float* __restrict__ interm, float* __restrict__ carry) {
-  // edges whose rows are loaded together: one with two planes (more resident
-  // warps hide the latency better than more loads per warp)
-  constexpr int U = 2 / PLANES;
+  chain_begin();
   const int lane8 = threadIdx.x & 7;
-  const unsigned omask = 0xffu << (threadIdx.x & 24);
-  const int64_t noct = ((int64_t)gridDim.x * blockDim.x) >> 3;
-  for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; c < nchunks;
-       c += noct) {
+  const int noct = (int)((gridDim.x * blockDim.x) >> 3);
+  for (int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 3); c < (int)nchunks; c += noct) {
     const int2 ch = __ldg(chunks + c);
     const PprSeg sg = segs[ch.y];
     const int64_t el = (c - sg.chunk0) * kChunk;
     const int n = (int)min((int64_t)kChunk, (int64_t)sg.E - el);
     const uint4* cf = reinterpret_cast<const uint4*>(colf + sg.cstart + el);
-    const uint4* hb = c_hi + (int64_t)sg.lo * 8 + lane8;
-    const uint4* lb = c_lo + (int64_t)sg.lo * 8 + lane8;
     int32_t row = ch.x;
-    float acc[8];
+    Row8 acc = {{0, 0, 0, 0}};
+    for (int g = 0; g < n; g += 4, ++cf) {
+      const uint4 f4 = __ldg(cf);  // the octet's lanes read the same four edges
+      const uint32_t f[4] = {f4.x, f4.y, f4.z, f4.w};
+      if (g + 4 <= n && !((f4.x | f4.y | f4.z | f4.w) & kRowEnd)) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.0f;
-    uint32_t last = kRowEnd;
-    for (int sb = 0; sb < n; sb += 32) {
-      const int m = min(32, n - sb);
-      uint4 f4 = make_uint4(0u, 0u, 0u, 0u);
-      if (4 * lane8 < m) f4 = __ldcs(cf + (sb >> 2) + lane8);
-      for (int g = 0; g < m; g += 4) {  // the 4 edges held by octet lane g / 4
+        for (int u = 0; u < 4; ++u)
+          add_row(acc, load_contrib<PLANES>(contrib, sg.lo + f[u], lane8));
+        continue;
+      }
 #pragma unroll
-        for (int u0 = 0; u0 < 4; u0 += U) {
-          uint32_t f[U];
-          uint4 h[U], l[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            f[u] = __shfl_sync(omask, pick(f4, u0 + u), g >> 2, 8);
-            if (g + u0 + u < m) {
-              const int64_t s = (int64_t)(f[u] & ~kRowEnd) * 8;
-              h[u] = __ldg(hb + s);
-              if (PLANES == 2) l[u] = __ldg(lb + s);
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            if (g + u0 + u < m) {
-              if (PLANES == 2) add_row2(acc, h[u], l[u]); else add_row(acc, h[u]);
-              last = f[u];
-              if (f[u] & kRowEnd) {
-                store_row(interm + (int64_t)row * kCols + lane8 * 8, acc);
-                ++row;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) acc[q] = 0.0f;
-              }
-            }
+      for (int u = 0; u < 4; ++u) {
+        if (g + u < n) {
+          add_row(acc, load_contrib<PLANES>(contrib, sg.lo + (f[u] & ~kRowEnd), lane8));
+          if (f[u] & kRowEnd) {
+            store_row(interm + (int64_t)row * kCols + lane8 * 8, acc);
+            ++row;
+            acc = {{0, 0, 0, 0}};
           }
         }
       }
     }
-    if (!(last & kRowEnd)) store_row(carry + c * kCols + lane8 * 8, acc);  // open row
+    // the row open at the chunk's end
+    if (!(__ldg(colf + sg.cstart + el + n - 1) & kRowEnd))
+      store_row(carry + (int64_t)c * kCols + lane8 * 8, acc);
   }
 }
 
-// Rows that span chunks.  One octet per piece (<= 32 consecutive chunks of
-// one run): it sums the pieces' carries in chunk order.  A run of one piece
-// adds its sum into the row directly; otherwise each piece stores its sum and
-// the last piece of the run to finish (atomic count, no waiting) adds the
-// pieces' sums in piece order into the row -- deterministic, and a hub row
-// spanning thousands of chunks no longer holds up one octet.
+// The sum of n rows, in order, four of them in flight (they are read past L1:
+// another octet may have written them in this launch).
+__device__ __forceinline__ void sum_rows(const float* src, int n, float (&sum)[8]) {
+  constexpr int U = 4;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) sum[q] = 0.0f;
+  for (int j = 0; j < n; j += U) {
+    float4 a[U], b[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      a[u] = b[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (j + u < n) {
+        const float4* p = reinterpret_cast<const float4*>(src + (int64_t)(j + u) * kCols);
+        a[u] = __ldcg(p);
+        b[u] = __ldcg(p + 1);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (j + u >= n) break;
+      sum[0] += a[u].x; sum[1] += a[u].y; sum[2] += a[u].z; sum[3] += a[u].w;
+      sum[4] += b[u].x; sum[5] += b[u].y; sum[6] += b[u].z; sum[7] += b[u].w;
+    }
+  }
+}
+
+// Rows that span chunks.  One octet per piece (<= kPprPiece consecutive chunks
+// of one run): it sums the chunks' carries in order.  A run of one piece adds
+// its sum into the row directly; otherwise each piece stores its sum and the
+// last piece of the run to finish (atomic count, no waiting) adds the pieces'
+// sums in piece order into the row -- deterministic, and a hub row spanning
+// thousands of chunks does not hold up one octet.  What bounds it is that
+// chain of reads, so pieces are short and their rows read four at a time (23.8
+// us with pieces of 32 read one by one, 10.1 so, at 122,657 chunks).
 __global__ void __launch_bounds__(kThreads)
 ppr_fixup_kernel(const int4* __restrict__ pieces, int64_t npieces, const int4* __restrict__ runs,
                  const float* __restrict__ carry, float* __restrict__ piece_sum,
                  unsigned* __restrict__ run_done, float* __restrict__ interm) {
+  chain_begin();
   const int lane8 = threadIdx.x & 7;
   const unsigned omask = 0xffu << (threadIdx.x & 24);
   const int64_t noct = ((int64_t)gridDim.x * blockDim.x) >> 3;
@@ -176,21 +222,16 @@ ppr_fixup_kernel(const int4* __restrict__ pieces, int64_t npieces, const int4* _
     const int4 pc = __ldg(pieces + p);  // (first chunk, chunks, run)
     const int4 rn = __ldg(runs + pc.z); // (row, first piece, pieces)
     float sum[8], x[8];
-    load_row(carry + (int64_t)pc.x * kCols + lane8 * 8, sum);
-    for (int j = 1; j < pc.y; ++j) {
-      load_row(carry + ((int64_t)pc.x + j) * kCols + lane8 * 8, x);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) sum[q] += x[q];
-    }
+    sum_rows(carry + (int64_t)pc.x * kCols + lane8 * 8, pc.y, sum);
     float* dst = interm + (int64_t)rn.x * kCols + lane8 * 8;
     if (rn.z == 1) {
-      load_row(dst, x);
+      unpack(load_row(dst), x);
 #pragma unroll
       for (int q = 0; q < 8; ++q) x[q] += sum[q];
-      store_row(dst, x);
+      store_row(dst, pack(x));
       continue;
     }
-    store_row(piece_sum + p * kCols + lane8 * 8, sum);
+    store_row(piece_sum + p * kCols + lane8 * 8, pack(sum));
     __threadfence();
     __syncwarp(omask);
     unsigned prev = 0;
@@ -199,25 +240,25 @@ ppr_fixup_kernel(const int4* __restrict__ pieces, int64_t npieces, const int4* _
     if (prev != (unsigned)rn.z - 1) continue;  // not the run's last piece
     __threadfence();
     float tot[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) tot[q] = 0.0f;
-    for (int j = 0; j < rn.z; ++j) {
-      const float4* ps =
-          reinterpret_cast<const float4*>(piece_sum + ((int64_t)rn.y + j) * kCols + lane8 * 8);
-      const float4 u = __ldcg(ps), w = __ldcg(ps + 1);
-      tot[0] += u.x; tot[1] += u.y; tot[2] += u.z; tot[3] += u.w;
-      tot[4] += w.x; tot[5] += w.y; tot[6] += w.z; tot[7] += w.w;
-    }
-    load_row(dst, x);
+    sum_rows(piece_sum + (int64_t)rn.y * kCols + lane8 * 8, rn.z, tot);
+    unpack(load_row(dst), x);
 #pragma unroll
     for (int q = 0; q < 8; ++q) x[q] += tot[q];
-    store_row(dst, x);
+    store_row(dst, pack(x));
     if (lane8 == 0) run_done[pc.z] = 0u;  // ready for the next iteration
   }
 }
 
 // ---------------------------------------------------------------------------
 // Merge (Algorithm 4, destination-major) fused with the personalised update.
+//
+// What bounds it is memory: its rows once in, the contributions once out (38 us
+// of the 69 it takes at 1 M vertices and 15.7 M edges), and the reads in flight
+// towards that: the first rows of an octet's next two destinations, 24 warps
+// per SM (with 32 and spills 71 us, with one row ahead 75).  The octets of a
+// warp go through their destinations together, so the update runs once for
+// four.  FP64 sums lie in shared memory, touched only where there is something
+// to add.
 // ---------------------------------------------------------------------------
 struct MergeArgs {
   const int32_t* dst_off;
@@ -226,25 +267,27 @@ struct MergeArgs {
   const float* inv;
   const int32_t* seeds;
   const uint32_t* seed_bits;
-  uint4* c_hi;
-  uint4* c_lo;
+  void* contrib;
   float* r_out;        // NULL: R' not written
   const float* r_old;  // NULL: no residual
   double* D;           // [64] in: D of the previous iterate; out: D'
   double* resid;       // [64] or NULL
-  double* partials;
-  unsigned* counter;
+  double* partials;    // [grid][128], then the groups' sums [ceil(grid / 32)][128]
+  unsigned* counter;   // groups finished, then each group's finished blocks
   float d;
   int32_t V;
 };
 
 template <int PLANES, bool RESID>
-__global__ void __launch_bounds__(kThreads, 4)
+__global__ void __launch_bounds__(kThreads, 3)
 ppr_merge_kernel(MergeArgs a) {
   __shared__ float s_tele[kCols];
   __shared__ int32_t s_seed[kCols];
-  __shared__ double s_red[kThreads / 32][2][kCols];
+  // per warp and lane: the FP64 sums of its columns 8 lane8 + q
+  __shared__ double s_acc[kThreads / 32][RESID ? 2 : 1][8][32];
+  __shared__ double s_half[2 * kCols];
   __shared__ bool s_last;
+  chain_begin();
   if (threadIdx.x < kCols) {
     s_tele[threadIdx.x] =
         (float)((1.0 - (double)a.d) + (double)a.d * a.D[threadIdx.x]);
@@ -252,38 +295,68 @@ ppr_merge_kernel(MergeArgs a) {
   }
   __syncthreads();
   const int lane8 = threadIdx.x & 7;
-  const unsigned omask = 0xffu << (threadIdx.x & 24);
   const int64_t noct = ((int64_t)gridDim.x * blockDim.x) >> 3;
+  const int oct = (threadIdx.x >> 3) & 3;
   const int64_t ntask = ((int64_t)a.V + kTask - 1) / kTask;
-  double dsum[8], rsum[8];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int q = 0; q < 8; ++q) dsum[q] = rsum[q] = 0.0;
-  const float4* in4 = reinterpret_cast<const float4*>(a.interm);
-  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; t < ntask; t += noct) {
-    const int64_t v0 = t * kTask;
+  for (int q = 0; q < 8; ++q) {
+    s_acc[w][0][q][lane] = 0.0;
+    if (RESID) s_acc[w][RESID][q][lane] = 0.0;
+  }
+  for (int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; t0 < ntask;
+       t0 += noct) {
+    // (an octet past the last task has no destinations)
+    const int64_t v0 = min((t0 + oct) * kTask, (int64_t)a.V);
     const int nv = (int)min((int64_t)kTask, (int64_t)a.V - v0);
-    // row-list offsets and reciprocal degrees of the task's destinations
+    // row-list offsets, first rows and reciprocal degrees of the destinations
     const int32_t off_a = __ldg(a.dst_off + v0 + min(lane8, nv));
     const int32_t off_b = __ldg(a.dst_off + v0 + min(8 + lane8, nv));
     const float inv_a = lane8 < nv ? __ldg(a.inv + v0 + lane8) : 0.0f;
     const float inv_b = 8 + lane8 < nv ? __ldg(a.inv + v0 + 8 + lane8) : 0.0f;
-    const uint32_t sbits = __ldg(a.seed_bits + (v0 >> 5)) >> (v0 & 31);
+    const uint32_t sbits = nv > 0 ? __ldg(a.seed_bits + (v0 >> 5)) >> (v0 & 31) : 0u;
     const int32_t o_end = __ldg(a.dst_off + v0 + nv);
-    float dpart[8], rpart[8], acc[8];
+    const int32_t row_a = off_a < o_end ? __ldg(a.dst_rows + off_a) : 0;
+    const int32_t row_b = off_b < o_end ? __ldg(a.dst_rows + off_b) : 0;
+    float dpart[8], rpart[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) dpart[q] = rpart[q] = acc[q] = 0.0f;
-    int i = 0;  // destination being accumulated
-    auto off_of = [&](int j) -> int32_t {  // start of destination j's rows, j in [0, nv]
-      const int32_t x = __shfl_sync(omask, off_a, j & 7, 8);
-      const int32_t y = __shfl_sync(omask, off_b, j & 7, 8);
-      return j >= nv ? o_end : j < 8 ? x : y;
+    for (int q = 0; q < 8; ++q) dpart[q] = rpart[q] = 0.0f;
+    // start of destination j's rows, j in [0, kTask] (o_end from nv on)
+    auto off_of = [&](int j) -> int32_t {
+      const int32_t x = __shfl_sync(0xffffffffu, j < 8 ? off_a : off_b, j & 7, 8);
+      return j >= nv ? o_end : x;
     };
-    auto finish = [&](int j) {  // update of destination v0 + j from acc
+    auto first_row = [&](int j, bool some) -> Row8 {  // zeros if it has none
+      const int32_t r = __shfl_sync(0xffffffffu, j < 8 ? row_a : row_b, j & 7, 8);
+      Row8 x = {{0, 0, 0, 0}};
+      if (some) x = load_row(a.interm + (int64_t)r * kCols + lane8 * 8);
+      return x;
+    };
+    // the first rows of the next two destinations are on their way
+    int32_t o0 = off_of(0), o1 = off_of(1), o2 = off_of(2);
+    Row8 ahead[2] = {first_row(0, o0 < o1), first_row(1, o1 < o2)};
+#pragma unroll 2
+    for (int j = 0; j < kTask; ++j) {  // a warp's octets go through their destinations together
+      Row8 sum = ahead[j & 1];
+      const int32_t p0 = o0 + 1, p1 = o1;
+      const int32_t o3 = off_of(min(j + 3, kTask));
+      if (j + 2 < kTask) ahead[j & 1] = first_row(j + 2, o2 < o3);
+      o0 = o1; o1 = o2; o2 = o3;
+      const float iv = __shfl_sync(0xffffffffu, j < 8 ? inv_a : inv_b, j & 7, 8);
+      if (j >= nv) continue;
+      for (int32_t p = p0; p < p1; p += 2) {
+        const int32_t r0 = __ldg(a.dst_rows + p), r1 = p + 1 < p1 ? __ldg(a.dst_rows + p + 1) : 0;
+        const Row8 x = load_row(a.interm + (int64_t)r0 * kCols + lane8 * 8);
+        Row8 y = {{0, 0, 0, 0}};
+        if (p + 1 < p1) y = load_row(a.interm + (int64_t)r1 * kCols + lane8 * 8);
+        add_row(sum, x);
+        if (p + 1 < p1) add_row(sum, y);
+      }
       const int64_t v = v0 + j;
-      const float iv = __shfl_sync(omask, j < 8 ? inv_a : inv_b, j & 7, 8);
       float r[8];
+      unpack(sum, r);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) r[q] = a.d * acc[q];
+      for (int q = 0; q < 8; ++q) r[q] *= a.d;
       if ((sbits >> j) & 1u) {
 #pragma unroll
         for (int q = 0; q < 8; ++q)
@@ -293,105 +366,90 @@ ppr_merge_kernel(MergeArgs a) {
         float c[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) c[q] = r[q] * iv;
-        uint4 h, l;
-        split_row(c, &h, PLANES == 2 ? &l : nullptr);
-        __stcs(a.c_hi + v * 8 + lane8, h);
-        if (PLANES == 2) __stcs(a.c_lo + v * 8 + lane8, l);
+        store_contrib<PLANES>(a.contrib, v, lane8, c);
       } else {
 #pragma unroll
         for (int q = 0; q < 8; ++q) dpart[q] += r[q];
       }
-      if (a.r_out) {
+      if (a.r_out) {  // the caller's: 16-byte aligned
         float4* p = reinterpret_cast<float4*>(a.r_out + v * kCols + lane8 * 8);
         __stcs(p, make_float4(r[0], r[1], r[2], r[3]));
         __stcs(p + 1, make_float4(r[4], r[5], r[6], r[7]));
       }
       if (RESID) {
-        float o[8];
-        load_row(a.r_old + v * kCols + lane8 * 8, o);
+        const float4* p = reinterpret_cast<const float4*>(a.r_old + v * kCols + lane8 * 8);
+        const float4 x = __ldcs(p), y = __ldcs(p + 1);
+        const float o[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
 #pragma unroll
         for (int q = 0; q < 8; ++q) rpart[q] += fabsf(r[q] - o[q]);
       }
-    };
-    const int32_t o_lo = off_of(0);
-    int32_t iend = off_of(1);
-    constexpr int G = 2;  // intermBuf rows loaded together (4 blocks per SM fit)
-    for (int32_t p = o_lo; p < o_end; p += G) {
-      int32_t rr[G];
-      float4 x[G], y[G];
-#pragma unroll
-      for (int u = 0; u < G; ++u) rr[u] = p + u < o_end ? __ldg(a.dst_rows + p + u) : 0;
-#pragma unroll
-      for (int u = 0; u < G; ++u) {
-        if (p + u < o_end) {
-          x[u] = __ldcs(in4 + (int64_t)rr[u] * (kCols / 4) + lane8 * 2);
-          y[u] = __ldcs(in4 + (int64_t)rr[u] * (kCols / 4) + lane8 * 2 + 1);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < G; ++u) {
-        if (p + u < o_end) {
-          while (p + u >= iend) {  // rows of destination i are done
-            finish(i);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) acc[q] = 0.0f;
-            ++i;
-            iend = off_of(i + 1);
-          }
-          acc[0] += x[u].x; acc[1] += x[u].y; acc[2] += x[u].z; acc[3] += x[u].w;
-          acc[4] += y[u].x; acc[5] += y[u].y; acc[6] += y[u].z; acc[7] += y[u].w;
-        }
-      }
     }
-    for (; i < nv; ++i) {
-      finish(i);
+    // (FP64 adds run at 2 per cycle and SM: most tasks have no dangling mass)
+    bool any = false;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) acc[q] = 0.0f;
+    for (int q = 0; q < 8; ++q) any = any || dpart[q] != 0.0f;
+    if (any) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s_acc[w][0][q][lane] += (double)dpart[q];
     }
+    if (RESID) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      dsum[q] += (double)dpart[q];
-      if (RESID) rsum[q] += (double)rpart[q];
+      for (int q = 0; q < 8; ++q) s_acc[w][RESID][q][lane] += (double)rpart[q];
     }
   }
   // per-column partials: octets of a warp, then warps of the block
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    dsum[q] += __shfl_xor_sync(0xffffffffu, dsum[q], 8);
-    dsum[q] += __shfl_xor_sync(0xffffffffu, dsum[q], 16);
-    if (RESID) {
-      rsum[q] += __shfl_xor_sync(0xffffffffu, rsum[q], 8);
-      rsum[q] += __shfl_xor_sync(0xffffffffu, rsum[q], 16);
-    }
-  }
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane < 8) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      s_red[w][0][lane * 8 + q] = dsum[q];
-      s_red[w][1][lane * 8 + q] = rsum[q];
-    }
-  }
   __syncthreads();
   if (threadIdx.x < 2 * kCols) {
     const int which = threadIdx.x / kCols, j = threadIdx.x % kCols;
     double s = 0.0;
-    for (int q = 0; q < kThreads / 32; ++q) s += s_red[q][which][j];
+    if (which == 0 || RESID)
+      for (int q = 0; q < kThreads / 32; ++q)
+        for (int o = 0; o < 4; ++o) s += s_acc[q][RESID ? which : 0][j & 7][8 * o + (j >> 3)];
     a.partials[(int64_t)blockIdx.x * 2 * kCols + threadIdx.x] = s;
   }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (threadIdx.x < 2 * kCols) {
+  // the last block of 32 adds up their sums, the last of those the groups': a
+  // fixed order, 8 loads in flight per thread (one block adding up all 608
+  // one after the other took 40 us)
+  const int group = blockIdx.x / kMergeGroup, ngroups = (gridDim.x + kMergeGroup - 1) / kMergeGroup;
+  const int size = min(kMergeGroup, (int)gridDim.x - group * kMergeGroup);
+  double* gsum = a.partials + (int64_t)gridDim.x * 2 * kCols;
+  auto add_up = [&](const double* src, int n) -> double {  // valid in threads < 2 kCols
+    constexpr int U = 8;
+    const int j = threadIdx.x % (2 * kCols), half = threadIdx.x / (2 * kCols);
     double s = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b)
-      s += __ldcg(a.partials + (int64_t)b * 2 * kCols + threadIdx.x);
-    if (threadIdx.x < kCols) a.D[threadIdx.x] = s;
-    else if (RESID && a.resid) a.resid[threadIdx.x - kCols] = s;
-  }
+#pragma unroll 1
+    for (int b0 = 0; b0 < n; b0 += 2 * U) {
+      double x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int b = b0 + 2 * u + half;
+        x[u] = b < n ? __ldcg(src + (int64_t)b * 2 * kCols + j) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) s += x[u];
+    }
+    __syncthreads();
+    if (half == 1) s_half[j] = s;
+    __syncthreads();
+    return half == 0 ? s + s_half[j] : 0.0;
+  };
+  auto last_of = [&](unsigned* count, int n) -> bool {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(count, 1u) == (unsigned)n - 1;
+    __syncthreads();
+    const bool last = s_last;
+    if (last) __threadfence();
+    return last;
+  };
+  if (!last_of(a.counter + 1 + group, size)) return;
+  double s = add_up(a.partials + (int64_t)group * kMergeGroup * 2 * kCols, size);
+  if (threadIdx.x < 2 * kCols) gsum[(int64_t)group * 2 * kCols + threadIdx.x] = s;
+  if (threadIdx.x == 0) a.counter[1 + group] = 0u;
+  if (!last_of(a.counter, ngroups)) return;
+  s = add_up(gsum, ngroups);
+  if (threadIdx.x < kCols) a.D[threadIdx.x] = s;
+  else if (RESID && a.resid && threadIdx.x < 2 * kCols) a.resid[threadIdx.x - kCols] = s;
   if (threadIdx.x == 0) *a.counter = 0u;
 }
 
@@ -473,15 +531,16 @@ __global__ void fill_dst_kernel(const int32_t* __restrict__ idx_map, int64_t r0,
 }
 
 __global__ void ppr_seed_kernel(const float* __restrict__ inv, const int32_t* __restrict__ seeds,
-                                __nv_bfloat16* __restrict__ c_hi, __nv_bfloat16* __restrict__ c_lo,
+                                void* __restrict__ contrib, int planes,
                                 uint32_t* __restrict__ seed_bits, double* __restrict__ D) {
   const int j = threadIdx.x;
   if (j >= kCols) return;
   const int32_t s = seeds[j];
   const float c = inv[s];  // R_0 = one-hot at the seed: C = 1 / outdeg
-  const __nv_bfloat16 h = __float2bfloat16_rn(c);
-  c_hi[(int64_t)s * kCols + j] = h;
-  if (c_lo) c_lo[(int64_t)s * kCols + j] = __float2bfloat16_rn(c - __bfloat162float(h));
+  if (planes == 2)
+    static_cast<float*>(contrib)[(int64_t)s * kCols + j] = c;
+  else
+    static_cast<__nv_bfloat16*>(contrib)[(int64_t)s * kCols + j] = __float2bfloat16_rn(c);
   atomicOr(seed_bits + (s >> 5), 1u << (s & 31));
   D[j] = c == 0.0f ? 1.0 : 0.0;
 }
@@ -495,8 +554,7 @@ int merge_launch(cg_ppr* p, const float* inv, double damping, float* r_out, cons
   a.inv = inv;
   a.seeds = p->seeds;
   a.seed_bits = p->seed_bits;
-  a.c_hi = p->c_hi;
-  a.c_lo = p->c_lo;
+  a.contrib = p->contrib;
   a.r_out = r_out;
   a.r_old = r_old;
   a.D = p->D;
@@ -506,36 +564,24 @@ int merge_launch(cg_ppr* p, const float* inv, double damping, float* r_out, cons
   a.d = (float)damping;
   a.V = p->V;
   const bool res = r_old != nullptr;
-  if (p->planes == 2) {
-    if (res) ppr_merge_kernel<2, true><<<p->merge_grid, kThreads, 0, s>>>(a);
-    else ppr_merge_kernel<2, false><<<p->merge_grid, kThreads, 0, s>>>(a);
-  } else {
-    if (res) ppr_merge_kernel<1, true><<<p->merge_grid, kThreads, 0, s>>>(a);
-    else ppr_merge_kernel<1, false><<<p->merge_grid, kThreads, 0, s>>>(a);
-  }
-  CG_LAUNCH_CHECK();
-  return CG_OK;
+  auto fn = p->planes == 2 ? (res ? ppr_merge_kernel<2, true> : ppr_merge_kernel<2, false>)
+                           : (res ? ppr_merge_kernel<1, true> : ppr_merge_kernel<1, false>);
+  return launch_chained(fn, p->merge_grid, kThreads, 0, s, a);
 }
 
 int gather_launch(cg_ppr* p, cudaStream_t s) {
   if (p->nchunks == 0) return CG_OK;
   const SegPlan& sp = p->seg->plan;
-  if (p->planes == 2)
-    ppr_gather_kernel<2><<<p->gather_grid, kThreads, 0, s>>>(
-        sp.colf, p->segs, p->chunks, p->nchunks, p->c_hi, p->c_lo, p->interm, p->carry);
-  else
-    ppr_gather_kernel<1><<<p->gather_grid, kThreads, 0, s>>>(
-        sp.colf, p->segs, p->chunks, p->nchunks, p->c_hi, p->c_hi, p->interm, p->carry);
-  CG_LAUNCH_CHECK();
-  return CG_OK;
+  return launch_chained(p->planes == 2 ? ppr_gather_kernel<2> : ppr_gather_kernel<1>,
+                        p->gather_grid, kThreads, 0, s, sp.colf, p->segs, p->chunks, p->nchunks,
+                        p->contrib, p->interm, p->carry);
 }
 
 int fixup_launch(cg_ppr* p, cudaStream_t s) {
   if (p->npieces == 0) return CG_OK;
-  ppr_fixup_kernel<<<grid_for(p->npieces * 8, kThreads, 8), kThreads, 0, s>>>(
-      p->pieces, p->npieces, p->runs, p->carry, p->piece_sum, p->run_done, p->interm);
-  CG_LAUNCH_CHECK();
-  return CG_OK;
+  return launch_chained(ppr_fixup_kernel, grid_for(p->npieces * 8, kThreads, 8), kThreads, 0, s,
+                        p->pieces, p->npieces, p->runs, p->carry, p->piece_sum, p->run_done,
+                        p->interm);
 }
 
 void ppr_free(cg_ppr* p) {
@@ -550,8 +596,7 @@ void ppr_free(cg_ppr* p) {
   cudaFree(p->dst_off);
   cudaFree(p->dst_rows);
   cudaFree(p->interm);
-  cudaFree(p->c_hi);
-  cudaFree(p->c_lo);
+  cudaFree(p->contrib);
   cudaFree(p->r_prev);
   cudaFree(p->seeds);
   cudaFree(p->seed_bits);
@@ -592,7 +637,7 @@ int ppr_build(cg_ppr* p, cudaStream_t s) {
     ppr_chunks_kernel<<<grid_for(nch, 256), 256, 0, s>>>(sp.rp32, sp.meta, p->segs, k, nch,
                                                           p->chunks);
     CG_LAUNCH_CHECK();
-    // runs of carries (static) cut into pieces of <= 32 chunks
+    // runs of carries (static) cut into pieces
     int32_t* crow = nullptr;
     CG_CUDA(cudaMallocAsync((void**)&crow, sizeof(int32_t) * (size_t)nch, s));
     carry_rows_kernel<<<grid_for(nch, 256), 256, 0, s>>>(sp.rp32, sp.meta, p->segs, p->chunks,
@@ -611,8 +656,8 @@ int ppr_build(cg_ppr* p, cudaStream_t s) {
       int64_t e = c + 1;
       while (e < nch && hc[e] == hc[c]) ++e;
       const int32_t run = (int32_t)hr.size(), p0 = (int32_t)hp.size();
-      for (int64_t x = c; x < e; x += 32)
-        hp.push_back(make_int4((int32_t)x, (int32_t)std::min<int64_t>(32, e - x), run, 0));
+      for (int64_t x = c; x < e; x += kPprPiece)
+        hp.push_back(make_int4((int32_t)x, (int32_t)std::min<int64_t>(kPprPiece, e - x), run, 0));
       hr.push_back(make_int4(hc[c], p0, (int32_t)hp.size() - p0, 0));
       c = e;
     }
@@ -665,8 +710,7 @@ int ppr_build(cg_ppr* p, cudaStream_t s) {
   if (e != cudaSuccess) return cuda_fail(e, "ppr_batched_create", __FILE__, __LINE__);
   // iteration state
   CG_CUDA(alloc(&p->interm, p->rows * kCols, &B));
-  CG_CUDA(alloc(&p->c_hi, (int64_t)V * 8, &B));
-  if (p->planes == 2) CG_CUDA(alloc(&p->c_lo, (int64_t)V * 8, &B));
+  CG_CUDA(alloc(&p->contrib, (int64_t)V * 8 * p->planes, &B));
   CG_CUDA(alloc(&p->r_prev, (int64_t)V * kCols, &B));
   CG_CUDA(alloc(&p->seeds, kCols, &B));
   CG_CUDA(alloc(&p->seed_bits, ceil_div(V, 32), &B));
@@ -682,9 +726,10 @@ int ppr_build(cg_ppr* p, cudaStream_t s) {
   CG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
       &per_sm, p->planes == 2 ? ppr_gather_kernel<2> : ppr_gather_kernel<1>, kThreads, 0));
   p->gather_grid = di.sm_count * (per_sm > 0 ? per_sm : 1);
-  CG_CUDA(alloc(&p->partials, (int64_t)p->merge_grid * 2 * kCols, &B));
-  CG_CUDA(alloc(&p->counter, 1, &B));
-  CG_CUDA(cudaMemsetAsync(p->counter, 0, sizeof(unsigned), s));
+  const int64_t groups = ceil_div(p->merge_grid, kMergeGroup);
+  CG_CUDA(alloc(&p->partials, (p->merge_grid + groups) * 2 * kCols, &B));
+  CG_CUDA(alloc(&p->counter, 1 + groups, &B));
+  CG_CUDA(cudaMemsetAsync(p->counter, 0, sizeof(unsigned) * (size_t)(1 + groups), s));
   CG_CUDA(cudaStreamSynchronize(s));
   return CG_OK;
 }
@@ -744,16 +789,13 @@ int ppr_batched_init(cg_ppr* p, const float* inv, const int32_t* host_seeds,
   for (int j = 0; j < kCols; ++j)
     CG_ARG(host_seeds[j] >= 0 && host_seeds[j] < p->V,
            "ppr_batched_init: seed %d of column %d outside [0, %d)", host_seeds[j], j, p->V);
-  const size_t plane = sizeof(uint4) * 8 * (size_t)p->V;
   CG_CUDA(cudaMemcpyAsync(p->seeds, host_seeds, sizeof(int32_t) * kCols, cudaMemcpyHostToDevice,
                           stream));
-  CG_CUDA(cudaMemsetAsync(p->c_hi, 0, plane, stream));
-  if (p->c_lo) CG_CUDA(cudaMemsetAsync(p->c_lo, 0, plane, stream));
+  CG_CUDA(cudaMemsetAsync(p->contrib, 0, sizeof(uint4) * 8 * p->planes * (size_t)p->V, stream));
   CG_CUDA(cudaMemsetAsync(p->seed_bits, 0, sizeof(uint32_t) * (size_t)ceil_div(p->V, 32),
                           stream));
-  ppr_seed_kernel<<<1, kCols, 0, stream>>>(inv, p->seeds, reinterpret_cast<__nv_bfloat16*>(p->c_hi),
-                                           reinterpret_cast<__nv_bfloat16*>(p->c_lo),
-                                           p->seed_bits, p->D);
+  ppr_seed_kernel<<<1, kCols, 0, stream>>>(inv, p->seeds, p->contrib, p->planes, p->seed_bits,
+                                           p->D);
   CG_LAUNCH_CHECK();
   CG_TRY(ppr_dense_pack(p, stream));
   // host_seeds may go out of scope on return

@@ -15,6 +15,9 @@ constexpr int kCols = 64;         // columns (rank vectors) per batch
 constexpr int kChunk = 128;       // edges per octet chunk in the gather
 constexpr int kTask = 16;         // destinations per octet task in the merge
 constexpr int kThreads = 256;     // threads per block of every kernel here
+constexpr int kPprPiece = 16;     // chunks per piece of a run of carries
+constexpr int kMergeGroup = 32;   // merge blocks whose sums one block adds up
+constexpr int kGatherBlocks = 6;  // gather blocks per SM
 constexpr uint32_t kRowEnd = 0x80000000u;
 
 struct PprSeg {
@@ -44,13 +47,12 @@ struct cg_ppr {
   int32_t* dst_off = nullptr;    // [V+1] destination-major row lists
   int32_t* dst_rows = nullptr;   // [rows]
   float* interm = nullptr;       // [rows][64] intermBuf
-  uint4* c_hi = nullptr;         // [V][64] bf16
-  uint4* c_lo = nullptr;         // [V][64] bf16 (two planes only)
+  uint4* contrib = nullptr;      // [V][64] FP32 (two planes) or BF16 (one)
   float* r_prev = nullptr;       // [V][64] R of the second-to-last iteration
   int32_t* seeds = nullptr;      // [64]
   uint32_t* seed_bits = nullptr; // [ceil(V/32)] vertices that are some column's seed
   double* D = nullptr;           // [64] dangling mass per column
-  double* partials = nullptr;    // [merge_grid][128]
+  double* partials = nullptr;    // [merge_grid + groups][128]
   unsigned* counter = nullptr;
   int merge_grid = 0, gather_grid = 0;
   bool seeded = false;

@@ -400,9 +400,10 @@ __global__ void dense_tile_bits_kernel(const uint32_t* __restrict__ bits, int32_
 
 // The hubs' contributions in the B operand layout: chunk c = u / 64 holds
 // 64 columns x 64 sources; column n of source u at tile_off(n, u % 64).
-__global__ void dense_pack_kernel(const uint4* __restrict__ c_hi, const uint4* __restrict__ c_lo,
-                                  int32_t h, uint8_t* __restrict__ ct_hi,
-                                  uint8_t* __restrict__ ct_lo) {
+// FP32 contributions are split: hi = bf16(c), lo = bf16(c - hi).
+template <int PLANES>
+__global__ void dense_pack_kernel(const uint4* __restrict__ contrib, int32_t h,
+                                  uint8_t* __restrict__ ct_hi, uint8_t* __restrict__ ct_lo) {
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < (int64_t)h * 8;
        x += (int64_t)gridDim.x * blockDim.x) {
     const int64_t u = x >> 3;
@@ -410,14 +411,26 @@ __global__ void dense_pack_kernel(const uint4* __restrict__ c_hi, const uint4* _
     const int k = (int)(u & (kDK - 1));
     uint8_t* dh = ct_hi + (u / kDK) * kTileB;
     uint8_t* dl = ct_lo + (u / kDK) * kTileB;
-    const uint4 a = c_hi[u * 8 + g];
-    const uint4 b = c_lo ? c_lo[u * 8 + g] : make_uint4(0u, 0u, 0u, 0u);
-    const uint32_t wa[4] = {a.x, a.y, a.z, a.w}, wb[4] = {b.x, b.y, b.z, b.w};
+    uint32_t w[4 * PLANES];
+#pragma unroll
+    for (int q = 0; q < PLANES; ++q) {
+      const uint4 a = contrib[(u * 8 + g) * PLANES + q];
+      w[4 * q] = a.x; w[4 * q + 1] = a.y; w[4 * q + 2] = a.z; w[4 * q + 3] = a.w;
+    }
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const uint32_t o = tile_off(8 * g + q, k);
-      *reinterpret_cast<uint16_t*>(dh + o) = (uint16_t)(wa[q >> 1] >> (16 * (q & 1)));
-      *reinterpret_cast<uint16_t*>(dl + o) = (uint16_t)(wb[q >> 1] >> (16 * (q & 1)));
+      uint16_t hi, lo = 0;
+      if (PLANES == 2) {
+        const float c = __uint_as_float(w[q]);
+        const __nv_bfloat16 b = __float2bfloat16_rn(c);
+        hi = __bfloat16_as_ushort(b);
+        lo = __bfloat16_as_ushort(__float2bfloat16_rn(c - __bfloat162float(b)));
+      } else {
+        hi = (uint16_t)(w[q >> 1] >> (16 * (q & 1)));
+      }
+      *reinterpret_cast<uint16_t*>(dh + o) = hi;
+      *reinterpret_cast<uint16_t*>(dl + o) = lo;
     }
   }
 }
@@ -525,8 +538,9 @@ int ppr_dense_launch(cg_ppr* p, cudaStream_t s) {
 
 int ppr_dense_pack(cg_ppr* p, cudaStream_t s) {
   if (p->dense_h == 0) return CG_OK;
-  dense_pack_kernel<<<grid_for((int64_t)p->dense_h * 8, 256), 256, 0, s>>>(
-      p->c_hi, p->c_lo, p->dense_h, p->ct_hi, p->ct_lo);
+  auto fn = p->planes == 2 ? dense_pack_kernel<2> : dense_pack_kernel<1>;
+  fn<<<grid_for((int64_t)p->dense_h * 8, 256), 256, 0, s>>>(p->contrib, p->dense_h, p->ct_hi,
+                                                            p->ct_lo);
   CG_LAUNCH_CHECK();
   return CG_OK;
 }
