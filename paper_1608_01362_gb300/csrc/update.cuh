@@ -18,18 +18,39 @@ constexpr int kMergeWarps = 8;  // warps per merge / update block
 // destination receives its partial sums in segment order (deterministic).
 //
 // The rows of up to 32 segments are handled as one flattened sequence
-// (segment-major, so flattened order is segment order): lane l holds the
-// inclusive prefix of the row counts of segment s0+l, and a flattened
-// position f belongs to the segment whose prefix first exceeds f (a binary
-// search over the lanes).  A warp loads 32*U consecutive flattened rows at
-// once, then applies them 32 at a time; inside one group of 32 lanes the rows
-// of one segment have distinct destinations, and different segments are
-// applied one after the other in ascending order.  An operator that is exact
-// in any order (min) applies a whole group at once with shared-memory
-// atomics instead.  A block whose segments hold a few rows each then costs
-// one memory round trip instead of one per segment, and a hub block's
-// segments with hundreds of rows keep 32*U loads in flight instead of 32.
+// (segment-major, so flattened order is segment order): lane l holds where the
+// rows of the l-th segment that has any begin in it.  A warp loads 32*U
+// consecutive flattened rows at once: the segments that begin among 32 of them
+// are one OR over the lanes, a row's segment the number of set bits up to it.
+// It then applies them 32 at a time; inside one group of 32 lanes the rows of
+// one segment have distinct destinations, and different segments are applied
+// one after the other in ascending order.  An operator that is exact in any
+// order (min) applies a whole group at once with shared-memory atomics instead.
+// A block whose segments hold a few rows each then costs one memory round trip
+// instead of one per segment, and a hub block's segments with hundreds of rows
+// keep 32*U loads in flight instead of 32.
+//
+// What bounds it is instructions (issue slots 68% taken), then memory: of 223
+// us at 32 M vertices and 33 segments, 133 are its bytes.  Finding a row's
+// segment by a binary search over the lanes and its turn by ballots, 85
+// instructions per 32 rows, took 279 us; groups of one segment, the most
+// common, apply without the loop (225 with it, 215 so).
 // ---------------------------------------------------------------------------
+
+// The place of the (n+1)-th set bit of m (31 if there are fewer).
+__device__ __forceinline__ int nth_bit(unsigned m, int n) {
+  int at = 0;
+#pragma unroll
+  for (int step = 16; step; step >>= 1) {
+    const int below = __popc(m & ((1u << step) - 1u));
+    if (n >= below) {
+      n -= below;
+      m >>= step;
+      at += step;
+    }
+  }
+  return at;
+}
 
 template <class Op>
 __device__ __forceinline__ void warp_merge(const int32_t* __restrict__ blk,
@@ -41,6 +62,7 @@ __device__ __forceinline__ void warp_merge(const int32_t* __restrict__ blk,
   constexpr int U = 4;  // groups of 32 flattened rows loaded together
   constexpr unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x & 31;
+  const unsigned upto = 0xffffffffu >> (31 - lane);  // this lane's bit and those below
   for (int i = lane; i < n; i += 32) acc[i] = Op::identity();
   __syncwarp();
   for (int s0 = 0; s0 < k; s0 += 32) {
@@ -50,27 +72,35 @@ __device__ __forceinline__ void warp_merge(const int32_t* __restrict__ blk,
       lo = __ldg(blk + mb * k + ls);
       hi = __ldg(blk + (mb + 1) * k + ls);
     }
-    // inclusive prefix of the row counts over the lanes' segments
-    int32_t pre = hi - lo;
+    // the segments that have rows, in order, one per lane: where their rows
+    // begin in the flattened sequence, and the row there
+    const unsigned some = __ballot_sync(kFull, hi > lo);
+    const int m = __popc(some), from = nth_bit(some, lane);
+    const int32_t first = __shfl_sync(kFull, lo, from);
+    const int32_t last = __shfl_sync(kFull, hi, from);
+    const int32_t cnt = lane < m ? last - first : 0;
+    int32_t pre = cnt;  // inclusive prefix
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int32_t t = __shfl_up_sync(kFull, pre, o);
       if (lane >= o) pre += t;
     }
-    const int32_t off = lo - (pre - (hi - lo));  // row index = flattened position + off
+    const int32_t start = lane < m ? pre - cnt : 0x7fffffff;
+    const int32_t off = first - (pre - cnt);  // row index = flattened position + off
     const int32_t total = __shfl_sync(kFull, pre, 31);
+    int before = -1;  // segment of the row before the group's
     for (int32_t base = 0; base < total; base += 32 * U) {
-      int32_t seg[U], dd[U];
+      unsigned begin[U];  // positions of the group where a segment begins
+      int32_t dd[U];
       T xx[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int32_t f = base + u * 32 + lane;
-        int j = 0;  // number of segments whose rows all precede f
-#pragma unroll
-        for (int step = 16; step; step >>= 1)
-          if (__shfl_sync(kFull, pre, j + step - 1) <= f) j += step;
+        const int32_t f0 = base + u * 32, f = f0 + lane;
+        const unsigned rel = (unsigned)(start - f0);
+        begin[u] = __reduce_or_sync(kFull, rel < 32u ? 1u << rel : 0u);
+        const int j = before + __popc(begin[u] & upto);
+        before += __popc(begin[u]);
         const int32_t row = f + __shfl_sync(kFull, off, j);
-        seg[u] = f < total ? j : 32;
         dd[u] = 0;
         xx[u] = Op::identity();
         if (f < total) {
@@ -78,26 +108,24 @@ __device__ __forceinline__ void warp_merge(const int32_t* __restrict__ blk,
           xx[u] = __ldcs(interm + row);
         }
       }
-      if constexpr (Op::kExactAnyOrder) {  // e.g. min: every row at once
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int64_t lv = (int64_t)dd[u] - v0;
-          if (seg[u] < 32 && (uint64_t)lv < (uint64_t)n) Op::atomic_op(acc + lv, xx[u]);
-        }
-        continue;
-      }
 #pragma unroll
       for (int u = 0; u < U; ++u) {  // apply in flattened (= segment) order
-        unsigned pend = __ballot_sync(kFull, seg[u] < 32);
-        while (pend) {
-          const int sj = __shfl_sync(kFull, seg[u], __ffs(pend) - 1);
-          const bool mine = seg[u] == sj;
-          if (mine) {
-            const int64_t lv = (int64_t)dd[u] - v0;
-            if ((uint64_t)lv < (uint64_t)n) acc[lv] = Op::op(acc[lv], xx[u]);
+        T* at = acc + (dd[u] - (int32_t)v0);
+        const bool ok = base + u * 32 + lane < total;
+        if constexpr (Op::kExactAnyOrder) {  // e.g. min: every row at once
+          if (ok) Op::atomic_op(at, xx[u]);
+        } else {
+          const unsigned inner = begin[u] & ~1u;
+          if (!inner) {  // one segment
+            if (ok) *at = Op::op(*at, xx[u]);
+            __syncwarp();
+          } else {
+            const int mine = __popc(inner & upto), n = __popc(inner);
+            for (int t = 0; t <= n; ++t) {
+              if (ok && mine == t) *at = Op::op(*at, xx[u]);
+              __syncwarp();
+            }
           }
-          __syncwarp();
-          pend &= ~__ballot_sync(kFull, mine);
         }
       }
     }
