@@ -74,7 +74,8 @@ struct cg_bc {
                                         // frontier (three levels in turn), vertices reached
   void* sort = nullptr;        // scratch of the scans and the sort
   size_t sort_bytes = 0;
-  unsigned long long* h_pin = nullptr;  // pinned host copy of count
+  unsigned long long* h_pin = nullptr;  // pinned host copy of count, and its ticket
+  unsigned long long ticket = 0;
   double alpha = 16.0;
   int32_t depth = 0;           // levels of the last source
   int32_t last_source = -1;
@@ -92,6 +93,7 @@ typedef unsigned long long u64;
 __global__ void bc_reset_kernel(int32_t V, int32_t* __restrict__ level,
                                 double* __restrict__ sigma, double* __restrict__ delta,
                                 uint32_t* __restrict__ xbits) {
+  if (!chain_begin()) return;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V;
        v += (int64_t)gridDim.x * blockDim.x) {
     level[v] = -1;
@@ -112,6 +114,7 @@ __global__ void bc_seed_kernel(int32_t s, const int64_t* __restrict__ out_off,
                                int32_t* __restrict__ level, double* __restrict__ sigma,
                                int32_t* __restrict__ list, int32_t* __restrict__ fpos,
                                int32_t* __restrict__ fgap, u64* __restrict__ count) {
+  if (!chain_begin()) return;
   level[s] = 0;
   sigma[s] = 1.0;
   const u64 deg = (u64)(out_off[s + 1] - out_off[s]);
@@ -219,6 +222,7 @@ __global__ void __launch_bounds__(kThreads)
 push_kernel(Frontier cur, int32_t n, int32_t m, const int64_t* __restrict__ out_off,
             const int32_t* __restrict__ out_dst, int32_t L, int32_t* __restrict__ level,
             double* __restrict__ sigma, Frontier nxt, u64* __restrict__ count) {
+  if (!chain_begin()) return;
   u64* next = count + (L + 1) % 3;
   if (blockIdx.x == 0 && threadIdx.x == 0) count[(L + 2) % 3] = 0ull;
   const int lane = threadIdx.x & 31;
@@ -308,6 +312,7 @@ struct ListRows {
 template <class F, bool WRITE>
 __global__ void __launch_bounds__(kThreads)
 compact_kernel(F f, int64_t n, int64_t* __restrict__ tsum) {
+  if (!chain_begin()) return;
   __shared__ u64 s_w[kThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t base = (int64_t)blockIdx.x * kCTile + (int64_t)w * (kItems * 32);
@@ -350,12 +355,10 @@ template <class F>
 int compact(cg_bc* h, const F& f, int64_t n, const int64_t** total, cudaStream_t s) {
   const int64_t tiles = ceil_div(n, kCTile);
   int64_t* scan = h->tsum + tiles;
-  compact_kernel<F, false><<<(unsigned)tiles, kThreads, 0, s>>>(f, n, h->tsum);
-  CG_LAUNCH_CHECK();
+  CG_TRY(launch_chained(compact_kernel<F, false>, (unsigned)tiles, kThreads, 0, s, f, n, h->tsum));
   Scratch ws(s, h->sort, h->sort_bytes);
   CG_TRY(exclusive_scan_i64(h->tsum, scan, tiles, s, &ws));
-  compact_kernel<F, true><<<(unsigned)tiles, kThreads, 0, s>>>(f, n, scan);
-  CG_LAUNCH_CHECK();
+  CG_TRY(launch_chained(compact_kernel<F, true>, (unsigned)tiles, kThreads, 0, s, f, n, scan));
   if (total) *total = scan + tiles;
   return CG_OK;
 }
@@ -398,6 +401,7 @@ __device__ __forceinline__ int pad8(int j) { return j + (j >> 3); }
 
 __global__ void __launch_bounds__(kThreads, 4)
 row_sum_kernel(RowSums a) {
+  if (!chain_begin()) return;
   __shared__ double s_all[kThreads / 32][kSub + kSub / 8];
   constexpr unsigned kFull = 0xffffffffu;
   constexpr int U = 4;  // batches of 32 edges whose reads are in flight together
@@ -492,6 +496,7 @@ row_sum_kernel(RowSums a) {
 }
 
 __global__ void __launch_bounds__(256) row_fix_kernel(RowSums a) {
+  if (!chain_begin()) return;
   const int64_t m = a.edges();
   const int64_t tile = (int64_t)tile_steps(m) * kSub;
   fix_runs<SumF64>(a.carry_row, a.carry, (m + tile - 1) / tile, a.out);
@@ -499,10 +504,8 @@ __global__ void __launch_bounds__(256) row_fix_kernel(RowSums a) {
 
 int row_sums(const RowSums& a, int64_t most_edges, cudaStream_t s) {
   const int64_t tiles = ceil_div(most_edges, kSub);
-  row_sum_kernel<<<grid_for(tiles * 32, kThreads, 4), kThreads, 0, s>>>(a);
-  CG_LAUNCH_CHECK();
-  row_fix_kernel<<<grid_for(tiles, 256, 4), 256, 0, s>>>(a);
-  CG_LAUNCH_CHECK();
+  CG_TRY(launch_chained(row_sum_kernel, grid_for(tiles * 32, kThreads, 4), kThreads, 0, s, a));
+  CG_TRY(launch_chained(row_fix_kernel, grid_for(tiles, 256, 4), 256, 0, s, a));
   return CG_OK;
 }
 
@@ -513,6 +516,7 @@ pull_update_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ 
                    const double* __restrict__ acc, const int64_t* __restrict__ out_off, int32_t L,
                    int32_t* __restrict__ level, double* __restrict__ sigma, Frontier nxt,
                    u64* __restrict__ count) {
+  if (!chain_begin()) return;
   u64* next = count + (L + 1) % 3;
   if (blockIdx.x == 0 && threadIdx.x == 0) count[(L + 2) % 3] = 0ull;
   const int64_t n = *packed >> 32;
@@ -536,6 +540,7 @@ pull_update_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ 
 
 __global__ void set_bits_kernel(const int32_t* __restrict__ list, int64_t n,
                                 uint32_t* __restrict__ bits, bool on) {
+  if (!chain_begin()) return;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     set_bit(bits, list[i], on);
@@ -549,6 +554,7 @@ __global__ void dependency_kernel(const int32_t* __restrict__ list, int64_t n, i
                                   double* __restrict__ delta, double* __restrict__ xval,
                                   uint32_t* __restrict__ xbits, double* __restrict__ bc,
                                   int32_t source) {
+  if (!chain_begin()) return;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t u = list[i];
@@ -582,10 +588,40 @@ __global__ void row_of_edge_kernel(const int64_t* __restrict__ off, int32_t V, i
   }
 }
 
-int read_counts(cg_bc* h, cudaStream_t s) {
-  CG_CUDA(cudaMemcpyAsync(h->h_pin, h->count, 4 * sizeof(u64), cudaMemcpyDeviceToHost, s));
-  CG_CUDA(cudaStreamSynchronize(s));
+// Writes the counts and, behind them, the ticket to the host's pinned copy.
+__device__ __forceinline__ void publish(const u64* count, volatile u64* pin, u64 ticket) {
+  for (int q = 0; q < 4; ++q) pin[q] = __ldcg(count + q);
+  __threadfence_system();
+  pin[4] = ticket;
+}
+
+__global__ void publish_kernel(const u64* count, u64* pin, u64 ticket) {
+  if (!chain_begin()) return;
+  publish(count, pin, ticket);
+}
+
+// Waits for the counts of the ticket: the host watches the pinned word that a
+// kernel writes (a copy and a synchronisation took 17 us of every level, this 8),
+// and asks the stream now and then whether it has failed.
+int wait_counts(cg_bc* h, cudaStream_t s) {
+  for (int spins = 1; __atomic_load_n(h->h_pin + 4, __ATOMIC_ACQUIRE) != h->ticket; ++spins) {
+    if (spins % 4096) continue;
+    const cudaError_t e = cudaStreamQuery(s);
+    if (e != cudaErrorNotReady && e != cudaSuccess)
+      return cuda_fail(e, "bc_run", __FILE__, __LINE__);
+    if (e == cudaSuccess) {  // all done: the word is there, or will never be
+      CG_CUDA(cudaStreamSynchronize(s));
+      if (__atomic_load_n(h->h_pin + 4, __ATOMIC_ACQUIRE) == h->ticket) break;
+      set_error("bc_run: the level's counts did not arrive");
+      return CG_ERR_CUDA;
+    }
+  }
   return CG_OK;
+}
+
+int read_counts(cg_bc* h, cudaStream_t s) {
+  CG_TRY(launch_chained(publish_kernel, 1, 1, 0, s, h->count, h->h_pin, ++h->ticket));
+  return wait_counts(h, s);
 }
 
 Frontier frontier(const cg_bc* h, int q) { return Frontier{h->flist[q], h->fpos[q], h->fgap[q]}; }
@@ -596,29 +632,27 @@ Frontier frontier(const cg_bc* h, int q) { return Frontier{h->flist[q], h->fpos[
 int pull_level(cg_bc* h, int32_t L, int32_t n, cudaStream_t s) {
   const int32_t V = h->V;
   const int cur = L & 1;
-  set_bits_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(h->flist[cur], n, h->xbits, true);
-  CG_LAUNCH_CHECK();
+  CG_TRY(launch_chained(set_bits_kernel, grid_for(n, kThreads), kThreads, 0, s, h->flist[cur], n,
+                        h->xbits, true));
   const int64_t* packed = nullptr;
   CG_TRY(compact(h, Unvisited{h->level, h->in_off, h->ids, h->pos, h->gap}, V, &packed, s));
   const RowSums a{h->pos, h->gap, 0, 0, 0, packed, h->in_src, h->xbits, h->sigma, h->acc,
                   h->carry, h->carry_row};
   CG_TRY(row_sums(a, h->E, s));
-  pull_update_kernel<<<grid_for(V, kThreads), kThreads, 0, s>>>(
-      h->ids, packed, h->acc, h->out_off, L, h->level, h->sigma, frontier(h, 1 - cur), h->count);
-  CG_LAUNCH_CHECK();
-  set_bits_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(h->flist[cur], n, h->xbits, false);
-  CG_LAUNCH_CHECK();
+  CG_TRY(launch_chained(pull_update_kernel, grid_for(V, kThreads), kThreads, 0, s, h->ids, packed,
+                        h->acc, h->out_off, L, h->level, h->sigma, frontier(h, 1 - cur),
+                        h->count));
+  CG_TRY(launch_chained(set_bits_kernel, grid_for(n, kThreads), kThreads, 0, s, h->flist[cur], n,
+                        h->xbits, false));
   return CG_OK;
 }
 
 int run_source(cg_bc* h, int32_t src, double* bc, cudaStream_t s) {
   const int32_t V = h->V;
-  bc_reset_kernel<<<grid_for(V, kThreads), kThreads, 0, s>>>(V, h->level, h->sigma, h->delta,
-                                                               h->xbits);
-  CG_LAUNCH_CHECK();
-  bc_seed_kernel<<<1, 1, 0, s>>>(src, h->out_off, h->level, h->sigma, h->flist[0], h->fpos[0],
-                                 h->fgap[0], h->count);
-  CG_LAUNCH_CHECK();
+  CG_TRY(launch_chained(bc_reset_kernel, grid_for(V, kThreads), kThreads, 0, s, V, h->level,
+                        h->sigma, h->delta, h->xbits));
+  CG_TRY(launch_chained(bc_seed_kernel, 1, 1, 0, s, src, h->out_off, h->level, h->sigma,
+                        h->flist[0], h->fpos[0], h->fgap[0], h->count));
   CG_TRY(read_counts(h, s));
   // per level: vertices, of them with out-edges, and these edges
   std::vector<int64_t> size(1, 1), rows, edges;
@@ -635,10 +669,9 @@ int run_source(cg_bc* h, int32_t src, double* bc, cudaStream_t s) {
       ++h->pull_levels;
     } else {  // push from the frontier's out-edges
       const int cur = L & 1;
-      push_kernel<<<grid_for(ceil_div(m, kPushTile) * 32, kThreads), kThreads, 0, s>>>(
-          frontier(h, cur), n, m, h->out_off, h->out_dst, L, h->level, h->sigma,
-          frontier(h, 1 - cur), h->count);
-      CG_LAUNCH_CHECK();
+      CG_TRY(launch_chained(push_kernel, grid_for(ceil_div(m, kPushTile) * 32, kThreads), kThreads,
+                            0, s, frontier(h, cur), n, m, h->out_off, h->out_dst, L, h->level,
+                            h->sigma, frontier(h, 1 - cur), h->count));
       ++h->push_levels;
     }
     CG_TRY(read_counts(h, s));
@@ -673,9 +706,8 @@ int run_source(cg_bc* h, int32_t src, double* bc, cudaStream_t s) {
                       h->out_dst, h->xbits, h->xval, h->acc, h->carry, h->carry_row};
       CG_TRY(row_sums(a, edges[L], s));
     }
-    dependency_kernel<<<grid_for(n, kThreads), kThreads, 0, s>>>(
-        list, n, summed, h->acc, h->sigma, h->delta, h->xval, h->xbits, bc, src);
-    CG_LAUNCH_CHECK();
+    CG_TRY(launch_chained(dependency_kernel, grid_for(n, kThreads), kThreads, 0, s, list, n,
+                          summed, h->acc, h->sigma, h->delta, h->xval, h->xbits, bc, src));
   }
   h->last_source = src;
   return CG_OK;
@@ -779,7 +811,8 @@ int bc_create(const int64_t* in_offsets, const int32_t* in_src, const int64_t* o
     h->carry_row = reinterpret_cast<int32_t*>(take(c4));
     h->count = reinterpret_cast<unsigned long long*>(take(256));
     h->sort = take(h->sort_bytes);
-    e = cudaHostAlloc((void**)&h->h_pin, 4 * sizeof(unsigned long long), 0);
+    e = cudaHostAlloc((void**)&h->h_pin, 5 * sizeof(unsigned long long), 0);
+    if (e == cudaSuccess) std::fill(h->h_pin, h->h_pin + 5, 0ull);
   }
   int st = e == cudaSuccess ? CG_OK : cuda_fail(e, "bc_create", __FILE__, __LINE__);
   if (st == CG_OK) {

@@ -150,8 +150,13 @@ int launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t
 // ---------------------------------------------------------------------------
 // Device helpers
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void chain_begin() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+// Always true, which only the machine knows: what stands behind
+// `if (!chain_begin()) return;` is not moved in front of it, not even a load
+// through the read-only path of what the kernel before has written.
+__device__ __forceinline__ bool chain_begin() {
+  unsigned go;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 1;" : "=r"(go)::"memory");
+  return go != 0u;
 }
 
 template <typename T>

@@ -17,7 +17,7 @@ lp_merge_update_kernel(const int32_t* __restrict__ blk, const int32_t* __restric
                        const int32_t* __restrict__ labels_in, int32_t* __restrict__ labels_out,
                        unsigned long long* __restrict__ changed) {
   extern __shared__ int32_t lp_acc_all[];
-  chain_begin();
+  if (!chain_begin()) return;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t mb = (int64_t)blockIdx.x * kMergeWarps + w;
   if (mb >= nb) return;

@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32, 6)
 merge_update_kernel(const int32_t* __restrict__ blk, const int32_t* __restrict__ idx_map,
                     const float* __restrict__ interm, int k, int nb, int B, PrArgs a) {
   extern __shared__ float acc_all[];
-  chain_begin();
+  if (!chain_begin()) return;
   const double D = *a.D_in;
   const int w = threadIdx.x >> 5;
   const int64_t mb = (int64_t)blockIdx.x * kMergeWarps + w;
@@ -46,7 +46,7 @@ merge_only_kernel(const int32_t* __restrict__ blk, const int32_t* __restrict__ i
                   typename Op::T* __restrict__ out) {
   using T = typename Op::T;
   extern __shared__ unsigned char raw[];
-  chain_begin();
+  if (!chain_begin()) return;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t mb = (int64_t)blockIdx.x * kMergeWarps + w;
   if (mb >= nb) return;

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks)
 ppr_gather_kernel(const uint32_t* __restrict__ colf, const PprSeg* __restrict__ segs,
                   const int2* __restrict__ chunks, int64_t nchunks, const void* __restrict__ contrib,
                   float* __restrict__ interm, float* __restrict__ carry) {
-  chain_begin();
+  if (!chain_begin()) return;
   const int lane8 = threadIdx.x & 7;
   const int noct = (int)((gridDim.x * blockDim.x) >> 3);
   for (int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 3); c < (int)nchunks; c += noct) {
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kThreads)
 ppr_fixup_kernel(const int4* __restrict__ pieces, int64_t npieces, const int4* __restrict__ runs,
                  const float* __restrict__ carry, float* __restrict__ piece_sum,
                  unsigned* __restrict__ run_done, float* __restrict__ interm) {
-  chain_begin();
+  if (!chain_begin()) return;
   const int lane8 = threadIdx.x & 7;
   const unsigned omask = 0xffu << (threadIdx.x & 24);
   const int64_t noct = ((int64_t)gridDim.x * blockDim.x) >> 3;
@@ -287,7 +287,7 @@ ppr_merge_kernel(MergeArgs a) {
   __shared__ double s_acc[kThreads / 32][RESID ? 2 : 1][8][32];
   __shared__ double s_half[2 * kCols];
   __shared__ bool s_last;
-  chain_begin();
+  if (!chain_begin()) return;
   if (threadIdx.x < kCols) {
     s_tele[threadIdx.x] =
         (float)((1.0 - (double)a.d) + (double)a.d * a.D[threadIdx.x]);

@@ -14,6 +14,7 @@ constexpr int kScanTile = kScanThreads * kScanItems;
 template <typename TI>
 __global__ void tile_reduce_kernel(const TI* __restrict__ in, int64_t n,
                                    int64_t* __restrict__ sums) {
+  if (!chain_begin()) return;
   __shared__ int64_t sh[32];
   const int64_t base = (int64_t)blockIdx.x * kScanTile;
   int64_t acc = 0;
@@ -33,6 +34,7 @@ template <typename TI>
 __global__ void tile_scan_kernel(const TI* __restrict__ in, int64_t n,
                                  const int64_t* __restrict__ tile_off,
                                  int64_t* __restrict__ out) {
+  if (!chain_begin()) return;
   __shared__ int64_t warp_tot[kScanThreads / 32];
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   int64_t v[kScanItems];
@@ -77,19 +79,17 @@ int exclusive_scan_impl(const TI* in, int64_t* out, int64_t n, cudaStream_t s, S
   }
   const int64_t tiles = ceil_div(n, kScanTile);
   if (tiles == 1) {
-    tile_scan_kernel<TI><<<1, kScanThreads, 0, s>>>(in, n, nullptr, out);
-    CG_LAUNCH_CHECK();
+    CG_TRY(launch_chained(tile_scan_kernel<TI>, 1, kScanThreads, 0, s, in, n, nullptr, out));
     return CG_OK;
   }
   Scratch own(s, scan_scratch(n));
   if (!ws) ws = &own;
   int64_t* buf = nullptr;  // tile sums [tiles], tile offsets [tiles+1]
   CG_CUDA(ws->get(&buf, 2 * tiles + 1));
-  tile_reduce_kernel<TI><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, buf);
-  CG_LAUNCH_CHECK();
+  CG_TRY(launch_chained(tile_reduce_kernel<TI>, (unsigned)tiles, kScanThreads, 0, s, in, n, buf));
   CG_TRY(exclusive_scan_impl<int64_t>(buf, buf + tiles, tiles, s, ws));
-  tile_scan_kernel<TI><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, buf + tiles, out);
-  CG_LAUNCH_CHECK();
+  CG_TRY(launch_chained(tile_scan_kernel<TI>, (unsigned)tiles, kScanThreads, 0, s, in, n,
+                        buf + tiles, out));
   return CG_OK;
 }
 
@@ -102,6 +102,7 @@ constexpr int kSortWarps = kSortThreads / 32;
 
 __global__ void radix_hist_kernel(const uint32_t* __restrict__ keys, int64_t n, int shift,
                                   int32_t* __restrict__ counts, int64_t ntiles) {
+  if (!chain_begin()) return;
   __shared__ int32_t h[256];
   for (int i = threadIdx.x; i < 256; i += kSortThreads) h[i] = 0;
   __syncthreads();
@@ -123,6 +124,7 @@ __global__ void radix_scatter_kernel(const uint32_t* __restrict__ kin,
                                      const int32_t* __restrict__ vin, int64_t n, int shift,
                                      const int64_t* __restrict__ offs, int64_t ntiles,
                                      uint32_t* __restrict__ kout, int32_t* __restrict__ vout) {
+  if (!chain_begin()) return;
   __shared__ int32_t wc[kSortWarps][256];
   for (int i = threadIdx.x; i < kSortWarps * 256; i += kSortThreads) (&wc[0][0])[i] = 0;
   __syncthreads();
@@ -214,12 +216,11 @@ int radix_sort_pairs(const uint32_t* keys_in, const int32_t* vals_in, uint32_t* 
     const bool to_out = ((passes - 1 - p) % 2) == 0;
     uint32_t* kdst = to_out ? keys_out : kb;
     int32_t* vdst = to_out ? vals_out : vb;
-    radix_hist_kernel<<<(unsigned)ntiles, kSortThreads, 0, s>>>(ksrc, n, 8 * p, counts, ntiles);
-    CG_LAUNCH_CHECK();
+    CG_TRY(launch_chained(radix_hist_kernel, (unsigned)ntiles, kSortThreads, 0, s, ksrc, n, 8 * p,
+                          counts, ntiles));
     CG_TRY(exclusive_scan_i32_to_i64(counts, offs, 256 * ntiles, s, ws));
-    radix_scatter_kernel<<<(unsigned)ntiles, kSortThreads, 0, s>>>(ksrc, vsrc, n, 8 * p, offs,
-                                                                    ntiles, kdst, vdst);
-    CG_LAUNCH_CHECK();
+    CG_TRY(launch_chained(radix_scatter_kernel, (unsigned)ntiles, kSortThreads, 0, s, ksrc, vsrc,
+                          n, 8 * p, offs, ntiles, kdst, vdst));
     ksrc = kdst;
     vsrc = vdst;
   }

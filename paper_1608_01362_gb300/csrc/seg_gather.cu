@@ -61,7 +61,7 @@ template <class Op>
 __global__ void __launch_bounds__(256)
 seg_fixup_kernel(const int32_t* __restrict__ carry_row, const typename Op::T* __restrict__ carry,
                  int64_t n, typename Op::T* __restrict__ out) {
-  chain_begin();
+  if (!chain_begin()) return;
   fix_runs<Op>(carry_row, carry, n, out);
 }
 
@@ -177,7 +177,7 @@ seg_gather_kernel(const uint32_t* __restrict__ colf, const typename Op::T* __res
                   const int32_t* __restrict__ seg_lo, int k, int32_t ct_begin, int32_t ct_end,
                   typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   constexpr int WARPS = THREADS / 32;
-  chain_begin();
+  if (!chain_begin()) return;
   const int w = threadIdx.x >> 5;
   const int32_t my_lo = ct_begin + (int32_t)blockIdx.x;
   const int32_t step = (int32_t)gridDim.x;
@@ -298,7 +298,7 @@ staged_gather_kernel(StagedTasks q, StagedShare sh, const typename Op::T* __rest
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ RangeSlots slots;
-  chain_begin();
+  if (!chain_begin()) return;
   staged_pieces<Op>(q, sh, x, out, carry, reinterpret_cast<T*>(smem_raw), THREADS, &slots);
   counters_done(sh.ranges.next, (int)gridDim.x, sh.done);
 }
@@ -317,7 +317,7 @@ affine_gather_kernel(StagedTasks q, const typename Op::T* __restrict__ x,
                      int m, int m2, unsigned* __restrict__ next_seg, unsigned* __restrict__ done,
                      typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   using T = typename Op::T;
-  chain_begin();
+  if (!chain_begin()) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
   __shared__ int32_t s_seg;
@@ -400,7 +400,7 @@ overlap_gather_kernel(StagedTasks q, StagedShare sh, const uint32_t* __restrict_
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ RangeSlots slots;
-  chain_begin();
+  if (!chain_begin()) return;
   if ((int)threadIdx.x < staged_threads)
     staged_pieces<Op>(q, sh, x, out, carry, reinterpret_cast<T*>(smem_raw), staged_threads, &slots);
   cached_queue<Op>(colf, x, nx, first_row, seg_cstart, seg_E, seg_chunk, seg_lo, m, k, next_chunk,
