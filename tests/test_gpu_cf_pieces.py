@@ -1,8 +1,7 @@
-"""The collaborative-filtering gather through segments of neighbours: several
-segments on both sides, runs of 128, 129, 256 and 257 ratings in one segment,
-vertices without ratings, every K and precision, ratings of 0 and 255, and the
-rule that leaves K = 16 and rows whose neighbours do not ascend to the gather
-from L2.
+"""The collaborative-filtering gather where its pieces and tasks meet their edges:
+rows of 15 to 33 ratings (pieces of 16 here), rows at the numbers of pieces from
+which a warp (8) or a block (64) updates a vertex, vertices without ratings,
+neighbours that ascend or not, every K and precision, ratings of 0 and 255.
 Every entry within the oracle's rounding bound for a sweep from the same
 factors (oracle.cf_sweep_bound: any summation tree)."""
 import numpy as np
@@ -29,10 +28,13 @@ def ratings():
     for u in range(U):
         if u % 97 == 0:
             rows.append(np.empty(0, np.int64))  # no ratings
-        elif u < 40:
-            rows.append(np.sort(rng.choice(800, [128, 129, 256, 257][u % 4], replace=False)))
-        else:
-            rows.append(np.unique((I * rng.random(85) ** 1.5).astype(np.int64)))
+        elif u < 160:
+            n = [15, 16, 17, 31, 33, 128, 129, 1024, 1025, 4000][u % 10]
+            rows.append(np.sort(rng.choice(I - 100, n, replace=False)))
+        else:  # items rated by about 6,100 and by 300 to 500 users among them
+            pick = np.unique((I * rng.random(40) ** 1.5).astype(np.int64))
+            few = 4450 + np.flatnonzero(rng.random(40) < 0.045)
+            rows.append(np.unique(np.concatenate([pick[pick < I - 110], few, [0] * (u < 6300)])))
     off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
     item = np.concatenate(rows).astype(np.int32)
     rate = rng.integers(0, 256, item.size).astype(np.uint8)
@@ -61,9 +63,7 @@ def test_sweep_within_bound(C, ratings, K, precision, ascending):
         d[1] = torch.as_tensor(item[perm].copy()).cuda()
         d[2] = torch.as_tensor(rate[perm].copy()).cuda()
     h = C.cf_create(U, I, K, precision, *d)
-    # from L2: one piece per 512 ratings; through segments: one per segment and vertex
-    plain = int(sum(-(-n // 512) for n in np.diff(off)))
-    assert (h.info["user_pieces"] == plain) == (not ascending or K == 16)
+    assert h.info["user_pieces"] == int(sum(-(-n // 16) for n in np.diff(off)))
     P0, Q0 = (0.05 * a for a in graphgen.cf_factors(U, I, K, seed=2))
     C.cf_set_factors(h, torch.as_tensor(P0.astype(np.float32)).cuda(),
                      torch.as_tensor(Q0.astype(np.float32)).cuda())
