@@ -339,7 +339,7 @@ affine_gather_kernel(StagedTasks q, const typename Op::T* __restrict__ x,
 }
 
 // L1/L2 chunks of segments [m, k) taken from a queue (a global counter of
-// chunks, kCachedGrab at a time): a warp's successive grabs only move forward,
+// chunks, kCachedGrab at a time or one): a warp's successive grabs only move forward,
 // so its segment is found by stepping.  The grab's chunks are prefetched into
 // L2 (TMA) when it is taken.
 constexpr int kCachedGrab = 4;
@@ -353,14 +353,17 @@ __device__ __forceinline__ void cached_queue(
     typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   const int lane = threadIdx.x & 31;
   const int32_t c_begin = (int32_t)seg_chunk[m], c_end = (int32_t)seg_chunk[k];
+  // one chunk at a time where there are few: with 80 per SM, four at a time, the
+  // last grabs outlast everything else (1 M vertices, 8 warps: 75 us, so 55)
+  const int grab = c_end - c_begin < (int32_t)gridDim.x * 512 ? 1 : kCachedGrab;
   int s = m;
   int32_t lo = 0, Es = 0, cstart = 0, cbase = 0, cnext = -1;
   for (;;) {
     int32_t c0 = 0;
-    if (lane == 0) c0 = (int32_t)atomicAdd(next_chunk, (unsigned)kCachedGrab);
+    if (lane == 0) c0 = (int32_t)atomicAdd(next_chunk, (unsigned)grab);
     c0 = __shfl_sync(0xffffffffu, c0, 0) + c_begin;
     if (c0 >= c_end) break;
-    const int32_t c1 = c0 + kCachedGrab < c_end ? c0 + kCachedGrab : c_end;
+    const int32_t c1 = c0 + grab < c_end ? c0 + grab : c_end;
     if (lane < c1 - c0) {  // lane u prefetches chunk c0 + u (1 KB of colf)
       const int32_t cu = c0 + lane;
       int su = s;
