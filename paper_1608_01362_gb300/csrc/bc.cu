@@ -90,6 +90,32 @@ constexpr int kSub = 256;        // edges a warp folds at once: 8 consecutive pe
 constexpr int kPushTile = 256;   // frontier edges per warp in a push
 typedef unsigned long long u64;
 
+// Where a level's counts go when it is done: the host's pinned words, the
+// ticket last.
+struct Mailbox {
+  u64* pin;
+  u64 ticket;
+};
+
+__device__ __forceinline__ void publish(const u64* count, const Mailbox& box) {
+  volatile u64* pin = box.pin;
+  for (int q = 0; q < 4; ++q) pin[q] = __ldcg(count + q);
+  __threadfence_system();
+  pin[4] = box.ticket;
+}
+
+// The same by the last block of a launch (count[4]: blocks done, cleared
+// again).  Every thread of the block calls it, when the block has counted.
+__device__ __forceinline__ void publish_last(u64* count, const Mailbox& box) {
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  __threadfence();
+  if (atomicAdd(count + 4, 1ull) != gridDim.x - 1) return;
+  __threadfence();
+  count[4] = 0ull;
+  publish(count, box);
+}
+
 __global__ void bc_reset_kernel(int32_t V, int32_t* __restrict__ level,
                                 double* __restrict__ sigma, double* __restrict__ delta,
                                 uint32_t* __restrict__ xbits) {
@@ -113,7 +139,7 @@ __device__ __forceinline__ void set_bit(uint32_t* bits, int32_t v, bool on) {
 __global__ void bc_seed_kernel(int32_t s, const int64_t* __restrict__ out_off,
                                int32_t* __restrict__ level, double* __restrict__ sigma,
                                int32_t* __restrict__ list, int32_t* __restrict__ fpos,
-                               int32_t* __restrict__ fgap, u64* __restrict__ count) {
+                               int32_t* __restrict__ fgap, u64* __restrict__ count, Mailbox box) {
   if (!chain_begin()) return;
   level[s] = 0;
   sigma[s] = 1.0;
@@ -122,8 +148,10 @@ __global__ void bc_seed_kernel(int32_t s, const int64_t* __restrict__ out_off,
   fpos[0] = 0;
   fgap[0] = (int32_t)out_off[s];
   count[0] = deg ? (1ull << 32) | deg : 0ull;
-  count[1] = count[2] = 0ull;
+  count[1] = count[2] = count[4] = 0ull;
   count[3] = 1ull;
+  __threadfence();
+  publish(count, box);
 }
 
 struct Frontier {
@@ -221,7 +249,7 @@ __device__ __forceinline__ void append_block(bool take, int32_t v,
 __global__ void __launch_bounds__(kThreads)
 push_kernel(Frontier cur, int32_t n, int32_t m, const int64_t* __restrict__ out_off,
             const int32_t* __restrict__ out_dst, int32_t L, int32_t* __restrict__ level,
-            double* __restrict__ sigma, Frontier nxt, u64* __restrict__ count) {
+            double* __restrict__ sigma, Frontier nxt, u64* __restrict__ count, Mailbox box) {
   if (!chain_begin()) return;
   u64* next = count + (L + 1) % 3;
   if (blockIdx.x == 0 && threadIdx.x == 0) count[(L + 2) % 3] = 0ull;
@@ -251,6 +279,7 @@ push_kernel(Frontier cur, int32_t n, int32_t m, const int64_t* __restrict__ out_
       append(take, w, out_off, nxt, next, count + 3);
     }
   }
+  publish_last(count, box);
 }
 
 // ---------------------------------------------------------------------------
@@ -505,7 +534,8 @@ __global__ void __launch_bounds__(256) row_fix_kernel(RowSums a) {
 int row_sums(const RowSums& a, int64_t most_edges, cudaStream_t s) {
   const int64_t tiles = ceil_div(most_edges, kSub);
   CG_TRY(launch_chained(row_sum_kernel, grid_for(tiles * 32, kThreads, 4), kThreads, 0, s, a));
-  CG_TRY(launch_chained(row_fix_kernel, grid_for(tiles, 256, 4), 256, 0, s, a));
+  if (tiles > 1)  // (one tile ends with its last row)
+    CG_TRY(launch_chained(row_fix_kernel, grid_for(tiles, 256, 4), 256, 0, s, a));
   return CG_OK;
 }
 
@@ -515,7 +545,7 @@ __global__ void __launch_bounds__(kThreads)
 pull_update_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ packed,
                    const double* __restrict__ acc, const int64_t* __restrict__ out_off, int32_t L,
                    int32_t* __restrict__ level, double* __restrict__ sigma, Frontier nxt,
-                   u64* __restrict__ count) {
+                   u64* __restrict__ count, Mailbox box) {
   if (!chain_begin()) return;
   u64* next = count + (L + 1) % 3;
   if (blockIdx.x == 0 && threadIdx.x == 0) count[(L + 2) % 3] = 0ull;
@@ -536,6 +566,7 @@ pull_update_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ 
     }
     append_block(take, v, out_off, nxt, next, count + 3);
   }
+  publish_last(count, box);
 }
 
 __global__ void set_bits_kernel(const int32_t* __restrict__ list, int64_t n,
@@ -588,20 +619,8 @@ __global__ void row_of_edge_kernel(const int64_t* __restrict__ off, int32_t V, i
   }
 }
 
-// Writes the counts and, behind them, the ticket to the host's pinned copy.
-__device__ __forceinline__ void publish(const u64* count, volatile u64* pin, u64 ticket) {
-  for (int q = 0; q < 4; ++q) pin[q] = __ldcg(count + q);
-  __threadfence_system();
-  pin[4] = ticket;
-}
-
-__global__ void publish_kernel(const u64* count, u64* pin, u64 ticket) {
-  if (!chain_begin()) return;
-  publish(count, pin, ticket);
-}
-
-// Waits for the counts of the ticket: the host watches the pinned word that a
-// kernel writes (a copy and a synchronisation took 17 us of every level, this 8),
+// Waits for the counts of the ticket: the host watches the pinned word that the
+// level's last block writes (a copy and a synchronisation took 17 us of every level),
 // and asks the stream now and then whether it has failed.
 int wait_counts(cg_bc* h, cudaStream_t s) {
   for (int spins = 1; __atomic_load_n(h->h_pin + 4, __ATOMIC_ACQUIRE) != h->ticket; ++spins) {
@@ -619,10 +638,8 @@ int wait_counts(cg_bc* h, cudaStream_t s) {
   return CG_OK;
 }
 
-int read_counts(cg_bc* h, cudaStream_t s) {
-  CG_TRY(launch_chained(publish_kernel, 1, 1, 0, s, h->count, h->h_pin, ++h->ticket));
-  return wait_counts(h, s);
-}
+// The mailbox of the launch that is next to be waited for.
+Mailbox mailbox(cg_bc* h) { return Mailbox{h->h_pin, ++h->ticket}; }
 
 Frontier frontier(const cg_bc* h, int q) { return Frontier{h->flist[q], h->fpos[q], h->fgap[q]}; }
 
@@ -641,7 +658,7 @@ int pull_level(cg_bc* h, int32_t L, int32_t n, cudaStream_t s) {
   CG_TRY(row_sums(a, h->E, s));
   CG_TRY(launch_chained(pull_update_kernel, grid_for(V, kThreads), kThreads, 0, s, h->ids, packed,
                         h->acc, h->out_off, L, h->level, h->sigma, frontier(h, 1 - cur),
-                        h->count));
+                        h->count, mailbox(h)));
   CG_TRY(launch_chained(set_bits_kernel, grid_for(n, kThreads), kThreads, 0, s, h->flist[cur], n,
                         h->xbits, false));
   return CG_OK;
@@ -652,8 +669,8 @@ int run_source(cg_bc* h, int32_t src, double* bc, cudaStream_t s) {
   CG_TRY(launch_chained(bc_reset_kernel, grid_for(V, kThreads), kThreads, 0, s, V, h->level,
                         h->sigma, h->delta, h->xbits));
   CG_TRY(launch_chained(bc_seed_kernel, 1, 1, 0, s, src, h->out_off, h->level, h->sigma,
-                        h->flist[0], h->fpos[0], h->fgap[0], h->count));
-  CG_TRY(read_counts(h, s));
+                        h->flist[0], h->fpos[0], h->fgap[0], h->count, mailbox(h)));
+  CG_TRY(wait_counts(h, s));
   // per level: vertices, of them with out-edges, and these edges
   std::vector<int64_t> size(1, 1), rows, edges;
   h->push_levels = h->pull_levels = 0;
@@ -671,10 +688,10 @@ int run_source(cg_bc* h, int32_t src, double* bc, cudaStream_t s) {
       const int cur = L & 1;
       CG_TRY(launch_chained(push_kernel, grid_for(ceil_div(m, kPushTile) * 32, kThreads), kThreads,
                             0, s, frontier(h, cur), n, m, h->out_off, h->out_dst, L, h->level,
-                            h->sigma, frontier(h, 1 - cur), h->count));
+                            h->sigma, frontier(h, 1 - cur), h->count, mailbox(h)));
       ++h->push_levels;
     }
-    CG_TRY(read_counts(h, s));
+    CG_TRY(wait_counts(h, s));
     if (h->h_pin[3] == reached) break;  // nothing new
     size.push_back((int64_t)(h->h_pin[3] - reached));
   }
