@@ -85,12 +85,14 @@ __global__ void first_row_kernel(const int32_t* __restrict__ rp,
   }
 }
 
-// One L1/L2 chunk: 256 edges of segment-local chunk j (global chunk c) of a
-// segment whose sources start at lo; lane l holds edges [8l, 8l + 8).
-constexpr int kCachedIPL = 8;
-constexpr int kCachedChunk = 32 * kCachedIPL;  // 256 edges
+// One L1/L2 chunk: segment-local chunk j (global chunk c) of 32 * IPL edges of a
+// segment whose sources start at lo; lane l holds edges [IPL l, IPL (l + 1)).
+// Eight edges per lane, or four where there are few edges: chunks are then few
+// per warp, and a launch is a chain of two of them (0.3 M edges 10.3 -> 8.1 us,
+// 3.1 M 18.0 -> 16.3, 8.8 M 41.9 -> 40.0, 22 M 89.0 -> 91.0, 66 M 260 -> 268).
+constexpr int64_t kFewCachedEdges = (int64_t)1 << 24;
 
-template <class Op>
+template <class Op, int IPL>
 __device__ __forceinline__ void cached_chunk(const uint32_t* __restrict__ colf,
                                              const typename Op::T* __restrict__ x, int32_t nx,
                                              int32_t lo, int32_t Es, int32_t cstart, int32_t j,
@@ -98,16 +100,19 @@ __device__ __forceinline__ void cached_chunk(const uint32_t* __restrict__ colf,
                                              typename Op::T* __restrict__ out,
                                              typename Op::T* __restrict__ carry) {
   using T = typename Op::T;
-  constexpr int IPL = kCachedIPL;
-  constexpr int CHUNK = kCachedChunk;
+  constexpr int CHUNK = 32 * IPL;
   const int lane = threadIdx.x & 31;
   const int32_t e0 = j * CHUNK;
   const int n = Es - e0 < CHUNK ? Es - e0 : CHUNK;
 
-  // 1. this lane's 8 edges (two 16-byte streaming loads; colf is padded)
+  // 1. this lane's edges (16-byte streaming loads; colf is padded)
   const uint4* p = reinterpret_cast<const uint4*>(colf + cstart + e0 + lane * IPL);
-  const uint4 qa = __ldcs(p), qb = __ldcs(p + 1);
-  const uint32_t cf[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+  uint32_t cf[IPL];
+#pragma unroll
+  for (int u = 0; u < IPL; u += 4) {
+    const uint4 q = __ldcs(p + u / 4);
+    cf[u] = q.x; cf[u + 1] = q.y; cf[u + 2] = q.z; cf[u + 3] = q.w;
+  }
   T v[IPL];
   uint32_t fl = 0;
   const int nl = n - lane * IPL;  // valid edges of this lane
@@ -168,7 +173,7 @@ __device__ __forceinline__ void cached_chunk(const uint32_t* __restrict__ colf,
 // The L1/L2 launch: every read of a segment in [ct_begin, ct_end) goes
 // through L1/L2.  Blocks take block-groups round-robin (the grid sweeps the
 // groups in order, which balances blocks when the cost per group varies).
-template <class Op, int THREADS>
+template <class Op, int THREADS, int IPL>
 __global__ void __launch_bounds__(THREADS, 2048 / THREADS)
 seg_gather_kernel(const uint32_t* __restrict__ colf, const typename Op::T* __restrict__ x,
                   int32_t nx, const int32_t* __restrict__ first_row,
@@ -204,8 +209,8 @@ seg_gather_kernel(const uint32_t* __restrict__ colf, const typename Op::T* __res
       ctnext = seg_ctile[s + 1];
     }
     const int32_t j = (ct - ctbase) * WARPS + w;  // chunk of this warp within the segment
-    if (j * kCachedChunk >= Es) continue;         // warp-uniform
-    cached_chunk<Op>(colf, x, nx, lo, Es, cstart, j, cbase + j, first_row[cbase + j], out,
+    if (j * 32 * IPL >= Es) continue;             // warp-uniform
+    cached_chunk<Op, IPL>(colf, x, nx, lo, Es, cstart, j, cbase + j, first_row[cbase + j], out,
                      carry);
   }
 }
@@ -344,7 +349,7 @@ affine_gather_kernel(StagedTasks q, const typename Op::T* __restrict__ x,
 // L2 (TMA) when it is taken.
 constexpr int kCachedGrab = 4;
 
-template <class Op>
+template <class Op, int IPL>
 __device__ __forceinline__ void cached_queue(
     const uint32_t* __restrict__ colf, const typename Op::T* __restrict__ x, int32_t nx,
     const int32_t* __restrict__ first_row, const int64_t* __restrict__ seg_cstart,
@@ -368,8 +373,8 @@ __device__ __forceinline__ void cached_queue(
       const int32_t cu = c0 + lane;
       int su = s;
       while (cu >= (int32_t)seg_chunk[su + 1]) ++su;
-      prefetch_l2(colf + seg_cstart[su] + (int64_t)(cu - (int32_t)seg_chunk[su]) * kCachedChunk,
-                  kCachedChunk * 4);
+      prefetch_l2(colf + seg_cstart[su] + (int64_t)(cu - (int32_t)seg_chunk[su]) * 32 * IPL,
+                  32 * IPL * 4);
     }
     for (int32_t c = c0; c < c1; ++c) {
       if (c >= cnext) {
@@ -380,7 +385,7 @@ __device__ __forceinline__ void cached_queue(
         cbase = (int32_t)seg_chunk[s];
         cnext = (int32_t)seg_chunk[s + 1];
       }
-      cached_chunk<Op>(colf, x, nx, lo, Es, cstart, c - cbase, c, first_row[c], out, carry);
+      cached_chunk<Op, IPL>(colf, x, nx, lo, Es, cstart, c - cbase, c, first_row[c], out, carry);
     }
   }
 }
@@ -391,7 +396,7 @@ __device__ __forceinline__ void cached_queue(
 // start, and the staged warps join that queue when their pieces run out.
 // The cold segments' random reads go to L2 while the staged warps read
 // shared memory, so the two kinds of lookup proceed side by side.
-template <class Op>
+template <class Op, int IPL>
 __global__ void __launch_bounds__(1024, 1)
 overlap_gather_kernel(StagedTasks q, StagedShare sh, const uint32_t* __restrict__ colf,
                       const typename Op::T* __restrict__ x, int32_t nx,
@@ -406,7 +411,7 @@ overlap_gather_kernel(StagedTasks q, StagedShare sh, const uint32_t* __restrict_
   if (!chain_begin()) return;
   if ((int)threadIdx.x < staged_threads)
     staged_pieces<Op>(q, sh, x, out, carry, reinterpret_cast<T*>(smem_raw), staged_threads, &slots);
-  cached_queue<Op>(colf, x, nx, first_row, seg_cstart, seg_E, seg_chunk, seg_lo, m, k, next_chunk,
+  cached_queue<Op, IPL>(colf, x, nx, first_row, seg_cstart, seg_E, seg_chunk, seg_lo, m, k, next_chunk,
                    out, carry);
   counters_done(next_chunk, 4 + (int)gridDim.x, sh.done);  // the ranges' lie behind it
 }
@@ -511,7 +516,8 @@ static int allow_tables() {
   const void* fns[] = {(const void*)staged_gather_kernel<Op, 1024>,
                        (const void*)staged_gather_kernel<Op, 512>,
                        (const void*)affine_gather_kernel<Op>,
-                       (const void*)overlap_gather_kernel<Op>};
+                       (const void*)overlap_gather_kernel<Op, 4>,
+                       (const void*)overlap_gather_kernel<Op, 8>};
   const int most = 4 * seg_table_capacity(1) + 16;
   for (const void* f : fns)
     CG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
@@ -582,11 +588,15 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   const int warps_b = 1024 / 32;
   const int tab_cap = (int)((tabmax + 3) & ~3LL);
   // chunks of the segments read through L1/L2
+  int64_t cached = 0;
+  for (int q = m2; q < k; ++q) cached += p->edge_base[q + 1] - p->edge_base[q];
+  p->cached_ipl = cached < kFewCachedEdges ? 4 : 8;
+  const int chunk_edges = 32 * p->cached_ipl;
   std::vector<int64_t> chunk(k + 1, 0);
   std::vector<int32_t> ctile(k + 1, 0), tn(k > 0 ? k : 1, 0);
   for (int q = 0; q < k; ++q) {
     chunk[q + 1] =
-        chunk[q] + (q < m2 ? 0 : ceil_div(p->edge_base[q + 1] - p->edge_base[q], kCachedChunk));
+        chunk[q] + (q < m2 ? 0 : ceil_div(p->edge_base[q + 1] - p->edge_base[q], chunk_edges));
     tn[q] = q < m2 ? (int32_t)(p->src_bounds[q + 1] - p->src_bounds[q]) : 0;
   }
   const int64_t ncached = chunk[k];
@@ -605,10 +615,10 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   }
   if (ncached > 0) {
     first_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
-        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, kCachedChunk, ncached, p->first_row);
+        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, chunk_edges, ncached, p->first_row);
     CG_LAUNCH_CHECK();
     open_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
-        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, kCachedChunk, ncached,
+        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, chunk_edges, ncached,
         p->carry_row);
     CG_LAUNCH_CHECK();
   }
@@ -702,7 +712,7 @@ static int launch_overlap(const SegPlan& p, const typename Op::T* x, int32_t nx,
                           typename Op::T* out, cudaStream_t s) {
   using T = typename Op::T;
   const size_t smem = staged_smem(p);
-  auto fn = overlap_gather_kernel<Op>;
+  auto fn = p.cached_ipl == 4 ? overlap_gather_kernel<Op, 4> : overlap_gather_kernel<Op, 8>;
   return launch_chained(fn, p.grid, 1024, smem, s, staged_tasks(p), staged_share(p), p.colf, x, nx,
                         p.first_row, p.seg_cstart, p.seg_E, p.seg_chunk, p.seg_lo, p.m, p.k,
                         1024 - 32 * p.overlap, p.counter, out, reinterpret_cast<T*>(p.carry));
@@ -733,7 +743,8 @@ int run_seg_gather(const SegPlan& p, const typename Op::T* x, int32_t nx, typena
   }
   // the rest through L1/L2: no shared memory, so the whole on-chip store is L1
   if ((phases & kPhaseCached) && p.n_ctiles > 0) {
-    CG_TRY(launch_chained(seg_gather_kernel<Op, 1024>, p.grid_l2, 1024, 0, s, p.colf, x, nx,
+    auto fn = p.cached_ipl == 4 ? seg_gather_kernel<Op, 1024, 4> : seg_gather_kernel<Op, 1024, 8>;
+    CG_TRY(launch_chained(fn, p.grid_l2, 1024, 0, s, p.colf, x, nx,
                           p.first_row, p.seg_cstart, p.seg_E, p.seg_chunk, p.seg_ctile, p.seg_lo,
                           p.k, 0, (int32_t)p.n_ctiles, out, reinterpret_cast<T*>(p.carry)));
   }

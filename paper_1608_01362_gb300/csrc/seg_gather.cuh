@@ -72,6 +72,7 @@ struct SegPlan {
   int m2 = 0;               // segments [m, m2): staged too, one block per segment (affine)
   double affine_head = 0.0;  // > 0: head threshold (edges per source) of the segment-affine
                             // plan; the table-sized segments after the head go one per block
+  int cached_ipl = 8;          // edges per lane of an L1/L2 chunk
   int grid_affine = 0;      // blocks of the segment-affine launch
   int64_t n_ctiles = 0;     // block-groups of the L1/L2 launch
   int grid = 0;             // staged launch blocks

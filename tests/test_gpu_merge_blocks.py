@@ -88,3 +88,21 @@ def test_start_counts_its_dangling_mass(C, V):
         assert D.item() == float((V + 2) // 3) * float(r)
         assert np.array_equal(rank.cpu().numpy(), np.full(V, r))
         assert np.array_equal(contrib.cpu().numpy(), r * inv)
+
+
+@pytest.mark.parametrize("drop", [0, 1])
+def test_chunks_of_the_cached_segments(C, drop):
+    """2^24 edges read through L1/L2, and one fewer: the two chunk sizes."""
+    import torch
+    V = 1 << 20
+    src = (np.arange(16) * 65536 + (np.arange(V) * 7919 % 65536)[:, None]).astype(np.int32).ravel()
+    src = src[:src.size - drop]
+    off = np.minimum(np.arange(V + 1, dtype=np.int64) * 16, src.size)
+    seg = C.pr_build_segments(torch.as_tensor(off).cuda(), torch.as_tensor(src).cuda(), 1)
+    assert seg.info["staged_segments"] == 0
+    x = (1 + np.arange(V) % 7).astype(np.float32)
+    want = np.add.reduceat(x[src], off[:-1])
+    out = torch.full((V,), -1.0, device="cuda")
+    for _ in range(2):
+        C.cg_seg_gather(seg, C.CG_OP_SUM_F32, torch.as_tensor(x).cuda(), out)
+        assert np.array_equal(out.cpu().numpy(), want)
