@@ -119,6 +119,7 @@ gather_tile_kernel(const RowEndT* __restrict__ row_end, const int32_t* __restric
   __shared__ T s_prev_val[THREADS];
   __shared__ int32_t s_prev_row[THREADS];
 
+  if (!chain_begin()) return;
   const int tid = threadIdx.x;
   const int64_t t = blockIdx.x;
   const int32_t r0 = tile_row[t], r1 = tile_row[t + 1];
@@ -237,6 +238,7 @@ __global__ void carry_fixup_kernel(const typename Op::T* __restrict__ carry,
                                    const int32_t* __restrict__ carry_row, int64_t ntiles,
                                    int64_t nrows, typename Op::T* __restrict__ out) {
   using T = typename Op::T;
+  if (!chain_begin()) return;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntiles;
        t += (int64_t)gridDim.x * blockDim.x) {
     const int32_t r = carry_row[t];
@@ -294,15 +296,14 @@ inline int64_t tile_plan_bytes(const TilePlan& p) { return 16 * (p.ntiles + 1); 
 template <class Op, bool PROBE, typename RowEndT>
 int run_tile_gather(const TilePlan& p, const RowEndT* row_end, const int32_t* col,
                     const typename Op::T* x, int32_t nx, typename Op::T* out, cudaStream_t s) {
+  using T = typename Op::T;
   if (p.ntiles == 0) return CG_OK;
-  gather_tile_kernel<Op, kTileThreads, kTileIPT, PROBE, RowEndT>
-      <<<(unsigned)p.ntiles, kTileThreads, 0, s>>>(
-          row_end, col, x, nx, p.tile_row, p.tile_edge, out,
-          reinterpret_cast<typename Op::T*>(p.carry), p.carry_row);
-  CG_LAUNCH_CHECK();
-  carry_fixup_kernel<Op><<<grid_for(p.ntiles, 256, 4), 256, 0, s>>>(
-      reinterpret_cast<const typename Op::T*>(p.carry), p.carry_row, p.ntiles, p.nrows, out);
-  CG_LAUNCH_CHECK();
+  T* carry = reinterpret_cast<T*>(p.carry);
+  CG_TRY(launch_chained(gather_tile_kernel<Op, kTileThreads, kTileIPT, PROBE, RowEndT>,
+                        (unsigned)p.ntiles, kTileThreads, 0, s, row_end, col, x, nx, p.tile_row,
+                        p.tile_edge, out, carry, p.carry_row));
+  CG_TRY(launch_chained(carry_fixup_kernel<Op>, grid_for(p.ntiles, 256, 4), 256, 0, s, carry,
+                        p.carry_row, p.ntiles, p.nrows, out));
   return CG_OK;
 }
 

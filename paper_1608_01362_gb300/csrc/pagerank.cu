@@ -440,9 +440,8 @@ int pr_iterate_plain(const cg_plain* p, const float* inv, const float* rank_in,
     a.counter = p->counter;
     a.V = p->V;
     a.seed = -1;
-    dense_update_kernel<<<(unsigned)ceil_div(nb, kMergeWarps), kMergeWarps * 32, smem,
-                          stream>>>(p->acc, B, nb, a);
-    CG_LAUNCH_CHECK();
+    CG_TRY(launch_chained(dense_update_kernel, (unsigned)ceil_div(nb, kMergeWarps),
+                          kMergeWarps * 32, smem, stream, p->acc, B, nb, a));
   }
   return CG_OK;
 }

@@ -257,6 +257,7 @@ __device__ __forceinline__ void block_finish(double dsum, double rsum, const PrA
 __global__ void __launch_bounds__(kMergeWarps * 32)
 dense_update_kernel(const float* __restrict__ sums, int B, int nb, PrArgs a) {
   extern __shared__ float acc_all[];
+  if (!chain_begin()) return;
   const double D = *a.D_in;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t mb = (int64_t)blockIdx.x * kMergeWarps + w;
