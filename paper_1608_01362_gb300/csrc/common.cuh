@@ -73,8 +73,14 @@ struct Scratch {
   char* cur = nullptr;
   size_t left = 0;
   explicit Scratch(cudaStream_t st, size_t first_slab = 0) : s(st), first(first_slab) {}
-  Scratch(cudaStream_t st, void* buffer, size_t bytes)  // over a buffer that a handle keeps
-      : s(st), first(0), cur(static_cast<char*>(buffer)), left(bytes) {}
+  // over a buffer that a handle or a caller keeps, where it is not too small
+  Scratch(cudaStream_t st, void* buffer, size_t bytes, size_t first_slab = 0)
+      : s(st), first(first_slab) {
+    if (bytes >= first_slab) {
+      cur = static_cast<char*>(buffer);
+      left = bytes;
+    }
+  }
   Scratch(const Scratch&) = delete;
   Scratch& operator=(const Scratch&) = delete;
   static size_t round(size_t b) { return (b + 255) & ~(size_t)255; }

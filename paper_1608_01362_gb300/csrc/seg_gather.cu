@@ -663,7 +663,6 @@ int seg_plan_carries(SegPlan* p, int64_t n) {
 
 void seg_plan_free(SegPlan* p) {
   cudaFree(p->colf);
-  cudaFree(p->cs);
   cudaFree(p->desc);
   cudaFree(p->meta);
   cudaFree(p->first_row);
@@ -671,7 +670,7 @@ void seg_plan_free(SegPlan* p) {
 }
 
 int64_t seg_plan_bytes(const SegPlan& p) {
-  return 4 * p.colf_len + p.cs_cap + 16 * p.desc_cap + 12 * p.carry_cap +
+  return 4 * p.colf_len + p.cs_cap + 12 * p.carry_cap +
          76 * (int64_t)p.k;
 }
 

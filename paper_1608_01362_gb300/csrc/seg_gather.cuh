@@ -43,7 +43,8 @@ struct SegPlan {
   uint8_t* cs = nullptr;           // staged segments' edge stream (staged_stream.cuh)
   int64_t cs_cap = 0;
   uint4* desc = nullptr;           // one descriptor per staged task
-  int64_t desc_cap = 0;
+  void* lent = nullptr;     // scratch that a caller of seg_plan_finish has at hand
+  size_t lent_bytes = 0;
   int32_t* seg_task = nullptr;     // [k+1] first staged task of each segment
   std::vector<int32_t> h_seg_task;
   int32_t head_tasks = 0;          // tasks of the segments [0, m)

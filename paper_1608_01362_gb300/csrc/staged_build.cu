@@ -193,10 +193,11 @@ int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s
   }
   const int64_t edges = p->edge_base[m2];
   const int64_t most = rows + edges / kStagedMost;  // rows and at most their full pieces
-  Scratch tmp(s, 6 * Scratch::round(4 * (size_t)most) + sort_scratch(most) +
-                     3 * Scratch::round(8 * (size_t)(nb + 1)) + 2 * Scratch::round(4 * (size_t)nb) +
-                     2 * scan_scratch(nb) + Scratch::round(8 * (size_t)(rows + 1)) +
-                     scan_scratch(rows) + Scratch::round(8 * (size_t)(m2 + 1)) + 4096);
+  Scratch tmp(s, p->lent, p->lent_bytes,
+              6 * Scratch::round(4 * (size_t)most) + sort_scratch(most) +
+                  3 * Scratch::round(8 * (size_t)(nb + 1)) + 2 * Scratch::round(4 * (size_t)nb) +
+                  2 * scan_scratch(nb) + Scratch::round(8 * (size_t)(rows + 1)) +
+                  scan_scratch(rows) + Scratch::round(8 * (size_t)(m2 + 1)) + 4096);
   int64_t *d_wbase = nullptr, *pos = nullptr, *start = nullptr, *task_base = nullptr,
           *unit_base = nullptr;
   uint32_t *key = nullptr, *skey = nullptr;
@@ -251,21 +252,17 @@ int staged_build(SegPlan* p, int m2, int pad, int64_t carry_base, cudaStream_t s
                           cudaMemcpyDeviceToHost, s));
   CG_CUDA(cudaStreamSynchronize(s));
   const int64_t ntasks = p->h_seg_task[k];
-  if (ntasks > p->desc_cap) {
+  // descriptors and stream, one allocation (desc owns it); the prefetch reads ahead
+  const int64_t db = (int64_t)Scratch::round(sizeof(uint4) * (size_t)ntasks);
+  const int64_t bytes = db + nunits * 32 + 2 * kStreamAhead;
+  if (bytes > p->cs_cap) {
     cudaFree(p->desc);
     p->desc = nullptr;
-    p->desc_cap = 0;
-    CG_CUDA(cudaMalloc((void**)&p->desc, sizeof(uint4) * (size_t)ntasks));
-    p->desc_cap = ntasks;
-  }
-  const int64_t cs_bytes = nunits * 32 + 2 * kStreamAhead;  // the prefetch reads ahead
-  if (cs_bytes > p->cs_cap) {
-    cudaFree(p->cs);
-    p->cs = nullptr;
     p->cs_cap = 0;
-    CG_CUDA(cudaMalloc((void**)&p->cs, (size_t)cs_bytes));
-    p->cs_cap = cs_bytes;
+    CG_CUDA(cudaMalloc((void**)&p->desc, (size_t)bytes));
+    p->cs_cap = bytes;
   }
+  p->cs = reinterpret_cast<uint8_t*>(p->desc) + db;
   staged_fill_kernel<<<grid_for(ntasks * 32, 256), 256, 0, s>>>(
       p->colf, p->rp32, p->meta, p->meta + (k + 1), p->meta + 2 * (k + 1), d_wbase, m2, item,
       rows, xrow, xpiece, start, task_base, unit_base, (int)nb, ntasks, pad, carry_base, place,
