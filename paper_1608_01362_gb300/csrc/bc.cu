@@ -625,23 +625,9 @@ __global__ void row_of_edge_kernel(const int64_t* __restrict__ off, int32_t V, i
   }
 }
 
-// Waits for the counts of the ticket: the host watches the pinned word that the
-// level's last block writes (a copy and a synchronisation took 17 us of every level),
-// and asks the stream now and then whether it has failed.
+// Waits for the counts of the last mailbox.
 int wait_counts(cg_bc* h, cudaStream_t s) {
-  for (int spins = 1; __atomic_load_n(h->h_pin + 4, __ATOMIC_ACQUIRE) != h->ticket; ++spins) {
-    if (spins % 4096) continue;
-    const cudaError_t e = cudaStreamQuery(s);
-    if (e != cudaErrorNotReady && e != cudaSuccess)
-      return cuda_fail(e, "bc_run", __FILE__, __LINE__);
-    if (e == cudaSuccess) {  // all done: the word is there, or will never be
-      CG_CUDA(cudaStreamSynchronize(s));
-      if (__atomic_load_n(h->h_pin + 4, __ATOMIC_ACQUIRE) == h->ticket) break;
-      set_error("bc_run: the level's counts did not arrive");
-      return CG_ERR_CUDA;
-    }
-  }
-  return CG_OK;
+  return wait_ticket(h->h_pin + 4, h->ticket, s, "bc_run");
 }
 
 // The mailbox of the launch that is next to be waited for.

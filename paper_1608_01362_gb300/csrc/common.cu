@@ -65,6 +65,22 @@ int grid_for(int64_t n, int threads, int per_sm) {
   return (int)(want < cap ? want : cap);
 }
 
+int wait_ticket(const unsigned long long* word, unsigned long long ticket, cudaStream_t s,
+                const char* what) {
+  for (int spins = 1; __atomic_load_n(word, __ATOMIC_ACQUIRE) != ticket; ++spins) {
+    if (spins % 4096) continue;
+    const cudaError_t e = cudaStreamQuery(s);
+    if (e != cudaErrorNotReady && e != cudaSuccess) return cuda_fail(e, what, __FILE__, __LINE__);
+    if (e == cudaSuccess) {  // all done: the word is there, or will never be
+      CG_CUDA(cudaStreamSynchronize(s));
+      if (__atomic_load_n(word, __ATOMIC_ACQUIRE) == ticket) break;
+      set_error("%s: a result did not reach the host", what);
+      return CG_ERR_CUDA;
+    }
+  }
+  return CG_OK;
+}
+
 }  // namespace cg
 
 extern "C" {

@@ -153,6 +153,12 @@ int launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t
   return CG_OK;
 }
 
+// Waits until a kernel on the stream has written the ticket to a pinned word:
+// the host watches the word (a copy and a synchronisation take 17 us) and asks
+// the stream now and then whether it has failed.
+int wait_ticket(const unsigned long long* word, unsigned long long ticket, cudaStream_t s,
+                const char* what);
+
 // ---------------------------------------------------------------------------
 // Device helpers
 // ---------------------------------------------------------------------------

@@ -35,6 +35,10 @@ struct cg_segmented {
   float* rank_tmp = nullptr;     // [V] ping-pong for multi-iteration calls
   float* contrib_tmp = nullptr;  // [V]
   int64_t bytes = 0;
+  // where a pass's count of changed labels goes, and its ticket (lp_run, from its
+  // first call on)
+  mutable unsigned long long* pin = nullptr;
+  mutable unsigned long long ticket = 0;
 };
 
 // The plain pull baseline: the caller's CSR plus a merge-path tiling.

@@ -443,6 +443,7 @@ int build_impl(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,
 }
 
 void free_segmented(cg_segmented* g) {
+  if (g->pin) cudaFreeHost(g->pin);
   cudaFree(g->idx_map);
   seg_plan_free(&g->plan);
 }
