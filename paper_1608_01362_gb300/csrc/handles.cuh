@@ -60,13 +60,17 @@ struct cg_plain {
 };
 
 namespace cg {
-// Destinations per warp of the merge: the caller's B, halved (down to 32) while
-// the GPU would have fewer than 48 such warps per SM.  One warp's merge is a
-// chain of dependent reads, so a small graph's time is that chain: with B = 512
-// a 20,011-vertex graph merged on 5 of 152 SMs (11.0 us, 4.9 with 32), a
-// 1 M-vertex graph on 13 warps per SM (18.8 us, 11.7 with 128); from about 4 M
-// vertices on B stays.
-int32_t merge_block(int32_t V, int32_t B, int sm_count);
+// Destinations per warp of the merge: the most, up to the caller's B and in
+// steps of 32, with which the warps make whole waves of 40 per SM (5 blocks).  One
+// warp's merge is a chain of dependent reads, so a small graph's time is that
+// chain, and a last wave that is nearly empty costs as much as a full one.  With
+// B = 512: 20,011 vertices merged on 5 of 152 SMs (11.0 us, 4.9 so), 300 K in 1.3
+// waves of 48 (20 iterations with the gathers 770 us, 661 so), 1 M 1198 and 1098, 4
+// M 2869 and 2762, 33 M in 9 waves of 48 or 11 of 40 (17.70 ms both).  A block of
+// hubs has rows in every one of the k segments: where that makes more than 3000
+// for one warp, up to three waves share them out (label propagation, 3 M
+// vertices, 9 segments: 1236 us in one wave, 1130 in two).
+int32_t merge_block(int32_t V, int32_t B, int32_t k, int sm_count);
 
 // Validate an in-edge CSR on the device (offsets monotone from 0 to E, every
 // source in [0, V)).  Synchronizes the stream.

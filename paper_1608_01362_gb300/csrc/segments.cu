@@ -338,7 +338,7 @@ int build_impl(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,
   g->nb = (int32_t)ceil_div(V, B);
   DeviceInfo di{};
   CG_TRY(device_info(&di));
-  g->mB = merge_block(V, B, di.sm_count);
+  g->mB = merge_block(V, B, k, di.sm_count);
   g->mnb = (int32_t)ceil_div(V, g->mB);
   const size_t e4 = Scratch::round(4 * (size_t)E), kt = (size_t)k * ntiles;
   Scratch tmp(s, e4 + Scratch::round(4 * kt) + Scratch::round(8 * (kt + 1)) +
@@ -450,10 +450,14 @@ void free_segmented(cg_segmented* g) {
 
 }  // namespace
 
-int32_t merge_block(int32_t V, int32_t B, int sm_count) {
-  int32_t b = B;
-  while (b > 32 && ceil_div(V, b) < (int64_t)sm_count * 48) b = std::max(32, (b + 1) / 2);
-  return b;
+int32_t merge_block(int32_t V, int32_t B, int32_t k, int sm_count) {
+  const int64_t wave = (int64_t)sm_count * 40;
+  auto in_waves = [&](int64_t w) {
+    return std::min<int64_t>(B, ceil_div(ceil_div(V, w * wave), 32) * 32);
+  };
+  int64_t waves = ceil_div(ceil_div(V, B), wave);
+  while (waves < 3 && in_waves(waves) * k > 3000) ++waves;
+  return (int32_t)in_waves(waves);
 }
 
 int validate_csr(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,

@@ -1,4 +1,4 @@
-"""The merge's own block size (the caller's, halved while there are few warps)
+"""The merge's own block size (the caller's, or one that makes whole waves of warps)
 and the counters that a launch leaves cleared for the next one: exact against
 numpy, over sizes at the edges of a block and over every way to run a gather."""
 import numpy as np
