@@ -135,7 +135,7 @@ typedef struct {
   int64_t rows;          /* total subgraph rows = sum_s |dst(s)| = q V */
   double q;              /* expansion factor rows / V (Section III-D) */
   int64_t device_bytes;  /* device memory held by the handle */
-  int64_t gather_tiles;  /* 256-edge chunks of one segment-processing pass */
+  int64_t gather_tiles;  /* staged tasks and L1/L2 chunks of one segment-processing pass */
   int32_t table_vertices; /* shared-memory table entries per staged block */
   int32_t ctas_per_sm;   /* staged-gather blocks per SM */
   int32_t gather_threads; /* threads per staged-gather block */
@@ -160,7 +160,8 @@ typedef struct {
  * The handle also owns the intermediate buffers (intermBuf) and the tiling
  * of the gather.  Inputs: device CSR as in the conventions; 1 <= k <= 1024;
  * 1 <= merge_block <= 6144 (a merge block's accumulator lives in one warp's
- * share of shared memory; 512 is a good default).  The call synchronizes the stream (it reads
+ * share of shared memory; 512 is a good default; the GPU's merge takes smaller
+ * blocks where these fill it better, the export is in merge_block's).  The call synchronizes the stream (it reads
  * segment sizes on the host).  Errors: CG_ERR_INVALID_ARG, CG_ERR_OOM,
  * CG_ERR_CUDA.  Empty segments are legal.
  */
@@ -209,7 +210,7 @@ int pr_plan_bounds(const int32_t *dev_outdeg, int32_t V, int32_t smem_vertices,
  * segment's source values into shared memory and serves every read of the
  * segment from there.  The other segments are read through L1/L2 by a
  * second launch (1024 threads, 2 blocks per SM, no shared memory).  threads:
- * 512 or 1024; ctas_per_sm <= 1024/threads (the staged kernel holds 64
+ * 512 or 1024; ctas_per_sm <= 1024/threads (the staged kernel holds up to 64
  * registers per thread): 1 at 1024 threads, 1 or 2 at 512.  Results do not
  * depend on it; CG_ERR_INVALID_ARG otherwise (the previous shape stays).
  * Default after pr_build_segments: 1024, 1, -1.  Synchronizes the stream.
@@ -302,7 +303,7 @@ int cg_seg_gather_phases(const cg_segmented *seg, int32_t op, const void *dev_x,
 
 /*
  * Cache-aware merge alone (Algorithm 4, Section III-C): for each block of
- * merge_block destinations (one warp per block, its accumulator in shared
+ * at most merge_block destinations (one warp per block, its accumulator in shared
  * memory), out[v] = identity (0 / INT32_MAX), then for each segment in
  * ascending order, for its rows i in the block,
  * out[idx_map[i]] = op(out[idx_map[i]], interm[i]).  dev_interm: rows
@@ -452,8 +453,9 @@ typedef struct cg_batch cg_batch;
  * graph's vertex range, dev_offsets (device int64[V_total+1]) are global edge
  * offsets, dev_src (device int32[E_total]) holds sources LOCAL to their graph
  * (in [0, V_g)).  Every graph has 1..65536 vertices and must fit one block's
- * shared memory (CG_ERR_UNSUPPORTED otherwise).  The arrays are copied into
- * the handle (flagged edges, per-graph out-degrees); synchronizes.
+ * shared memory (CG_ERR_UNSUPPORTED otherwise); offsets must not decrease
+ * (CG_ERR_INVALID_ARG).  The arrays are copied into the handle (the staged edge
+ * stream, per-graph out-degrees); synchronizes.
  */
 int pr_batch_create(int32_t G, const int64_t *host_vbase, const int64_t *dev_offsets,
                     const int32_t *dev_src, cg_batch **out, cudaStream_t stream);
