@@ -327,6 +327,8 @@ int cf_pieces_build(CfPieces* c, int64_t n, int64_t R, int K, const int64_t* off
   c->poff = reinterpret_cast<int64_t*>(c->slab + rb + sb);
   c->gpart = reinterpret_cast<float*>(c->slab + rb + sb + pb);
   CG_CUDA(cudaMemcpyAsync(c->poff, poff, 8 * (size_t)(n + 1), cudaMemcpyDeviceToDevice, s));
+  // (an update before the first gather only decays the factors)
+  CG_CUDA(cudaMemsetAsync(c->gpart, 0, 4 * (size_t)nslots * K, s));
   if (np == 0) return CG_OK;
   CG_CUDA(tmp.get(&key, np));
   CG_CUDA(tmp.get(&skey, np));

@@ -91,3 +91,24 @@ def test_sweep_within_bound(C, ratings, K, precision, ascending):
     s64 = O.cf_sweep_bound(U, I, off, item, three, ioff, iuser, three, P, Q, LAM, STEP,
                            u_store=u_store)
     assert abs(float(sse.item()) - s64[2]) <= s64[5]
+
+
+def test_update_before_a_gather_only_decays(C, ratings):
+    import torch
+    U, I, off, item, rate = ratings
+    d = _item_major(C, U, I, off, item, rate)
+    rng = np.random.default_rng(1)
+    P0, Q0 = (rng.random((n, 32)).astype(np.float32) for n in (U, I))
+    Pg, Qg = torch.empty((U, 32), device="cuda"), torch.empty((I, 32), device="cuda")
+    for sweeps in (3, 0):  # the second handle may get the memory that the first one used
+        h = C.cf_create(U, I, 32, 0, *d)
+        C.cf_set_factors(h, torch.as_tensor(P0).cuda(), torch.as_tensor(Q0).cuda())
+        if sweeps:
+            C.cf_sweep(h, sweeps, LAM, STEP)
+            del h
+    C.cf_sweep_phase(h, 2, LAM, STEP)
+    C.cf_sweep_phase(h, 3, LAM, STEP)
+    C.cf_get_factors(h, Pg, Qg)
+    for got, x in ((Pg, P0), (Qg, Q0)):  # two products and a sum, rounded in FP32
+        want = x.astype(np.float64) * (1.0 - STEP * LAM)
+        assert np.all(np.abs(got.cpu().numpy() - want) <= 4 * 2.0 ** -24 * x)
