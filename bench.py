@@ -134,7 +134,8 @@ class ClockSampler:
                 "samples": len(self.rows)}
 
 
-KERNEL_SOURCES = ("seg_gather.cu", "seg_gather.cuh", "pagerank.cu", "update.cuh", "gather.cuh")
+KERNEL_SOURCES = ("seg_gather.cu", "seg_gather.cuh", "staged_stream.cuh", "staged_build.cu",
+                  "ranges.cuh", "carry_runs.cuh", "pagerank.cu", "update.cuh", "gather.cuh")
 
 
 def kernel_source_hash():
