@@ -416,10 +416,14 @@ overlap_gather_kernel(StagedTasks q, StagedShare sh, const uint32_t* __restrict_
   counters_done(next_chunk, 4 + (int)gridDim.x, sh.done);  // the ranges' lie behind it
 }
 
-// Block b's first task: equal stretches of the stream.
+// Block b's first task: equal stretches of the stream (no tasks: empty shares).
 __global__ void staged_share_kernel(const uint4* __restrict__ desc, int32_t ntasks, int grid,
                                     int32_t* __restrict__ blk_task) {
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b <= grid; b += gridDim.x * blockDim.x) {
+    if (ntasks == 0) {
+      blk_task[b] = 0;
+      continue;
+    }
     const uint4 e = desc[ntasks - 1];
     const int64_t total = (int64_t)e.x + (e.y >> 16);
     const int64_t want = total * b / grid;
@@ -486,7 +490,7 @@ int seg_plan_alloc(int64_t E, int k, const std::vector<int64_t>& edge_base,
   p->seg_task = w + 4 * n;
   p->counter = reinterpret_cast<unsigned*>(w + 5 * n);
   p->blk_task = w + 5 * n + 4 + most;
-  CG_CUDA(cudaMemsetAsync(p->counter, 0, 4 * (4 + most), s));
+  CG_CUDA(cudaMemsetAsync(p->counter, 0, 4 * ((4 + most) + (most + 1)), s));  // and the shares
   std::vector<int64_t> up(4 * n, 0);  // edge_base, cstart, bounds, then seg_E and seg_lo
   int32_t* eo = reinterpret_cast<int32_t*>(up.data() + 3 * n);
   for (size_t q = 0; q < n; ++q) {
@@ -576,15 +580,12 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
       ++m2;
     }
   }
-  // one overlapped launch needs both kinds of segment and the 1024 x 1 shape
-  bool cached_edges = false;
-  for (int q = m2; q < k; ++q) cached_edges |= p->edge_base[q + 1] > p->edge_base[q];
+  // one overlapped launch needs the 1024 x 1 shape
   if (p->overlap_request > 0 && (threads != 1024 || ctas_per_sm != 1)) {
     set_error("gather overlap needs 1024 threads and 1 block per SM (got %d x %d)", threads,
               ctas_per_sm);
     return CG_ERR_INVALID_ARG;
   }
-  p->overlap = (m > 0 && cached_edges) ? p->overlap_request : 0;
   const int warps_b = 1024 / 32;
   const int tab_cap = (int)((tabmax + 3) & ~3LL);
   // chunks of the segments read through L1/L2
@@ -634,14 +635,15 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   // the staged launch: one block per resident slot, or per task where there are fewer
   // (every SM serves the L1/L2 queue too in an overlapped launch)
   const int32_t head = p->h_seg_task[m];
+  // one overlapped launch needs tasks of both kinds (staged segments can all be
+  // empty: they have no tasks, and the blocks no shares)
+  p->overlap = (head > 0 && cached > 0) ? p->overlap_request : 0;
   p->grid = (int)std::max<int64_t>(1, std::min<int64_t>(head, (int64_t)di.sm_count * ctas_per_sm));
   if (p->overlap > 0) p->grid = di.sm_count;
   p->head_tasks = head;
-  if (head > 0) {
-    staged_share_kernel<<<grid_for(p->grid + 1, 128), 128, 0, s>>>(p->desc, head, p->grid,
-                                                                   p->blk_task);
-    CG_LAUNCH_CHECK();
-  }
+  staged_share_kernel<<<grid_for(p->grid + 1, 128), 128, 0, s>>>(p->desc, head, p->grid,
+                                                                 p->blk_task);
+  CG_LAUNCH_CHECK();
   p->grid_l2 = (int)std::max<int64_t>(
       1, std::min<int64_t>(p->n_ctiles, (int64_t)di.sm_count * 2));
   CG_CUDA(cudaStreamSynchronize(s));
