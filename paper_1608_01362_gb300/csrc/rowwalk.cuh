@@ -53,7 +53,8 @@ struct RowWalk {
     const int lane = threadIdx.x & 31;
     int32_t lo = 0, hi = n;  // row lo begins at or before e, row hi behind it
     while (hi - lo > 1) {
-      const int32_t step = (hi - lo + 32) / 33;  // probes lo + step, lo + 2 step, ...
+      // probes lo + step, lo + 2 step, ... (unsigned: hi - lo goes up to 2^31 - 1)
+      const int32_t step = (int32_t)(((uint32_t)(hi - lo) + 32u) / 33u);
       const int64_t p = (int64_t)lo + (int64_t)step * (lane + 1);
       const bool le = p < hi && (int32_t)(__ldg(off + p) - origin) <= e;
       const int c = __popc(__ballot_sync(0xffffffffu, le));
