@@ -65,8 +65,10 @@ __global__ void relabel_len_kernel(const int64_t* __restrict__ offsets,
 // and reads its source at the same place of the old row.  Bound by the random
 // 4-byte reads of new_of_old (L2 sectors).  65.2 M edges: 2.49 ms with a warp
 // per row (15 edges a row, most lanes idle) -> 0.43 ms.
+// (PosT: int64 where there are 2^31 edges and more.)
 constexpr int kRelabelTile = 1024;
 
+template <typename PosT>
 __global__ void __launch_bounds__(256)
 relabel_copy_kernel(const int64_t* __restrict__ offsets, const int32_t* __restrict__ src,
                     const int32_t* __restrict__ new_of_old,
@@ -76,18 +78,18 @@ relabel_copy_kernel(const int64_t* __restrict__ offsets, const int32_t* __restri
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t n = min(E, out_offsets[V]);  // an old_of_new that is no permutation
-  RowWalk<int64_t> walk(out_offsets, V, (int32_t)out_offsets[V]);
+  RowWalk<int64_t, PosT> walk(out_offsets, V, (PosT)n);
   for (int64_t b = ((((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5)) * kRelabelTile; b < n;
        b += nw * kRelabelTile) {
-    walk.seek((int32_t)b);
+    walk.seek((PosT)b);
     for (int i = 0; i < kRelabelTile && b + i < n; i += 32 * U) {
       int64_t at[U];
       int32_t u[U];
 #pragma unroll
       for (int j = 0; j < U; ++j) {
         const int64_t e = b + i + 32 * j + lane;
-        int32_t st, en;
-        const int32_t r = walk.row_of((int32_t)e, e < n, &st, &en);
+        PosT st, en;
+        const int32_t r = walk.row_of((PosT)e, e < n, &st, &en);
         at[j] = -1;
         if (e < n) {
           const int64_t o = __ldg(old_of_new + r);  // in [0, V): its row is not empty
@@ -235,7 +237,8 @@ int cg_relabel_csr(const int64_t* offsets, const int32_t* src, int32_t V, int64_
   CG_LAUNCH_CHECK();
   CG_TRY(exclusive_scan_i64(len, out_offsets, V, stream, &tmp));
   if (E > 0) {
-    relabel_copy_kernel<<<grid_for(ceil_div(E, kRelabelTile) * 32, 256), 256, 0, stream>>>(
+    auto fn = E < 0x7FFFFFFFLL ? relabel_copy_kernel<int32_t> : relabel_copy_kernel<int64_t>;
+    fn<<<grid_for(ceil_div(E, kRelabelTile) * 32, 256), 256, 0, stream>>>(
         offsets, src, new_of_old, old_of_new, V, E, out_offsets, out_src);
     CG_LAUNCH_CHECK();
   }

@@ -15,23 +15,26 @@
 
 namespace cg {
 
-// At most 2^31 - 1 edges; OffT is the stored offset type.
-template <typename OffT>
+// OffT is the stored offset type, PosT holds an edge's place: 32 bits below 2^31
+// edges (rows that begin behind the last edge walked are taken to begin there).
+template <typename OffT, typename PosT = int32_t>
 struct RowWalk {
   const OffT* off;  // off[r] - origin: first edge of row r < n
   int32_t n;        // rows
-  int32_t total;    // edges, the end of row n - 1
-  int32_t origin;
+  PosT total;       // edges walked, the end of row n - 1
+  PosT origin;
   int32_t r0;       // first row of the window
-  int32_t start;    // its first edge
-  int32_t end;      // this lane's row end: that of row r0 + lane (the total past row n - 1)
-  int32_t ahead;    // the same of the next 32 rows, read ahead
+  PosT start;       // its first edge
+  PosT end;         // this lane's row end: that of row r0 + lane (the total past row n - 1)
+  PosT ahead;       // the same of the next 32 rows, read ahead
 
-  __device__ __forceinline__ RowWalk(const OffT* o, int32_t rows, int32_t edges, int32_t org = 0)
+  __device__ __forceinline__ RowWalk(const OffT* o, int32_t rows, PosT edges, PosT org = 0)
       : off(o), n(rows), total(edges), origin(org), r0(0), start(0), end(0), ahead(0) {}
 
-  __device__ __forceinline__ int32_t first_of(int64_t r) const {
-    return r < n ? (int32_t)(__ldg(off + r) - origin) : total;
+  __device__ __forceinline__ PosT first_of(int64_t r) const {
+    if (r >= n) return total;
+    const OffT at = __ldg(off + r) - (OffT)origin;
+    return at < (OffT)total ? (PosT)at : total;
   }
   __device__ __forceinline__ void window(int32_t r) {
     const int lane = threadIdx.x & 31;
@@ -49,14 +52,14 @@ struct RowWalk {
   }
 
   // window at the row of edge e (uniform in the warp): the last r with off[r] <= e
-  __device__ __forceinline__ void seek(int32_t e) {
+  __device__ __forceinline__ void seek(PosT e) {
     const int lane = threadIdx.x & 31;
     int32_t lo = 0, hi = n;  // row lo begins at or before e, row hi behind it
     while (hi - lo > 1) {
       // probes lo + step, lo + 2 step, ... (unsigned: hi - lo goes up to 2^31 - 1)
       const int32_t step = (int32_t)(((uint32_t)(hi - lo) + 32u) / 33u);
       const int64_t p = (int64_t)lo + (int64_t)step * (lane + 1);
-      const bool le = p < hi && (int32_t)(__ldg(off + p) - origin) <= e;
+      const bool le = p < hi && __ldg(off + p) - (OffT)origin <= (OffT)e;
       const int c = __popc(__ballot_sync(0xffffffffu, le));
       const int64_t nh = (int64_t)lo + (int64_t)step * (c + 1);
       lo += step * c;
@@ -67,14 +70,14 @@ struct RowWalk {
 
   // Row of this lane's edge e, the row's first edge and its end; lanes' edges
   // ascend with the lane, ok tells which lanes have one (a prefix of the warp).
-  __device__ __forceinline__ int32_t row_of(int32_t e, bool ok, int32_t* row_start,
-                                            int32_t* row_end) {
+  __device__ __forceinline__ int32_t row_of(PosT e, bool ok, PosT* row_start, PosT* row_end) {
     const unsigned full = 0xffffffffu;
-    int32_t row = 0, st = 0, en = 0;
+    int32_t row = 0;
+    PosT st = 0, en = 0;
     unsigned todo = __ballot_sync(full, ok);
     while (todo) {
       const int first = __ffs(todo) - 1;
-      const int32_t ef = __shfl_sync(full, e, first);
+      const PosT ef = __shfl_sync(full, e, first);
       if (ef >= __shfl_sync(full, end, 31)) {  // past the window
         advance();
         if (ef >= __shfl_sync(full, end, 31)) seek(ef);
@@ -84,8 +87,8 @@ struct RowWalk {
       for (int s = 16; s; s >>= 1)
         if (__shfl_sync(full, end, j + s - 1) <= e) j += s;
       // j = 31 may also mean that all 32 end before e
-      const int32_t ej = __shfl_sync(full, end, j);
-      const int32_t sj = __shfl_sync(full, end, j > 0 ? j - 1 : 0);
+      const PosT ej = __shfl_sync(full, end, j);
+      const PosT sj = __shfl_sync(full, end, j > 0 ? j - 1 : 0);
       const bool mine = ((todo >> (threadIdx.x & 31)) & 1u) && e < ej;
       if (mine) {
         row = r0 + j;
