@@ -5,20 +5,40 @@ namespace cg {
 namespace {
 
 // Out-degree by counting sources, one reduction per edge: bound by the L2's
-// atomics (65.2 M edges: 390 us; combining equal sources of a warp with
-// match_any first took 495 us, they are too rare to pay for it).
+// atomics.  A warp combines the equal ones of 32 edges first (match_any) while it
+// meets any: it looks at the first of every four batches, and combines the
+// batches of four looks in a row from one that had equal sources on.  65 M edges:
+// RMAT 382 us (511 combining always, 378 never), one source in every edge 1337
+// (1337, 41,760), in every 16th 1645 (1653, 2846), sources V x^6 3694 (3680, 5758).
 __global__ void __launch_bounds__(256)
 out_degree_kernel(const int32_t* __restrict__ src, int64_t E, int32_t V,
                   int32_t* __restrict__ outdeg) {
-  constexpr int U = 4;
+  constexpr int U = 4, kLooks = 4;
+  constexpr unsigned kFull = 0xffffffffu;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += stride * U) {
+  const int lane = threadIdx.x & 31;
+  int left = 0;  // looks whose batches are still combined
+  // (base is that of lane 0: the warp stays together)
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < E;
+       base += stride * U) {
     int32_t u[U];
 #pragma unroll
-    for (int j = 0; j < U; ++j) u[j] = e + j * stride < E ? __ldcs(src + e + j * stride) : -1;
+    for (int j = 0; j < U; ++j) {
+      const int64_t e = base + lane + j * stride;
+      u[j] = e < E ? __ldcs(src + e) : -1;
+      if (u[j] >= V) u[j] = -1;  // out of range: ignored
+    }
 #pragma unroll
-    for (int j = 0; j < U; ++j)
-      if (u[j] >= 0 && u[j] < V) atomicAdd(outdeg + u[j], 1);  // others are ignored
+    for (int j = 0; j < U; ++j) {
+      if (j == 0 || left > 0) {
+        const unsigned peers =
+            __match_any_sync(kFull, u[j] >= 0 ? (unsigned)u[j] : (0x80000000u | (unsigned)lane));
+        if (j == 0) left = __any_sync(kFull, peers & (peers - 1)) ? kLooks : max(left - 1, 0);
+        if (u[j] >= 0 && lane == __ffs(peers) - 1) atomicAdd(outdeg + u[j], __popc(peers));
+      } else if (u[j] >= 0) {
+        atomicAdd(outdeg + u[j], 1);
+      }
+    }
   }
 }
 
