@@ -111,7 +111,7 @@ cf_rows_kernel(const int4* __restrict__ recs, int32_t ntasks, int32_t nn,
   const char* mine = static_cast<const char*>(self) + sub * kPart;
   const char* rows = static_cast<const char*>(other) + sub * kPart;
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  float se = 0.0f, sc = 0.0f;  // squared errors and what their FP32 sum has dropped
+  double se = 0.0;  // squared errors: FP32 within a piece, FP64 over the pieces
   for (int32_t task = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); task < ntasks;
        task += nw) {
     const int64_t slot = (int64_t)task * G + grp;
@@ -189,16 +189,12 @@ cf_rows_kernel(const int4* __restrict__ recs, int32_t ntasks, int32_t nn,
       for (int q = 0; q < NP; q += 2)
         __stcs(reinterpret_cast<ulonglong2*>(dst + 2 * q), make_ulonglong2(g[q], g[q + 1]));
     }
-    if (SSE) {  // compensated: the lane's sum runs over many pieces
-      const float a = se + te2, z = a - se;
-      sc += (se - (a - z)) + (te2 - z);
-      se = a;
-    }
+    if (SSE) se += (double)te2;
   }
   if (!SSE) return;
   __shared__ double sh[32];
   __shared__ bool s_last;
-  const double bs = block_sum<double, kRowThreads>((double)se + (double)sc, sh);
+  const double bs = block_sum<double, kRowThreads>(se, sh);
   if (threadIdx.x == 0) {
     partials[blockIdx.x] = bs;
     __threadfence();
