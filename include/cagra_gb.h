@@ -19,8 +19,11 @@
  *    on the host before anything is enqueued; on error nothing is enqueued
  *    and cg_last_error_message() (thread-local) explains.  Calls that must
  *    read a device result on the host (noted below) synchronize the stream.
- *  - No entry point spins on device flags; a kernel waits on another only for its
- *    end, in stream order.
+ *  - No kernel waits on a flag: one kernel waits on another only for its end, in
+ *    stream order.  The host does in two calls, lp_run (once per pass) and
+ *    bc_run (once per level): it polls a pinned word that a kernel on the
+ *    stream writes (asleep in between when that takes more than 5 ms), and the
+ *    call returns an error if the stream fails.
  *  - Handles are bound to the device that was current when they were built;
  *    use them with that device current.
  */

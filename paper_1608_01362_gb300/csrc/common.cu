@@ -1,7 +1,9 @@
 // Host-side helpers: status strings, thread-local error text, device info.
 #include <stdarg.h>
 
+#include <chrono>
 #include <mutex>
+#include <thread>
 
 #include "common.cuh"
 
@@ -67,18 +69,23 @@ int grid_for(int64_t n, int threads, int per_sm) {
 
 int wait_ticket(const unsigned long long* word, unsigned long long ticket, cudaStream_t s,
                 const char* what) {
-  for (int spins = 1; __atomic_load_n(word, __ATOMIC_ACQUIRE) != ticket; ++spins) {
+  using clock = std::chrono::steady_clock;
+  const clock::time_point start = clock::now();
+  for (unsigned spins = 1;; ++spins) {
+    if (__atomic_load_n(word, __ATOMIC_ACQUIRE) == ticket) return CG_OK;
     if (spins % 4096) continue;
     const cudaError_t e = cudaStreamQuery(s);
-    if (e != cudaErrorNotReady && e != cudaSuccess) return cuda_fail(e, what, __FILE__, __LINE__);
     if (e == cudaSuccess) {  // all done: the word is there, or will never be
-      CG_CUDA(cudaStreamSynchronize(s));
-      if (__atomic_load_n(word, __ATOMIC_ACQUIRE) == ticket) break;
+      if (__atomic_load_n(word, __ATOMIC_ACQUIRE) == ticket) return CG_OK;
       set_error("%s: a result did not reach the host", what);
       return CG_ERR_CUDA;
     }
+    if (e != cudaErrorNotReady) return cuda_fail(e, what, __FILE__, __LINE__);
+    // a long wait (other work in front of it on the stream) leaves the core to
+    // others: from 5 ms on, sleeps of a 64th of the time waited so far
+    const clock::duration waited = clock::now() - start;
+    if (waited > std::chrono::milliseconds(5)) std::this_thread::sleep_for(waited / 64);
   }
-  return CG_OK;
 }
 
 }  // namespace cg

@@ -154,8 +154,9 @@ int launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t
 }
 
 // Waits until a kernel on the stream has written the ticket to a pinned word:
-// the host watches the word (a copy and a synchronisation take 17 us) and asks
-// the stream now and then whether it has failed.
+// the host watches the word (a copy and a synchronisation take 17 us), asks the
+// stream now and then whether it has failed, and sleeps in between when the wait
+// gets long.
 int wait_ticket(const unsigned long long* word, unsigned long long ticket, cudaStream_t s,
                 const char* what);
 
