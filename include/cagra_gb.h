@@ -198,7 +198,8 @@ int cg_segmented_stats(const cg_segmented *seg, int64_t *q_rows_total, double *q
  * source values as fill half of this GPU's L2, from its device properties).
  * dev_outdeg: int32[V]
  * of the (clustered) graph.  Writes k+1 bounds to host_bounds (capacity
- * k_max+1) and k to *k_out.  Synchronizes (reads the degrees on the host).
+ * k_max+1) and k to *k_out, 1 <= k <= k_max.  Synchronizes (reads sums of the
+ * degrees on the host).
  */
 int pr_plan_bounds(const int32_t *dev_outdeg, int32_t V, int32_t smem_vertices,
                    double min_avg_degree, int32_t max_global_vertices,

@@ -648,7 +648,11 @@ int pr_plan_bounds(const int32_t* dev_outdeg, int32_t V, int32_t smem_vertices,
     const int64_t end = std::max(lo, sums[nr]);
     const int64_t left_k = k_max - ((int64_t)b.size() - 1) - (end < V && end > lo ? 1 : 0);
     if (left_k < 1) {
-      b.back() = V;  // no room: the last shared-memory segment absorbs the rest
+      // no room: the last shared-memory segment absorbs the rest
+      if (b.size() > 1)
+        b.back() = V;
+      else
+        b.push_back(V);  // (there is none)
     } else {
       if (end > lo) {
         int64_t parts = std::max<int64_t>(1, ceil_div(end - lo, max_global_vertices));

@@ -1,0 +1,21 @@
+"""Segment plans with room for few segments: always a partition of [0, V) in 1 to
+k_max segments."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("k_max", [1, 2, 3, 4])
+@pytest.mark.parametrize("V", [1, 2, 33, 5000])
+@pytest.mark.parametrize("smem", [0, 16, 600])
+def test_plan_is_a_partition(V, smem, k_max):
+    import torch
+    from paper_1608_01362_gb300 import cagra as C
+    rng = np.random.default_rng(V)
+    deg = np.sort(rng.integers(0, 40, V))[::-1].astype(np.int32).copy()
+    for tail in (0, 1, V // 3, V):
+        deg[V - tail:] = 0
+        b = C.pr_plan_bounds(torch.as_tensor(deg).cuda(), smem, 10.0, 100, k_max)
+        assert 1 <= len(b) - 1 <= k_max, b
+        assert b[0] == 0 and b[-1] == V and np.all(np.diff(b) >= 0), b
