@@ -456,9 +456,10 @@ typedef struct cg_batch cg_batch;
  * in-edge CSR -- host_vbase (host int64[G+1], vbase[0] = 0) gives each
  * graph's vertex range, dev_offsets (device int64[V_total+1]) are global edge
  * offsets, dev_src (device int32[E_total]) holds sources LOCAL to their graph
- * (in [0, V_g)).  Every graph has 1..65536 vertices and must fit one block's
- * shared memory (CG_ERR_UNSUPPORTED otherwise); offsets must not decrease
- * (CG_ERR_INVALID_ARG).  The arrays are copied into the handle (the staged edge
+ * (in [0, V_g)).  Every graph has 1..65536 vertices, must fit one block's
+ * shared memory and has fewer than 2^31 - 1 edges (CG_ERR_UNSUPPORTED
+ * otherwise); the batch as a whole may have more, and any number of graphs.
+ * Offsets must not decrease (CG_ERR_INVALID_ARG).  The arrays are copied into the handle (the staged edge
  * stream, per-graph out-degrees); synchronizes.
  */
 int pr_batch_create(int32_t G, const int64_t *host_vbase, const int64_t *dev_offsets,
@@ -469,13 +470,14 @@ int pr_batch_destroy(cg_batch *batch);
 int pr_batch_set_threads(cg_batch *batch, int32_t threads);
 
 /*
- * PageRank of every graph of the batch in ONE persistent launch: r_0 = 1/V_g,
+ * PageRank of every graph of the batch in ONE persistent launch (one per 2^18
+ * graphs, 2^30 vertices or 2^30 edges): r_0 = 1/V_g,
  * `iterations` normalised iterations with uniform dangling redistribution
  * (the same arithmetic as pr_iterate on each graph alone).  Graphs are taken
  * largest first by an atomic counter; a block runs all iterations of its
  * graph on chip.  dev_rank: float[V_total] receives the ranks (graph g's at
  * vbase[g]); dev_resid: double[G*iterations] (graph-major) or NULL.  Stream-
- * ordered and capturable in a CUDA graph (a memset and one kernel).
+ * ordered and capturable in a CUDA graph (a memset and a kernel per launch).
  */
 int pr_batch_run(cg_batch *batch, int32_t iterations, double damping, float *dev_rank,
                  double *dev_resid, cudaStream_t stream);

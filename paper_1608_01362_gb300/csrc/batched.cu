@@ -27,14 +27,16 @@
 
 #include "staged_stream.cuh"
 
-struct cg_batch {
-  int device = 0;
+namespace cg {
+
+// Consecutive graphs that are laid out and launched together.
+struct BatchPart {
   int32_t G = 0;
+  int64_t g0 = 0, v0 = 0, e0 = 0;  // first graph, vertex and edge
   int64_t V = 0, E = 0, rows = 0;
   int32_t vmax = 0;
-  std::vector<int64_t> h_vbase, h_ebase;
-  cg::SegPlan plan;           // the graphs as staged segments: tasks, stream, carries
-  int64_t* vbase = nullptr;   // [G+1] first vertex of each graph
+  SegPlan plan;               // the graphs as staged segments: tasks, stream, carries
+  int64_t* vbase = nullptr;   // [G+1] first vertex of each graph (from v0 on)
   int32_t* order = nullptr;   // [G] graphs by edge count, descending
   int32_t* ndang = nullptr;   // [G]
   int32_t* xbase = nullptr;   // [G+1] first carry of each graph
@@ -43,6 +45,23 @@ struct cg_batch {
   float* inv = nullptr;       // [V]
   float* sums = nullptr;      // [V] row sums of graphs too large to keep them on chip
   unsigned* counter = nullptr;
+  int64_t bytes = 0;
+};
+
+// A part ends before it has more than this many graphs, vertices or edges (a
+// graph of more edges has one to itself): its places then fit 32 bits, and the
+// scratch of its build, 4 KB per graph, stays below 1 GB.  A batch within one part
+// is one launch.
+constexpr int64_t kPartGraphs = (int64_t)1 << 18;
+constexpr int64_t kPartVertices = (int64_t)1 << 30;
+constexpr int64_t kPartEdges = (int64_t)1 << 30;
+
+}  // namespace cg
+
+struct cg_batch {
+  int device = 0;
+  int32_t G = 0;
+  std::vector<cg::BatchPart> parts;
   int threads = 1024;
   int64_t bytes = 0;
 };
@@ -50,6 +69,17 @@ struct cg_batch {
 namespace cg {
 namespace {
 
+// The edge offsets at the graphs' first vertices.
+__global__ void batch_ebase_kernel(const int64_t* __restrict__ offsets,
+                                   const int64_t* __restrict__ vbase, int G,
+                                   int64_t* __restrict__ ebase) {
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g <= G;
+       g += (int64_t)gridDim.x * blockDim.x)
+    ebase[g] = offsets[vbase[g]];
+}
+
+// (Offsets, sources and bases below are those of a part: vertices and edges are
+// counted from its first ones, offsets from its first edge, e0, on.)
 __global__ void batch_degree_kernel(const int32_t* __restrict__ src, const int64_t* __restrict__ ebase,
                                     const int64_t* __restrict__ vbase, int G, int64_t E,
                                     int32_t* __restrict__ outdeg) {
@@ -84,13 +114,14 @@ __global__ void batch_rows_kernel(const int64_t* __restrict__ offsets,
                                   const int64_t* __restrict__ rowpos,  // exclusive scan of nonempty
                                   const int64_t* __restrict__ vbase,
                                   const int64_t* __restrict__ ebase,
-                                  const int64_t* __restrict__ cstart, int G, int64_t V, int pad,
+                                  const int64_t* __restrict__ cstart, int G, int64_t V, int64_t e0,
+                                  int pad,
                                   uint32_t* __restrict__ colf, int32_t* __restrict__ row_ptr,
                                   int32_t* __restrict__ idx) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < V; v += nw) {
-    const int64_t lo = offsets[v], hi = offsets[v + 1];
+    const int64_t lo = offsets[v] - e0, hi = offsets[v + 1] - e0;
     if (hi <= lo) continue;
     int a = 0, b = G + 1;
     while (a < b) {
@@ -276,7 +307,7 @@ batch_pagerank_kernel(BatchArgs a) {
   }
 }
 
-void free_batch(cg_batch* b) {
+void free_part(BatchPart* b) {
   seg_plan_free(&b->plan);
   cudaFree(b->vbase);
   cudaFree(b->order);
@@ -289,6 +320,10 @@ void free_batch(cg_batch* b) {
   cudaFree(b->counter);
 }
 
+void free_batch(cg_batch* b) {
+  for (BatchPart& p : b->parts) free_part(&p);
+}
+
 // row_base[g] = first non-empty row of graph g.
 __global__ void batch_row_base_kernel(const int64_t* __restrict__ rowpos,
                                       const int64_t* __restrict__ vbase, int G,
@@ -298,35 +333,22 @@ __global__ void batch_row_base_kernel(const int64_t* __restrict__ rowpos,
 }
 
 // the entry behind the largest contrib vector that holds the sum's identity
-int batch_pad(const cg_batch* b) { return (b->vmax + 3) & ~3; }
+int batch_pad(const BatchPart& b) { return (b.vmax + 3) & ~3; }
 
-int build_batch(cg_batch* b, const int64_t* offsets, const int32_t* src, cudaStream_t s) {
+// Lays out one part (its G, g0, v0, e0, V, E and vmax are set); vbase and ebase:
+// its graphs' first vertices and edges, counted from its own first ones.
+int build_part(BatchPart* b, const std::vector<int64_t>& vbase, const std::vector<int64_t>& ebase,
+               const int64_t* offsets, const int32_t* src, cudaStream_t s) {
   const int G = b->G;
-  // per-graph edge bases from the offsets (host reads G+1 values)
-  b->h_ebase.assign(G + 1, 0);
-  for (int g = 0; g <= G; ++g)
-    CG_CUDA(cudaMemcpyAsync(&b->h_ebase[g], offsets + b->h_vbase[g], sizeof(int64_t),
-                            cudaMemcpyDeviceToHost, s));
-  CG_CUDA(cudaStreamSynchronize(s));
-  if (b->h_ebase[0] != 0) {
-    set_error("pr_batch_create: offsets must start at 0");
-    return CG_ERR_INVALID_ARG;
-  }
-  for (int g = 0; g < G; ++g)
-    if (b->h_ebase[g + 1] < b->h_ebase[g]) {
-      set_error("pr_batch_create: offsets decrease across graph %d", g);
-      return CG_ERR_INVALID_ARG;
-    }
-  b->E = b->h_ebase[G];
   std::vector<int32_t> order(G);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-    return b->h_ebase[x + 1] - b->h_ebase[x] > b->h_ebase[y + 1] - b->h_ebase[y];
+    return ebase[x + 1] - ebase[x] > ebase[y + 1] - ebase[y];
   });
   const int64_t V = b->V, E = b->E;
-  CG_TRY(seg_plan_alloc(E, G, b->h_ebase, b->h_vbase, &b->plan, s));
+  CG_TRY(seg_plan_alloc(E, G, ebase, vbase, &b->plan, s));
   SegPlan* p = &b->plan;
-  const int64_t* ebase = p->meta + (G + 1);
+  const int64_t* d_ebase = p->meta + (G + 1);
   const int64_t* cstart = p->meta + 2 * (G + 1);
   CG_CUDA(cudaMalloc((void**)&b->vbase, sizeof(int64_t) * (G + 1)));
   CG_CUDA(cudaMalloc((void**)&b->order, sizeof(int32_t) * G));
@@ -335,7 +357,7 @@ int build_batch(cg_batch* b, const int64_t* offsets, const int32_t* src, cudaStr
   CG_CUDA(cudaMalloc((void**)&b->inv, sizeof(float) * (size_t)V));
   CG_CUDA(cudaMalloc((void**)&b->sums, sizeof(float) * (size_t)V));
   CG_CUDA(cudaMalloc((void**)&b->counter, sizeof(unsigned)));
-  CG_CUDA(cudaMemcpyAsync(b->vbase, b->h_vbase.data(), sizeof(int64_t) * (G + 1),
+  CG_CUDA(cudaMemcpyAsync(b->vbase, vbase.data(), sizeof(int64_t) * (G + 1),
                           cudaMemcpyHostToDevice, s));
   CG_CUDA(cudaMemcpyAsync(b->order, order.data(), sizeof(int32_t) * G, cudaMemcpyHostToDevice, s));
   // scratch: out-degree, non-empty flags and their scan
@@ -351,7 +373,7 @@ int build_batch(cg_batch* b, const int64_t* offsets, const int32_t* src, cudaStr
   CG_CUDA(cudaMemsetAsync(bad, 0, sizeof(int32_t), s));
   CG_CUDA(cudaMemsetAsync(outdeg, 0, sizeof(int32_t) * (size_t)V, s));
   if (E > 0) {
-    batch_degree_kernel<<<grid_for(E, 256), 256, 0, s>>>(src, ebase, b->vbase, G, E, outdeg);
+    batch_degree_kernel<<<grid_for(E, 256), 256, 0, s>>>(src, d_ebase, b->vbase, G, E, outdeg);
     CG_LAUNCH_CHECK();
   }
   batch_inv_kernel<<<grid_for(V, 256), 256, 0, s>>>(outdeg, V, b->inv, offsets, nonempty, bad);
@@ -377,13 +399,13 @@ int build_batch(cg_batch* b, const int64_t* offsets, const int32_t* src, cudaStr
   const int32_t end = (int32_t)E;
   CG_CUDA(cudaMemcpyAsync(b->row_ptr + b->rows, &end, sizeof(int32_t), cudaMemcpyHostToDevice, s));
   batch_rows_kernel<<<grid_for(V * 32, 256, 16), 256, 0, s>>>(
-      offsets, src, rowpos, b->vbase, ebase, cstart, G, V, batch_pad(b), p->colf, b->row_ptr,
-      b->idx);
+      offsets, src, rowpos, b->vbase, d_ebase, cstart, G, V, b->e0, batch_pad(*b), p->colf,
+      b->row_ptr, b->idx);
   CG_LAUNCH_CHECK();
   p->rows = b->rows;
   p->rp32 = b->row_ptr;
   p->row_base = rbase;
-  CG_TRY(staged_build(p, G, batch_pad(b), 0, s, b->idx));
+  CG_TRY(staged_build(p, G, batch_pad(*b), 0, s, b->idx));
   batch_xbase_kernel<<<grid_for(G + 1, 256), 256, 0, s>>>(p->carry_row, p->ncarry, p->meta, G,
                                                           b->xbase);
   CG_LAUNCH_CHECK();
@@ -393,6 +415,109 @@ int build_batch(cg_batch* b, const int64_t* offsets, const int32_t* src, cudaStr
   p->colf = nullptr;
   p->colf_len = 0;
   b->bytes = seg_plan_bytes(*p) + 8 * V + 8 * (b->rows + 1) + 20 * (int64_t)(G + 1);
+  return CG_OK;
+}
+
+int build_batch(cg_batch* b, const int64_t* vbase, const int64_t* offsets, const int32_t* src,
+                cudaStream_t s) {
+  const int G = b->G;
+  std::vector<int64_t> ebase(G + 1, 0);
+  {
+    Scratch tmp(s, 2 * Scratch::round(8 * (size_t)(G + 1)));
+    int64_t *d_v = nullptr, *d_e = nullptr;
+    CG_CUDA(tmp.get(&d_v, G + 1));
+    CG_CUDA(tmp.get(&d_e, G + 1));
+    CG_CUDA(cudaMemcpyAsync(d_v, vbase, sizeof(int64_t) * (G + 1), cudaMemcpyHostToDevice, s));
+    batch_ebase_kernel<<<grid_for(G + 1, 256), 256, 0, s>>>(offsets, d_v, G, d_e);
+    CG_LAUNCH_CHECK();
+    CG_CUDA(cudaMemcpyAsync(ebase.data(), d_e, sizeof(int64_t) * (G + 1), cudaMemcpyDeviceToHost,
+                            s));
+    CG_CUDA(cudaStreamSynchronize(s));
+  }
+  if (ebase[0] != 0) {
+    set_error("pr_batch_create: offsets must start at 0");
+    return CG_ERR_INVALID_ARG;
+  }
+  for (int g = 0; g < G; ++g) {
+    if (ebase[g + 1] < ebase[g]) {
+      set_error("pr_batch_create: offsets decrease across graph %d", g);
+      return CG_ERR_INVALID_ARG;
+    }
+    if (ebase[g + 1] - ebase[g] >= 0x7FFFFFFFLL) {
+      set_error("pr_batch_create: graph %d has 2^31 - 1 edges or more", g);
+      return CG_ERR_UNSUPPORTED;
+    }
+  }
+  for (int64_t g = 0; g < G;) {
+    int64_t h = g + 1;
+    while (h < G && h - g < kPartGraphs && vbase[h + 1] - vbase[g] <= kPartVertices &&
+           ebase[h + 1] - ebase[g] <= kPartEdges)
+      ++h;
+    b->parts.emplace_back();
+    BatchPart& p = b->parts.back();
+    p.G = (int32_t)(h - g);
+    p.g0 = g;
+    p.v0 = vbase[g];
+    p.e0 = ebase[g];
+    p.V = vbase[h] - p.v0;
+    p.E = ebase[h] - p.e0;
+    std::vector<int64_t> vb(p.G + 1), eb(p.G + 1);
+    for (int32_t q = 0; q <= p.G; ++q) {
+      vb[q] = vbase[g + q] - p.v0;
+      eb[q] = ebase[g + q] - p.e0;
+      if (q > 0) p.vmax = std::max(p.vmax, (int32_t)(vb[q] - vb[q - 1]));
+    }
+    CG_TRY(build_part(&p, vb, eb, offsets + p.v0, src + p.e0, s));
+    b->bytes += p.bytes;
+    g = h;
+  }
+  return CG_OK;
+}
+
+int run_part(const BatchPart& b, int threads, int32_t iterations, double damping, float* rank,
+             double* resid, cudaStream_t stream) {
+  DeviceInfo di{};
+  CG_TRY(device_info(&di));
+  // contrib, the identity and, behind them, row sums for as many vertices as fit,
+  // up to the largest graph's
+  const int pad = batch_pad(b);
+  const size_t least = sizeof(float) * (size_t)(pad + 4);
+  const size_t most = (size_t)(232448 - 2048);
+  const size_t smem = std::max(least, std::min(2 * least, most));
+  BatchArgs a;
+  a.tasks = StagedTasks{b.plan.cs, b.plan.desc, b.plan.seg_task, pad};
+  a.idx = b.idx;
+  a.xbase = b.xbase;
+  a.xrow = b.plan.carry_row;
+  a.carry = (float*)b.plan.carry;
+  a.inv = b.inv;
+  a.vbase = b.vbase;
+  a.order = b.order;
+  a.ndang = b.ndang;
+  a.sums = b.sums;
+  a.rank = rank + b.v0;
+  a.resid = resid ? resid + b.g0 * iterations : nullptr;
+  a.counter = b.counter;
+  a.G = b.G;
+  a.iters = iterations;
+  a.room = (int)((smem - least) / sizeof(float));
+  a.d = (float)damping;
+  const int per_sm = std::max(1, std::min(1024 / threads,
+                                          (int)(232448 / std::max<size_t>(smem + 2048, 1))));
+  const int grid = std::min<int>(b.G, di.sm_count * per_sm);
+  CG_CUDA(cudaMemsetAsync(b.counter, 0, sizeof(unsigned), stream));
+  const void* fn = threads == 1024 ? (const void*)batch_pagerank_kernel<1024>
+                   : threads == 512 ? (const void*)batch_pagerank_kernel<512>
+                                    : (const void*)batch_pagerank_kernel<256>;
+  if (smem > 48 * 1024)
+    CG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (threads == 1024)
+    batch_pagerank_kernel<1024><<<grid, 1024, smem, stream>>>(a);
+  else if (threads == 512)
+    batch_pagerank_kernel<512><<<grid, 512, smem, stream>>>(a);
+  else
+    batch_pagerank_kernel<256><<<grid, 256, smem, stream>>>(a);
+  CG_LAUNCH_CHECK();
   return CG_OK;
 }
 
@@ -420,16 +545,13 @@ int pr_batch_create(int32_t G, const int64_t* host_vbase, const int64_t* offsets
   cg_batch* b = new cg_batch();
   CG_CUDA(cudaGetDevice(&b->device));
   b->G = G;
-  b->V = host_vbase[G];
-  b->vmax = vmax;
-  b->h_vbase.assign(host_vbase, host_vbase + G + 1);
   const int cap = (int)((232448 - 2048) / 4);  // shared memory of one block, in floats
   if (vmax > cap) {
     delete b;
     set_error("pr_batch_create: largest graph (%d vertices) exceeds shared memory", vmax);
     return CG_ERR_UNSUPPORTED;
   }
-  int st = build_batch(b, offsets, src, stream);
+  int st = build_batch(b, host_vbase, offsets, src, stream);
   if (st != CG_OK) {
     cudaStreamSynchronize(stream);
     free_batch(b);
@@ -466,48 +588,8 @@ int pr_batch_run(cg_batch* b, int32_t iterations, double damping, float* rank,
   CG_ARG(b && rank, "pr_batch_run: null argument");
   CG_ARG(iterations >= 1, "pr_batch_run: iterations must be >= 1");
   CG_ARG(damping >= 0.0 && damping <= 1.0, "pr_batch_run: damping must be in [0, 1]");
-  DeviceInfo di{};
-  CG_TRY(device_info(&di));
-  // contrib and the identity; where a block has the SM to itself, row sums
-  // behind them for as many vertices as fit, otherwise up to the largest graph's
-  const int pad = batch_pad(b);
-  const size_t least = sizeof(float) * (size_t)(pad + 4);
-  const size_t most = (size_t)(232448 - 2048);
-  const size_t smem = std::max(least, std::min(2 * least, most));
-  BatchArgs a;
-  a.tasks = StagedTasks{b->plan.cs, b->plan.desc, b->plan.seg_task, pad};
-  a.idx = b->idx;
-  a.xbase = b->xbase;
-  a.xrow = b->plan.carry_row;
-  a.carry = (float*)b->plan.carry;
-  a.inv = b->inv;
-  a.vbase = b->vbase;
-  a.order = b->order;
-  a.ndang = b->ndang;
-  a.sums = b->sums;
-  a.rank = rank;
-  a.resid = resid;
-  a.counter = b->counter;
-  a.G = b->G;
-  a.iters = iterations;
-  a.room = (int)((smem - least) / sizeof(float));
-  a.d = (float)damping;
-  const int per_sm = std::max(1, std::min(1024 / b->threads,
-                                          (int)(232448 / std::max<size_t>(smem + 2048, 1))));
-  const int grid = std::min<int>(b->G, di.sm_count * per_sm);
-  CG_CUDA(cudaMemsetAsync(b->counter, 0, sizeof(unsigned), stream));
-  const void* fn = b->threads == 1024 ? (const void*)batch_pagerank_kernel<1024>
-                   : b->threads == 512 ? (const void*)batch_pagerank_kernel<512>
-                                       : (const void*)batch_pagerank_kernel<256>;
-  if (smem > 48 * 1024)
-    CG_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  if (b->threads == 1024)
-    batch_pagerank_kernel<1024><<<grid, 1024, smem, stream>>>(a);
-  else if (b->threads == 512)
-    batch_pagerank_kernel<512><<<grid, 512, smem, stream>>>(a);
-  else
-    batch_pagerank_kernel<256><<<grid, 256, smem, stream>>>(a);
-  CG_LAUNCH_CHECK();
+  for (const BatchPart& p : b->parts)
+    CG_TRY(run_part(p, b->threads, iterations, damping, rank, resid, stream));
   return CG_OK;
 }
 

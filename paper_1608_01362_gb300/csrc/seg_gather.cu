@@ -465,10 +465,6 @@ int seg_plan_alloc(int64_t E, int k, const std::vector<int64_t>& edge_base,
     p->h_cstart[q + 1] = p->h_cstart[q] + ((Eq + 7) & ~7LL);
   }
   p->colf_len = p->h_cstart[k] + kMaxChunkEdges;  // chunks may read past their segment's end
-  if (p->colf_len >= 0x7FFFFFFFLL) {
-    set_error("segmented gather: padded edge array exceeds 2^31 entries");
-    return CG_ERR_UNSUPPORTED;
-  }
   CG_CUDA(cudaMalloc((void**)&p->colf, sizeof(uint32_t) * p->colf_len));
   // The segments' arrays, one allocation and one upload: meta (row_base, which
   // the caller's build writes, edge_base, cstart, bounds), then seg_E and

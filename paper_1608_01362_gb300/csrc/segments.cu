@@ -373,6 +373,10 @@ int build_impl(const int64_t* offsets, const int32_t* src, int32_t V, int64_t E,
   }
   CG_CUDA(cudaStreamSynchronize(s));  // edge_base
   CG_TRY(seg_plan_alloc(E, k, g->edge_base, bounds, &g->plan, s));
+  if (g->plan.colf_len >= 0x7FFFFFFFLL) {  // the gathers keep places in it in 32 bits
+    set_error("segmented gather: padded edge array exceeds 2^31 entries");
+    return CG_ERR_UNSUPPORTED;
+  }
   SegPlan* p = &g->plan;
   int64_t* d_rb = p->meta;
   int64_t* m_eb = p->meta + (k + 1);
