@@ -14,7 +14,8 @@
 // written by the last iteration alone unless residuals are asked for.
 // Graphs are handed out largest first through an atomic counter, so the
 // biggest ones start first and small ones fill in behind (longest processing
-// time first).  Nothing waits on another block.
+// time first).  Nothing waits on another block.  Tiny graphs that come in thousands
+// are handed out last, to a warp each, and have plain rows (kTinyGraphs below).
 //
 // The earlier kernel walked 256-edge chunks of 32-bit flagged sources with a
 // scan per chunk, stored the row sums in row order, scattered them into the
@@ -34,19 +35,40 @@ struct BatchPart {
   int32_t G = 0;
   int64_t g0 = 0, v0 = 0, e0 = 0;  // first graph, vertex and edge
   int64_t V = 0, E = 0, rows = 0;
-  int32_t vmax = 0;
+  int32_t nstaged = 0;        // graphs that are not tiny
+  int32_t vmax = 0, tmax = 0; // vertices of the largest of them and of the largest tiny one
   SegPlan plan;               // the graphs as staged segments: tasks, stream, carries
   int64_t* vbase = nullptr;   // [G+1] first vertex of each graph (from v0 on)
-  int32_t* order = nullptr;   // [G] graphs by edge count, descending
+  int32_t* order = nullptr;   // [G] graphs by edge count, descending, the tiny ones last
   int32_t* ndang = nullptr;   // [G]
   int32_t* xbase = nullptr;   // [G+1] first carry of each graph
   int32_t* row_ptr = nullptr; // [rows+1] first edge of each non-empty row
   int32_t* idx = nullptr;     // [rows] local destination of each non-empty row
   float* inv = nullptr;       // [V]
   float* sums = nullptr;      // [V] row sums of graphs too large to keep them on chip
+  longlong2* tiny = nullptr;  // [G] a tiny graph's first source and row start, (-1, -) for
+                              // the others; NULL where there is no tiny one
+  uint16_t* trow = nullptr;   // where the tiny graphs' rows begin among their sources (one
+                              // entry more than rows), and these; same allocation as tiny
+  uint8_t* tcol = nullptr;
   unsigned* counter = nullptr;
   int64_t bytes = 0;
 };
+
+// Tiny graphs, where there are thousands, have plain rows in place of staged
+// tasks, which take 0.6 to 2 KB for every length class that a graph's rows meet
+// (kept for 20,000 graphs of 25 vertices and 50 edges: 134 MB so, 10 MB with plain
+// rows), and a warp each in place of a block.  Up to the limits below no batch of
+// 4,096 and more was slower than with a block each, at 256 threads per block,
+// where blocks are fastest (4.66 ms at 1024 threads and 1.19 at 256 for those
+// 20,000, 0.28 and 0.26 so; 12,000 of 64 vertices and 1,024 edges 0.54 of the
+// time; 7,800 of 64 and 1,536: 0.96).  One graph on its own takes up to three
+// times as long on a warp, hence only from kTinyGraphs on.
+constexpr int kTinyVertices = 255;
+constexpr int kTinyEdges = 1280;
+constexpr int kTinyRow = 255;  // edges of the longest row
+constexpr int kTinyGraphs = 4096;
+constexpr uint8_t kOutside = 255;  // a source outside its graph
 
 // A part ends before it has more than this many graphs, vertices or edges (a
 // graph of more edges has one to itself): its places then fit 32 bits, and the
@@ -69,13 +91,37 @@ struct cg_batch {
 namespace cg {
 namespace {
 
-// The edge offsets at the graphs' first vertices.
-__global__ void batch_ebase_kernel(const int64_t* __restrict__ offsets,
-                                   const int64_t* __restrict__ vbase, int G,
-                                   int64_t* __restrict__ ebase) {
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g <= G;
-       g += (int64_t)gridDim.x * blockDim.x)
-    ebase[g] = offsets[vbase[g]];
+// The edge offsets at the graphs' first vertices, and whether a graph is tiny:
+// a warp per graph.
+__global__ void batch_look_kernel(const int64_t* __restrict__ offsets,
+                                  const int64_t* __restrict__ vbase, int G,
+                                  int64_t* __restrict__ ebase, uint8_t* __restrict__ tiny) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g <= G; g += nw) {
+    const int64_t v0 = vbase[g], v1 = g < G ? vbase[g + 1] : v0;
+    if (lane == 0) ebase[g] = offsets[v0];
+    if (g == G) break;
+    bool fits = v1 - v0 <= kTinyVertices;
+    if (fits) fits = offsets[v1] - offsets[v0] <= kTinyEdges;
+    if (fits)
+      for (int64_t v = v0 + lane; v < v1; v += 32) {
+        const int64_t n = offsets[v + 1] - offsets[v];
+        fits = fits && n >= 0 && n <= kTinyRow;
+      }
+    fits = __all_sync(0xffffffffu, fits);
+    if (lane == 0) tiny[g] = fits;
+  }
+}
+
+// The graph that vertex v lies in: the last g with vbase[g] <= v.
+__device__ __forceinline__ int graph_of(const int64_t* __restrict__ vbase, int G, int64_t v) {
+  int lo = 0, hi = G + 1;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (vbase[mid] <= v) lo = mid + 1; else hi = mid;
+  }
+  return lo - 1;
 }
 
 // (Offsets, sources and bases below are those of a part: vertices and edges are
@@ -85,59 +131,73 @@ __global__ void batch_degree_kernel(const int32_t* __restrict__ src, const int64
                                     int32_t* __restrict__ outdeg) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E;
        e += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = G + 1;  // graph of edge e: last g with ebase[g] <= e
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (ebase[mid] <= e) lo = mid + 1; else hi = mid;
-    }
-    const int g = lo - 1;
+    const int g = graph_of(ebase, G, e);
     const int32_t u = src[e];
     if (u >= 0 && (int64_t)u < vbase[g + 1] - vbase[g]) atomicAdd(outdeg + vbase[g] + u, 1);
   }
 }
 
+// (nonempty: of the rows that become staged ones)
 __global__ void batch_inv_kernel(const int32_t* __restrict__ outdeg, int64_t V,
                                  float* __restrict__ inv, const int64_t* __restrict__ offsets,
+                                 const int64_t* __restrict__ vbase, int G,
+                                 const longlong2* __restrict__ tiny,
                                  int32_t* __restrict__ nonempty, int32_t* __restrict__ bad) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V;
        v += (int64_t)gridDim.x * blockDim.x) {
     inv[v] = outdeg[v] > 0 ? 1.0f / (float)outdeg[v] : 0.0f;
-    nonempty[v] = offsets[v + 1] > offsets[v] ? 1 : 0;
+    bool staged = offsets[v + 1] > offsets[v];
+    if (staged && tiny) staged = tiny[graph_of(vbase, G, v)].x < 0;
+    nonempty[v] = staged ? 1 : 0;
     if (offsets[v + 1] < offsets[v]) atomicExch(bad, 1);
   }
 }
 
 // Non-empty rows (in vertex order): their starts and local destinations, and
-// their sources in the plan's padded layout.
+// their sources in the plan's padded layout; the tiny graphs' rows.  sbase: the
+// graphs' first edges among the staged ones.
+struct RowsOut {
+  uint32_t* colf;
+  int32_t* row_ptr;
+  int32_t* idx;
+  const longlong2* tiny;
+  uint16_t* trow;
+  uint8_t* tcol;
+};
 __global__ void batch_rows_kernel(const int64_t* __restrict__ offsets,
                                   const int32_t* __restrict__ src,
                                   const int64_t* __restrict__ rowpos,  // exclusive scan of nonempty
                                   const int64_t* __restrict__ vbase,
                                   const int64_t* __restrict__ ebase,
+                                  const int64_t* __restrict__ sbase,
                                   const int64_t* __restrict__ cstart, int G, int64_t V, int64_t e0,
-                                  int pad,
-                                  uint32_t* __restrict__ colf, int32_t* __restrict__ row_ptr,
-                                  int32_t* __restrict__ idx) {
+                                  int pad, RowsOut out) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < V; v += nw) {
     const int64_t lo = offsets[v] - e0, hi = offsets[v + 1] - e0;
-    if (hi <= lo) continue;
-    int a = 0, b = G + 1;
-    while (a < b) {
-      const int mid = (a + b) >> 1;
-      if (vbase[mid] <= v) a = mid + 1; else b = mid;
-    }
-    const int g = a - 1;
+    if (hi <= lo && !out.tiny) continue;
+    const int g = graph_of(vbase, G, v);
     const int32_t n = (int32_t)(vbase[g + 1] - vbase[g]);
-    if (lane == 0) {
-      idx[rowpos[v]] = (int32_t)(v - vbase[g]);
-      row_ptr[rowpos[v]] = (int32_t)lo;
+    const int64_t eb = ebase[g];
+    const longlong2 t = out.tiny ? out.tiny[g] : make_longlong2(-1, 0);
+    if (t.x >= 0) {
+      uint16_t* row = out.trow + t.y + (v - vbase[g]);
+      if (lane == 0) {
+        row[0] = (uint16_t)(lo - eb);
+        if (v + 1 == vbase[g + 1]) row[1] = (uint16_t)(hi - eb);
+      }
+    } else if (lane == 0 && hi > lo) {
+      out.idx[rowpos[v]] = (int32_t)(v - vbase[g]);
+      out.row_ptr[rowpos[v]] = (int32_t)(lo - eb + sbase[g]);
     }
-    const int64_t shift = cstart[g] - ebase[g];
     for (int64_t e = lo + lane; e < hi; e += 32) {
       const int32_t u = src[e];  // a source outside its graph contributes nothing
-      colf[e + shift] = (uint32_t)u < (uint32_t)n ? (uint32_t)u : (uint32_t)pad;
+      const bool inside = (uint32_t)u < (uint32_t)n;
+      if (t.x >= 0)
+        out.tcol[t.x + (e - eb)] = inside ? (uint8_t)u : kOutside;
+      else
+        out.colf[cstart[g] + (e - eb)] = inside ? (uint32_t)u : (uint32_t)pad;
     }
   }
 }
@@ -187,18 +247,149 @@ struct BatchArgs {
   const int32_t* order;
   const int32_t* ndang;
   float* sums;
+  const longlong2* tiny;
+  const uint16_t* trow;
+  const uint8_t* tcol;
   float* rank;     // [V] result (and the previous iterate where residuals are asked for)
   double* resid;   // [G * iters] or NULL
   unsigned* counter;
   int G;
+  int nstaged;     // graphs that a block solves; behind them in `order` the tiny ones,
+  int bundle;      // so many of which a block's warps take at once, one each
+  int stride;      // floats of a tiny graph's vector (a warp has it and its row sums)
   int iters;
   int room;        // floats of dynamic shared memory behind the contrib vector
   float d;
 };
 
+// x at source e of a row of n, 0 behind its end and where the source is outside.
+__device__ __forceinline__ float tiny_at(const uint8_t* __restrict__ col, int e, int n,
+                                         const float* x) {
+  const int u = e < n ? __ldg(col + e) : kOutside;
+  return u != kOutside ? x[u] : 0.0f;
+}
+
+// The row sums of vertices v0 .. v0 + 31 (v: this lane's, with n sources from col
+// on), each in the order in which a staged task adds it: up to 8 sources one after
+// the other; up to 16 the even and the odd ones apart, a lane per row; up to 16
+// 2^lg so on each of 2^lg lanes (here four, with up to four of those lanes' parts
+// each, for eight rows at a time), then a tree over the lanes.
+__device__ __forceinline__ void tiny_rows(const uint8_t* __restrict__ col, int lo, int n, int v,
+                                          int v0, const float* x, float* sums) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31, sub = lane & 3, grp = lane >> 2;
+  if (n <= 16) {
+    float a = 0.0f, b = 0.0f;
+    for (int e = 0; e < n; e += 4) {
+      const uint8_t* c = col + lo;
+      const float w[4] = {tiny_at(c, e, n, x), tiny_at(c, e + 1, n, x), tiny_at(c, e + 2, n, x),
+                          tiny_at(c, e + 3, n, x)};
+      if (n <= 8) {
+        a += w[0]; a += w[1]; a += w[2]; a += w[3];
+      } else {
+        a += w[0]; b += w[1]; a += w[2]; b += w[3];
+      }
+    }
+    if (v >= 0) sums[v] = a + b;
+  }
+  for (unsigned rest = __ballot_sync(kFull, n > 16); rest;) {
+    unsigned t = rest;  // the group takes the grp-th row of the rest
+    for (int q = 0; q < grp; ++q) t &= t - 1;
+    const int at = t ? __ffs(t) - 1 : 0;
+    const uint8_t* c = col + __shfl_sync(kFull, lo, at);
+    const int len = __shfl_sync(kFull, n, at), m = t ? len : 0;
+    const int lg = m <= 16 ? 0 : 28 - __clz(m - 1);  // m <= 16 << lg
+    float w[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int l = sub + 4 * k;
+      if (l >= 1 << lg) break;
+      float a = 0.0f, b = 0.0f;
+      for (int e = l; e < m; e += 4 << lg) {
+        const float y[4] = {tiny_at(c, e, m, x), tiny_at(c, e + (1 << lg), m, x),
+                            tiny_at(c, e + (2 << lg), m, x), tiny_at(c, e + (3 << lg), m, x)};
+        a += y[0]; b += y[1]; a += y[2]; b += y[3];
+      }
+      w[k] = a + b;
+    }
+    __syncwarp();
+    const int parts = __any_sync(kFull, m > 64) ? 4 : 1;  // (the other parts are 0)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (k >= parts) break;
+      w[k] += __shfl_xor_sync(kFull, w[k], 1);
+      w[k] += __shfl_xor_sync(kFull, w[k], 2);
+    }
+    if (sub == 0 && t) sums[v0 + at] = (w[0] + w[1]) + (w[2] + w[3]);
+    for (int q = 0; q < 8; ++q) rest &= rest - 1;
+  }
+}
+
+// All iterations of tiny graph g on one warp; x: contrib, and a.stride floats
+// behind it the row sums.  Every sum is taken in the order of the block's way (a
+// graph's ranks do not depend on the batch it is in).  Not inlined: the staged
+// graphs' code keeps its registers.
+__device__ __noinline__ void tiny_solve(const BatchArgs& a, int g, float* x) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int64_t vb = a.vbase[g];
+  const int V = (int)(a.vbase[g + 1] - vb);
+  const longlong2 first = a.tiny[g];
+  const uint16_t* row = a.trow + first.y;
+  const uint8_t* col = a.tcol + first.x;
+  const float* inv = a.inv + vb;
+  float* rank = a.rank + vb;
+  float* sums = x + a.stride;
+  const bool residuals = a.resid != nullptr;
+  const float base = (1.0f - a.d) / (float)V, r0 = 1.0f / (float)V;
+  const double invV = 1.0 / (double)V;
+  __syncwarp();  // the warp's previous graph is done with the vectors
+  for (int v = lane; v < V; v += 32) {
+    if (residuals) rank[v] = r0;
+    x[v] = r0 * __ldg(inv + v);
+  }
+  double D = (double)a.ndang[g] * (double)r0;
+  __syncwarp();
+  for (int it = 0; it < a.iters; ++it) {
+    const bool write = residuals || it == a.iters - 1;
+    for (int v0 = 0; v0 < V; v0 += 32) {
+      const int v = v0 + lane < V ? v0 + lane : -1;
+      const int lo = v >= 0 ? __ldg(row + v) : 0, hi = v >= 0 ? __ldg(row + v + 1) : 0;
+      tiny_rows(col, lo, hi - lo, v, v0, x, sums);
+    }
+    __syncwarp();
+    const float Dv = (float)(D * invV);
+    double dd = 0.0, rr = 0.0;  // lane c: those of vertices 32 c .. 32 c + 31, summed in FP32
+    for (int c = 0; 32 * c < V; ++c) {
+      const int v = 32 * c + lane;
+      float dpart = 0.0f, rpart = 0.0f;
+      if (v < V) {
+        const float iv = __ldg(inv + v);
+        const float r = base + a.d * (sums[v] + Dv);
+        if (residuals) rpart = fabsf(r - rank[v]);
+        if (write) rank[v] = r;
+        x[v] = r * iv;
+        if (iv == 0.0f) dpart = r;
+      }
+      const float d = __shfl_sync(kFull, warp_sum(dpart), 0);
+      if (lane == c) dd = (double)d;
+      if (residuals) {
+        const float q = __shfl_sync(kFull, warp_sum(rpart), 0);
+        if (lane == c) rr = (double)q;
+      }
+    }
+    D = __shfl_sync(kFull, warp_sum(dd), 0);
+    if (residuals) {
+      rr = warp_sum(rr);
+      if (lane == 0) a.resid[(int64_t)g * a.iters + it] = rr;
+    }
+    __syncwarp();
+  }
+}
+
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
-batch_pagerank_kernel(BatchArgs a) {
+batch_pagerank_kernel(const __grid_constant__ BatchArgs a) {
   constexpr int WARPS = THREADS / 32;
   extern __shared__ __align__(16) float xs[];  // contrib, the identity, then the row sums
   __shared__ int s_g;
@@ -210,12 +401,18 @@ batch_pagerank_kernel(BatchArgs a) {
   for (;;) {
     __syncthreads();
     if (tid == 0) {
-      const unsigned q = atomicAdd(a.counter, 1u);
-      s_g = (int)q < a.G ? a.order[q] : -1;
+      const int q = (int)atomicAdd(a.counter, 1u);
+      const int64_t t = a.nstaged + (int64_t)(q - a.nstaged) * a.bundle;  // first of a bundle
+      s_g = q < a.nstaged ? a.order[q] : t < a.G ? -1 - (int)t : INT32_MIN;
     }
     __syncthreads();
     const int g = s_g;
-    if (g < 0) break;
+    if (g < 0) {
+      if (g == INT32_MIN) break;
+      const int t = -1 - g + w;  // (staged graphs are all handed out before)
+      if (w < a.bundle && t < a.G) tiny_solve(a, a.order[t], xs + w * 2 * a.stride);
+      continue;
+    }
     const int64_t vb = a.vbase[g];
     const int V = (int)(a.vbase[g + 1] - vb);
     const int32_t t0 = a.tasks.seg_task[g], t1 = a.tasks.seg_task[g + 1];
@@ -317,6 +514,7 @@ void free_part(BatchPart* b) {
   cudaFree(b->idx);
   cudaFree(b->inv);
   cudaFree(b->sums);
+  cudaFree(b->tiny);
   cudaFree(b->counter);
 }
 
@@ -335,20 +533,42 @@ __global__ void batch_row_base_kernel(const int64_t* __restrict__ rowpos,
 // the entry behind the largest contrib vector that holds the sum's identity
 int batch_pad(const BatchPart& b) { return (b.vmax + 3) & ~3; }
 
-// Lays out one part (its G, g0, v0, e0, V, E and vmax are set); vbase and ebase:
+// Lays out one part (its G, g0, v0, e0, V and E are set); vbase and ebase:
 // its graphs' first vertices and edges, counted from its own first ones.
 int build_part(BatchPart* b, const std::vector<int64_t>& vbase, const std::vector<int64_t>& ebase,
-               const int64_t* offsets, const int32_t* src, cudaStream_t s) {
+               std::vector<uint8_t> is_tiny, const int64_t* offsets, const int32_t* src,
+               cudaStream_t s) {
   const int G = b->G;
+  if (std::count(is_tiny.begin(), is_tiny.end(), 1) < kTinyGraphs)
+    std::fill(is_tiny.begin(), is_tiny.end(), 0);
+  // the staged graphs' edges, and the tiny graphs' places
+  std::vector<int64_t> sbase(G + 1, 0);
+  std::vector<longlong2> tiny(G, make_longlong2(-1, 0));
+  int64_t ncol = 0, nrow = 0;
+  for (int g = 0; g < G; ++g) {
+    const int64_t n = ebase[g + 1] - ebase[g];
+    sbase[g + 1] = sbase[g] + (is_tiny[g] ? 0 : n);
+    const int32_t vertices = (int32_t)(vbase[g + 1] - vbase[g]);
+    if (!is_tiny[g]) {
+      ++b->nstaged;
+      b->vmax = std::max(b->vmax, vertices);
+    } else {
+      b->tmax = std::max(b->tmax, vertices);
+      tiny[g] = make_longlong2(ncol, nrow);
+      ncol += n;
+      nrow += vbase[g + 1] - vbase[g] + 1;
+    }
+  }
   std::vector<int32_t> order(G);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+    if (is_tiny[x] != is_tiny[y]) return is_tiny[x] < is_tiny[y];
     return ebase[x + 1] - ebase[x] > ebase[y + 1] - ebase[y];
   });
   const int64_t V = b->V, E = b->E;
-  CG_TRY(seg_plan_alloc(E, G, ebase, vbase, &b->plan, s));
+  CG_TRY(seg_plan_alloc(sbase[G], G, sbase, vbase, &b->plan, s));
   SegPlan* p = &b->plan;
-  const int64_t* d_ebase = p->meta + (G + 1);
+  const int64_t* d_sbase = p->meta + (G + 1);
   const int64_t* cstart = p->meta + 2 * (G + 1);
   CG_CUDA(cudaMalloc((void**)&b->vbase, sizeof(int64_t) * (G + 1)));
   CG_CUDA(cudaMalloc((void**)&b->order, sizeof(int32_t) * G));
@@ -360,9 +580,21 @@ int build_part(BatchPart* b, const std::vector<int64_t>& vbase, const std::vecto
   CG_CUDA(cudaMemcpyAsync(b->vbase, vbase.data(), sizeof(int64_t) * (G + 1),
                           cudaMemcpyHostToDevice, s));
   CG_CUDA(cudaMemcpyAsync(b->order, order.data(), sizeof(int32_t) * G, cudaMemcpyHostToDevice, s));
-  // scratch: out-degree, non-empty flags and their scan
+  const size_t tiny_bytes = nrow > 0 ? 16 * (size_t)G + 2 * (size_t)nrow + (size_t)ncol : 0;
+  if (nrow > 0) {
+    CG_CUDA(cudaMalloc((void**)&b->tiny, tiny_bytes));
+    b->trow = reinterpret_cast<uint16_t*>(b->tiny + G);
+    b->tcol = reinterpret_cast<uint8_t*>(b->trow + nrow);
+    CG_CUDA(cudaMemcpyAsync(b->tiny, tiny.data(), sizeof(longlong2) * G, cudaMemcpyHostToDevice,
+                            s));
+  }
+  // scratch: out-degree, non-empty flags and their scan, the graphs' first edges
   Scratch tmp(s, 2 * Scratch::round(4 * (size_t)V) + Scratch::round(8 * (size_t)(V + 1)) +
-                     scan_scratch(V) + 256);
+                     scan_scratch(V) + 256 + Scratch::round(8 * (size_t)(G + 1)));
+  int64_t* d_ebase = nullptr;
+  CG_CUDA(tmp.get(&d_ebase, G + 1));
+  CG_CUDA(cudaMemcpyAsync(d_ebase, ebase.data(), sizeof(int64_t) * (G + 1),
+                          cudaMemcpyHostToDevice, s));
   int32_t *outdeg = nullptr, *nonempty = nullptr;
   int64_t* rowpos = nullptr;
   int32_t* bad = nullptr;
@@ -376,7 +608,8 @@ int build_part(BatchPart* b, const std::vector<int64_t>& vbase, const std::vecto
     batch_degree_kernel<<<grid_for(E, 256), 256, 0, s>>>(src, d_ebase, b->vbase, G, E, outdeg);
     CG_LAUNCH_CHECK();
   }
-  batch_inv_kernel<<<grid_for(V, 256), 256, 0, s>>>(outdeg, V, b->inv, offsets, nonempty, bad);
+  batch_inv_kernel<<<grid_for(V, 256), 256, 0, s>>>(outdeg, V, b->inv, offsets, b->vbase, G,
+                                               b->tiny, nonempty, bad);
   CG_LAUNCH_CHECK();
   batch_dangling_kernel<<<std::min(G, 4096), 256, 0, s>>>(outdeg, b->vbase, G, b->ndang);
   CG_LAUNCH_CHECK();
@@ -396,11 +629,11 @@ int build_part(BatchPart* b, const std::vector<int64_t>& vbase, const std::vecto
   b->rows = rbase[G];
   CG_CUDA(cudaMalloc((void**)&b->idx, sizeof(int32_t) * (size_t)(b->rows + 1)));
   CG_CUDA(cudaMalloc((void**)&b->row_ptr, sizeof(int32_t) * (size_t)(b->rows + 1)));
-  const int32_t end = (int32_t)E;
+  const int32_t end = (int32_t)sbase[G];
   CG_CUDA(cudaMemcpyAsync(b->row_ptr + b->rows, &end, sizeof(int32_t), cudaMemcpyHostToDevice, s));
   batch_rows_kernel<<<grid_for(V * 32, 256, 16), 256, 0, s>>>(
-      offsets, src, rowpos, b->vbase, d_ebase, cstart, G, V, b->e0, batch_pad(*b), p->colf,
-      b->row_ptr, b->idx);
+      offsets, src, rowpos, b->vbase, d_ebase, d_sbase, cstart, G, V, b->e0, batch_pad(*b),
+      RowsOut{p->colf, b->row_ptr, b->idx, b->tiny, b->trow, b->tcol});
   CG_LAUNCH_CHECK();
   p->rows = b->rows;
   p->rp32 = b->row_ptr;
@@ -414,7 +647,8 @@ int build_part(BatchPart* b, const std::vector<int64_t>& vbase, const std::vecto
   cudaFree(p->colf);
   p->colf = nullptr;
   p->colf_len = 0;
-  b->bytes = seg_plan_bytes(*p) + 8 * V + 8 * (b->rows + 1) + 20 * (int64_t)(G + 1);
+  b->bytes = seg_plan_bytes(*p) + 8 * V + 8 * (b->rows + 1) + 20 * (int64_t)(G + 1) +
+             (int64_t)tiny_bytes;
   return CG_OK;
 }
 
@@ -422,14 +656,19 @@ int build_batch(cg_batch* b, const int64_t* vbase, const int64_t* offsets, const
                 cudaStream_t s) {
   const int G = b->G;
   std::vector<int64_t> ebase(G + 1, 0);
+  std::vector<uint8_t> tiny(G, 0);
   {
-    Scratch tmp(s, 2 * Scratch::round(8 * (size_t)(G + 1)));
+    Scratch tmp(s, 2 * Scratch::round(8 * (size_t)(G + 1)) + Scratch::round((size_t)G));
     int64_t *d_v = nullptr, *d_e = nullptr;
+    uint8_t* d_t = nullptr;
+    CG_CUDA(tmp.get(&d_t, G));
     CG_CUDA(tmp.get(&d_v, G + 1));
     CG_CUDA(tmp.get(&d_e, G + 1));
     CG_CUDA(cudaMemcpyAsync(d_v, vbase, sizeof(int64_t) * (G + 1), cudaMemcpyHostToDevice, s));
-    batch_ebase_kernel<<<grid_for(G + 1, 256), 256, 0, s>>>(offsets, d_v, G, d_e);
+    batch_look_kernel<<<grid_for(((int64_t)G + 1) * 32, 256), 256, 0, s>>>(offsets, d_v, G, d_e,
+                                                                           d_t);
     CG_LAUNCH_CHECK();
+    CG_CUDA(cudaMemcpyAsync(tiny.data(), d_t, (size_t)G, cudaMemcpyDeviceToHost, s));
     CG_CUDA(cudaMemcpyAsync(ebase.data(), d_e, sizeof(int64_t) * (G + 1), cudaMemcpyDeviceToHost,
                             s));
     CG_CUDA(cudaStreamSynchronize(s));
@@ -465,9 +704,9 @@ int build_batch(cg_batch* b, const int64_t* vbase, const int64_t* offsets, const
     for (int32_t q = 0; q <= p.G; ++q) {
       vb[q] = vbase[g + q] - p.v0;
       eb[q] = ebase[g + q] - p.e0;
-      if (q > 0) p.vmax = std::max(p.vmax, (int32_t)(vb[q] - vb[q - 1]));
     }
-    CG_TRY(build_part(&p, vb, eb, offsets + p.v0, src + p.e0, s));
+    CG_TRY(build_part(&p, vb, eb, {tiny.begin() + g, tiny.begin() + h}, offsets + p.v0, src + p.e0,
+                      s));
     b->bytes += p.bytes;
     g = h;
   }
@@ -483,8 +722,11 @@ int run_part(const BatchPart& b, int threads, int32_t iterations, double damping
   const int pad = batch_pad(b);
   const size_t least = sizeof(float) * (size_t)(pad + 4);
   const size_t most = (size_t)(232448 - 2048);
-  const size_t smem = std::max(least, std::min(2 * least, most));
-  BatchArgs a;
+  // (a tiny graph's contrib and row sums per warp)
+  const int stride = (b.tmax + 3) & ~3, warps = threads / 32;
+  const size_t smem = std::max({least, std::min(2 * least, most),
+                                sizeof(float) * (size_t)(2 * stride * warps)});
+  BatchArgs a{};
   a.tasks = StagedTasks{b.plan.cs, b.plan.desc, b.plan.seg_task, pad};
   a.idx = b.idx;
   a.xbase = b.xbase;
@@ -495,16 +737,23 @@ int run_part(const BatchPart& b, int threads, int32_t iterations, double damping
   a.order = b.order;
   a.ndang = b.ndang;
   a.sums = b.sums;
+  a.tiny = b.tiny;
+  a.tcol = b.tcol;
+  a.trow = b.trow;
   a.rank = rank + b.v0;
   a.resid = resid ? resid + b.g0 * iterations : nullptr;
   a.counter = b.counter;
   a.G = b.G;
   a.iters = iterations;
   a.room = (int)((smem - least) / sizeof(float));
+  a.nstaged = b.nstaged;
+  a.stride = stride;
   a.d = (float)damping;
   const int per_sm = std::max(1, std::min(1024 / threads,
                                           (int)(232448 / std::max<size_t>(smem + 2048, 1))));
-  const int grid = std::min<int>(b.G, di.sm_count * per_sm);
+  const int ntiny = b.G - b.nstaged, slots = di.sm_count * per_sm;
+  a.bundle = std::max(1, std::min(warps, (int)ceil_div(ntiny, slots)));
+  const int grid = std::min<int>(b.nstaged + (int)ceil_div(ntiny, a.bundle), slots);
   CG_CUDA(cudaMemsetAsync(b.counter, 0, sizeof(unsigned), stream));
   const void* fn = threads == 1024 ? (const void*)batch_pagerank_kernel<1024>
                    : threads == 512 ? (const void*)batch_pagerank_kernel<512>
