@@ -116,9 +116,9 @@ __device__ __forceinline__ void publish_last(u64* count, const Mailbox& box) {
   publish(count, box);
 }
 
-__global__ void bc_reset_kernel(int32_t V, int32_t* __restrict__ level,
-                                double* __restrict__ sigma, double* __restrict__ delta,
-                                uint32_t* __restrict__ xbits) {
+__global__ void bc_reset_kernel(int32_t V, int32_t* level,
+                                double* sigma, double* delta,
+                                uint32_t* xbits) {
   if (!chain_begin()) return;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V;
        v += (int64_t)gridDim.x * blockDim.x) {
@@ -136,10 +136,10 @@ __device__ __forceinline__ void set_bit(uint32_t* bits, int32_t v, bool on) {
     atomicAnd(bits + (v >> 5), ~(1u << (v & 31)));
 }
 
-__global__ void bc_seed_kernel(int32_t s, const int64_t* __restrict__ out_off,
-                               int32_t* __restrict__ level, double* __restrict__ sigma,
-                               int32_t* __restrict__ list, int32_t* __restrict__ fpos,
-                               int32_t* __restrict__ fgap, u64* __restrict__ count, Mailbox box) {
+__global__ void bc_seed_kernel(int32_t s, const int64_t* out_off,
+                               int32_t* level, double* sigma,
+                               int32_t* list, int32_t* fpos,
+                               int32_t* fgap, u64* count, Mailbox box) {
   if (!chain_begin()) return;
   level[s] = 0;
   sigma[s] = 1.0;
@@ -162,7 +162,7 @@ struct Frontier {
 
 // The vertices found at this level by the warp: those with out-edges join the
 // next frontier at places reserved together with their out-edges' places.
-__device__ __forceinline__ void append(bool take, int32_t v, const int64_t* __restrict__ out_off,
+__device__ __forceinline__ void append(bool take, int32_t v, const int64_t* out_off,
                                        const Frontier& f, u64* next, u64* reached) {
   const unsigned full = 0xffffffffu;
   const unsigned found = __ballot_sync(full, take);
@@ -171,8 +171,8 @@ __device__ __forceinline__ void append(bool take, int32_t v, const int64_t* __re
   int64_t o0 = 0;
   int32_t deg = 0;
   if (take) {
-    o0 = __ldg(out_off + v);
-    deg = (int32_t)(__ldg(out_off + v + 1) - o0);
+    o0 = __ldca(out_off + v);
+    deg = (int32_t)(__ldca(out_off + v + 1) - o0);
   }
   const unsigned m = __ballot_sync(full, deg > 0);
   int32_t incl = deg;  // a warp's degrees sum to at most E < 2^31 (its vertices are distinct)
@@ -200,7 +200,7 @@ __device__ __forceinline__ void append(bool take, int32_t v, const int64_t* __re
 // its 256 vertices, where a warp's would queue up behind each other on the two
 // counters.
 __device__ __forceinline__ void append_block(bool take, int32_t v,
-                                             const int64_t* __restrict__ out_off,
+                                             const int64_t* out_off,
                                              const Frontier& f, u64* next, u64* reached) {
   __shared__ u64 s_w[kThreads / 32], s_base;
   __shared__ int s_found;
@@ -211,8 +211,8 @@ __device__ __forceinline__ void append_block(bool take, int32_t v,
   int64_t o0 = 0;
   u64 val = 0;
   if (take) {
-    o0 = __ldg(out_off + v);
-    const u64 deg = (u64)(__ldg(out_off + v + 1) - o0);
+    o0 = __ldca(out_off + v);
+    const u64 deg = (u64)(__ldca(out_off + v + 1) - o0);
     if (deg) val = (1ull << 32) | deg;
   }
   u64 incl = val;
@@ -247,9 +247,9 @@ __device__ __forceinline__ void append_block(bool take, int32_t v,
 // Push: the frontier's n vertices and m out-edges, kPushTile edges per warp.
 // The counts of the level after next are cleared for it.
 __global__ void __launch_bounds__(kThreads)
-push_kernel(Frontier cur, int32_t n, int32_t m, const int64_t* __restrict__ out_off,
-            const int32_t* __restrict__ out_dst, int32_t L, int32_t* __restrict__ level,
-            double* __restrict__ sigma, Frontier nxt, u64* __restrict__ count, Mailbox box) {
+push_kernel(Frontier cur, int32_t n, int32_t m, const int64_t* out_off,
+            const int32_t* out_dst, int32_t L, int32_t* level,
+            double* sigma, Frontier nxt, u64* count, Mailbox box) {
   if (!chain_begin()) return;
   u64* next = count + (L + 1) % 3;
   if (blockIdx.x == 0 && threadIdx.x == 0) count[(L + 2) % 3] = 0ull;
@@ -266,8 +266,8 @@ push_kernel(Frontier cur, int32_t n, int32_t m, const int64_t* __restrict__ out_
       bool take = false;
       int32_t w = 0;
       if (e < m) {
-        const int32_t u = __ldg(cur.list + j);
-        w = __ldcs(out_dst + (e + __ldg(cur.gap + j)));
+        const int32_t u = __ldca(cur.list + j);
+        w = __ldcs(out_dst + (e + __ldca(cur.gap + j)));
         // a target seen visited on an earlier level needs no atomic; one that
         // reads unvisited takes the compare-and-swap (it may lose to another
         // edge of this level, which then reads L + 1)
@@ -284,7 +284,8 @@ push_kernel(Frontier cur, int32_t n, int32_t m, const int64_t* __restrict__ out_
 
 // ---------------------------------------------------------------------------
 // Compactions: a value per item, its exclusive prefix, and what to write there
-// (tile sums, their scan, a second pass over the items).
+// (tile sums, their scan, a second pass over the items).  What an item's writing
+// needs (more) is read for all of a thread's items before any is written.
 // ---------------------------------------------------------------------------
 constexpr int kItems = 8;                      // per thread, 32 at a time per warp
 constexpr int kCTile = kThreads * kItems;
@@ -297,14 +298,15 @@ struct Unvisited {
   int32_t* pos;
   int32_t* gap;
   __device__ u64 operator()(int64_t v) const {
-    if (__ldg(level + v) != -1) return 0ull;
-    const u64 d = (u64)(__ldg(in_off + v + 1) - __ldg(in_off + v));
+    if (__ldca(level + v) != -1) return 0ull;
+    const u64 d = (u64)(__ldca(in_off + v + 1) - __ldca(in_off + v));
     return d ? (1ull << 32) | d : 0ull;
   }
-  __device__ void put(int64_t v, u64 val, u64 before) const {
+  __device__ int64_t more(int64_t v) const { return __ldca(in_off + v); }
+  __device__ void put(int64_t v, int64_t row, u64 before) const {
     ids[before >> 32] = (int32_t)v;
     pos[before >> 32] = (int32_t)(before & 0xffffffffull);
-    gap[before >> 32] = (int32_t)(__ldg(in_off + v) - (int64_t)(before & 0xffffffffull));
+    gap[before >> 32] = (int32_t)(row - (int64_t)(before & 0xffffffffull));
   }
 };
 
@@ -314,10 +316,13 @@ struct Reached {
   const int64_t* out_off;
   int32_t* ids;
   uint32_t* keys;
-  __device__ u64 operator()(int64_t v) const { return __ldg(level + v) >= 0; }
-  __device__ void put(int64_t v, u64, u64 before) const {
+  __device__ u64 operator()(int64_t v) const { return __ldca(level + v) >= 0; }
+  __device__ int64_t more(int64_t v) const {
+    return (int64_t)__ldca(level + v) << 1 | (__ldca(out_off + v + 1) == __ldca(out_off + v));
+  }
+  __device__ void put(int64_t v, int64_t key, u64 before) const {
     ids[before] = (int32_t)v;
-    keys[before] = ((uint32_t)level[v] << 1) | (out_off[v + 1] == out_off[v]);
+    keys[before] = (uint32_t)key;
   }
 };
 
@@ -328,28 +333,31 @@ struct ListRows {
   int32_t* pos;
   int32_t* gap;
   __device__ u64 operator()(int64_t i) const {
-    const int32_t u = __ldg(list + i);
-    return (u64)(__ldg(out_off + u + 1) - __ldg(out_off + u)) | 1ull << 63;
+    const int32_t u = __ldca(list + i);
+    return (u64)(__ldca(out_off + u + 1) - __ldca(out_off + u)) | 1ull << 63;
   }
-  __device__ void put(int64_t i, u64, u64 before) const {
+  __device__ int64_t more(int64_t i) const { return __ldca(out_off + __ldca(list + i)); }
+  __device__ void put(int64_t i, int64_t row, u64 before) const {
     const int32_t p = (int32_t)(before & 0x7fffffffull);
     pos[i] = p;
-    gap[i] = (int32_t)__ldg(out_off + __ldg(list + i)) - p;
+    gap[i] = (int32_t)row - p;
   }
 };
 
 template <class F, bool WRITE>
 __global__ void __launch_bounds__(kThreads)
-compact_kernel(F f, int64_t n, int64_t* __restrict__ tsum) {
+compact_kernel(F f, int64_t n, int64_t* tsum) {
   if (!chain_begin()) return;
   __shared__ u64 s_w[kThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t base = (int64_t)blockIdx.x * kCTile + (int64_t)w * (kItems * 32);
   u64 v[kItems], sum = 0;
+  int64_t more[WRITE ? kItems : 1];
 #pragma unroll
   for (int r = 0; r < kItems; ++r) {
     const int64_t i = base + r * 32 + lane;
     v[r] = i < n ? f(i) : 0ull;
+    if (WRITE) more[r] = v[r] ? f.more(i) : 0;
     sum += v[r] & ~(1ull << 63);
   }
   for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -374,7 +382,7 @@ compact_kernel(F f, int64_t n, int64_t* __restrict__ tsum) {
       const u64 y = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += y;
     }
-    if (v[r]) f.put(base + r * 32 + lane, x, run + incl - x);
+    if (v[r]) f.put(base + r * 32 + lane, more[r], run + incl - x);
     run += __shfl_sync(0xffffffffu, incl, 31);
   }
 }
@@ -463,7 +471,7 @@ row_sum_kernel(RowSums a) {
           if (q0 + u == 0) row0 = walk.row;
           const uint32_t f = walk.batch((int32_t)(b + (q0 + u) * 32), &r);
           if (lane == q0 + u) ends = f;
-          w[u] = e < t1 ? (int32_t)e + __ldg(a.gap + r) : -1;  // place in vadj
+          w[u] = e < t1 ? (int32_t)e + __ldca(a.gap + r) : -1;  // place in vadj
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -473,10 +481,10 @@ row_sum_kernel(RowSums a) {
         bool hit[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          hit[u] = w[u] >= 0 && ((__ldg(a.bits + (w[u] >> 5)) >> (w[u] & 31)) & 1u);
+          hit[u] = w[u] >= 0 && ((__ldca(a.bits + (w[u] >> 5)) >> (w[u] & 31)) & 1u);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          sv[pad8((q0 + u) * 32 + lane)] = hit[u] ? __ldg(a.x + w[u]) : 0.0;
+          sv[pad8((q0 + u) * 32 + lane)] = hit[u] ? __ldca(a.x + w[u]) : 0.0;
       }
       __syncwarp();
       const uint32_t fl = (__shfl_sync(kFull, ends, lane >> 2) >> (8 * (lane & 3))) & 0xFFu;
@@ -548,10 +556,10 @@ int row_sums(const RowSums& a, int64_t most_edges, cudaStream_t s) {
 // After the pull's sums: one with a non-zero sum (a frontier in-neighbour) is on
 // level L+1.
 __global__ void __launch_bounds__(kThreads)
-pull_update_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ packed,
-                   const double* __restrict__ acc, const int64_t* __restrict__ out_off, int32_t L,
-                   int32_t* __restrict__ level, double* __restrict__ sigma, Frontier nxt,
-                   u64* __restrict__ count, Mailbox box) {
+pull_update_kernel(const int32_t* ids, const int64_t* packed,
+                   const double* acc, const int64_t* out_off, int32_t L,
+                   int32_t* level, double* sigma, Frontier nxt,
+                   u64* count, Mailbox box) {
   if (!chain_begin()) return;
   u64* next = count + (L + 1) % 3;
   if (blockIdx.x == 0 && threadIdx.x == 0) count[(L + 2) % 3] = 0ull;
@@ -575,8 +583,8 @@ pull_update_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ 
   publish_last(count, box);
 }
 
-__global__ void set_bits_kernel(const int32_t* __restrict__ list, int64_t n,
-                                uint32_t* __restrict__ bits, bool on) {
+__global__ void set_bits_kernel(const int32_t* list, int64_t n,
+                                uint32_t* bits, bool on) {
   if (!chain_begin()) return;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -586,10 +594,10 @@ __global__ void set_bits_kernel(const int32_t* __restrict__ list, int64_t n,
 // A level's n listed vertices, the first `summed` of them with gathered sums (0
 // for the others): delta, bc += delta (not for the source) and x = (1 + delta)
 // / sigma for the next level up.
-__global__ void dependency_kernel(const int32_t* __restrict__ list, int64_t n, int64_t summed,
-                                  const double* __restrict__ sums, const double* __restrict__ sigma,
-                                  double* __restrict__ delta, double* __restrict__ xval,
-                                  uint32_t* __restrict__ xbits, double* __restrict__ bc,
+__global__ void dependency_kernel(const int32_t* list, int64_t n, int64_t summed,
+                                  const double* sums, const double* sigma,
+                                  double* delta, double* xval,
+                                  uint32_t* xbits, double* bc,
                                   int32_t source) {
   if (!chain_begin()) return;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -598,9 +606,10 @@ __global__ void dependency_kernel(const int32_t* __restrict__ list, int64_t n, i
     const double sg = sigma[u];
     double d = 0.0;
     if (i < summed) {
+      const double before = bc[u];
       d = sg * sums[i];
       delta[u] = d;
-      if (u != source) bc[u] += d;
+      if (u != source) bc[u] = before + d;
     }
     xval[u] = (1.0 + d) / sg;
     set_bit(xbits, u, true);

@@ -13,8 +13,8 @@ namespace cg {
 // (The run lists this replaces were made by the host from a copy of the rows,
 // 0.7 ms of a new 65 M-edge graph.)
 template <class Op>
-__device__ __forceinline__ void fix_runs(const int32_t* __restrict__ carry_row,
-                                         const typename Op::T* __restrict__ carry, int64_t n,
+__device__ __forceinline__ void fix_runs(const int32_t* carry_row,
+                                         const typename Op::T* carry, int64_t n,
                                          typename Op::T* __restrict__ out) {
   using T = typename Op::T;
   constexpr unsigned kFull = 0xffffffffu;
@@ -23,10 +23,10 @@ __device__ __forceinline__ void fix_runs(const int32_t* __restrict__ carry_row,
   for (int64_t c0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) << 5; c0 < n;
        c0 += step) {
     const int64_t c = c0 + lane;
-    const int32_t r = c < n ? __ldg(carry_row + c) : -1;
+    const int32_t r = c < n ? __ldca(carry_row + c) : -1;
     int32_t prev = __shfl_up_sync(kFull, r, 1), next = __shfl_down_sync(kFull, r, 1);
-    if (lane == 0) prev = c0 > 0 ? __ldg(carry_row + c0 - 1) : -1;
-    if (lane == 31) next = c0 + 32 < n ? __ldg(carry_row + c0 + 32) : -1;
+    if (lane == 0) prev = c0 > 0 ? __ldca(carry_row + c0 - 1) : -1;
+    if (lane == 31) next = c0 + 32 < n ? __ldca(carry_row + c0 + 32) : -1;
     T S = r >= 0 ? carry[c] : Op::identity();
     int h = r < 0 || r != prev;  // a run begins (or none lies) here
 #pragma unroll
@@ -48,7 +48,7 @@ __device__ __forceinline__ void fix_runs(const int32_t* __restrict__ carry_row,
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int64_t i = b + 32 * u + lane;
-        const unsigned m = __ballot_sync(kFull, i < n && __ldg(carry_row + (i < n ? i : 0)) == row);
+        const unsigned m = __ballot_sync(kFull, i < n && __ldca(carry_row + (i < n ? i : 0)) == row);
         const int len = !more ? 0 : m == kFull ? 32 : __ffs(~m) - 1;
         if (lane < len) v = Op::op(v, carry[i]);
         more = more && len == 32;

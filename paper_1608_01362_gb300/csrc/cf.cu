@@ -72,12 +72,12 @@ template <bool BF16>
 __device__ __forceinline__ void load8(const void* p0, int64_t row, int K, int d0, float (&y)[8]) {
   const int64_t at = row * K + d0;
   if (BF16) {
-    const uint4 h = __ldg(reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(p0) + at));
+    const uint4 h = __ldca(reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(p0) + at));
     y[0] = b_lo(h.x); y[1] = b_hi(h.x); y[2] = b_lo(h.y); y[3] = b_hi(h.y);
     y[4] = b_lo(h.z); y[5] = b_hi(h.z); y[6] = b_lo(h.w); y[7] = b_hi(h.w);
   } else {
     const float4* f = reinterpret_cast<const float4*>(static_cast<const float*>(p0) + at);
-    const float4 a = __ldg(f), b = __ldg(f + 1);
+    const float4 a = __ldca(f), b = __ldca(f + 1);
     y[0] = a.x; y[1] = a.y; y[2] = a.z; y[3] = a.w;
     y[4] = b.x; y[5] = b.y; y[6] = b.z; y[7] = b.w;
   }
@@ -98,7 +98,7 @@ __device__ __forceinline__ void store8(void* p0, int64_t row, int K, int d0, con
 
 // Four pieces' gradients (their slots, -1: none) into g, in order.
 template <int K>
-__device__ __forceinline__ void add_pieces(const float* __restrict__ gpart, const int32_t (&slot)[4],
+__device__ __forceinline__ void add_pieces(const float* gpart, const int32_t (&slot)[4],
                                            int d0, float (&g)[8]) {
   float4 a[4], b[4];
 #pragma unroll
@@ -172,7 +172,7 @@ cf_update_kernel(UpdateRows a) {
     for (int64_t p = a.poff[v] + grp; p < p1; p += U * GROUPS) {
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        slot[u] = p + u * GROUPS < p1 ? __ldg(a.slots + p + u * GROUPS) : -1;
+        slot[u] = p + u * GROUPS < p1 ? __ldca(a.slots + p + u * GROUPS) : -1;
       add_pieces<K>(a.gpart, slot, d0, g);
     }
 #pragma unroll
@@ -203,7 +203,7 @@ cf_update_kernel(UpdateRows a) {
     for (int64_t p = a.poff[v] + grp; p < p1; p += U * GROUPS) {
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        slot[u] = p + u * GROUPS < p1 ? __ldg(a.slots + p + u * GROUPS) : -1;
+        slot[u] = p + u * GROUPS < p1 ? __ldca(a.slots + p + u * GROUPS) : -1;
       add_pieces<K>(a.gpart, slot, d0, g);
     }
     __syncwarp();
@@ -223,7 +223,7 @@ cf_update_kernel(UpdateRows a) {
     for (int q = 0; q < 8; ++q) g[q] = 0.0f;
     for (int64_t p = p0; p < p1; p += U) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) slot[u] = p + u < p1 ? __ldg(a.slots + p + u) : -1;
+      for (int u = 0; u < U; ++u) slot[u] = p + u < p1 ? __ldca(a.slots + p + u) : -1;
       add_pieces<K>(a.gpart, slot, d0, g);
     }
     update_vertex<LANES, BF16>(a, v, d0, g);

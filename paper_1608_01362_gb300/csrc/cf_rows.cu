@@ -97,11 +97,11 @@ int blocks_per_sm(int K) { return K == 16 ? Lanes<16>::kBlocks : Lanes<32>::kBlo
 
 template <int K, bool BF16, bool SSE>
 __global__ void __launch_bounds__(kRowThreads, Lanes<K>::kBlocks)
-cf_rows_kernel(const int4* __restrict__ recs, int32_t ntasks, int32_t nn,
-               const int32_t* __restrict__ nbr, const uint8_t* __restrict__ rate,
-               const void* __restrict__ self, const void* __restrict__ other,
-               float* __restrict__ gpart, double* __restrict__ partials,
-               unsigned* __restrict__ counter, double* __restrict__ sse_out) {
+cf_rows_kernel(const int4* recs, int32_t ntasks, int32_t nn,
+               const int32_t* nbr, const uint8_t* rate,
+               const void* self, const void* other,
+               float* gpart, double* partials,
+               unsigned* counter, double* sse_out) {
   constexpr unsigned kFull = 0xffffffffu;
   constexpr int LANES = Lanes<K>::n, EL = K / LANES, NP = EL / 2, G = 32 / LANES;
   constexpr int kRow = K * (BF16 ? 2 : 4), kPart = EL * (BF16 ? 2 : 4);
@@ -115,7 +115,7 @@ cf_rows_kernel(const int4* __restrict__ recs, int32_t ntasks, int32_t nn,
   for (int32_t task = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); task < ntasks;
        task += nw) {
     const int64_t slot = (int64_t)task * G + grp;
-    const int4 rec = __ldg(recs + slot);
+    const int4 rec = __ldca(recs + slot);
     const int64_t at = (int64_t)(((u64)(uint32_t)rec.y << 32) | (uint32_t)rec.x);
     const int len = rec.z;
     const int32_t* nb = nbr + at + sub;
@@ -128,12 +128,12 @@ cf_rows_kernel(const int4* __restrict__ recs, int32_t ntasks, int32_t nn,
     for (int q = 0; q < NP; ++q) g[q] = 0ull;
     uint32_t un = 0, rn = 0, um = 0, rm = 0;  // this chunk's rating and the next one's
     if (sub < len) {
-      un = (uint32_t)__ldg(nb);
-      rn = __ldg(rt);
+      un = (uint32_t)*nb;
+      rn = *rt;
     }
     if (sub + LANES < len) {
-      um = (uint32_t)__ldg(nb + LANES);
-      rm = __ldg(rt + LANES);
+      um = (uint32_t)nb[LANES];
+      rm = rt[LANES];
     }
     float te2 = 0.0f;
     const int longest = __shfl_sync(kFull, len, 0);
@@ -145,8 +145,8 @@ cf_rows_kernel(const int4* __restrict__ recs, int32_t ntasks, int32_t nn,
       un = um;
       rn = rm;
       if (c + 2 * LANES + sub < len) {
-        um = (uint32_t)__ldg(nb + c + 2 * LANES);
-        rm = __ldg(rt + c + 2 * LANES);
+        um = (uint32_t)nb[c + 2 * LANES];
+        rm = rt[c + 2 * LANES];
       }
 #pragma unroll
       for (int h = 0; h < LANES; h += 4) {  // four ratings of the group at a time

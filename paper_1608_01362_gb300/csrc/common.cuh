@@ -135,6 +135,10 @@ int radix_sort_pairs(const uint32_t* keys_in, const int32_t* vals_in,
 // (griddepcontrol.launch_dependents): its waiting blocks then hold registers
 // and shared memory, and with them L1, that the running kernel still wants
 // (1835 us at 1 M vertices; 27.1 ms instead of 19.1 at 32 M).
+// The blocks of such a kernel exist before the kernel in front of it has ended, so
+// nothing that they read counts as read-only for as long as they run: they take no
+// read-only-path load (__ldg, or what the compiler makes of a __restrict__
+// pointer), but plain ones (__ldca, __ldcs, __ldcg).
 // ---------------------------------------------------------------------------
 template <typename... P, typename... A>
 int launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem,
@@ -164,8 +168,7 @@ int wait_ticket(const unsigned long long* word, unsigned long long ticket, cudaS
 // Device helpers
 // ---------------------------------------------------------------------------
 // Always true, which only the machine knows: what stands behind
-// `if (!chain_begin()) return;` is not moved in front of it, not even a load
-// through the read-only path of what the kernel before has written.
+// `if (!chain_begin()) return;` is not moved in front of it.
 __device__ __forceinline__ bool chain_begin() {
   unsigned go;
   asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 1;" : "=r"(go)::"memory");

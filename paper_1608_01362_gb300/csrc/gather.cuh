@@ -51,9 +51,9 @@ struct MinI32 {
   static __device__ __forceinline__ void atomic_op(T* p, T v) { atomicMin(p, v); }
 };
 
-// Read-only random load of a gathered vertex value (L1-cached).
+// Random load of a gathered vertex value (L1-cached).
 template <typename T>
-__device__ __forceinline__ T ld_gather(const T* p) { return __ldg(p); }
+__device__ __forceinline__ T ld_gather(const T* p) { return __ldca(p); }
 
 __device__ __forceinline__ int pad32(int p) { return p + (p >> 5); }
 
@@ -97,11 +97,11 @@ __global__ void tile_partition_kernel(const RowEndT* __restrict__ row_end, int64
 // index); col: global source IDs; PROBE sends every gathered read to x[0].
 template <class Op, int THREADS, int IPT, bool PROBE, typename RowEndT>
 __global__ void __launch_bounds__(THREADS)
-gather_tile_kernel(const RowEndT* __restrict__ row_end, const int32_t* __restrict__ col,
-                   const typename Op::T* __restrict__ x, int32_t nx,
-                   const int32_t* __restrict__ tile_row, const int32_t* __restrict__ tile_edge,
-                   typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry,
-                   int32_t* __restrict__ carry_row) {
+gather_tile_kernel(const RowEndT* row_end, const int32_t* col,
+                   const typename Op::T* x, int32_t nx,
+                   const int32_t* tile_row, const int32_t* tile_edge,
+                   typename Op::T* out, typename Op::T* carry,
+                   int32_t* carry_row) {
   using T = typename Op::T;
   constexpr int TILE = THREADS * IPT;
   constexpr int WARPS = THREADS / 32;
@@ -234,9 +234,9 @@ gather_tile_kernel(const RowEndT* __restrict__ row_end, const int32_t* __restric
 // Fold the tile carries into the rows they belong to, in tile order: the
 // first tile of each run of tiles carrying the same row sums the run.
 template <class Op>
-__global__ void carry_fixup_kernel(const typename Op::T* __restrict__ carry,
-                                   const int32_t* __restrict__ carry_row, int64_t ntiles,
-                                   int64_t nrows, typename Op::T* __restrict__ out) {
+__global__ void carry_fixup_kernel(const typename Op::T* carry,
+                                   const int32_t* carry_row, int64_t ntiles,
+                                   int64_t nrows, typename Op::T* out) {
   using T = typename Op::T;
   if (!chain_begin()) return;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntiles;

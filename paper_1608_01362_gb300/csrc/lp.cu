@@ -14,9 +14,9 @@ namespace {
 // to *changed.  With a pin, the last block to finish (done) writes the sum and
 // the ticket there and clears both counters for the next pass.
 __global__ void __launch_bounds__(kMergeWarps * 32)
-lp_merge_update_kernel(const int32_t* __restrict__ blk, const int32_t* __restrict__ idx_map,
-                       const int32_t* __restrict__ interm, int k, int nb, int B, int32_t V,
-                       const int32_t* __restrict__ labels_in, int32_t* __restrict__ labels_out,
+lp_merge_update_kernel(const int32_t* blk, const int32_t* idx_map,
+                       const int32_t* interm, int k, int nb, int B, int32_t V,
+                       const int32_t* labels_in, int32_t* labels_out,
                        unsigned long long* changed, unsigned* done,
                        volatile unsigned long long* pin, unsigned long long ticket) {
   extern __shared__ int32_t lp_acc_all[];

@@ -20,8 +20,8 @@ namespace {
 
 // Cache-aware merge (Algorithm 4) fused with the vertex update.
 __global__ void __launch_bounds__(kMergeWarps * 32, 6)
-merge_update_kernel(const int32_t* __restrict__ blk, const int32_t* __restrict__ idx_map,
-                    const float* __restrict__ interm, int k, int nb, int B, PrArgs a) {
+merge_update_kernel(const int32_t* blk, const int32_t* idx_map,
+                    const float* interm, int k, int nb, int B, PrArgs a) {
   extern __shared__ float acc_all[];
   if (!chain_begin()) return;
   const double D = *a.D_in;
@@ -41,9 +41,9 @@ merge_update_kernel(const int32_t* __restrict__ blk, const int32_t* __restrict__
 // Generic merge (Algorithm 4 alone) with identity fill.
 template <class Op>
 __global__ void __launch_bounds__(kMergeWarps * 32)
-merge_only_kernel(const int32_t* __restrict__ blk, const int32_t* __restrict__ idx_map,
-                  const typename Op::T* __restrict__ interm, int k, int nb, int B, int32_t V,
-                  typename Op::T* __restrict__ out) {
+merge_only_kernel(const int32_t* blk, const int32_t* idx_map,
+                  const typename Op::T* interm, int k, int nb, int B, int32_t V,
+                  typename Op::T* out) {
   using T = typename Op::T;
   extern __shared__ unsigned char raw[];
   if (!chain_begin()) return;

@@ -68,7 +68,7 @@ __device__ __forceinline__ Row8 load_contrib(const void* c, uint32_t row, int la
                  : "=l"(x.p[0]), "=l"(x.p[1]), "=l"(x.p[2]), "=l"(x.p[3])
                  : "l"(p));
   } else {
-    const uint4 h = __ldg(static_cast<const uint4*>(c) + ((int64_t)row * 8 + lane8));
+    const uint4 h = __ldca(static_cast<const uint4*>(c) + ((int64_t)row * 8 + lane8));
     x.p[0] = pair(bf_lo(h.x), bf_hi(h.x));
     x.p[1] = pair(bf_lo(h.y), bf_hi(h.y));
     x.p[2] = pair(bf_lo(h.z), bf_hi(h.z));
@@ -134,14 +134,14 @@ __device__ __forceinline__ void store_contrib(void* c, int64_t v, int lane8, con
 // ---------------------------------------------------------------------------
 template <int PLANES>
 __global__ void __launch_bounds__(kThreads, kGatherBlocks)
-ppr_gather_kernel(const uint32_t* __restrict__ colf, const PprSeg* __restrict__ segs,
-                  const int2* __restrict__ chunks, int64_t nchunks, const void* __restrict__ contrib,
-                  float* __restrict__ interm, float* __restrict__ carry) {
+ppr_gather_kernel(const uint32_t* colf, const PprSeg* segs,
+                  const int2* chunks, int64_t nchunks, const void* contrib,
+                  float* interm, float* carry) {
   if (!chain_begin()) return;
   const int lane8 = threadIdx.x & 7;
   const int noct = (int)((gridDim.x * blockDim.x) >> 3);
   for (int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 3); c < (int)nchunks; c += noct) {
-    const int2 ch = __ldg(chunks + c);
+    const int2 ch = __ldca(chunks + c);
     const PprSeg sg = segs[ch.y];
     const int64_t el = (c - sg.chunk0) * kChunk;
     const int n = (int)min((int64_t)kChunk, (int64_t)sg.E - el);
@@ -149,7 +149,7 @@ ppr_gather_kernel(const uint32_t* __restrict__ colf, const PprSeg* __restrict__ 
     int32_t row = ch.x;
     Row8 acc = {{0, 0, 0, 0}};
     for (int g = 0; g < n; g += 4, ++cf) {
-      const uint4 f4 = __ldg(cf);  // the octet's lanes read the same four edges
+      const uint4 f4 = __ldca(cf);  // the octet's lanes read the same four edges
       const uint32_t f[4] = {f4.x, f4.y, f4.z, f4.w};
       if (g + 4 <= n && !((f4.x | f4.y | f4.z | f4.w) & kRowEnd)) {
 #pragma unroll
@@ -170,7 +170,7 @@ ppr_gather_kernel(const uint32_t* __restrict__ colf, const PprSeg* __restrict__ 
       }
     }
     // the row open at the chunk's end
-    if (!(__ldg(colf + sg.cstart + el + n - 1) & kRowEnd))
+    if (!(__ldca(colf + sg.cstart + el + n - 1) & kRowEnd))
       store_row(carry + (int64_t)c * kCols + lane8 * 8, acc);
   }
 }
@@ -210,17 +210,17 @@ __device__ __forceinline__ void sum_rows(const float* src, int n, float (&sum)[8
 // chain of reads, so pieces are short and their rows read four at a time (23.8
 // us with pieces of 32 read one by one, 10.1 so, at 122,657 chunks).
 __global__ void __launch_bounds__(kThreads)
-ppr_fixup_kernel(const int4* __restrict__ pieces, int64_t npieces, const int4* __restrict__ runs,
-                 const float* __restrict__ carry, float* __restrict__ piece_sum,
-                 unsigned* __restrict__ run_done, float* __restrict__ interm) {
+ppr_fixup_kernel(const int4* pieces, int64_t npieces, const int4* runs,
+                 const float* carry, float* piece_sum,
+                 unsigned* run_done, float* interm) {
   if (!chain_begin()) return;
   const int lane8 = threadIdx.x & 7;
   const unsigned omask = 0xffu << (threadIdx.x & 24);
   const int64_t noct = ((int64_t)gridDim.x * blockDim.x) >> 3;
   for (int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; p < npieces;
        p += noct) {
-    const int4 pc = __ldg(pieces + p);  // (first chunk, chunks, run)
-    const int4 rn = __ldg(runs + pc.z); // (row, first piece, pieces)
+    const int4 pc = __ldca(pieces + p);  // (first chunk, chunks, run)
+    const int4 rn = __ldca(runs + pc.z); // (row, first piece, pieces)
     float sum[8], x[8];
     sum_rows(carry + (int64_t)pc.x * kCols + lane8 * 8, pc.y, sum);
     float* dst = interm + (int64_t)rn.x * kCols + lane8 * 8;
@@ -310,14 +310,14 @@ ppr_merge_kernel(MergeArgs a) {
     const int64_t v0 = min((t0 + oct) * kTask, (int64_t)a.V);
     const int nv = (int)min((int64_t)kTask, (int64_t)a.V - v0);
     // row-list offsets, first rows and reciprocal degrees of the destinations
-    const int32_t off_a = __ldg(a.dst_off + v0 + min(lane8, nv));
-    const int32_t off_b = __ldg(a.dst_off + v0 + min(8 + lane8, nv));
-    const float inv_a = lane8 < nv ? __ldg(a.inv + v0 + lane8) : 0.0f;
-    const float inv_b = 8 + lane8 < nv ? __ldg(a.inv + v0 + 8 + lane8) : 0.0f;
-    const uint32_t sbits = nv > 0 ? __ldg(a.seed_bits + (v0 >> 5)) >> (v0 & 31) : 0u;
-    const int32_t o_end = __ldg(a.dst_off + v0 + nv);
-    const int32_t row_a = off_a < o_end ? __ldg(a.dst_rows + off_a) : 0;
-    const int32_t row_b = off_b < o_end ? __ldg(a.dst_rows + off_b) : 0;
+    const int32_t off_a = __ldca(a.dst_off + v0 + min(lane8, nv));
+    const int32_t off_b = __ldca(a.dst_off + v0 + min(8 + lane8, nv));
+    const float inv_a = lane8 < nv ? __ldca(a.inv + v0 + lane8) : 0.0f;
+    const float inv_b = 8 + lane8 < nv ? __ldca(a.inv + v0 + 8 + lane8) : 0.0f;
+    const uint32_t sbits = nv > 0 ? __ldca(a.seed_bits + (v0 >> 5)) >> (v0 & 31) : 0u;
+    const int32_t o_end = __ldca(a.dst_off + v0 + nv);
+    const int32_t row_a = off_a < o_end ? __ldca(a.dst_rows + off_a) : 0;
+    const int32_t row_b = off_b < o_end ? __ldca(a.dst_rows + off_b) : 0;
     float dpart[8], rpart[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) dpart[q] = rpart[q] = 0.0f;
@@ -345,7 +345,7 @@ ppr_merge_kernel(MergeArgs a) {
       const float iv = __shfl_sync(0xffffffffu, j < 8 ? inv_a : inv_b, j & 7, 8);
       if (j >= nv) continue;
       for (int32_t p = p0; p < p1; p += 2) {
-        const int32_t r0 = __ldg(a.dst_rows + p), r1 = p + 1 < p1 ? __ldg(a.dst_rows + p + 1) : 0;
+        const int32_t r0 = __ldca(a.dst_rows + p), r1 = p + 1 < p1 ? __ldca(a.dst_rows + p + 1) : 0;
         const Row8 x = load_row(a.interm + (int64_t)r0 * kCols + lane8 * 8);
         Row8 y = {{0, 0, 0, 0}};
         if (p + 1 < p1) y = load_row(a.interm + (int64_t)r1 * kCols + lane8 * 8);

@@ -65,13 +65,13 @@ __device__ __forceinline__ bool next_range(const RangeShare& sh, int nt, RangeSl
 }
 
 // Which of m segments holds task t (first[q]: segment q's first task, ascending).
-__device__ __forceinline__ int segment_of_task(const int32_t* __restrict__ first, int m,
+__device__ __forceinline__ int segment_of_task(const int32_t* first, int m,
                                                int32_t t) {
   const int lane = threadIdx.x & 31;
   int s = 0;  // segments whose tasks all precede t
   for (int i = 0; i < m; i += 32) {
     const unsigned bal =
-        __ballot_sync(0xffffffffu, i + lane < m && __ldg(first + i + lane + 1) <= t);
+        __ballot_sync(0xffffffffu, i + lane < m && __ldca(first + i + lane + 1) <= t);
     s += __popc(bal);
     if (bal != 0xffffffffu) break;
   }

@@ -17,8 +17,12 @@ namespace cg {
 
 // OffT is the stored offset type, PosT holds an edge's place: 32 bits below 2^31
 // edges (rows that begin behind the last edge walked are taken to begin there).
-template <typename OffT, typename PosT = int32_t>
+// CHAINED: for kernels that are launched chained.
+template <typename OffT, typename PosT = int32_t, bool CHAINED = false>
 struct RowWalk {
+  static __device__ __forceinline__ OffT load(const OffT* p) {
+    return CHAINED ? __ldca(p) : __ldg(p);
+  }
   const OffT* off;  // off[r] - origin: first edge of row r < n
   int32_t n;        // rows
   PosT total;       // edges walked, the end of row n - 1
@@ -33,7 +37,7 @@ struct RowWalk {
 
   __device__ __forceinline__ PosT first_of(int64_t r) const {
     if (r >= n) return total;
-    const OffT at = __ldg(off + r) - (OffT)origin;
+    const OffT at = load(off + r) - (OffT)origin;
     return at < (OffT)total ? (PosT)at : total;
   }
   __device__ __forceinline__ void window(int32_t r) {
@@ -59,7 +63,7 @@ struct RowWalk {
       // probes lo + step, lo + 2 step, ... (unsigned: hi - lo goes up to 2^31 - 1)
       const int32_t step = (int32_t)(((uint32_t)(hi - lo) + 32u) / 33u);
       const int64_t p = (int64_t)lo + (int64_t)step * (lane + 1);
-      const bool le = p < hi && __ldg(off + p) - (OffT)origin <= (OffT)e;
+      const bool le = p < hi && load(off + p) - (OffT)origin <= (OffT)e;
       const int c = __popc(__ballot_sync(0xffffffffu, le));
       const int64_t nh = (int64_t)lo + (int64_t)step * (c + 1);
       lo += step * c;
@@ -108,7 +112,7 @@ struct RowWalk {
 // the window's ends, and a lane's row is a population count away: about 15
 // instructions per 32 edges, no search.
 struct DenseWalk {
-  RowWalk<int32_t> w;
+  RowWalk<int32_t, int32_t, true> w;
   int32_t row;    // row of the next batch's first edge
 
   __device__ __forceinline__ DenseWalk(const int32_t* pos, int32_t rows, int32_t edges,

@@ -12,8 +12,8 @@ constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;
 
 template <typename TI>
-__global__ void tile_reduce_kernel(const TI* __restrict__ in, int64_t n,
-                                   int64_t* __restrict__ sums) {
+__global__ void tile_reduce_kernel(const TI* in, int64_t n,
+                                   int64_t* sums) {
   if (!chain_begin()) return;
   __shared__ int64_t sh[32];
   const int64_t base = (int64_t)blockIdx.x * kScanTile;
@@ -31,9 +31,9 @@ __global__ void tile_reduce_kernel(const TI* __restrict__ in, int64_t n,
 // consecutive items.  tile_off: exclusive offsets of the tiles (or NULL for a
 // single tile).  out[n] receives the grand total (written by the last tile).
 template <typename TI>
-__global__ void tile_scan_kernel(const TI* __restrict__ in, int64_t n,
-                                 const int64_t* __restrict__ tile_off,
-                                 int64_t* __restrict__ out) {
+__global__ void tile_scan_kernel(const TI* in, int64_t n,
+                                 const int64_t* tile_off,
+                                 int64_t* out) {
   if (!chain_begin()) return;
   __shared__ int64_t warp_tot[kScanThreads / 32];
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
@@ -100,8 +100,8 @@ constexpr int kSortRounds = 16;                       // items per thread
 constexpr int kSortTile = kSortThreads * kSortRounds;  // 4096
 constexpr int kSortWarps = kSortThreads / 32;
 
-__global__ void radix_hist_kernel(const uint32_t* __restrict__ keys, int64_t n, int shift,
-                                  int32_t* __restrict__ counts, int64_t ntiles) {
+__global__ void radix_hist_kernel(const uint32_t* keys, int64_t n, int shift,
+                                  int32_t* counts, int64_t ntiles) {
   if (!chain_begin()) return;
   __shared__ int32_t h[256];
   for (int i = threadIdx.x; i < 256; i += kSortThreads) h[i] = 0;
@@ -120,10 +120,10 @@ __global__ void radix_hist_kernel(const uint32_t* __restrict__ keys, int64_t n, 
 // Stable scatter of one tile: warp w owns items [w*512, w*512+512) of the
 // tile, visited in rounds of 32 consecutive items, so (warp, round, lane)
 // order is the input order.  Equal digits are ranked with __match_any_sync.
-__global__ void radix_scatter_kernel(const uint32_t* __restrict__ kin,
-                                     const int32_t* __restrict__ vin, int64_t n, int shift,
-                                     const int64_t* __restrict__ offs, int64_t ntiles,
-                                     uint32_t* __restrict__ kout, int32_t* __restrict__ vout) {
+__global__ void radix_scatter_kernel(const uint32_t* kin,
+                                     const int32_t* vin, int64_t n, int shift,
+                                     const int64_t* offs, int64_t ntiles,
+                                     uint32_t* kout, int32_t* vout) {
   if (!chain_begin()) return;
   __shared__ int32_t wc[kSortWarps][256];
   for (int i = threadIdx.x; i < kSortWarps * 256; i += kSortThreads) (&wc[0][0])[i] = 0;
@@ -135,11 +135,14 @@ __global__ void radix_scatter_kernel(const uint32_t* __restrict__ kin,
   int32_t v[kSortRounds];
   int32_t lr[kSortRounds];
 #pragma unroll
-  for (int r = 0; r < kSortRounds; ++r) {
+  for (int r = 0; r < kSortRounds; ++r) {  // all reads first: none moves over a barrier
     const int64_t i = base + r * 32 + lane;
-    const bool ok = i < n;
-    k[r] = ok ? kin[i] : 0u;
-    v[r] = ok ? vin[i] : 0;
+    k[r] = i < n ? kin[i] : 0u;
+    v[r] = i < n ? vin[i] : 0;
+  }
+#pragma unroll
+  for (int r = 0; r < kSortRounds; ++r) {
+    const bool ok = base + r * 32 + lane < n;
     const unsigned d = (k[r] >> shift) & 255u;
     const unsigned key = ok ? d : (0x100u | (unsigned)lane);  // unique for idle lanes
     const unsigned peers = __match_any_sync(0xffffffffu, key);
@@ -158,14 +161,18 @@ __global__ void radix_scatter_kernel(const uint32_t* __restrict__ kin,
     }
   }
   __syncthreads();
+  int64_t pos[kSortRounds];  // (and none over the stores below)
 #pragma unroll
   for (int r = 0; r < kSortRounds; ++r) {
-    const int64_t i = base + r * 32 + lane;
-    if (i < n) {
-      const unsigned d = (k[r] >> shift) & 255u;
-      const int64_t pos = offs[(int64_t)d * ntiles + blockIdx.x] + wc[w][d] + lr[r];
-      kout[pos] = k[r];
-      vout[pos] = v[r];
+    const unsigned d = (k[r] >> shift) & 255u;
+    pos[r] = base + r * 32 + lane < n
+                 ? offs[(int64_t)d * ntiles + blockIdx.x] + wc[w][d] + lr[r] : -1;
+  }
+#pragma unroll
+  for (int r = 0; r < kSortRounds; ++r) {
+    if (pos[r] >= 0) {
+      kout[pos[r]] = k[r];
+      vout[pos[r]] = v[r];
     }
   }
 }

@@ -59,8 +59,8 @@ __global__ void open_row_kernel(const int32_t* __restrict__ rp,
 
 template <class Op>
 __global__ void __launch_bounds__(256)
-seg_fixup_kernel(const int32_t* __restrict__ carry_row, const typename Op::T* __restrict__ carry,
-                 int64_t n, typename Op::T* __restrict__ out) {
+seg_fixup_kernel(const int32_t* carry_row, const typename Op::T* carry,
+                 int64_t n, typename Op::T* out) {
   if (!chain_begin()) return;
   fix_runs<Op>(carry_row, carry, n, out);
 }
@@ -93,8 +93,8 @@ __global__ void first_row_kernel(const int32_t* __restrict__ rp,
 constexpr int64_t kFewCachedEdges = (int64_t)1 << 24;
 
 template <class Op, int IPL>
-__device__ __forceinline__ void cached_chunk(const uint32_t* __restrict__ colf,
-                                             const typename Op::T* __restrict__ x, int32_t nx,
+__device__ __forceinline__ void cached_chunk(const uint32_t* colf,
+                                             const typename Op::T* x, int32_t nx,
                                              int32_t lo, int32_t Es, int32_t cstart, int32_t j,
                                              int32_t c, int32_t frow,
                                              typename Op::T* __restrict__ out,
@@ -121,7 +121,7 @@ __device__ __forceinline__ void cached_chunk(const uint32_t* __restrict__ colf,
     const bool ok = u < nl;
     const int32_t src = lo + (int32_t)(cf[u] & ~kRowEndFlag);
     if (ok) fl |= (cf[u] >> 31) << u;
-    v[u] = (ok && (uint32_t)src < (uint32_t)nx) ? __ldg(x + src) : Op::identity();
+    v[u] = (ok && (uint32_t)src < (uint32_t)nx) ? __ldca(x + src) : Op::identity();
   }
 
   // 2. rows ended before this lane (exclusive warp prefix of flag counts)
@@ -175,12 +175,12 @@ __device__ __forceinline__ void cached_chunk(const uint32_t* __restrict__ colf,
 // groups in order, which balances blocks when the cost per group varies).
 template <class Op, int THREADS, int IPL>
 __global__ void __launch_bounds__(THREADS, 2048 / THREADS)
-seg_gather_kernel(const uint32_t* __restrict__ colf, const typename Op::T* __restrict__ x,
-                  int32_t nx, const int32_t* __restrict__ first_row,
-                  const int64_t* __restrict__ seg_cstart, const int32_t* __restrict__ seg_E,
-                  const int64_t* __restrict__ seg_chunk, const int32_t* __restrict__ seg_ctile,
-                  const int32_t* __restrict__ seg_lo, int k, int32_t ct_begin, int32_t ct_end,
-                  typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
+seg_gather_kernel(const uint32_t* colf, const typename Op::T* x,
+                  int32_t nx, const int32_t* first_row,
+                  const int64_t* seg_cstart, const int32_t* seg_E,
+                  const int64_t* seg_chunk, const int32_t* seg_ctile,
+                  const int32_t* seg_lo, int k, int32_t ct_begin, int32_t ct_end,
+                  typename Op::T* out, typename Op::T* carry) {
   constexpr int WARPS = THREADS / 32;
   if (!chain_begin()) return;
   const int w = threadIdx.x >> 5;
@@ -220,7 +220,7 @@ seg_gather_kernel(const uint32_t* __restrict__ colf, const typename Op::T* __res
 // flight at once and pass no register), 4-byte ones otherwise.  The caller's
 // next barrier publishes the table.
 template <typename T>
-__device__ __forceinline__ void stage_table(const T* __restrict__ src, int n, T* dst, int tid,
+__device__ __forceinline__ void stage_table(const T* src, int n, T* dst, int tid,
                                             int nt) {
   static_assert(sizeof(T) == 4, "4-byte values");
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
@@ -253,7 +253,7 @@ struct StagedShare {
 // reads at 64 bytes per cycle and SM, and two barriers per piece.)
 template <class Op>
 __device__ __forceinline__ void staged_pieces(
-    const StagedTasks& q, const StagedShare& sh, const typename Op::T* __restrict__ x,
+    const StagedTasks& q, const StagedShare& sh, const typename Op::T* x,
     typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry, typename Op::T* tab,
     int nt, RangeSlots* slots) {
   using T = typename Op::T;
@@ -265,7 +265,7 @@ __device__ __forceinline__ void staged_pieces(
   while (next_range(sh.ranges, nt, slots, &v, &t, &hi)) {
     while (t < hi) {
       const int sn = segment_of_task(q.seg_task, sh.m, t);
-      const int32_t te = __ldg(q.seg_task + sn + 1);
+      const int32_t te = __ldca(q.seg_task + sn + 1);
       if (sn != s) {
         s = sn;
         group_sync(nt);  // every warp is done reading the previous table
@@ -298,8 +298,8 @@ __device__ __forceinline__ void counters_done(unsigned* counters, int n, unsigne
 // The staged launch: every thread of the block runs the staged schedule.
 template <class Op, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
-staged_gather_kernel(StagedTasks q, StagedShare sh, const typename Op::T* __restrict__ x,
-                     typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
+staged_gather_kernel(StagedTasks q, StagedShare sh, const typename Op::T* x,
+                     typename Op::T* out, typename Op::T* carry) {
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ RangeSlots slots;
@@ -317,10 +317,10 @@ staged_gather_kernel(StagedTasks q, StagedShare sh, const typename Op::T* __rest
 // instead of one per block.
 template <class Op>
 __global__ void __launch_bounds__(1024, 1)
-affine_gather_kernel(StagedTasks q, const typename Op::T* __restrict__ x,
-                     const int32_t* __restrict__ seg_lo, const int32_t* __restrict__ seg_tab,
-                     int m, int m2, unsigned* __restrict__ next_seg, unsigned* __restrict__ done,
-                     typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
+affine_gather_kernel(StagedTasks q, const typename Op::T* x,
+                     const int32_t* seg_lo, const int32_t* seg_tab,
+                     int m, int m2, unsigned* next_seg, unsigned* done,
+                     typename Op::T* out, typename Op::T* carry) {
   using T = typename Op::T;
   if (!chain_begin()) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -351,10 +351,10 @@ constexpr int kCachedGrab = 4;
 
 template <class Op, int IPL>
 __device__ __forceinline__ void cached_queue(
-    const uint32_t* __restrict__ colf, const typename Op::T* __restrict__ x, int32_t nx,
-    const int32_t* __restrict__ first_row, const int64_t* __restrict__ seg_cstart,
-    const int32_t* __restrict__ seg_E, const int64_t* __restrict__ seg_chunk,
-    const int32_t* __restrict__ seg_lo, int m, int k, unsigned* __restrict__ next_chunk,
+    const uint32_t* colf, const typename Op::T* x, int32_t nx,
+    const int32_t* first_row, const int64_t* seg_cstart,
+    const int32_t* seg_E, const int64_t* seg_chunk,
+    const int32_t* seg_lo, int m, int k, unsigned* __restrict__ next_chunk,
     typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   const int lane = threadIdx.x & 31;
   const int32_t c_begin = (int32_t)seg_chunk[m], c_end = (int32_t)seg_chunk[k];
@@ -398,13 +398,13 @@ __device__ __forceinline__ void cached_queue(
 // shared memory, so the two kinds of lookup proceed side by side.
 template <class Op, int IPL>
 __global__ void __launch_bounds__(1024, 1)
-overlap_gather_kernel(StagedTasks q, StagedShare sh, const uint32_t* __restrict__ colf,
-                      const typename Op::T* __restrict__ x, int32_t nx,
-                      const int32_t* __restrict__ first_row,
-                      const int64_t* __restrict__ seg_cstart, const int32_t* __restrict__ seg_E,
-                      const int64_t* __restrict__ seg_chunk, const int32_t* __restrict__ seg_lo,
-                      int m, int k, int staged_threads, unsigned* __restrict__ next_chunk,
-                      typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
+overlap_gather_kernel(StagedTasks q, StagedShare sh, const uint32_t* colf,
+                      const typename Op::T* x, int32_t nx,
+                      const int32_t* first_row,
+                      const int64_t* seg_cstart, const int32_t* seg_E,
+                      const int64_t* seg_chunk, const int32_t* seg_lo,
+                      int m, int k, int staged_threads, unsigned* next_chunk,
+                      typename Op::T* out, typename Op::T* carry) {
   using T = typename Op::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ RangeSlots slots;

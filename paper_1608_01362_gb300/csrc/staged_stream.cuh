@@ -119,7 +119,7 @@ struct StagedTasks {
 };
 
 // A lane's first 8 words of a task (fewer where the task has fewer).
-__device__ __forceinline__ void load_words(const uint8_t* __restrict__ base, uint32_t word,
+__device__ __forceinline__ void load_words(const uint8_t* base, uint32_t word,
                                            uint32_t (&w)[8]) {
   const int lane = threadIdx.x & 31;
   const int nw = (int)((word >> 8) & 0xFFu);
@@ -137,7 +137,7 @@ __device__ __forceinline__ void load_words(const uint8_t* __restrict__ base, uin
 // A lane's R rows of L edges each; pp: the rows' positions.
 template <class Op, int L>
 __device__ __forceinline__ void short_rows_task(const uint32_t (&w)[8],
-                                                const uint8_t* __restrict__ pp,
+                                                const uint8_t* pp,
                                                 const typename Op::T* tab,
                                                 typename Op::T* __restrict__ out) {
   using T = typename Op::T;
@@ -184,7 +184,7 @@ __device__ __forceinline__ void fold_words(const uint32_t (&w)[8], const typenam
 // Rows on 2^lg adjacent lanes each, NW words per lane; pp: their positions.
 template <class Op, int NW>
 __device__ __forceinline__ void lane_rows_task(const uint32_t (&w)[8],
-                                               const uint8_t* __restrict__ pp, int lg,
+                                               const uint8_t* pp, int lg,
                                                const typename Op::T* tab,
                                                typename Op::T* __restrict__ out) {
   using T = typename Op::T;
@@ -199,7 +199,7 @@ __device__ __forceinline__ void lane_rows_task(const uint32_t (&w)[8],
 
 // One task (at base) whose first words are loaded.
 template <class Op>
-__device__ __forceinline__ void fold_task(const uint8_t* __restrict__ base, uint32_t word,
+__device__ __forceinline__ void fold_task(const uint8_t* base, uint32_t word,
                                           int32_t row, const uint32_t (&w)[8],
                                           const typename Op::T* tab,
                                           typename Op::T* __restrict__ out,
@@ -269,13 +269,13 @@ __device__ __forceinline__ void staged_run(const StagedTasks& q, int32_t t0, int
                                            typename Op::T* __restrict__ carry) {
   int32_t t = t0 + w;
   if (t >= t1) return;
-  uint4 d = __ldg(q.desc + t);
+  uint4 d = __ldca(q.desc + t);
   for (;;) {
     const uint8_t* base = q.cs + (size_t)d.x * 32;
     uint32_t c[8];
     load_words(base, d.y, c);
     const int32_t tn = t + warps;
-    const uint4 dn = __ldg(q.desc + min(tn, t1 - 1));
+    const uint4 dn = __ldca(q.desc + min(tn, t1 - 1));
     if (threadIdx.x == 0 && dn.x > d.x)
       prefetch_l2(base + kStreamAhead, min((dn.x - d.x) * 32, (uint32_t)kStreamAhead));
     fold_task<Op>(base, d.y, (int32_t)d.z, c, tab, out, carry);

@@ -53,9 +53,9 @@ __device__ __forceinline__ int nth_bit(unsigned m, int n) {
 }
 
 template <class Op>
-__device__ __forceinline__ void warp_merge(const int32_t* __restrict__ blk,
-                                           const int32_t* __restrict__ idx_map,
-                                           const typename Op::T* __restrict__ interm, int k,
+__device__ __forceinline__ void warp_merge(const int32_t* blk,
+                                           const int32_t* idx_map,
+                                           const typename Op::T* interm, int k,
                                            int nb, int64_t mb, int64_t v0, int n,
                                            typename Op::T* acc) {
   using T = typename Op::T;
@@ -69,8 +69,8 @@ __device__ __forceinline__ void warp_merge(const int32_t* __restrict__ blk,
     const int ls = s0 + lane;
     int32_t lo = 0, hi = 0;
     if (ls < k) {  // block-major: the lanes read consecutive words
-      lo = __ldg(blk + mb * k + ls);
-      hi = __ldg(blk + (mb + 1) * k + ls);
+      lo = __ldca(blk + mb * k + ls);
+      hi = __ldca(blk + (mb + 1) * k + ls);
     }
     // the segments that have rows, in order, one per lane: where their rows
     // begin in the flattened sequence, and the row there
@@ -255,7 +255,7 @@ __device__ __forceinline__ void block_finish(double dsum, double rsum, const PrA
 
 // Plain path: the gathered sums are already dense.
 __global__ void __launch_bounds__(kMergeWarps * 32)
-dense_update_kernel(const float* __restrict__ sums, int B, int nb, PrArgs a) {
+dense_update_kernel(const float* sums, int B, int nb, PrArgs a) {
   extern __shared__ float acc_all[];
   if (!chain_begin()) return;
   const double D = *a.D_in;
