@@ -587,8 +587,7 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   // chunks of the segments read through L1/L2
   int64_t cached = 0;
   for (int q = m2; q < k; ++q) cached += p->edge_base[q + 1] - p->edge_base[q];
-  p->cached_ipl = cached < kFewCachedEdges ? 4 : 8;
-  const int chunk_edges = 32 * p->cached_ipl;
+  const int cached_ipl = cached < kFewCachedEdges ? 4 : 8, chunk_edges = 32 * cached_ipl;
   std::vector<int64_t> chunk(k + 1, 0);
   std::vector<int32_t> ctile(k + 1, 0), tn(k > 0 ? k : 1, 0);
   for (int q = 0; q < k; ++q) {
@@ -597,6 +596,7 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
     tn[q] = q < m2 ? (int32_t)(p->src_bounds[q + 1] - p->src_bounds[q]) : 0;
   }
   const int64_t ncached = chunk[k];
+  p->ready = false;
   // the staged segments' tasks; the carries of their full pieces follow the chunks'
   CG_TRY(staged_build(p, m2, tab_cap, ncached, s));
   for (int q = 0; q < k; ++q)  // block-groups of the L1/L2 launch
@@ -619,6 +619,7 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
         p->carry_row);
     CG_LAUNCH_CHECK();
   }
+  p->cached_ipl = cached_ipl;
   p->threads = threads;
   p->ctas_per_sm = ctas_per_sm;
   p->tab_cap = tab_cap;
@@ -643,6 +644,7 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   p->grid_l2 = (int)std::max<int64_t>(
       1, std::min<int64_t>(p->n_ctiles, (int64_t)di.sm_count * 2));
   CG_CUDA(cudaStreamSynchronize(s));
+  p->ready = true;
   return CG_OK;
 }
 
@@ -718,6 +720,10 @@ static int launch_overlap(const SegPlan& p, const typename Op::T* x, int32_t nx,
 template <class Op>
 int run_seg_gather(const SegPlan& p, const typename Op::T* x, int32_t nx, typename Op::T* out,
                    cudaStream_t s, int phases) {
+  if (!p.ready) {
+    set_error("segmented gather: its last configuration failed; configure it again");
+    return CG_ERR_UNSUPPORTED;
+  }
   if (p.nchunks == 0) return CG_OK;
   using T = typename Op::T;
   if (p.overlap > 0) {  // both kinds in one launch, counted as the staged phase

@@ -65,6 +65,7 @@ struct SegPlan {
   int64_t ncarry = 0, carry_cap = 0;
   const int32_t* rp32 = nullptr;   // subgraph row starts (owned by the handle)
   std::vector<int64_t> h_cstart, src_bounds, edge_base, row_base;
+  bool ready = false;       // configured (false where a configuration failed half way)
   int threads = 1024;       // staged-segment launch shape
   int ctas_per_sm = 1;
   int tab_cap = 0;          // table entries of the staged launch (its largest segment)
@@ -98,7 +99,8 @@ int seg_plan_finish(SegPlan* p, const int32_t* rp32, int64_t rows,
                     const std::vector<int64_t>& row_base, cudaStream_t s);
 
 // Launch shape: threads per block (512 or 1024), blocks per SM, table size
-// (-1: the capacity; 0: none).  Synchronizes the stream.
+// (-1: the capacity; 0: none).  Synchronizes the stream.  CG_ERR_INVALID_ARG changes
+// nothing; after another error no gather runs until a configuration succeeds.
 int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertices,
                        cudaStream_t s);
 

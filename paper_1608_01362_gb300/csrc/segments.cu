@@ -570,7 +570,11 @@ int pr_set_gather_config(cg_segmented* g, int32_t threads, int32_t ctas_per_sm,
                          int32_t table_vertices, cudaStream_t stream) {
   CG_ARG(g != nullptr, "pr_set_gather_config: null handle");
   CG_ARG(table_vertices >= -1, "pr_set_gather_config: table_vertices must be >= -1");
-  return seg_plan_configure(&g->plan, threads, ctas_per_sm, table_vertices, stream);
+  const int t = g->plan.threads, c = g->plan.ctas_per_sm, tab = g->plan.table_request;
+  const int rc = seg_plan_configure(&g->plan, threads, ctas_per_sm, table_vertices, stream);
+  if (!g->plan.ready)  // it failed half way (memory): back to the previous one, if that goes
+    seg_plan_configure(&g->plan, t, c, tab, stream);
+  return rc;
 }
 
 int pr_set_gather_overlap(cg_segmented* g, int32_t cached_warps, cudaStream_t stream) {
