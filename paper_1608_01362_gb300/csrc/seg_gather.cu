@@ -343,11 +343,13 @@ affine_gather_kernel(StagedTasks q, const typename Op::T* x,
   counters_done(next_seg, 1, done);
 }
 
-// L1/L2 chunks of segments [m, k) taken from a queue (a global counter of
-// chunks, kCachedGrab at a time or one): a warp's successive grabs only move forward,
-// so its segment is found by stepping.  The grab's chunks are prefetched into
-// L2 (TMA) when it is taken.
-constexpr int kCachedGrab = 4;
+// L1/L2 chunks of segments [m, k) taken from a queue (a global counter of chunks,
+// kCachedGrab at a time): a warp's successive grabs only move forward, so its segment
+// is found by stepping.  Two at a time: with one the counter and the search cost (4
+// M vertices, 8 warps per block: 128 us, 119 so), with four the last grabs outlast
+// the rest (0.5 M, 4 warps: 40 us, 30 so).  Pulling a grab's edges into L2 when it is
+// taken was of no use (33 M, 2 warps: 1051 us with, 1014 without).
+constexpr int kCachedGrab = 2;
 
 template <class Op, int IPL>
 __device__ __forceinline__ void cached_queue(
@@ -358,24 +360,14 @@ __device__ __forceinline__ void cached_queue(
     typename Op::T* __restrict__ out, typename Op::T* __restrict__ carry) {
   const int lane = threadIdx.x & 31;
   const int32_t c_begin = (int32_t)seg_chunk[m], c_end = (int32_t)seg_chunk[k];
-  // one chunk at a time where there are few: with 80 per SM, four at a time, the
-  // last grabs outlast everything else (1 M vertices, 8 warps: 75 us, so 55)
-  const int grab = c_end - c_begin < (int32_t)gridDim.x * 512 ? 1 : kCachedGrab;
   int s = m;
   int32_t lo = 0, Es = 0, cstart = 0, cbase = 0, cnext = -1;
   for (;;) {
     int32_t c0 = 0;
-    if (lane == 0) c0 = (int32_t)atomicAdd(next_chunk, (unsigned)grab);
+    if (lane == 0) c0 = (int32_t)atomicAdd(next_chunk, (unsigned)kCachedGrab);
     c0 = __shfl_sync(0xffffffffu, c0, 0) + c_begin;
     if (c0 >= c_end) break;
-    const int32_t c1 = c0 + grab < c_end ? c0 + grab : c_end;
-    if (lane < c1 - c0) {  // lane u prefetches chunk c0 + u (1 KB of colf)
-      const int32_t cu = c0 + lane;
-      int su = s;
-      while (cu >= (int32_t)seg_chunk[su + 1]) ++su;
-      prefetch_l2(colf + seg_cstart[su] + (int64_t)(cu - (int32_t)seg_chunk[su]) * 32 * IPL,
-                  32 * IPL * 4);
-    }
+    const int32_t c1 = min(c0 + kCachedGrab, c_end);
     for (int32_t c = c0; c < c1; ++c) {
       if (c >= cnext) {
         while (c >= (int32_t)seg_chunk[s + 1]) ++s;
