@@ -57,12 +57,30 @@ __global__ void open_row_kernel(const int32_t* __restrict__ rp,
   }
 }
 
+template <class Op, bool TILES>
+__global__ void __launch_bounds__(256)
+seg_fixup_kernel(const int32_t* carry_row, const typename Op::T* carry, int64_t n,
+                 typename Op::T* out, const typename Op::T* tiles) {
+  if (!chain_begin()) return;
+  fix_runs<Op, TILES>(carry_row, carry, n, out, tiles);
+}
+
 template <class Op>
 __global__ void __launch_bounds__(256)
-seg_fixup_kernel(const int32_t* carry_row, const typename Op::T* carry,
-                 int64_t n, typename Op::T* out) {
+carry_tiles_kernel(const int32_t* carry_row, const typename Op::T* carry, int64_t n,
+                   typename Op::T* tiles) {
   if (!chain_begin()) return;
-  fix_runs<Op>(carry_row, carry, n, out);
+  carry_tile_sums<Op>(carry_row, carry, n, tiles);
+}
+
+// Does a row have all of kLongRun aligned carries?
+__global__ void long_runs_kernel(const int32_t* __restrict__ carry_row, int64_t n,
+                                 unsigned* __restrict__ found) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n / kLongRun;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t r = carry_row[t * kLongRun];
+    if (r >= 0 && carry_row[(t + 1) * kLongRun - 1] == r) *found = 1u;
+  }
 }
 
 // Subgraph row of each chunk's first edge (chunks of `size` edges; the staged
@@ -465,7 +483,7 @@ int seg_plan_alloc(int64_t E, int k, const std::vector<int64_t>& edge_base,
   DeviceInfo di{};
   CG_TRY(device_info(&di));
   const size_t n = (size_t)k + 1, most = (size_t)di.sm_count * 2;  // blocks of any staged shape
-  const size_t words = 2 * 4 * n + 2 * n + 2 * n + 3 * n + (4 + most) + (most + 1);
+  const size_t words = 2 * 4 * n + 2 * n + 2 * n + 3 * n + (4 + most) + (most + 1) + 1;
   CG_CUDA(cudaMalloc((void**)&p->meta, 4 * words));
   int32_t* w = reinterpret_cast<int32_t*>(p->meta) + 2 * 4 * n;
   p->seg_cstart = p->meta + 2 * n;
@@ -478,6 +496,7 @@ int seg_plan_alloc(int64_t E, int k, const std::vector<int64_t>& edge_base,
   p->seg_task = w + 4 * n;
   p->counter = reinterpret_cast<unsigned*>(w + 5 * n);
   p->blk_task = w + 5 * n + 4 + most;
+  p->found = reinterpret_cast<unsigned*>(p->blk_task + most + 1);
   CG_CUDA(cudaMemsetAsync(p->counter, 0, 4 * ((4 + most) + (most + 1)), s));  // and the shares
   std::vector<int64_t> up(4 * n, 0);  // edge_base, cstart, bounds, then seg_E and seg_lo
   int32_t* eo = reinterpret_cast<int32_t*>(up.data() + 3 * n);
@@ -611,6 +630,14 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
         p->carry_row);
     CG_LAUNCH_CHECK();
   }
+  unsigned long_runs = 0;
+  if (p->ncarry >= kLongRun) {
+    CG_CUDA(cudaMemsetAsync(p->found, 0, sizeof(unsigned), s));
+    long_runs_kernel<<<grid_for(p->ncarry / kLongRun, 256), 256, 0, s>>>(p->carry_row, p->ncarry,
+                                                                         p->found);
+    CG_LAUNCH_CHECK();
+    CG_CUDA(cudaMemcpyAsync(&long_runs, p->found, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+  }
   p->cached_ipl = cached_ipl;
   p->threads = threads;
   p->ctas_per_sm = ctas_per_sm;
@@ -636,6 +663,7 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   p->grid_l2 = (int)std::max<int64_t>(
       1, std::min<int64_t>(p->n_ctiles, (int64_t)di.sm_count * 2));
   CG_CUDA(cudaStreamSynchronize(s));
+  p->long_runs = long_runs != 0;
   p->ready = true;
   return CG_OK;
 }
@@ -646,9 +674,10 @@ int seg_plan_carries(SegPlan* p, int64_t n) {
   cudaFree(p->first_row);
   p->first_row = nullptr;
   p->carry_cap = 0;
-  CG_CUDA(cudaMalloc((void**)&p->first_row, 3 * sizeof(int32_t) * (size_t)n));
+  CG_CUDA(cudaMalloc((void**)&p->first_row, sizeof(int32_t) * (size_t)(3 * n + n / kCarryTile)));
   p->carry_row = p->first_row + n;
   p->carry = p->first_row + 2 * n;
+  p->carry_tiles = p->first_row + 3 * n;
   p->carry_cap = n;
   return CG_OK;
 }
@@ -744,8 +773,14 @@ int run_seg_gather(const SegPlan& p, const typename Op::T* x, int32_t nx, typena
                           p.k, 0, (int32_t)p.n_ctiles, out, reinterpret_cast<T*>(p.carry)));
   }
   if ((phases & kPhaseFixup) && p.ncarry > 0) {
-    CG_TRY(launch_chained(seg_fixup_kernel<Op>, grid_for(p.ncarry, 256, 8), 256, 0, s, p.carry_row,
-                          reinterpret_cast<const T*>(p.carry), p.ncarry, out));
+    const T* carry = reinterpret_cast<const T*>(p.carry);
+    T* tiles = reinterpret_cast<T*>(p.carry_tiles);
+    if (p.long_runs)
+      CG_TRY(launch_chained(carry_tiles_kernel<Op>, grid_for(p.ncarry / kCarryTile * 32, 256, 8),
+                            256, 0, s, p.carry_row, carry, p.ncarry, tiles));
+    auto fn = p.long_runs ? seg_fixup_kernel<Op, true> : seg_fixup_kernel<Op, false>;
+    CG_TRY(launch_chained(fn, grid_for(p.ncarry, 256, 8), 256, 0, s, p.carry_row, carry, p.ncarry,
+                          out, tiles));
   }
   return CG_OK;
 }

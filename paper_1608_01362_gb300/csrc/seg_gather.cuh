@@ -62,7 +62,9 @@ struct SegPlan {
   int32_t* first_row = nullptr;    // subgraph row of each L1/L2 chunk's first edge
   int32_t* carry_row = nullptr;    // [ncarry] the row a carry belongs to (-1: none)
   void* carry = nullptr;           // [ncarry] 4-byte values
+  void* carry_tiles = nullptr;     // [ncarry / 256] sums of them, for plans with long_runs
   int64_t ncarry = 0, carry_cap = 0;
+  bool long_runs = false;          // a row has hundreds of carries (carry_runs.cuh)
   const int32_t* rp32 = nullptr;   // subgraph row starts (owned by the handle)
   std::vector<int64_t> h_cstart, src_bounds, edge_base, row_base;
   bool ready = false;       // configured (false where a configuration failed half way)
@@ -81,6 +83,7 @@ struct SegPlan {
   unsigned* counter = nullptr;  // next L1/L2 chunk (overlap), next segment-affine segment, blocks
                                 // finished of either, tasks taken of each staged block's range;
                                 // zero between launches (the last block of each clears them)
+  unsigned* found = nullptr;    // a word for the configuration
   int overlap_request = 0;  // warps per block given to the L1/L2 segments (0: two launches)
   int overlap = 0;          // the same, in effect (0 when one kind of segment is absent)
   int grid_l2 = 0;          // unstaged launch blocks (1024 threads, 2 per SM)
