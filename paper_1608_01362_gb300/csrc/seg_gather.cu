@@ -535,6 +535,44 @@ static int allow_tables() {
   return CG_OK;
 }
 
+// The staged segments' tasks, the L1/L2 segments' chunks and the carries of both.
+static int layout(SegPlan* p, int m2, int pad, int chunk_edges, const std::vector<int64_t>& chunk,
+                  const std::vector<int32_t>& ctile, const std::vector<int32_t>& tn,
+                  cudaStream_t s) {
+  const int k = p->k;
+  const int64_t ncached = chunk[k];
+  // the carries of the staged rows' full pieces follow the chunks'
+  CG_TRY(staged_build(p, m2, pad, ncached, s));
+  // seg_chunk, seg_ctile, seg_tab lie one behind the other
+  const size_t n = (size_t)k + 1;
+  std::vector<int32_t> up(4 * n, 0);
+  std::copy(chunk.begin(), chunk.end(), reinterpret_cast<int64_t*>(up.data()));
+  std::copy(ctile.begin(), ctile.end(), up.begin() + 2 * n);
+  std::copy(tn.begin(), tn.begin() + k, up.begin() + 3 * n);
+  CG_CUDA(cudaMemcpyAsync(p->seg_chunk, up.data(), sizeof(int32_t) * up.size(),
+                          cudaMemcpyHostToDevice, s));
+  if (ncached > 0) {
+    first_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
+        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, chunk_edges, ncached, p->first_row);
+    CG_LAUNCH_CHECK();
+    open_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
+        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, chunk_edges, ncached,
+        p->carry_row);
+    CG_LAUNCH_CHECK();
+  }
+  unsigned long_runs = 0;
+  if (p->ncarry >= kLongRun) {
+    CG_CUDA(cudaMemsetAsync(p->found, 0, sizeof(unsigned), s));
+    long_runs_kernel<<<grid_for(p->ncarry / kLongRun, 256), 256, 0, s>>>(p->carry_row, p->ncarry,
+                                                                         p->found);
+    CG_LAUNCH_CHECK();
+    CG_CUDA(cudaMemcpyAsync(&long_runs, p->found, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+    CG_CUDA(cudaStreamSynchronize(s));
+  }
+  p->long_runs = long_runs != 0;
+  return CG_OK;
+}
+
 int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertices,
                        cudaStream_t s) {
   CG_TRY(allow_tables<SumF32>());
@@ -607,38 +645,16 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
     tn[q] = q < m2 ? (int32_t)(p->src_bounds[q + 1] - p->src_bounds[q]) : 0;
   }
   const int64_t ncached = chunk[k];
-  p->ready = false;
-  // the staged segments' tasks; the carries of their full pieces follow the chunks'
-  CG_TRY(staged_build(p, m2, tab_cap, ncached, s));
   for (int q = 0; q < k; ++q)  // block-groups of the L1/L2 launch
     ctile[q + 1] = ctile[q] + (int32_t)ceil_div(chunk[q + 1] - chunk[q], warps_b);
-  {  // seg_chunk, seg_ctile, seg_tab lie one behind the other
-    const size_t n = (size_t)k + 1;
-    std::vector<int32_t> up(4 * n, 0);
-    std::copy(chunk.begin(), chunk.end(), reinterpret_cast<int64_t*>(up.data()));
-    std::copy(ctile.begin(), ctile.end(), up.begin() + 2 * n);
-    std::copy(tn.begin(), tn.begin() + k, up.begin() + 3 * n);
-    CG_CUDA(cudaMemcpyAsync(p->seg_chunk, up.data(), sizeof(int32_t) * up.size(),
-                            cudaMemcpyHostToDevice, s));
-  }
-  if (ncached > 0) {
-    first_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
-        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, chunk_edges, ncached, p->first_row);
-    CG_LAUNCH_CHECK();
-    open_row_kernel<<<grid_for(ncached, 256), 256, 0, s>>>(
-        p->rp32, p->meta, p->meta + (k + 1), p->seg_chunk, k, chunk_edges, ncached,
-        p->carry_row);
-    CG_LAUNCH_CHECK();
-  }
-  unsigned long_runs = 0;
-  if (p->ncarry >= kLongRun) {
-    CG_CUDA(cudaMemsetAsync(p->found, 0, sizeof(unsigned), s));
-    long_runs_kernel<<<grid_for(p->ncarry / kLongRun, 256), 256, 0, s>>>(p->carry_row, p->ncarry,
-                                                                         p->found);
-    CG_LAUNCH_CHECK();
-    CG_CUDA(cudaMemcpyAsync(&long_runs, p->found, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-  }
+  // tasks, chunks and carries stay where they come out as they are (another shape or
+  // overlap with the same segments staged)
+  const bool same = p->ready && p->m2 == m2 && p->tab_cap == tab_cap &&
+                    p->cached_ipl == cached_ipl && p->ncached == ncached;
+  p->ready = false;
+  if (!same) CG_TRY(layout(p, m2, tab_cap, chunk_edges, chunk, ctile, tn, s));
   p->cached_ipl = cached_ipl;
+  p->ncached = ncached;
   p->threads = threads;
   p->ctas_per_sm = ctas_per_sm;
   p->tab_cap = tab_cap;
@@ -663,7 +679,6 @@ int seg_plan_configure(SegPlan* p, int threads, int ctas_per_sm, int tab_vertice
   p->grid_l2 = (int)std::max<int64_t>(
       1, std::min<int64_t>(p->n_ctiles, (int64_t)di.sm_count * 2));
   CG_CUDA(cudaStreamSynchronize(s));
-  p->long_runs = long_runs != 0;
   p->ready = true;
   return CG_OK;
 }

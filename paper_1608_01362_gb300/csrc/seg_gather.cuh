@@ -77,6 +77,7 @@ struct SegPlan {
   double affine_head = 0.0;  // > 0: head threshold (edges per source) of the segment-affine
                             // plan; the table-sized segments after the head go one per block
   int cached_ipl = 8;          // edges per lane of an L1/L2 chunk
+  int64_t ncached = 0;         // L1/L2 chunks
   int grid_affine = 0;      // blocks of the segment-affine launch
   int64_t n_ctiles = 0;     // block-groups of the L1/L2 launch
   int grid = 0;             // staged launch blocks
