@@ -364,10 +364,7 @@ int codec_dispatch(cg_bipartite* h, const float* P, const float* Q, float* Pout,
 }
 
 void cf_free(cg_bipartite* h) {
-  for (int s = 0; s < 2; ++s) {
-    cf_pieces_free(&h->side[s]);
-    cudaFree(h->wide[s]);
-  }
+  for (int s = 0; s < 2; ++s) cf_pieces_free(&h->side[s]);  // with the lists
   cudaFree(h->P);  // with Q, the partials and the counter
   delete h;
 }
@@ -390,14 +387,13 @@ __global__ void many_pieces_kernel(const int64_t* __restrict__ poff, int64_t n, 
 int build_pieces(cg_bipartite* h, int side, cudaStream_t s) {
   const int64_t* off = side == 0 ? h->uoff : h->ioff;
   const int64_t n = side == 0 ? h->U : h->I;
-  CG_TRY(cf_pieces_build(&h->side[side], n, h->R, h->K, off, s));
+  CG_TRY(cf_pieces_build(&h->side[side], n, h->R, h->K, off, kCfWarp, s));
   const CfPieces& c = h->side[side];
   h->bytes += c.bytes;
   // vertices with many pieces get a warp or a whole block in the update
-  const int32_t cap = (int32_t)(c.npieces / kCfWarp + 1);
-  CG_CUDA(cudaMalloc((void**)&h->wide[side], sizeof(int32_t) * ((size_t)cap + 2)));
-  h->bytes += 4 * ((int64_t)cap + 2);
-  int32_t* count = h->wide[side] + cap;
+  const int32_t cap = c.most_many;
+  h->wide[side] = c.many;
+  int32_t* count = c.many + cap;
   CG_CUDA(cudaMemsetAsync(count, 0, 2 * sizeof(int32_t), s));
   if (n > 0) {
     many_pieces_kernel<<<grid_for(n, 256), 256, 0, s>>>(c.poff, n, cap, h->wide[side],

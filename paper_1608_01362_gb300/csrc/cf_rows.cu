@@ -287,7 +287,8 @@ int cf_rows_gather(const CfPieces& c, int K, bool bf16, int64_t nn, const int32_
   return run(c, nn, nbr, rate, self, other, with_sse, partials, counter, sse, grid, s);
 }
 
-int cf_pieces_build(CfPieces* c, int64_t n, int64_t R, int K, const int64_t* off, cudaStream_t s) {
+int cf_pieces_build(CfPieces* c, int64_t n, int64_t R, int K, const int64_t* off, int few,
+                    cudaStream_t s) {
   *c = CfPieces();
   int grid = 0;
   CG_TRY(cf_rows_grid(K, &grid));
@@ -314,14 +315,17 @@ int cf_pieces_build(CfPieces* c, int64_t n, int64_t R, int K, const int64_t* off
   const int64_t np = c->npieces;
   c->ntasks = (int32_t)ceil_div(np, G);
   const int64_t nslots = (int64_t)c->ntasks * G;
+  c->most_many = (int32_t)(np / few + 1);
   const size_t rb = Scratch::round(16 * (size_t)nslots), sb = Scratch::round(4 * (size_t)np),
-               pb = Scratch::round(8 * (size_t)(n + 1));
-  c->bytes = (int64_t)(rb + sb + pb) + 4 * nslots * K;
+               pb = Scratch::round(8 * (size_t)(n + 1)),
+               mb = Scratch::round(4 * ((size_t)c->most_many + 2));
+  c->bytes = (int64_t)(rb + sb + pb + mb) + 4 * nslots * K;
   CG_CUDA(cudaMalloc((void**)&c->slab, (size_t)c->bytes + 256));
   c->recs = reinterpret_cast<int4*>(c->slab);
   c->slots = reinterpret_cast<int32_t*>(c->slab + rb);
   c->poff = reinterpret_cast<int64_t*>(c->slab + rb + sb);
-  c->gpart = reinterpret_cast<float*>(c->slab + rb + sb + pb);
+  c->many = reinterpret_cast<int32_t*>(c->slab + rb + sb + pb);
+  c->gpart = reinterpret_cast<float*>(c->slab + rb + sb + pb + mb);
   CG_CUDA(cudaMemcpyAsync(c->poff, poff, 8 * (size_t)(n + 1), cudaMemcpyDeviceToDevice, s));
   // (an update before the first gather only decays the factors)
   CG_CUDA(cudaMemsetAsync(c->gpart, 0, 4 * (size_t)nslots * K, s));

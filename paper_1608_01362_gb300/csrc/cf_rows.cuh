@@ -17,12 +17,16 @@ struct CfPieces {
                                // word, ratings, vertex); unused: 0 ratings
   int32_t* slots = nullptr;    // [npieces] a vertex's pieces' slots, in rating order
   int64_t* poff = nullptr;     // [n+1] first piece of each vertex
+  int32_t* many = nullptr;     // [most_many + 2] a list of vertices with many pieces (cf.cu)
+  int32_t most_many = 0;
   float* gpart = nullptr;      // [slots][K] piece gradients
   int64_t bytes = 0;
 };
 
-// Lay out one side: n vertices with R ratings, K dimensions.  Synchronizes.
-int cf_pieces_build(CfPieces* c, int64_t n, int64_t R, int K, const int64_t* off, cudaStream_t s);
+// Lay out one side: n vertices with R ratings, K dimensions; room for a list of
+// vertices that have more than `few` pieces.  Synchronizes.
+int cf_pieces_build(CfPieces* c, int64_t n, int64_t R, int K, const int64_t* off, int few,
+                    cudaStream_t s);
 void cf_pieces_free(CfPieces* c);
 
 // Piece gradients of one side into c.gpart; with_sse (side 0): the squared
