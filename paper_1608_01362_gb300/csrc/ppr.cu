@@ -130,10 +130,12 @@ __device__ __forceinline__ void store_contrib(void* c, int64_t v, int lane8, con
 // instructions for four octets' edge, 32 of them unpacking.  Rows in flight
 // per octet beyond the one or two that fit in 40 registers, or more than 6
 // blocks per SM, cost (two rows at 5 blocks 316 us, 7 blocks 296): they evict
-// one another from L2 and the edge words from L1.
+// one another from L2 and the edge words from L1.  One plane's rows are half as
+// long and take 8 blocks (uniform graph of 1 M vertices and 16 M edges in 4 segments
+// 446 us, 477 with 6; RMAT of as many 227 and 226; 4 M uniform edges 129 and 198).
 // ---------------------------------------------------------------------------
 template <int PLANES>
-__global__ void __launch_bounds__(kThreads, kGatherBlocks)
+__global__ void __launch_bounds__(kThreads, kGatherBlocks[PLANES])
 ppr_gather_kernel(const uint32_t* colf, const PprSeg* segs,
                   const int2* chunks, int64_t nchunks, const void* contrib,
                   float* interm, float* carry) {

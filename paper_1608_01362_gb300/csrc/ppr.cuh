@@ -17,7 +17,7 @@ constexpr int kTask = 16;         // destinations per octet task in the merge
 constexpr int kThreads = 256;     // threads per block of every kernel here
 constexpr int kPprPiece = 16;     // chunks per piece of a run of carries
 constexpr int kMergeGroup = 32;   // merge blocks whose sums one block adds up
-constexpr int kGatherBlocks = 6;  // gather blocks per SM
+constexpr int kGatherBlocks[3] = {0, 8, 6};  // gather blocks per SM, by planes
 constexpr uint32_t kRowEnd = 0x80000000u;
 
 struct PprSeg {
