@@ -38,20 +38,21 @@ struct BatchPart {
   int32_t nstaged = 0;        // graphs that are not tiny
   int32_t vmax = 0, tmax = 0; // vertices of the largest of them and of the largest tiny one
   SegPlan plan;               // the graphs as staged segments: tasks, stream, carries
+  char* slab = nullptr;       // one allocation that holds the arrays up to sums
   int64_t* vbase = nullptr;   // [G+1] first vertex of each graph (from v0 on)
   int32_t* order = nullptr;   // [G] graphs by edge count, descending, the tiny ones last
   int32_t* ndang = nullptr;   // [G]
   int32_t* xbase = nullptr;   // [G+1] first carry of each graph
-  int32_t* row_ptr = nullptr; // [rows+1] first edge of each non-empty row
-  int32_t* idx = nullptr;     // [rows] local destination of each non-empty row
+  unsigned* counter = nullptr;
   float* inv = nullptr;       // [V]
   float* sums = nullptr;      // [V] row sums of graphs too large to keep them on chip
+  int32_t* row_ptr = nullptr; // [rows+1] first edge of each non-empty row
+  int32_t* idx = nullptr;     // [rows] local destination of each, in the same allocation
   longlong2* tiny = nullptr;  // [G] a tiny graph's first source and row start, (-1, -) for
                               // the others; NULL where there is no tiny one
   uint16_t* trow = nullptr;   // where the tiny graphs' rows begin among their sources (one
                               // entry more than rows), and these; same allocation as tiny
   uint8_t* tcol = nullptr;
-  unsigned* counter = nullptr;
   int64_t bytes = 0;
 };
 
@@ -506,16 +507,9 @@ batch_pagerank_kernel(const __grid_constant__ BatchArgs a) {
 
 void free_part(BatchPart* b) {
   seg_plan_free(&b->plan);
-  cudaFree(b->vbase);
-  cudaFree(b->order);
-  cudaFree(b->ndang);
-  cudaFree(b->xbase);
+  cudaFree(b->slab);
   cudaFree(b->row_ptr);
-  cudaFree(b->idx);
-  cudaFree(b->inv);
-  cudaFree(b->sums);
   cudaFree(b->tiny);
-  cudaFree(b->counter);
 }
 
 void free_batch(cg_batch* b) {
@@ -570,13 +564,16 @@ int build_part(BatchPart* b, const std::vector<int64_t>& vbase, const std::vecto
   SegPlan* p = &b->plan;
   const int64_t* d_sbase = p->meta + (G + 1);
   const int64_t* cstart = p->meta + 2 * (G + 1);
-  CG_CUDA(cudaMalloc((void**)&b->vbase, sizeof(int64_t) * (G + 1)));
-  CG_CUDA(cudaMalloc((void**)&b->order, sizeof(int32_t) * G));
-  CG_CUDA(cudaMalloc((void**)&b->ndang, sizeof(int32_t) * G));
-  CG_CUDA(cudaMalloc((void**)&b->xbase, sizeof(int32_t) * (G + 1)));
-  CG_CUDA(cudaMalloc((void**)&b->inv, sizeof(float) * (size_t)V));
-  CG_CUDA(cudaMalloc((void**)&b->sums, sizeof(float) * (size_t)V));
-  CG_CUDA(cudaMalloc((void**)&b->counter, sizeof(unsigned)));
+  const size_t g8 = Scratch::round(8 * (size_t)(G + 1)), g4 = Scratch::round(4 * (size_t)(G + 1)),
+               v4 = Scratch::round(4 * (size_t)V);
+  CG_CUDA(cudaMalloc((void**)&b->slab, g8 + 3 * g4 + 256 + 2 * v4));
+  b->vbase = reinterpret_cast<int64_t*>(b->slab);
+  b->order = reinterpret_cast<int32_t*>(b->slab + g8);
+  b->ndang = reinterpret_cast<int32_t*>(b->slab + g8 + g4);
+  b->xbase = reinterpret_cast<int32_t*>(b->slab + g8 + 2 * g4);
+  b->counter = reinterpret_cast<unsigned*>(b->slab + g8 + 3 * g4);
+  b->inv = reinterpret_cast<float*>(b->slab + g8 + 3 * g4 + 256);
+  b->sums = reinterpret_cast<float*>(b->slab + g8 + 3 * g4 + 256 + v4);
   CG_CUDA(cudaMemcpyAsync(b->vbase, vbase.data(), sizeof(int64_t) * (G + 1),
                           cudaMemcpyHostToDevice, s));
   CG_CUDA(cudaMemcpyAsync(b->order, order.data(), sizeof(int32_t) * G, cudaMemcpyHostToDevice, s));
@@ -627,8 +624,8 @@ int build_part(BatchPart* b, const std::vector<int64_t>& vbase, const std::vecto
     return CG_ERR_INVALID_ARG;
   }
   b->rows = rbase[G];
-  CG_CUDA(cudaMalloc((void**)&b->idx, sizeof(int32_t) * (size_t)(b->rows + 1)));
-  CG_CUDA(cudaMalloc((void**)&b->row_ptr, sizeof(int32_t) * (size_t)(b->rows + 1)));
+  CG_CUDA(cudaMalloc((void**)&b->row_ptr, sizeof(int32_t) * 2 * (size_t)(b->rows + 1)));
+  b->idx = b->row_ptr + b->rows + 1;
   const int32_t end = (int32_t)sbase[G];
   CG_CUDA(cudaMemcpyAsync(b->row_ptr + b->rows, &end, sizeof(int32_t), cudaMemcpyHostToDevice, s));
   batch_rows_kernel<<<grid_for(V * 32, 256, 16), 256, 0, s>>>(

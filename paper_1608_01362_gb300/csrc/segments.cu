@@ -26,7 +26,7 @@ namespace cg {
 namespace {
 
 constexpr int kMaxSegments = 1024;
-constexpr int32_t kFewDegrees = 1 << 14;  // see pr_plan_bounds
+constexpr int32_t kFewDegrees = 1 << 16;  // see pr_plan_bounds
 constexpr int kSplitThreads = 256;
 constexpr int kSplitWarps = kSplitThreads / 32;
 constexpr int kSplitRounds = 8;                               // edges per thread
@@ -628,8 +628,9 @@ int pr_plan_bounds(const int32_t* dev_outdeg, int32_t V, int32_t smem_vertices,
   // the out-edges of each table-sized range, and the end of the sources that have
   // any: on the device (copying the degrees to the host and adding them there took 4
   // ms of a 4 M-vertex graph's 21 ms from CSR to ranks), but from a copy of the
-  // degrees where these are so few that this is faster than scratch and a kernel
-  // (3,000 vertices: 23 us, 31 with the kernel; 20,000: 28 to 31 either way)
+  // degrees where these are few: scratch and a kernel take 31 us, but 80 where the
+  // pool has given its memory back (3,000 vertices from a copy 23 us, 30,000 33, 65,536
+  // 47)
   const int64_t nr = smem_vertices > 0 ? std::min<int64_t>(ceil_div(V, smem_vertices), k_max) : 0;
   std::vector<int64_t> sums(nr + 1, 0);
   if (V <= kFewDegrees) {
