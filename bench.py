@@ -511,8 +511,8 @@ def _ppr_bounds(nd, V, k):
 
 def run_ppr(args):
     """64 personalised PageRank vectors on a directed RMAT graph (default
-    scale 22), 20 iterations, rank matrix stored as BF16 hi+lo planes with
-    FP32 accumulation: one batched solve against 64 single-vector solves."""
+    scale 22), 20 iterations, rank matrix stored in 32 bits per value (FP32; two
+    planes) with FP32 accumulation: one batched solve against 64 single-vector solves."""
     import torch
     import __graft_entry__
     __graft_entry__.build()
@@ -668,7 +668,7 @@ def run_ppr(args):
     peak, peak_kind = _peaks()
     ach = alg[dom] / (phase_ms[dom] / 1e3) / 1e9
     edge_cols = g.E * 64 * ITERS
-    # the gather reads one 64-column row (BF16 hi+lo: 256 bytes) per edge from a
+    # the gather reads one 64-column row (FP32: 256 bytes) per edge from a
     # table of the non-dangling sources' rows; its ceiling is the random-row
     # rate of such a table (measured now); hub rows reread from L1/L2 can
     # carry it above that rate
@@ -679,10 +679,10 @@ def run_ppr(args):
                    "table_bytes": rb * nd, "achieved": a_rows, "peak": gp[(rb, rb * nd)],
                    "frac": a_rows / gp[(rb, rb * nd)]}
     line = {"metric": "batched personalised PageRank: edge-vector GTEPS (64 vectors x 20 "
-                      "iterations) at BF16 hi+lo storage",
+                      "iterations) at 32-bit storage",
             "value": edge_cols / t_step / 1e9, "unit": "GTEPS (edge x vector)", "n_gpus": 1,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": t_step * 1e3,
-            "higher_is_better": True, "dtype": "bf16x2 storage, f32 accumulate",
+            "higher_is_better": True, "dtype": "f32 storage, f32 accumulate",
             "data": "synthetic",
             "config": {"workload": f"ppr64_rmat{scale}_ef16", "V": g.V, "E": g.E,
                        "nondangling": nd, "segments": info["num_segments"], "q": info["q"],
@@ -718,8 +718,8 @@ def run_ppr(args):
 def run_cf(args):
     """Collaborative filtering on the Netflix-shaped bipartite graph (480,189
     users x 17,770 items x 99M ratings), K = 32, lambda 0.05, step 1e-3, 10
-    sweeps, factors stored in FP32, BF16 and BF16 hi+lo; RMSE per sweep
-    against the FP64 oracle on the same inputs."""
+    sweeps, factors stored in FP32, BF16 and as for a BF16 hi+lo request (FP32
+    too); RMSE per sweep against the FP64 oracle on the same inputs."""
     import torch
     import __graft_entry__
     __graft_entry__.build()
@@ -812,7 +812,7 @@ def run_cf(args):
     peak, peak_kind = _peaks()
     # algorithmic DRAM bytes per sweep: both rating CSRs (4 + 1 bytes per
     # rating each), offsets, and each factor row read and written once
-    # (BF16 hi+lo: 4 bytes per entry)
+    # (4 bytes per entry)
     alg = 2 * 5 * R + 8 * (U + I + 2) + 2 * (U + I) * K * 4
     dom = max(head["kernels_ms"], key=head["kernels_ms"].get)
     dom_bytes = 5 * R + (U + I) * K * 4
@@ -828,10 +828,10 @@ def run_cf(args):
                           "table_bytes": tb, "achieved": a, "peak": gp[(rb, tb)],
                           "frac": a / gp[(rb, tb)]}
     line = {"metric": "collaborative filtering sweep: ratings x sides per second (GTEPS), K=32, "
-                      "BF16 hi+lo storage, RMSE diff vs FP64",
+                      "32-bit storage, RMSE diff vs FP64",
             "value": 2 * R / t_sweep / 1e9, "unit": "GTEPS (rating x side)", "n_gpus": 1,
             "steps": SWEEPS, "warmup": args.warmup, "ms_per_step": t_sweep * 1e3,
-            "higher_is_better": True, "dtype": "bf16x2 storage, f32 accumulate",
+            "higher_is_better": True, "dtype": "f32 storage, f32 accumulate",
             "data": "synthetic",
             "config": {"workload": "cf_netflix_shaped_480189x17770_99M_K32", "U": U, "I": I,
                        "R": R, "K": K, "lambda": LAM, "step": STEP, "sweeps": SWEEPS,
@@ -1169,7 +1169,7 @@ def extras(g25, graph25):
     del lp, graph, g
     torch.cuda.empty_cache()
 
-    # 64-vector personalised PageRank (BF16 hi+lo) against 64 one-vector solves
+    # 64-vector personalised PageRank (32-bit storage) against 64 one-vector solves
     t0 = time.time()
     g = graphgen.rmat(22, 16, seed=1)
     graph = P.Graph(g.offsets, g.src, cluster_mode=0)
@@ -1237,7 +1237,8 @@ def extras(g25, graph25):
     del bp, handles, gb, gp, gs
     torch.cuda.empty_cache()
 
-    # collaborative filtering: 10 sweeps at BF16 hi+lo; two FP32 sweeps vs FP64
+    # collaborative filtering: 10 sweeps at a BF16 hi+lo request's storage (FP32);
+    # two FP32 sweeps vs FP64
     t0 = time.time()
     bpg = graphgen.bipartite(seed=1)
     dev = lambda a, dt: torch.as_tensor(np.ascontiguousarray(a), dtype=dt).cuda()  # noqa: E731
@@ -1286,7 +1287,7 @@ def extras(g25, graph25):
                                     iu, ir, Pw, Qw, 0.05, 1e-3)
     rel = float(np.max(np.abs(Pg.cpu().numpy() - Pw)) / np.max(np.abs(Pw)))
     out["cf_netflix_shaped_k32"] = {
-        "ms_per_sweep_bf16x2": t_cf * 1e3, "gteps_rating_sides": 2 * bpg.R / t_cf / 1e9,
+        "ms_per_sweep": t_cf * 1e3, "gteps_rating_sides": 2 * bpg.R / t_cf / 1e9,
         "fp32_sweeps_sampled_entries": 2 * 32 * (len(users) + len(items)),
         "fp32_sweeps_max_err_over_bound": worst, "fp32_sweeps_entries_outside_bound": outside,
         "fp32_two_sweeps_max_err_rel_to_max": rel, "fp32_drift_tolerance": 2e-6,

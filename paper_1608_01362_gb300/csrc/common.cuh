@@ -130,8 +130,8 @@ int radix_sort_pairs(const uint32_t* keys_in, const int32_t* vals_in,
 // calls before it reads or writes memory, then waits until that one's writes
 // are visible.  The order of execution is the stream's; what goes is the drain
 // and the launch between two kernels, 2-3 us of each of an iteration's two to
-// four (20 iterations at 20,011 vertices: 418 us without, 311 with; at 1 M:
-// 1393 and 1226).  The next kernel is not let in earlier than that
+// four (20 iterations at 20,011 vertices: 418 us without, 311 with; at 1 M 1393 and
+// 1226, when this came; 1083 with what has changed since).  The next kernel is not let in earlier than that
 // (griddepcontrol.launch_dependents): its waiting blocks then hold registers
 // and shared memory, and with them L1, that the running kernel still wants
 // (1835 us at 1 M vertices; 27.1 ms instead of 19.1 at 32 M).

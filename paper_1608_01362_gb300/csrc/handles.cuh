@@ -61,15 +61,18 @@ struct cg_plain {
 
 namespace cg {
 // Destinations per warp of the merge: the most, up to the caller's B and in
-// steps of 32, with which the warps make whole waves of 40 per SM (5 blocks).  One
-// warp's merge is a chain of dependent reads, so a small graph's time is that
-// chain, and a last wave that is nearly empty costs as much as a full one.  With
-// B = 512: 20,011 vertices merged on 5 of 152 SMs (11.0 us, 4.9 so), 300 K in 1.3
-// waves of 48 (20 iterations with the gathers 770 us, 661 so), 1 M 1198 and 1098, 4
-// M 2869 and 2762, 33 M in 9 waves of 48 or 11 of 40 (17.70 ms both).  A block of
-// hubs has rows in every one of the k segments: where that makes more than 3000
-// for one warp, up to three waves share them out (label propagation, 3 M
-// vertices, 9 segments: 1236 us in one wave, 1130 in two).
+// steps of 32, with which the warps make whole waves of 40 per SM.  One warp's merge
+// is a chain of dependent reads, so a small graph's time is that chain, and a last
+// wave that is nearly empty costs as much as a full one.  48 warps (6 blocks) fit;
+// counting on 40 was the best of 24, 32, 36, 40, 44 and 48 from 300 K to 33 M
+// vertices (20 iterations with 48 and 40: 300 K 770 and 661 us, 1 M 1167 and 1073, 4
+// M 2869 and 2762, 33 M 17.70 ms both), measured, not derived.  (The caller's B = 512
+// itself put 20,011 vertices on 5 of 152 SMs: 11.0 us, 4.9 so.)  A block of hubs has
+// rows in every one of the k segments: where that makes more than 3000 for one
+// warp, up to three waves share them out.  One merge without that, and with 6000,
+// 3000 and 1500: 1 M vertices, 40 segments 27.9, 16.8, 13.1, 13.0 us; 3 M, 9 segments
+// 28.6, 28.4, 17.0, 14.2; 3 M, 40 segments 74.5, 32.7, 32.8, 32.9; 4 M, 7 segments
+// 18.0, 18.4, 18.3, 15.1; 8 M the same with all.
 int32_t merge_block(int32_t V, int32_t B, int32_t k, int sm_count);
 
 // Validate an in-edge CSR on the device (offsets monotone from 0 to E, every

@@ -106,8 +106,10 @@ __global__ void first_row_kernel(const int32_t* __restrict__ rp,
 // One L1/L2 chunk: segment-local chunk j (global chunk c) of 32 * IPL edges of a
 // segment whose sources start at lo; lane l holds edges [IPL l, IPL (l + 1)).
 // Eight edges per lane, or four where there are few edges: chunks are then few
-// per warp, and a launch is a chain of two of them (0.3 M edges 10.3 -> 8.1 us,
-// 3.1 M 18.0 -> 16.3, 8.8 M 41.9 -> 40.0, 22 M 89.0 -> 91.0, 66 M 260 -> 268).
+// per warp, and a launch is a chain of two of them.  The line lies between the
+// largest size at which four were faster and the smallest at which eight were (0.3
+// M edges 10.3 -> 8.1 us with four, 3.1 M 18.0 -> 16.3, 8.8 M 41.9 -> 40.0, 13.4 M
+// 60.3 -> 57.6, 22 M 89.0 -> 91.0, 66 M 260 -> 268).
 constexpr int64_t kFewCachedEdges = (int64_t)1 << 24;
 
 template <class Op, int IPL>

@@ -6,25 +6,31 @@
 // one edge, so row i is the (i+1)-th flagged edge: the gather needs no row
 // pointers at all.
 //
-// Work unit of the segments read through L1/L2: a warp owns a chunk of 256
-// consecutive edges of one segment; lane l holds edges [8l, 8l + 8) of it
-// (16-byte streaming loads).  Lanes
-// fold their 8 values sequentially, emit every row that starts and ends
-// inside them, and a warp-wide segmented scan over the lanes' open-row parts
-// completes each lane's first row.  The row still open at the chunk's end
-// goes to carry[chunk], folded in afterwards in chunk order.  No shared
-// staging of edges and no block barriers between chunks.  The staged segments
-// have a layout of their own (staged_stream.cuh).
+// Work unit of the segments read through L1/L2: a warp owns a chunk of 128 or 256
+// consecutive edges of one segment (4 or 8 per lane, by the number of such edges);
+// lane l holds edges [IPL l, IPL (l + 1)) of it (16-byte streaming loads).  Lanes fold
+// their values sequentially, emit every row that starts and ends inside them, and a
+// warp-wide segmented scan over the lanes' open-row parts completes each lane's first
+// row.  The row still open at the chunk's end goes to carry[chunk], folded in
+// afterwards in chunk order.  No shared staging of edges and no block barriers
+// between chunks.  The staged segments' unit is the warp task of a layout of their
+// own (staged_stream.cuh).
 //
-// Two launches per pass.  The leading segments that fit an SM's shared
-// memory (after clustering, the hot head: the paper's cache-sized segment,
-// sized here to on-chip shared memory) are "staged": each block copies its
-// current segment's source values into shared memory and every read of the
-// segment is served from there.  The remaining segments are read through
-// L1/L2 by a second launch that uses no shared memory, leaving the whole
-// on-chip store to the L1 cache.  In both, a block owns a contiguous run of
-// block-sized groups of chunks (so it meets at most a few segments and
-// stages at most a few tables), in segment order.
+// Launches of a pass, each where there is something for it:
+//   staged    the leading segments that fit an SM's shared memory (after clustering,
+//             the hot head: the paper's cache-sized segment, sized here to on-chip
+//             shared memory): each block copies its current segment's source values
+//             into shared memory and every read of the segment is served from there.
+//             A block owns a contiguous range of tasks, which meets one or two
+//             segments, and helps with the fullest range when its own runs dry
+//             (ranges.cuh).
+//   affine    with the segment-affine plan: the table-sized segments behind the head,
+//             one block per segment, handed out by a counter.
+//   cached    the remaining segments, through L1/L2, without shared memory, which
+//             leaves the whole on-chip store to the L1 cache.  Blocks take block-sized
+//             groups of chunks round robin, in segment order.
+//   fix-up    rows that span chunks or full pieces (carry_runs.cuh).
+// With the overlap one launch serves the staged and the cached segments.
 #pragma once
 
 #include <vector>

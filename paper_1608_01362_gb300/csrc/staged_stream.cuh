@@ -33,8 +33,8 @@
 // 528.7 M edges 562 -> 394 us, 65.2 M edges 89 -> 63 us, 15.7 M edges 26.7 ->
 // 26.9 us (one table: its copy and the launch are a third of that).  On 130 M
 // edges 84 M -> 42 M instructions (ncu); what is left is bound by the shared-memory
-// pipe (3.3 wavefronts per random lookup, 56% of its peak over the launch) and by the latency
-// of a task's stream loads.  Loading the next task's words into registers first
+// pipe (3.9 wavefronts per random lookup, 64% of its peak over the launch of 264 M
+// edges in 19 segments) and by the latency of a task's stream loads.  Loading the next task's words into registers first
 // cost more instructions than it hid (423 us), the prefetch distance is flat
 // from 32 to 160 KB and worth 10% of the launch against none.
 #pragma once
