@@ -708,7 +708,7 @@ void seg_plan_free(SegPlan* p) {
 }
 
 int64_t seg_plan_bytes(const SegPlan& p) {
-  return 4 * p.colf_len + p.cs_cap + 12 * p.carry_cap +
+  return 4 * p.colf_len + p.cs_cap + 12 * p.carry_cap + 4 * (p.carry_cap / kCarryTile) +
          76 * (int64_t)p.k;
 }
 
